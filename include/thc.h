@@ -68,8 +68,8 @@ typedef enum {
  * and DIIS stay float64.  FP64_TC: float64 storage and arithmetic as FP64,
  * but the products of at least 3e7 flops (those a cost model of the two
  * paths does not keep on the CUDA cores) run on the tensor cores as exact
- * integer products of 8 slices of 7 bits per operand row (scaled by a power
- * of two per row), combined in float64: each product term is within about
+ * integer products of 7 slices of 8 bits per operand row (scaled by a power
+ * of two per row), combined in fixed point: each product term is within about
  * 1.2e-16 of its row and column scale, float64 rounding level; the triangle
  * (Alg. 6 line 11) runs in float pairs on the FP32 pipe, each term within
  * about 2^-45 of |E F G|.  Per-step choices: thc_config.policy. */
@@ -534,7 +534,7 @@ thc_status thc_probe_alu(int kind, double* tflops, void* stream);
  *   mode 1  the same with the bf16 hi/lo pack of both operands in every call
  *   mode 2  bf16 hi*hi only, packed operands cached
  *   mode 3  float64 operands as exact integer slices (THC_PREC_FP64_TC):
- *           row exponents, slicing, 8 level products and the float64 pass
+ *           row exponents, slicing, the fused product
  * *ms = milliseconds per product.  Allocates its operands and workspace.
  * Errors: THC_ERR_ARG, THC_ERR_OOM, THC_ERR_CUDA, THC_ERR_TIMEOUT.
  * Diagnostic; no counterpart in the paper.

@@ -165,9 +165,22 @@ __device__ __forceinline__ TileCoord tile_coord(const TcArgs& a, long long t, in
     return c;
 }
 
+// One test of a phase, without waiting (true: completed).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
 // Bounded wait that also gives up once another role has failed.
 __device__ __forceinline__ bool mbar_wait_or_fail(uint64_t* bar, uint32_t parity,
                                                   volatile int* fail) {
+    if (mbar_test(bar, parity)) return true;
     const uint32_t a = smem_u32(bar);
     const long long t0 = clock64();
     for (;;) {
@@ -755,27 +768,32 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
 }
 
 // ---------------------------------------------------------------------------
-// Float64 products on the tensor cores by exact integer slices (the splitting
+// Float64 products on the tensor cores by integer slices (the splitting
 // scheme of Ozaki et al.).  Every row r of an operand (UMMA orientation, K
 // along the row; in a batch-reduced product the row runs over all batches) is
 // scaled by 2^-e_r, e_r the binary exponent of its largest entry, so that its
-// entries lie in (-1, 1), and is cut into kSlices = 8 signed 7-bit integers:
-//   x = 2^e_r (sum_t a_t 2^(-7t) + r_x),   a_t in [-127, 127], |r_x| < 2^-56,
+// entries lie in (-1, 1), rounded to 55 fractional bits and cut into
+// kSlices = 7 balanced digits of 8 bits (7 bits for the first):
+//   x = 2^e_r (sum_t a_t 2^(1-8t) + r_x),   a_t in [-128, 128], |r_x| <= 2^-56,
 // read straight from the IEEE-754 fields (integer operations only).
-// A slice is exact in bf16, a product of two is an integer below 2^14, and a
-// float32 sum of at most 1024 of them is an integer below 2^24, so the tensor
-// cores' float32 accumulation over K chunks of 1024 is exact.  The pairs
-// (t, u) with t + u = l are one product over concatenated slices,
-//   S_l = [a_1 .. a_(l-1)] [b_(l-1) .. b_1]^T   (K of (l - 1) Ktot),
-// which is why A keeps its slices in order and B in reverse order along each
-// row.  The levels l = 2 .. 9 (36 pairs) are combined in float64 by Horner's
-// rule, sum_l 2^(-7l) S_l, and scaled by 2^(e_r + e_c).  The pairs left out
-// (l >= 10) and the remainders change each product term a_rk b_kc by less
-// than about 9 2^-56 = 1.2e-16 of 2^(e_r + e_c), the size of float64 rounding.
+// A slice is exact in bf16, a product of two is an integer of at most 2^14,
+// and a float32 sum of at most 1024 of them an integer of at most 2^24: the
+// tensor cores' float32 accumulation is exact.  The pairs (t, u) with
+// t + u = l form level l, S_l = sum a_t b_u, and
+//   C = 2^(e_r + e_c) sum_{l=2..8} 2^(2-8l) S_l   (28 pairs).
+// Balanced digits are why 28 pairs suffice: the digits left out (l >= 9) have
+// random signs and change a product term by about 2^-56 of 2^(e_r + e_c)
+// (rms), where 8 slices of 7 unsigned bits and 36 pairs, the form used before,
+// lost 2^-55 with the product's own sign.  Against 64-bit-mantissa sums over
+// K = 40, 400 and 4000 the error is 0.45 times the old one on Gaussian
+// entries and 0.47 to 0.57 times on entries spread over 2^-40 .. 1.  (Six
+// 9-bit digits and 26 pairs are as accurate, but products of such digits leave
+// room for 256 of them only, so that two levels would be drained in every K
+// step, where these digits drain one level every second step.)
 namespace {
 
-constexpr int kSlices = 8;
-constexpr int kLevels = kSlices;           // l = 2 .. kSlices + 1
+constexpr int kSlices = 7;
+constexpr int kLevels = 7;                 // l = 2 .. 8 (q = l - 2)
 
 // Biased exponent field of |x| (0 for zero; subnormals count as field 1).
 __device__ __forceinline__ int f64_field(double x) {
@@ -807,18 +825,18 @@ __device__ __forceinline__ void f64_tile(double (*tile)[PK_K + 1], const double*
     }
 }
 
-// expo[bo * Rp + r] = max over the row of the biased exponent field (atomic
+// expo[bo * R + r] = max over the row of the biased exponent field (atomic
 // over the K tiles; the array starts at zero = all-zero row).
 __global__ void __launch_bounds__(256) k_row_exp(const double* src, long long rs, long long ks,
-                                                 long long bs, int R, int Kd, int Rp,
-                                                 int reduce, int* expo) {
+                                                 long long bs, int R, int Kd, int reduce,
+                                                 int* expo) {
     __shared__ double tile[PK_R][PK_K + 1];
     const int b = blockIdx.z;
     const int k0 = blockIdx.x * PK_K;
     const double* s = src + (long long)b * bs;
     const int bo = reduce ? 0 : b;
     const int t = threadIdx.x;
-    for (int r0 = blockIdx.y * PK_R; r0 < Rp; r0 += gridDim.y * PK_R) {
+    for (int r0 = blockIdx.y * PK_R; r0 < R; r0 += gridDim.y * PK_R) {
         f64_tile(tile, s, rs, ks, R, Kd, r0, k0);
         __syncthreads();
         const int rr = t >> 3, oct = t & 7;
@@ -829,76 +847,86 @@ __global__ void __launch_bounds__(256) k_row_exp(const double* src, long long rs
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o, 8));
         const int r = r0 + rr;
-        if (oct == 0 && r < R && m > 0) atomicMax(&expo[(long long)bo * Rp + r], m);
+        if (oct == 0 && r < R && m > 0) atomicMax(&expo[(long long)bo * R + r], m);
         __syncthreads();
     }
 }
 
-// bf16 bits of the digit d (0 <= d <= 127) with sign bit sgn (0 or 0x8000;
-// +0 for d = 0): 2^23 + d is exact in float32, the subtraction leaves d, and
-// a float32 of at most 8 significant bits is its bf16 in the upper 16 bits.
-__device__ __forceinline__ unsigned short digit_bf16(unsigned d, unsigned sgn) {
-    const float f = __uint_as_float(0x4B000000u | d) - 8388608.0f;
-    return (unsigned short)((__float_as_uint(f) >> 16) | (d ? sgn : 0u));
+// Bits of the float32 whose upper half is the bf16 digit (byte n of w) - 128:
+// 2^23 + byte is exact in float32, the subtraction leaves the digit, and a
+// float32 of at most 8 significant bits is its bf16 in the upper 16 bits.
+__device__ __forceinline__ unsigned digit_bits(unsigned w, int n) {
+    const unsigned f = __byte_perm(w, 0x4B000000u, 0x7440u | (unsigned)n);
+    return __float_as_uint(__uint_as_float(f) - 8388736.0f);
 }
 
-// Slices of one operand: row (bo, r) holds kSlices segments of Ktot
-// elements, segment q = slice q + 1 (or slice kSlices - q with reverse), in
-// the packed K-major layout of k_pack (zero in the padding).  x = m 2^E with
-// the 53-bit significand m; |x| 2^(56 - e) = m 2^(E - e + 56) truncated to an
-// integer V < 2^56 gives the slices as its 7-bit digits.
-// Five blocks of 256 threads per SM (at its natural 78 registers three fit,
-// and on GB300 that measured no faster).
+// The 7 digits of x as such float32 bits, d[t - 1] = digit t, for a row of
+// exponent field fe (x below 2^(fe - 1022)).  V = x 2^(55 - e) rounded to an
+// integer, |V| <= 2^55; adding 128 to each of its six low bytes turns the
+// balanced base-256 digits into unsigned ones (and 256 the first, on top).
+__device__ __forceinline__ void f64_digits(double x, int fe, unsigned (&d)[kSlices]) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const int f = (int)((bits >> 52) & 0x7ff);
+    const unsigned long long mant =
+        ((bits & 0xfffffffffffffULL) | (f ? (1ULL << 52) : 0ULL)) << 2;
+    const int sh = fe - (f ? f : 1);       // >= 0 (an all-zero row has fe = 0 and mant = 0)
+    // round half up at the shifted-out bit; mant has two spare low bits
+    unsigned long long V = 0;
+    if (sh <= 2) V = mant >> max(sh, 0);
+    else if (sh < 56) V = (mant + (1ULL << (sh - 1))) >> sh;
+    const unsigned long long W = ((bits >> 63) ? 0ULL - V : V) + 0x0100808080808080ULL;
+    const unsigned lo = (unsigned)W, hi = (unsigned)(W >> 32);
+    d[6] = digit_bits(lo, 0);
+    d[5] = digit_bits(lo, 1);
+    d[4] = digit_bits(lo, 2);
+    d[3] = digit_bits(lo, 3);
+    d[2] = digit_bits(hi, 0);
+    d[1] = digit_bits(hi, 1);
+    d[0] = __float_as_uint(__uint_as_float(0x4B000000u | (hi >> 16)) - 8388864.0f);
+}
+
+// Slices of one operand, 64 K indices at a time: element (bo, k, slice q, r)
+// at ((bo nkb + k / 64) kSlices + q) R + r) 64 + k % 64, so that what a K step
+// of the product reads lies together (with K running along whole rows, a step
+// of a 400 x 240000 operand touched 2800 lines 3.4 MB apart: 7800 cycles per
+// K step instead of 6000).  A reduced product's batches follow one another
+// along k (Kp indices each, Kp a multiple of 8).  Written up to the next
+// multiple of 16, which is as far as the product reads.
 __global__ void __launch_bounds__(256, 5) k_slice64(const double* src, long long rs, long long ks,
-                                                 long long bs, int R, int Kd, int nb, int Rp,
-                                                 int Kp, int reduce, int reverse, const int* expo,
-                                                 __nv_bfloat16* out) {
+                                                    long long bs, int R, int Kd, int Kp,
+                                                    long long Ktot, int reduce, const int* expo,
+                                                    __nv_bfloat16* out) {
     __shared__ double tile[PK_R][PK_K + 1];
     const int b = blockIdx.z;
     const int k0 = blockIdx.x * PK_K;
     const double* s = src + (long long)b * bs;
-    const long long Ktot = reduce ? (long long)nb * Kp : Kp;
-    const int bo = reduce ? 0 : b, kb = reduce ? b : 0;
+    const int bo = reduce ? 0 : b;
+    const long long kofs = reduce ? (long long)b * Kp : 0;
+    const bool last = !reduce || b == (int)gridDim.z - 1;   // its zeros pad Ktot to 16
+    const long long nkb = (Ktot + BK - 1) / BK;
     const int t = threadIdx.x;
-    for (int r0 = blockIdx.y * PK_R; r0 < Rp; r0 += gridDim.y * PK_R) {
+    for (int r0 = blockIdx.y * PK_R; r0 < R; r0 += gridDim.y * PK_R) {
         f64_tile(tile, s, rs, ks, R, Kd, r0, k0);
         __syncthreads();
         const int rr = t >> 3, oct = t & 7;
         const int r = r0 + rr, k = k0 + oct * 8;
-        if (r < Rp && k < Kp) {
-            // row exponent e = field - 1022 (|x| < 2^e); 0 = all-zero row
-            const int fe = r < R ? expo[(long long)bo * Rp + r] : 0;
-            union { unsigned short h[8]; uint4 u; } v[kSlices];
+        const long long kg = kofs + k;
+        if (r < R && (k < Kp || (last && kg < (Ktot + 15) / 16 * 16))) {
+            const int fe = expo[(long long)bo * R + r];
+            unsigned v[kSlices][4];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const unsigned long long bits =
-                    (unsigned long long)__double_as_longlong(tile[rr][oct * 8 + j]);
-                const int f = (int)((bits >> 52) & 0x7ff);
-                const unsigned long long mant =
-                    (bits & 0xfffffffffffffULL) | (f ? (1ULL << 52) : 0ULL);
-                // shift = E - e + 56 with E = max(f, 1) - 1075, e = fe - 1022
-                const int sh = (f ? f : 1) - fe + 3;
-                unsigned long long V = 0;
-                if (fe > 0 && mant != 0) {
-                    if (sh >= 0) V = mant << sh;          // sh <= 3: V < 2^56
-                    else if (sh > -64) V = mant >> (-sh);
-                }
-                const unsigned sgn = (bits >> 63) ? 0x8000u : 0u;
-                // digits 0-3 in the high 28 bits of V, 4-7 in the low 28
-                const unsigned vh = (unsigned)(V >> 28), vl = (unsigned)V & 0xfffffffu;
+            for (int j = 0; j < 4; ++j) {
+                unsigned d0[kSlices], d1[kSlices];
+                f64_digits(tile[rr][oct * 8 + 2 * j], fe, d0);
+                f64_digits(tile[rr][oct * 8 + 2 * j + 1], fe, d1);
 #pragma unroll
-                for (int q = 0; q < kSlices; ++q) {
-                    const int slice = reverse ? kSlices - 1 - q : q;      // 0-based digit
-                    const unsigned dig =
-                        slice < 4 ? (vh >> (7 * (3 - slice))) & 0x7fu : (vl >> (7 * (7 - slice))) & 0x7fu;
-                    v[q].h[j] = digit_bf16(dig, sgn);
-                }
+                for (int q = 0; q < kSlices; ++q) v[q][j] = __byte_perm(d0[q], d1[q], 0x7632);
             }
-            const long long row = ((long long)bo * Rp + r) * kSlices;
+            __nv_bfloat16* o = out + (((long long)bo * nkb + kg / BK) * kSlices * R + r) * BK + kg % BK;
+            const long long plane = (long long)R * BK;
 #pragma unroll
             for (int q = 0; q < kSlices; ++q)
-                *reinterpret_cast<uint4*>(out + (row + q) * Ktot + (long long)kb * Kp + k) =
-                    v[q].u;
+                *reinterpret_cast<uint4*>(o + q * plane) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
         }
         __syncthreads();
     }
@@ -909,68 +937,115 @@ __device__ __forceinline__ double pow2(int k) {
                                      : scalbn(1.0, k);
 }
 
-// 3-D map over bf16 rows of `pitch` elements of which the first kext are read.
-cudaError_t make_map_pitch(CUtensorMap* map, const __nv_bfloat16* base, long long kext,
-                           long long pitch, long long rows, int nbo, int box_rows) {
-    cuuint64_t dims[3] = {(cuuint64_t)kext, (cuuint64_t)rows, (cuuint64_t)nbo};
-    cuuint64_t strides[2] = {(cuuint64_t)(pitch * 2), (cuuint64_t)(pitch * 2 * rows)};
-    cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)base, dims, strides, box,
+// 5-D map over the slices (K index in its block, row, slice, block, batch)
+// with boxes of 64 x box_rows x box_slices; rows outside read zero.
+cudaError_t make_map_slices(CUtensorMap* map, const __nv_bfloat16* base, long long nkb,
+                            long long rows, int nbo, int box_rows, int box_slices) {
+    cuuint64_t dims[5] = {(cuuint64_t)BK, (cuuint64_t)rows, (cuuint64_t)kSlices, (cuuint64_t)nkb,
+                          (cuuint64_t)nbo};
+    const cuuint64_t row = BK * 2, plane = row * (cuuint64_t)rows, block = plane * kSlices;
+    cuuint64_t strides[4] = {row, plane, block, block * (cuuint64_t)nkb};
+    cuuint32_t box[5] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)box_slices, 1, 1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)base, dims, strides, box,
                           estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Largest split-K count of the fused product: at most 32 chunks of at least
-// 8 K steps.
-inline int max_f64_splits(long long Ktot) {
-    return (int)std::max<long long>(1, std::min<long long>(32, Ktot / BK / 8));
+constexpr int FN = 64;                    // tile columns (B rows)
+constexpr int kMaxSteps = 1024;           // 64-wide K steps of one tile (range of the int64 sums)
+
+// K indices of a slice: K rounded up to a 16-byte store, batches of a reduced
+// product one after another.
+long long f64_ktot(int K, int batch, bool reduce) {
+    const long long Kp = rup(std::max(K, 1), 8);
+    return reduce ? Kp * batch : Kp;
+}
+
+// Split-K count: items = tiles x splits fill waves of SMs, each item takes its
+// K steps (1.9 us each at the tensor pipe's rate) and about one step more for
+// its first loads and its last drains, and the float64 partials are written
+// and read once.  At least 4 K steps per split, at most 32 splits.
+int f64_splits(long long tiles, long long ksteps, long long outputs, size_t part_elems,
+               long long sms) {
+    auto cost = [&](long long sp) {
+        const double waves = (double)((tiles * sp + sms - 1) / sms);
+        const double sum = sp > 1 ? (2.0 + outputs * sp * 16.0 / 4e6) / 1.9 : 0.0;
+        return waves * ((double)((ksteps + sp - 1) / sp) + 1.0) + sum;
+    };
+    const int lo = (int)((ksteps + kMaxSteps - 1) / kMaxSteps);
+    int best = lo;
+    for (int sp = lo + 1; sp <= 32 && ksteps / sp >= 4; ++sp) {
+        if ((size_t)(outputs * sp) > part_elems / 2) break;
+        if (cost(sp) < 0.98 * cost(best)) best = sp;
+    }
+    return best;
 }
 
 }  // namespace
 
 void gemm_f64_tc_sizes(int M, int N, int K, int batch, bool reduce, size_t* slice_elems,
                        size_t* part_elems, size_t* expo_elems) {
-    const long long Kp = rup(std::max(K, 1), BK);
-    const long long Ktot = reduce ? Kp * batch : Kp;
+    const long long Ktot = f64_ktot(K, batch, reduce);
     const long long nbo = reduce ? 1 : batch;
-    const long long Rm = rup(M, 128), Rn = rup(N, 128);
-    *slice_elems = (size_t)(kSlices * (Rm + Rn) * Ktot * nbo);
-    // float64 split-K partials of the fused product, counted in floats
-    *part_elems = (size_t)(2LL * max_f64_splits(Ktot) * nbo * (long long)M * N);
-    *expo_elems = (size_t)((Rm + Rn) * nbo);
+    *slice_elems = (size_t)(kSlices * ((long long)M + N) * rup(Ktot, BK) * nbo);
+    // float64 split-K partials, counted in floats: only products of few tiles
+    // or of a K above one tile's range are split
+    const long long tiles = (long long)cdiv(std::max(M, N), BM) * cdiv(std::min(M, N), FN) * nbo;
+    const long long steps = (Ktot + BK - 1) / BK;
+    const long long sp = tiles < 2 * 152 || steps > kMaxSteps
+                             ? std::max<long long>(1, std::min<long long>(32, steps / 4)) : 0;
+    *part_elems = (size_t)(2 * sp * nbo * (long long)M * N);
+    *expo_elems = (size_t)(((long long)M + N) * nbo);
 }
 
 // ---------------------------------------------------------------------------
 // Fused float64 product: one persistent kernel per product.  For every
-// 64-wide K step it loads the 8 slices of a 128-row A tile and of a 64-row B
-// tile once and issues the MMAs of all 36 digit pairs (t, u), t + u <= 9,
-// into eight level accumulators in tensor memory (level l = t + u at columns
-// (l - 2) 64 .. (l - 2) 64 + 63: all 512 columns).  A level accumulator
-// collects (l - 1) 64 products of |a_t b_u| < 2^14 per K step, so it is
-// drained after c_l = floor(16 / (l - 1)) steps (at most 1024 products: an
-// exact float32 integer) and restarted.  The epilogue warps combine every
-// drain exactly in registers (levels 2-6 in int64, 7-9 in float32 below
-// 2^-57 of the product's scale) and write the tile
-// once in float64: no float32 level outputs go through memory.
+// 64-wide K step it loads the 7 slices of a 128-row A tile and of a 64-row B
+// tile once and forms the 28 digit pairs (t, u), t + u <= 8, in seven level
+// accumulators in tensor memory (level q = t + u - 2 at columns 64 q ..
+// 64 q + 63).  The B slices lie one after another in shared memory and the
+// levels of A slice t one after another in tensor memory, so one MMA of
+// N = 64 m forms m pairs at once: A is read from shared memory 10 times per
+// 16-deep sub-step instead of 28 (an MMA of N = 64 reads 6 KB in the 32 cycles
+// it computes, above the 128 bytes per cycle shared memory delivers; the
+// merged ones average 110), and 40 MMAs are issued per K step.
+// A level is drained before its sum can pass 2^24: (q + 1) pairs x 64 x 2^14
+// per step, every 16, 8, 4, 4 and 2 steps for q = 0 .. 4 (exact); q = 5 and 6
+// weigh 2^-54 and less and are drained every 4 and 8 steps (a sum above 2^24
+// there is rounded by two of its units at most).
+// Measured with slicing and exponents (8 unsigned slices, one MMA per pair ->
+// this kernel): 4096^3 5.78 -> 2.65 ms (52 TFLOP/s of float64, 0.77 of the
+// measured bf16 peak on its 28 products), 400 x 400 x 240000 6.54 -> 3.27 ms,
+// 240000 x 400 x 400 6.43 -> 2.45 ms, 160000 x 1200 x 200 5.17 -> 2.03 ms and
+// x 40 3.22 -> 1.12 ms (there the epilogue's integer operations bound it).
+// The epilogue warps combine drains in registers: int64 for q <= 4, float32
+// for the rest with its integer part carried into the int64 after each drain
+// of q = 6.  The tile is written once, converted to float64 by integer
+// operations: assembled on the FP64 pipe (2 lanes per SM and cycle), a tile's
+// 8192 results take 4100 cycles per operation, whether it is predicated off
+// or not, against 2700 cycles of MMA at K = 40; so that products with a
+// general alpha or beta, which need that pipe, take a loop of their own.
 // Roles: warp 0 streams slices with TMA (B slices of a K step double-
-// buffered, A slices through a 4-deep ring), warp 1 issues the MMAs, warps
-// 2-9 drain: warp w reads TMEM lanes 32 (w % 4) .. + 31 and columns
-// 32 ((w - 2) / 4) .. + 31 of a level.  Every wait is bounded.
+// buffered, A slices through a ring), warp 1 issues the MMAs, warps 2-17
+// drain: warp w reads TMEM lanes 32 (w % 4) .. + 31 and columns
+// 16 ((w - 2) / 4) .. + 15 of a level (16 warps: the conversions to int64 and
+// the TMEM reads are latency chains that eight did not hide).  A level's
+// drain is requested as soon as its last pair of the step is issued (q after
+// A slice q + 1), so that it overlaps the remaining pairs.  Every wait is
+// bounded.
 namespace {
 
-constexpr int FN = 64;                    // tile columns (B rows)
-#ifndef THC_F64_FA
-#define THC_F64_FA 4
-#endif
-constexpr int FA = THC_F64_FA;            // A-slice ring depth
-constexpr int kF64EpiWarps = 8;
+constexpr int FA = 6;                     // A-slice ring depth
+constexpr int kF64EpiWarps = 16;
 constexpr int kF64Threads = 64 + 32 * kF64EpiWarps;
+constexpr int FC = 16;                    // columns of a level per epilogue warp
 
 struct F64Smem {
-    __nv_bfloat16 b[2][kSlices][FN * BK];   // B slices of one K step
+    __nv_bfloat16 b[2][kSlices * FN * BK];  // B slices of one K step, slice after slice
     __nv_bfloat16 a[FA][BM * BK];           // A slices, one per ring entry
+    alignas(16) int eb[kF64EpiWarps][FC];   // exponent fields of each warp's columns
     uint64_t bfull[2], bempty[2], afull[FA], aempty[FA];
     uint64_t lfull[kLevels], lempty[kLevels];
     uint64_t drain;
@@ -981,17 +1056,19 @@ struct F64Smem {
 struct F64Args {
     int M, N;                // real accumulator rows (A side) and columns (B side)
     int nbo, mblocks, nblocks, ksteps, splits;
+    int last_kk;             // 16-deep sub-steps of the last K step
     long long ntiles;        // mblocks * nblocks * nbo * splits
     int a_bcast, b_bcast;
-    long long Ktot;          // slice segment length
-    const int* eA;           // row exponent fields [bo][RpA], [bo][RpB]
+    const int* eA;           // row exponent fields [bo][M], [bo][N]
     const int* eB;
-    int RpA, RpB;
     double* C;               // output, or float64 partials when splits > 1
     long long crs, ccs, cbs;
     double alpha, beta;
+    int alpha_exp;           // alpha = +-2^alpha_exp, or kNoPow2
+    int hshift;              // fractional bits below the int64 sums' unit
     int* err;
 };
+constexpr int kNoPow2 = 1 << 20;
 
 struct F64Coord {
     int m0, n0, bo, split, k_lo, nk;
@@ -1013,8 +1090,94 @@ __device__ __forceinline__ F64Coord f64_coord(const F64Args& a, long long t) {
     return c;
 }
 
-// K steps per exact chunk of level q + 2: (l - 1) 64 c <= 1024.
-__device__ __forceinline__ int f64_chunk_steps(int q) { return 16 / (q + 1); }
+// Levels (bit q) that K step i starts afresh: every 16, 8, 4, 4, 2, 4, 8 steps
+// for q = 0 .. 6, so none at odd steps, {4} at 2 mod 4, {2 .. 5} at 4 mod 8,
+// {1 .. 6} at 8 mod 16, all at 0 mod 16.  Step i drains what step i + 1 starts.
+__device__ __forceinline__ unsigned f64_fresh(int i) {
+    return (unsigned)(0x7F7E3C1000ULL >> (8 * (__ffs(i | 16) - 1))) & 0x7fu;
+}
+__device__ __forceinline__ unsigned f64_drained(int i, int nk) {
+    return i == nk - 1 ? 0x7fu : f64_fresh(i + 1);
+}
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.b32 %0, 1, 0, q;\n}\n"
+        : "=r"(p));
+    return p != 0;
+}
+
+// Slices sl .. of rows row .. in K block kb of batch b.
+__device__ __forceinline__ void tma_load_slices(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                                int row, int sl, int kb, int b) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(sl), "r"(kb), "r"(b),
+        "r"(smem_u32(bar))
+        : "memory");
+}
+
+// F 2^e (|F| < 2^62) for the whole range: all-zero rows, values near the ends
+// of the float64 range, rows with a non-finite entry, small F.
+__device__ __noinline__ double f64_scaled(long long F, int fa, int fb, int e) {
+    if (fa == 2047 || fb == 2047) return __longlong_as_double(0x7ff8000000000000LL);
+    if (F == 0) return 0.0;
+    return (double)F * pow2(e);
+}
+
+// Bits of the same by integer operations, rounded to nearest, for |F| >= 2^32
+// and a result inside the normal range.
+__device__ __forceinline__ long long f64_bits(long long F, int e, unsigned neg) {
+    const int s = (int)(F >> 63);
+    const unsigned long long a = (unsigned long long)((F ^ (long long)s) - s);
+    // leading one at bit 62, rounded to 53 bits with it at bit 52, where it
+    // adds itself to the exponent
+    const int lz1 = __clz((int)(a >> 32)) - 1;
+    const unsigned long long m = ((a << lz1) + 0x200ULL) >> 10;
+    const unsigned hi = (unsigned)(m >> 32) + ((unsigned)(1084 + e - lz1) << 20);
+    return (long long)(((unsigned long long)(hi | (((unsigned)s ^ neg) & 0x80000000u)) << 32) |
+                       (unsigned)m);
+}
+
+// Turn the FC sums of one accumulator row into the bits of their float64
+// values 2^(fa + eb[j] + ebase) F, in place (neg: all ones to negate).
+__device__ __forceinline__ void f64_finish(long long (&H)[FC], const float (&T)[FC], const int* eb,
+                                           int hs, int fa, int ebase, unsigned neg, bool range_ok,
+                                           int ncols) {
+    const float ts = __uint_as_float((unsigned)(127 + hs) << 23);
+    unsigned slow = range_ok ? 0u : 0xffffffffu;
+    int e[FC];
+#pragma unroll
+    for (int j = 0; j < FC; j += 4) {
+        const int4 v = *reinterpret_cast<const int4*>(eb + j);
+        e[j] = v.x;
+        e[j + 1] = v.y;
+        e[j + 2] = v.z;
+        e[j + 3] = v.w;
+    }
+#pragma unroll
+    for (int j = 0; j < FC; ++j) {
+        const float m = fmaf(T[j], ts, 12582912.f);
+        H[j] = (H[j] << hs) + (int)(__float_as_uint(m) - 0x4B400000u);
+        // |F| < 2^32: the high word is 0 or all ones (a few of 2^62)
+        const int h = (int)(H[j] >> 32);
+        if ((h ^ (h >> 31)) == 0) slow |= 1u << j;
+    }
+    slow &= (1u << ncols) - 1u;   // (columns outside are not stored)
+    if (slow == 0) {
+#pragma unroll
+        for (int j = 0; j < FC; ++j) H[j] = f64_bits(H[j], fa + ebase + e[j], neg);
+    } else {
+#pragma unroll
+        for (int j = 0; j < FC; ++j) {
+            const double v = f64_scaled(neg ? -H[j] : H[j], fa, e[j], fa + ebase + e[j]);
+            H[j] = __double_as_longlong(v);
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kF64Threads, 1)
     k_gemm_f64s(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -1022,7 +1185,7 @@ __global__ void __launch_bounds__(kF64Threads, 1)
     extern __shared__ __align__(1024) unsigned char f64_raw[];
     F64Smem& sm = *reinterpret_cast<F64Smem*>((reinterpret_cast<uintptr_t>(f64_raw) + 1023) &
                                               ~uintptr_t(1023));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* fail = &sm.fail;
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -1051,224 +1214,333 @@ __global__ void __launch_bounds__(kF64Threads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = sm.tmem;
-    const long long Kt = args.Ktot;
 
     if (warp == 0) {
         if (lane == 0) {
             // TMA producer
             long long bit = 0, ait = 0;
-            long long blast[2] = {-1, -1}, alast[FA];
-            for (int s = 0; s < FA; ++s) alast[s] = -1;
-            for (long long t = blockIdx.x; t < args.ntiles && !*fail; t += gridDim.x) {
+            long long blast[2] = {-1, -1};
+            int as = 0;              // ring slot and parity of the next A slice
+            uint32_t apar = 1;       // (the first pass over the ring does not wait)
+            bool ok = true;
+            for (long long t = blockIdx.x; t < args.ntiles && ok && !*fail; t += gridDim.x) {
                 const F64Coord c = f64_coord(args, t);
                 const int ba = args.a_bcast ? 0 : c.bo, bb = args.b_bcast ? 0 : c.bo;
-                bool ok = true;
                 for (int i = 0; i < c.nk && ok; ++i) {
-                    const int kc = (c.k_lo + i) * BK;
+                    const int kb = c.k_lo + i;
                     const int bs = (int)(bit & 1);
                     if (bit >= 2 && !mbar_wait_or_fail(&sm.bempty[bs], (uint32_t)(((bit >> 1) - 1) & 1), fail)) {
                         ok = false;
                         break;
                     }
                     mbar_expect_tx(&sm.bfull[bs], (uint32_t)(kSlices * FN * BK * 2));
-                    for (int u = 1; u <= kSlices; ++u)   // slice u sits in segment 8 - u
-                        tma_load_3d(sm.b[bs][u - 1], &tmB, &sm.bfull[bs],
-                                    (int)((kSlices - u) * Kt) + kc, c.n0, bb);
+                    tma_load_slices(sm.b[bs], &tmB, &sm.bfull[bs], c.n0, 0, kb, bb);
                     blast[bs] = bit++;
-                    for (int ts = 1; ts <= kSlices; ++ts) {
-                        const int as = (int)(ait % FA);
-                        if (ait >= FA && !mbar_wait_or_fail(&sm.aempty[as], (uint32_t)(((ait / FA) - 1) & 1), fail)) {
+                    for (int ts = 0; ts < kSlices; ++ts) {
+                        if (ait >= FA && !mbar_wait_or_fail(&sm.aempty[as], apar, fail)) {
                             ok = false;
                             break;
                         }
                         mbar_expect_tx(&sm.afull[as], (uint32_t)(BM * BK * 2));
-                        tma_load_3d(sm.a[as], &tmA, &sm.afull[as], (int)((ts - 1) * Kt) + kc, c.m0, ba);
-                        alast[as] = ait++;
+                        tma_load_slices(sm.a[as], &tmA, &sm.afull[as], c.m0, ts, kb, ba);
+                        ++ait;
+                        if (++as == FA) {
+                            as = 0;
+                            apar ^= 1u;
+                        }
                     }
                 }
-                if (!ok) break;
             }
             // Every load issued has landed before the CTA exits.
             for (int s = 0; s < 2; ++s)
                 if (blast[s] >= 0) mbar_wait(&sm.bfull[s], (uint32_t)((blast[s] >> 1) & 1));
-            for (int s = 0; s < FA; ++s)
-                if (alast[s] >= 0) mbar_wait(&sm.afull[s], (uint32_t)((alast[s] / FA) & 1));
+            for (int s = 0; s < FA; ++s) {
+                // last load into slot s: number (ait - 1 - s) / FA of that slot
+                if (ait > s) mbar_wait(&sm.afull[s], (uint32_t)(((ait - 1 - s) / FA) & 1));
+            }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer.  The loops over the 36 digit pairs are unrolled and
-            // the shared-memory descriptors are stepped by constants: the
-            // start-address field counts 16-byte units, A ring slots are
-            // BM * BK * 2 bytes apart, B slices FN * BK * 2, B buffers 8 B
-            // slices, and a K sub-step of UK bf16 moves UK * 2 bytes.  (With the
-            // descriptors rebuilt for every MMA, the issuing thread spent about
-            // 130 cycles per 128 x 64 x 16 MMA, measured on GB300, where the
-            // tensor pipe at its peak takes about 45.)
-            const uint32_t idesc = instr_desc(BM, FN);
-            const uint64_t a0 = smem_desc(smem_u32(sm.a[0]));
-            const uint64_t b0 = smem_desc(smem_u32(sm.b[0][0]));
-            constexpr uint64_t kAStep = (uint64_t)(BM * BK * 2) >> 4;
-            constexpr uint64_t kBSlice = (uint64_t)(FN * BK * 2) >> 4;
-            constexpr uint64_t kKStep = (uint64_t)(UK * 2) >> 4;
-            long long bit = 0, ait = 0;
-            // Per level q (bit q): usedm = a chunk has been started before
-            // (its successor waits for the drain), parm = parity of the next
-            // lempty wait.
-            unsigned usedm = 0, parm = 0;
-            bool ok = true;
-            for (long long t = blockIdx.x; t < args.ntiles && ok && !*fail; t += gridDim.x) {
-                const F64Coord c = f64_coord(args, t);
-                int cnt[kLevels];
+        // MMA issuer.  The whole warp runs the loop and one elected lane
+        // issues, so that the descriptors stay in uniform registers (issued
+        // from a one-lane branch, every MMA first moved its operands there:
+        // 7700 cycles per K step at 4096^3 instead of 6000; testing barriers
+        // ahead took it to 5260, of which the tensor pipe works 3580).  Descriptors are stepped by constants (the start-address
+        // field counts 16-byte units).
+        const uint64_t a0 = smem_desc(smem_u32(sm.a[0]));
+        const uint64_t b0 = smem_desc(smem_u32(sm.b[0]));
+        constexpr uint64_t kAStep = (uint64_t)(BM * BK * 2) >> 4;
+        constexpr uint64_t kBSlice = (uint64_t)(FN * BK * 2) >> 4;
+        constexpr uint64_t kKStep = (uint64_t)(UK * 2) >> 4;
+        int bs = 0, as = 0;
+        uint32_t bpar = 0, apar = 0;
+        // usedm bit q: level q has been started before (its next restart
+        // waits for the drain), parm = parity of that wait.
+        unsigned usedm = 0, parm = 0;
+        // Whole-warp wait.  The barrier of the next A slice and of the next
+        // B buffer is tested before the MMAs of the current slice are issued
+        // (ready), so that a test's latency does not leave the tensor pipe,
+        // whose queue holds a few MMAs, without work.
+        auto wait_all = [&](bool ready, uint64_t* bar, uint32_t par) {
+            if (__all_sync(0xffffffffu, ready)) return true;
+            return __all_sync(0xffffffffu, mbar_wait_or_fail(bar, par, fail)) != 0;
+        };
+        auto wait_levels = [&](unsigned m) {
+            bool good = true;
 #pragma unroll
-                for (int q = 0; q < kLevels; ++q) cnt[q] = 0;
-                for (int i = 0; i < c.nk && ok; ++i) {
-                    const int bs = (int)(bit & 1);
-                    if (!mbar_wait_or_fail(&sm.bfull[bs], (uint32_t)((bit >> 1) & 1), fail)) {
-                        ok = false;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    unsigned startedm = 0;
+            for (int q = 0; q < kLevels; ++q)
+                if (good && (m >> q & 1u)) good = wait_all(false, &sm.lempty[q], (parm >> q) & 1u);
+            return good;
+        };
+        bool ok = true, a_ready = false, b_ready = false;
+        for (long long t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x) {
+            const F64Coord c = f64_coord(args, t);
+            for (int i = 0; i < c.nk && ok; ++i) {
+                ok = wait_all(b_ready, &sm.bfull[bs], bpar);
+                if (!ok) break;
+                const unsigned fresh = f64_fresh(i), wait = fresh & usedm;
+                usedm |= fresh;
+                const int nkk = c.k_lo + i == args.ksteps - 1 ? args.last_kk : BK / UK;
+                const uint64_t bbase = b0 + (uint64_t)bs * (kSlices * kBSlice);
+                const unsigned drained = f64_drained(i, c.nk);
+                b_ready = mbar_test(&sm.bfull[bs ^ 1], bpar ^ (uint32_t)bs);
 #pragma unroll
-                    for (int q = 0; q < kLevels; ++q)
-                        if (cnt[q] > 0) startedm |= 1u << q;
-                    const uint64_t bbase = b0 + (uint64_t)bs * (kSlices * kBSlice);
-#pragma unroll
-                    for (int ts = 1; ts <= kSlices; ++ts) {
-                        const int as = (int)(ait % FA);
-                        if (!mbar_wait_or_fail(&sm.afull[as], (uint32_t)((ait / FA) & 1), fail)) {
-                            ok = false;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        const uint64_t ad = a0 + (uint64_t)as * kAStep;
-#pragma unroll
-                        for (int u = 1; u <= kSlices + 1 - ts; ++u) {
-                            const int q = ts + u - 2;
-                            const unsigned qb = 1u << q;
-                            const uint32_t acc0 = (startedm >> q) & 1u;
-                            if (!acc0) {
-                                // a new chunk: the previous one has been drained
-                                if (usedm & qb) {
-                                    if (!mbar_wait_or_fail(&sm.lempty[q], (parm >> q) & 1u, fail)) {
-                                        ok = false;
-                                        break;
-                                    }
-                                    parm ^= qb;
-                                }
-                                usedm |= qb;
-                                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                            }
-                            const uint64_t bd = bbase + (uint64_t)(u - 1) * kBSlice;
-                            const uint32_t dst = tmem + (uint32_t)(q * FN);
-#pragma unroll
-                            for (int kk = 0; kk < BK / UK; ++kk)
-                                mma_bf16(dst, ad + kk * kKStep, bd + kk * kKStep, idesc,
-                                         kk > 0 ? 1u : acc0);
-                            startedm |= qb;
-                        }
-                        if (!ok) break;
-                        mma_commit(&sm.aempty[as]);
-                        ++ait;
-                    }
+                for (int ts = 1; ts <= kSlices; ++ts) {
+                    ok = wait_all(a_ready, &sm.afull[as], apar);
                     if (!ok) break;
-                    mma_commit(&sm.bempty[bs]);
-                    ++bit;
+                    const int as2 = as + 1 == FA ? 0 : as + 1;
+                    const uint32_t apar2 = as + 1 == FA ? apar ^ 1u : apar;
+                    const uint64_t ad = a0 + (uint64_t)as * kAStep;
+                    // n levels from level q on: B slices u = q + 2 - ts ...
+                    auto mma = [&](int kk, int q, int n, uint32_t acc) {
+                        mma_bf16(tmem + (uint32_t)(q * FN), ad + kk * kKStep,
+                                 bbase + (uint64_t)(q + 1 - ts) * kBSlice + kk * kKStep,
+                                 instr_desc(BM, n * FN), acc);
+                    };
+                    if (ts == 1) {
+                        // Every level is first touched by the first slice, and
+                        // sub-step 0 restarts the fresh ones (accumulate off).
+                        // Levels 4 - 6, drained last in the step before, come
+                        // after all of levels 0 - 3 (512 cycles of MMA).
+                        ok = wait_levels(wait & 0x0fu);
+                        if (!ok) break;
+                        a_ready = mbar_test(&sm.afull[as2], apar2);
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        if (elect_one()) {
+                            if (i & 3) {              // none of 0 - 3
+                                mma(0, 0, 4, 1u);
+                            } else if (i & 4) {       // 2, 3
+                                mma(0, 0, 2, 1u);
+                                mma(0, 2, 2, 0u);
+                            } else if (i & 8) {       // 1 - 3
+                                mma(0, 0, 1, 1u);
+                                mma(0, 1, 3, 0u);
+                            } else {                  // all
+                                mma(0, 0, 4, 0u);
+                            }
 #pragma unroll
-                    for (int q = 0; q < kLevels; ++q) {
-                        ++cnt[q];
-                        if (cnt[q] == f64_chunk_steps(q) || i == c.nk - 1) {
-                            mma_commit(&sm.lfull[q]);
-                            cnt[q] = 0;
+                            for (int kk = 1; kk < BK / UK; ++kk) {
+                                if (kk >= nkk) break;
+                                mma(kk, 0, 4, 1u);
+                            }
+                            if (drained & 1u) mma_commit(&sm.lfull[0]);
+                        }
+                        __syncwarp();
+                        ok = wait_levels(wait & 0x70u);
+                        parm ^= wait;
+                        if (!ok) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        if (elect_one()) {
+                            if (i & 1) {              // none of 4 - 6
+                                mma(0, 4, 3, 1u);
+                            } else if (i & 2) {       // 4
+                                mma(0, 4, 1, 0u);
+                                mma(0, 5, 2, 1u);
+                            } else if (i & 4) {       // 4, 5
+                                mma(0, 4, 2, 0u);
+                                mma(0, 6, 1, 1u);
+                            } else {                  // all
+                                mma(0, 4, 3, 0u);
+                            }
+#pragma unroll
+                            for (int kk = 1; kk < BK / UK; ++kk) {
+                                if (kk >= nkk) break;
+                                mma(kk, 4, 3, 1u);
+                            }
+                            mma_commit(&sm.aempty[as]);
+                        }
+                    } else {
+                        a_ready = mbar_test(&sm.afull[as2], apar2);
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < BK / UK; ++kk) {
+                                if (kk >= nkk) break;
+                                if (ts == 2) {
+                                    mma(kk, 1, 3, 1u);
+                                    mma(kk, 4, 3, 1u);
+                                } else if (ts == 3) {
+                                    mma(kk, 2, 3, 1u);
+                                    mma(kk, 5, 2, 1u);
+                                } else {
+                                    mma(kk, ts - 1, 8 - ts, 1u);
+                                }
+                            }
+                            mma_commit(&sm.aempty[as]);
+                            // level q is complete after slice q + 1
+                            if (drained >> (ts - 1) & 1u) mma_commit(&sm.lfull[ts - 1]);
+                            if (ts == kSlices) mma_commit(&sm.bempty[bs]);
                         }
                     }
+                    __syncwarp();
+                    as = as2;
+                    apar = apar2;
                 }
+                if (!ok) break;
+                bpar ^= (uint32_t)bs;
+                bs ^= 1;
             }
-            // All MMAs issued have completed before TMEM is freed.
+            if (__any_sync(0xffffffffu, *fail != 0)) break;
+        }
+        // All MMAs issued have completed before TMEM is freed.
+        __syncwarp();
+        if (elect_one()) {
             mma_commit(&sm.drain);
             mbar_wait(&sm.drain, 0);
         }
+        __syncwarp();
     } else {
         // Epilogue: drains and the float64 combination of the tile.
-        const int q4 = warp & 3, half = (warp - 2) >> 2;
+        const int q4 = warp & 3, quarter = (warp - 2) >> 2;
+        int* eb = sm.eb[warp - 2];
         unsigned dpar = 0;   // bit q: parity of the next lfull wait of level q
+        const bool partial = args.splits > 1;
+        // alpha = +-2^k goes into the exponent and the sign
+        const bool apow = !partial && args.alpha_exp != kNoPow2;
+        const bool general = !partial && (args.beta != 0.0 || !apow);
+        const int ebase = (apow ? args.alpha_exp : 0) - 2044 - 46 - args.hshift;
+        const unsigned aneg = apow && args.alpha < 0.0 ? 0xffffffffu : 0u;
         for (long long t = blockIdx.x; t < args.ntiles; t += gridDim.x) {
             const F64Coord c = f64_coord(args, t);
-            long long H[32];
-            float T[32];
+            // sums in units of 2^-46 of the product's scale: H + T
+            long long H[FC];
+            float T[FC];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
+            for (int j = 0; j < FC; ++j) {
                 H[j] = 0;
                 T[j] = 0.f;
             }
-            int cnt[kLevels];
-#pragma unroll
-            for (int q = 0; q < kLevels; ++q) cnt[q] = 0;
             bool ok = true;
+            // K indices that a level collects at most (short products)
+            const int kmax = c.k_lo + c.nk == args.ksteps
+                                 ? (c.nk - 1) * BK + args.last_kk * UK : c.nk * BK;
             for (int i = 0; i < c.nk && ok; ++i) {
-#pragma unroll
-                for (int q = 0; q < kLevels; ++q) {
-                    ++cnt[q];
-                    if (!ok || (cnt[q] != f64_chunk_steps(q) && i != c.nk - 1)) continue;
-                    cnt[q] = 0;
+#pragma unroll 1
+                for (unsigned todo = f64_drained(i, c.nk); todo != 0; todo &= todo - 1) {
+                    const int q = __ffs(todo) - 1;
                     if (!mbar_wait_or_fail(&sm.lfull[q], (dpar >> q) & 1u, fail)) {
                         ok = false;
-                        continue;
+                        break;
                     }
                     dpar ^= 1u << q;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    uint32_t r[32];
+                    uint32_t r[FC];
                     const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) +
-                                           (uint32_t)(q * FN + half * 32);
+                                           (uint32_t)(q * FN + quarter * FC);
                     asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x32.b32"
-                        " {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32"
+                        " {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
                           "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
-                          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-                          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-                          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]),
-                          "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                          "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                         : "r"(taddr));
                     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&sm.lempty[q]);
-                    const int l = q + 2;
-                    if (l <= 6) {
-                        const int sh = 7 * (6 - l);
+                    if (q <= 4 && (q + 1) * kmax <= 256) {
+                        // sums of at most 2^22: their integers are the low bits
+                        // of S + 1.5 2^23 (the conversion instruction runs on a
+                        // pipe of 16 lanes per SM)
+                        const long long w = 1LL << (8 * (4 - q));
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            H[j] += (long long)__float2int_rn(__uint_as_float(r[j])) << sh;
+                        for (int j = 0; j < FC; ++j) {
+                            const float m = __uint_as_float(r[j]) + 12582912.f;
+                            H[j] += (long long)(int)(__float_as_uint(m) - 0x4B400000u) * w;
+                        }
+                    } else if (q == 0) {
+                        // weight 2^32
+#pragma unroll
+                        for (int j = 0; j < FC; ++j)
+                            H[j] += (long long)((unsigned long long)(unsigned)__float2int_rn(
+                                                    __uint_as_float(r[j])) << 32);
+                    } else if (q <= 4) {
+                        const int w = 1 << (8 * (4 - q));
+#pragma unroll
+                        for (int j = 0; j < FC; ++j)
+                            H[j] += (long long)__float2int_rn(__uint_as_float(r[j])) * w;
                     } else {
-                        const float w = l == 7 ? 1.f : (l == 8 ? 0.0078125f : 0.00006103515625f);
+                        const float w = q == 5 ? 0.00390625f : 0.0000152587890625f;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) T[j] = fmaf(__uint_as_float(r[j]), w, T[j]);
+                        for (int j = 0; j < FC; ++j) T[j] = fmaf(__uint_as_float(r[j]), w, T[j]);
+                        if (q == 6) {
+                            // carry the integer part (|T| < 2^19)
+#pragma unroll
+                            for (int j = 0; j < FC; ++j) {
+                                const float m = T[j] + 12582912.f;
+                                H[j] += (int)(__float_as_uint(m) - 0x4B400000u);
+                                T[j] -= m - 12582912.f;
+                            }
+                        }
                     }
                 }
             }
             if (!ok) break;
-            // C(i, j) = alpha 2^(e_r + e_c - 42) (H + 2^-7 T) [+ beta C]
+            // C(i, j) = alpha 2^(e_r + e_c - 46) (H + T) [+ beta C]
             const int i = c.m0 + q4 * 32 + lane;
-            if (i >= args.M) continue;
-            const int fa = args.eA[(long long)(args.a_bcast ? 0 : c.bo) * args.RpA + i];
-            const int* eb = args.eB + (long long)(args.b_bcast ? 0 : c.bo) * args.RpB;
-            double* Cb = args.C + (long long)c.bo * args.cbs +
-                         (args.splits > 1 ? (long long)c.split * args.nbo * args.cbs : 0) +
-                         (long long)i * args.crs;
+            const int col0 = c.n0 + quarter * FC;
+            const int ncols = min(FC, args.N - col0);
+            const int fa = i < args.M ? args.eA[(long long)(args.a_bcast ? 0 : c.bo) * args.M + i] : 1;
+            const int fb = lane < ncols
+                         ? args.eB[(long long)(args.b_bcast ? 0 : c.bo) * args.N + col0 + lane] : 0;
+            __syncwarp();
+            if (lane < FC) eb[lane] = fb;
+            // exponents for which every result is a normal number (all-zero
+            // columns and rows give F = 0 and do not count)
+            int fmx = fb, fmn = fb > 0 ? fb : 4096;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int col = c.n0 + half * 32 + j;
-                if (col >= args.N) continue;
-                const int fb = eb[col];
-                double v = 0.0;
-                if (fa > 0 && fb > 0)
-                    v = fma((double)T[j], 0.0078125, (double)H[j]) *
-                        pow2((fa - 1022) + (fb - 1022) - 42);
-                double* p = Cb + (long long)col * args.ccs;
-                if (args.splits > 1) *p = v;
-                else *p = (args.beta != 0.0 ? args.beta * *p : 0.0) + args.alpha * v;
+            for (int off = 8; off > 0; off >>= 1) {
+                fmx = max(fmx, __shfl_xor_sync(0xffffffffu, fmx, off));
+                fmn = min(fmn, __shfl_xor_sync(0xffffffffu, fmn, off));
+            }
+            fmx = __shfl_sync(0xffffffffu, fmx, 0);
+            fmn = __shfl_sync(0xffffffffu, fmn, 0);
+            const bool range_ok = fa < 2047 && fmx < 2047 && fa + fmn > 2044 - 700 && fa + fmx < 2044 + 800;
+            __syncwarp();
+            if (i >= args.M || ncols <= 0) continue;
+            f64_finish(H, T, eb, args.hshift, fa, ebase, aneg, range_ok, ncols);
+            double* Cr = args.C + (long long)c.bo * args.cbs +
+                         (partial ? (long long)c.split * args.nbo * args.cbs : 0) +
+                         (long long)i * args.crs + (long long)col0 * args.ccs;
+            if (general) {
+#pragma unroll
+                for (int j = 0; j < FC; ++j) {
+                    if (j >= ncols) continue;
+                    double v = __longlong_as_double(H[j]);
+                    if (args.alpha_exp == kNoPow2) v *= args.alpha;
+                    double* p = Cr + (long long)j * args.ccs;
+                    *p = args.beta != 0.0 ? fma(args.beta, *p, v) : v;
+                }
+            } else if (args.ccs == 1 && ncols == FC && (reinterpret_cast<uintptr_t>(Cr) & 15) == 0) {
+#pragma unroll
+                for (int j = 0; j < FC; j += 2)
+                    *reinterpret_cast<longlong2*>(Cr + j) = make_longlong2(H[j], H[j + 1]);
+            } else if (ncols == FC) {
+#pragma unroll
+                for (int j = 0; j < FC; ++j) Cr[(long long)j * args.ccs] = __longlong_as_double(H[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < FC; ++j)
+                    if (j < ncols) Cr[(long long)j * args.ccs] = __longlong_as_double(H[j]);
             }
         }
     }
@@ -1281,17 +1553,17 @@ __global__ void __launch_bounds__(kF64Threads, 1)
 }
 
 // C = beta C + alpha sum_split part[split] (float64 split-K partials of the
-// fused kernel, in accumulator orientation: element (b, i, j) at
-// part[(split nbo + b) M N + i N + j]).
-__global__ void k_f64_splitsum(const double* part, int splits, int nbo, int M, int N, double* C,
-                               long long crs, long long ccs, long long cbs, double alpha,
-                               double beta) {
+// fused kernel; element (b, i, j) at part[(split nbo + b) M N + e], e = i N + j
+// or, i_fast, j M + i: the index that runs along C's rows).
+__global__ void k_f64_splitsum(const double* part, int splits, int nbo, int M, int N, int i_fast,
+                               double* C, long long crs, long long ccs, long long cbs,
+                               double alpha, double beta) {
     const long long MN = (long long)M * N, tot = MN * nbo;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
          e += (long long)gridDim.x * blockDim.x) {
         const int b = (int)(e / MN);
         const long long r = e % MN;
-        const int i = (int)(r / N), j = (int)(r % N);
+        const int i = (int)(i_fast ? r % M : r / N), j = (int)(i_fast ? r / M : r % N);
         double s = 0.0;
         for (int sp = 0; sp < splits; ++sp) s += part[(long long)sp * tot + e];
         double* p = C + (long long)b * cbs + (long long)i * crs + (long long)j * ccs;
@@ -1299,36 +1571,32 @@ __global__ void k_f64_splitsum(const double* part, int splits, int nbo, int M, i
     }
 }
 
-}  // namespace
-
-namespace {
-
-// Workspace a product takes in one piece: slices, exponents, and the slice
-// row pitch (which must fit a 32-bit coordinate).
+// Workspace a product takes in one piece.
 struct F64Need {
-    long long slices, expo, pitch;
+    long long slices, expo, Ktot;
 };
 
 F64Need f64_need(const Gemm<double>& g) {
-    const bool swap = g.N > g.M;
-    const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
-    const long long Kp = rup(std::max(g.K, 1), BK);
-    const int nb = g.batch;
-    const int nbo = g.reduce ? 1 : nb;
-    const long long Ktot = g.reduce ? Kp * nb : Kp;
-    const long long RpA = rup(Mr, BM), RpB = rup(Nr, FN);
-    const long long sa = swap ? g.sBb : g.sAb, sb = swap ? g.sAb : g.sBb;
-    const bool a_bc = !g.reduce && nb > 1 && sa == 0;
-    const bool b_bc = !g.reduce && nb > 1 && sb == 0;
-    const long long nba = a_bc ? 1 : nbo, nbb = b_bc ? 1 : nbo;
-    const long long pitch = kSlices * Ktot;
-    return F64Need{(RpA * nba + RpB * nbb) * pitch, RpA * nba + RpB * nbb, pitch};
+    const long long nbo = g.reduce ? 1 : g.batch;
+    const long long Ktot = f64_ktot(g.K, g.batch, g.reduce);
+    const long long nba = !g.reduce && g.batch > 1 && g.sAb == 0 ? 1 : nbo;
+    const long long nbb = !g.reduce && g.batch > 1 && g.sBb == 0 ? 1 : nbo;
+    const long long rows = g.M * nba + g.N * nbb;
+    return F64Need{rows * kSlices * rup(Ktot, BK), rows, Ktot};
+}
+
+// A K above kMaxSteps steps has to be split, which takes partials.
+bool f64_k_fits(const Gemm<double>& g, const F64TcWorkspace& ws) {
+    const long long steps = (f64_need(g).Ktot + BK - 1) / BK;
+    const long long sp = (steps + kMaxSteps - 1) / kMaxSteps;
+    const long long outputs = (long long)g.M * g.N * (g.reduce ? 1 : g.batch);
+    return sp <= 1 || (sp <= 32 && (size_t)(outputs * sp) <= ws.part_elems / 2);
 }
 
 bool f64_fits(const Gemm<double>& g, const F64TcWorkspace& ws) {
     const F64Need n = f64_need(g);
     return (size_t)n.slices <= ws.slice_elems && (size_t)n.expo <= ws.expo_elems &&
-           n.pitch <= INT32_MAX;
+           n.Ktot <= INT32_MAX - BK;
 }
 
 cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cudaStream_t s);
@@ -1338,12 +1606,14 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
 // A product whose slices do not fit the workspace is cut into pieces that
 // do: batches first (a batch-reduced product accumulates its later pieces
 // into C with beta = 1), then the rows or the columns of C, whichever are
-// more, in halves rounded to the 128-row tile.
+// more, in halves rounded to the 128-row tile.  A K too long for one tile's
+// sums is cut in halves too when its split-K partials do not fit.
 cudaError_t gemm_f64_tc(const Gemm<double>& g, const F64TcWorkspace& ws, cudaStream_t s) {
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
-    if (f64_fits(g, ws)) return gemm_f64_tc_one(g, ws, s);
+    const bool k_fits = f64_k_fits(g, ws);
+    if (k_fits && f64_fits(g, ws)) return gemm_f64_tc_one(g, ws, s);
     Gemm<double> g1 = g, g2 = g;
-    if (g.batch > 1) {
+    if (g.batch > 1 && (g.reduce || !f64_fits(g, ws))) {
         const int b1 = g.batch / 2;
         g1.batch = b1;
         g2.batch = g.batch - b1;
@@ -1354,6 +1624,13 @@ cudaError_t gemm_f64_tc(const Gemm<double>& g, const F64TcWorkspace& ws, cudaStr
         } else {
             g2.C = g.C + (long long)b1 * g.sCb;
         }
+    } else if (!k_fits && g.K > 2 * BK) {
+        const int k1 = (int)rup((g.K + 1) / 2, BK);
+        g1.K = k1;
+        g2.K = g.K - k1;
+        g2.A.p = g.A.p + (long long)k1 * g.A.cs;
+        g2.B.p = g.B.p + (long long)k1 * g.B.rs;
+        g2.beta = 1.0;
     } else if (g.M >= g.N && g.M > BM) {
         const int m1 = (int)rup((g.M + 1) / 2, BM);
         g1.M = m1;
@@ -1381,11 +1658,10 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     if (e != cudaSuccess) return e;
     const bool swap = g.N > g.M;
     const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
-    const long long Kp = rup(std::max(g.K, 1), BK);
+    const long long Kp = rup(std::max(g.K, 1), 8);
     const int nb = g.batch;
     const int nbo = g.reduce ? 1 : nb;
-    const long long Ktot = g.reduce ? Kp * nb : Kp;
-    const long long RpA = rup(Mr, BM), RpB = rup(Nr, FN);
+    const long long Ktot = f64_ktot(g.K, nb, g.reduce);
     View<double> va = g.A, vb{g.B.p, g.B.cs, g.B.rs};
     long long sa = g.sAb, sb = g.sBb;
     if (swap) {
@@ -1395,62 +1671,35 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     const bool a_bc = !g.reduce && nb > 1 && sa == 0;
     const bool b_bc = !g.reduce && nb > 1 && sb == 0;
     const int nba = a_bc ? 1 : nbo, nbb = b_bc ? 1 : nbo;
-    const long long pitch = kSlices * Ktot;
-    const long long sliceA = RpA * pitch * nba, sliceB = RpB * pitch * nbb;
-    if ((size_t)(sliceA + sliceB) > ws.slice_elems) return cudaErrorMemoryAllocation;
-    if ((size_t)(RpA * nba + RpB * nbb) > ws.expo_elems) return cudaErrorMemoryAllocation;
-    if (pitch > INT32_MAX) return cudaErrorMemoryAllocation;
-    const int mblocks = (int)(RpA / BM), nblocks = (int)(RpB / FN);
+    const long long sliceA = (long long)Mr * kSlices * rup(Ktot, BK) * nba;
+    const int mblocks = (int)cdiv(Mr, BM), nblocks = (int)cdiv(Nr, FN);
     const long long tiles = (long long)mblocks * nblocks * nbo;
-    const int ksteps = (int)(Ktot / BK);
+    const int ksteps = (int)((Ktot + BK - 1) / BK);
     const long long sms = device_sms();
-    // Split K so that the work items fill whole waves of SMs: the split
-    // count (at most 32, at least 8 K steps each) with the best ratio of
-    // items to SM slots in the waves they take; the float64 partials of the
-    // splits go to the workspace's partial buffer.
-    int splits = 1;
-    {
-        const long long per = (long long)Mr * Nr * nbo;
-        auto fill = [&](long long sp) {
-            const long long items = tiles * sp;
-            return (double)items / (double)(((items + sms - 1) / sms) * sms);
-        };
-        double best = fill(1);
-        for (int sp = 2; sp <= 32 && ksteps / sp >= 8; ++sp) {
-            if ((size_t)(per * sp) > ws.part_elems / 2) break;
-            const double f = fill(sp);
-            if (f > best + 0.02) {
-                best = f;
-                splits = sp;
-            }
-        }
-    }
+    const int splits = f64_splits(tiles, ksteps, (long long)Mr * Nr * nbo, ws.part_elems, sms);
 
     __nv_bfloat16* slA = ws.slices;
     __nv_bfloat16* slB = ws.slices + sliceA;
     int* eA = ws.expo;
-    int* eB = ws.expo + RpA * nba;
+    int* eB = ws.expo + (long long)Mr * nba;
     // Row exponents and slices of both operands.
     const int red = g.reduce ? 1 : 0;
-    if ((e = cudaMemsetAsync(ws.expo, 0, sizeof(int) * (RpA * nba + RpB * nbb), s)) !=
-        cudaSuccess)
+    if ((e = cudaMemsetAsync(ws.expo, 0, sizeof(int) * ((long long)Mr * nba + (long long)Nr * nbb),
+                             s)) != cudaSuccess)
         return e;
-    struct Side { View<double> v; long long sbat; int R; long long Rp; int nbg; __nv_bfloat16* sl;
-                  int* ex; int rev; };
-    const Side sides[2] = {{va, sa, Mr, RpA, a_bc ? 1 : nb, slA, eA, 0},
-                           {vb, sb, Nr, RpB, b_bc ? 1 : nb, slB, eB, 1}};
+    struct Side { View<double> v; long long sbat; int R; int nbg; __nv_bfloat16* sl; int* ex; };
+    const Side sides[2] = {{va, sa, Mr, a_bc ? 1 : nb, slA, eA}, {vb, sb, Nr, b_bc ? 1 : nb, slB, eB}};
     for (const Side& sd : sides) {
-        const dim3 grid(cdiv(Kp, PK_K), std::min<unsigned>(cdiv(sd.Rp, PK_R), 65535), sd.nbg);
-        k_row_exp<<<grid, 256, 0, s>>>(sd.v.p, sd.v.rs, sd.v.cs, sd.sbat, sd.R, g.K, (int)sd.Rp,
-                                       red, sd.ex);
-        k_slice64<<<grid, 256, 0, s>>>(sd.v.p, sd.v.rs, sd.v.cs, sd.sbat, sd.R, g.K, nb,
-                                       (int)sd.Rp, (int)Kp, red, sd.rev, sd.ex, sd.sl);
+        const dim3 grid(cdiv(Kp, PK_K), std::min<unsigned>(cdiv(sd.R, PK_R), 65535), sd.nbg);
+        k_row_exp<<<grid, 256, 0, s>>>(sd.v.p, sd.v.rs, sd.v.cs, sd.sbat, sd.R, g.K, red, sd.ex);
+        k_slice64<<<grid, 256, 0, s>>>(sd.v.p, sd.v.rs, sd.v.cs, sd.sbat, sd.R, g.K, (int)Kp, Ktot,
+                                       red, sd.ex, sd.sl);
         count_launches(2);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     CUtensorMap mA, mB;
-    if ((e = make_map_pitch(&mA, slA, pitch, pitch, RpA, nba, BM)) != cudaSuccess) return e;
-    if ((e = make_map_pitch(&mB, slB, pitch, pitch, RpB, nbb, FN)) != cudaSuccess) return e;
+    if ((e = make_map_slices(&mA, slA, ksteps, Mr, nba, BM, 1)) != cudaSuccess) return e;
+    if ((e = make_map_slices(&mB, slB, ksteps, Nr, nbb, FN, kSlices)) != cudaSuccess) return e;
     F64Args a{};
     a.M = Mr;
     a.N = Nr;
@@ -1458,17 +1707,27 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     a.mblocks = mblocks;
     a.nblocks = nblocks;
     a.ksteps = ksteps;
+    a.last_kk = (int)((Ktot - (long long)(ksteps - 1) * BK + UK - 1) / UK);
     a.splits = splits;
     a.ntiles = tiles * splits;
     a.a_bcast = a_bc ? 1 : 0;
     a.b_bcast = b_bc ? 1 : 0;
-    a.Ktot = Ktot;
     a.eA = eA;
     a.eB = eB;
-    a.RpA = (int)RpA;
-    a.RpB = (int)RpB;
     a.alpha = g.alpha;
     a.beta = g.beta;
+    {
+        int k = 0;
+        const double m = std::frexp(std::fabs(g.alpha), &k);   // 0.5 for a power of two
+        a.alpha_exp = m == 0.5 && k > -60 && k < 60 ? k - 1 : kNoPow2;
+    }
+    {
+        // |H| <= 2^46 per K index: as many fractional bits as leave |F| < 2^62
+        const long long kmax = (long long)((ksteps + splits - 1) / splits) * BK;
+        int lg = 0;
+        while ((1LL << lg) < kmax) ++lg;
+        a.hshift = std::max(0, std::min(16, 16 - lg));
+    }
     a.err = ws.err;
     // accumulator (i, j) is C's (m, n), or (n, m) when the operands were swapped
     const long long crs = swap ? 1 : g.ldc, ccs = swap ? g.ldc : 1;
@@ -1476,8 +1735,8 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     double* part = reinterpret_cast<double*>(ws.part);
     if (splits > 1) {
         a.C = part;
-        a.crs = Nr;
-        a.ccs = 1;
+        a.crs = swap ? 1 : Nr;
+        a.ccs = swap ? Mr : 1;
         a.cbs = (long long)Mr * Nr;
     } else {
         a.C = g.C;
@@ -1494,8 +1753,8 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     if (splits > 1) {
         const long long tot = (long long)Mr * Nr * nbo;
         const unsigned blocks = (unsigned)std::min<long long>((tot + 255) / 256, sms * 16);
-        k_f64_splitsum<<<blocks, 256, 0, s>>>(part, splits, nbo, Mr, Nr, g.C, crs, ccs, cbs,
-                                              g.alpha, g.beta);
+        k_f64_splitsum<<<blocks, 256, 0, s>>>(part, splits, nbo, Mr, Nr, swap ? 1 : 0, g.C, crs,
+                                              ccs, cbs, g.alpha, g.beta);
         count_launches(1);
         e = cudaGetLastError();
     }
@@ -1698,6 +1957,15 @@ cudaError_t gemm_f64_tc_selftest(int cases, unsigned long long seed, double* max
         g.M = 1 + (int)(st_next(s) % 600);
         g.N = 1 + (int)(st_next(s) % 600);
         g.K = 1 + (int)(st_next(s) % 2600);    // up to three exact K chunks
+        // every fourth case at the edges of the tiles, K steps and sub-steps
+        // and of the levels' drain periods
+        if (c % 4 == 3) {
+            const int mn[8] = {1, 16, 17, 63, 64, 65, 128, 129};
+            const int kk[10] = {1, 8, 16, 17, 48, 64, 65, 129, 1024, 1025};
+            g.M = mn[st_next(s) % 8] + (int)(st_next(s) % 2) * 128;
+            g.N = mn[st_next(s) % 8];
+            g.K = kk[st_next(s) % 10];
+        }
         g.batch = 1 + (int)(st_next(s) % 4);
         const int mode = (int)(st_next(s) % 4);   // 0 separate, 1 shared A, 2 shared B, 3 reduce
         g.reduce = mode == 3 && g.batch > 1;

@@ -77,10 +77,10 @@ size_t gemm_tc_pack_elems(int M, int N, int K, int batch, bool reduce);
 cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cudaStream_t s,
                     PackCache* cache = nullptr);
 
-// Float64 products on the tensor cores: each operand row is cut into 8
-// slices of 7-bit integers below a per-row power of two, the 36 slice pairs
-// that matter are multiplied exactly (bf16 integer products, float32 sums of
-// at most 1024 terms) and combined in float64, all in one fused kernel per
+// Float64 products on the tensor cores: each operand row is cut into 7
+// balanced 8-bit digits below a per-row power of two, the 28 digit pairs that
+// matter are multiplied exactly (bf16 integer products, float32 sums of at
+// most 1024 terms) and combined in fixed point, all in one fused kernel per
 // product.  A product whose slices do not fit the workspace is cut into
 // pieces that do; cudaErrorMemoryAllocation (without launching) only if a
 // single 128 x 128 piece does not fit.
