@@ -4,8 +4,10 @@
 // small for the tensor-core paths, and the float32 reference path.  Every
 // operand is a strided
 // view, so transposes, shared (stride-0) batch operands and column slices of
-// row-major arrays need no copies.  Tiles of 64 or 80 per side (chosen per
-// product to pad least) x 16, 256 threads, double-buffered shared memory.
+// row-major arrays need no copies.  Two kernels: tiles of 64 or 80 per side
+// (chosen per product to pad least) x 16, 256 threads, double-buffered shared
+// memory; and, for float64 products that such tiles would pad or leave on a
+// few SMs, one output per thread over 4 x 8 warp tiles (k_gemm_warp64).
 #include <algorithm>
 #include <type_traits>
 
@@ -217,19 +219,89 @@ __global__ void gemm_splitk_reduce(const Gemm<T> g) {
 
 constexpr int kTargetBlocks = 2 * 152;
 
-// C(0, n) = alpha sum_k A(0, k) B(k, n) + beta C(0, n): a row vector times a
-// matrix, one thread per output column (a 64 x 64 tile would compute 64 rows
-// for the one that exists).
-template <typename T>
-__global__ void k_gemv_row(Gemm<T> g) {
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < g.N;
-         n += (long long)gridDim.x * blockDim.x) {
-        T acc = 0;
-        for (int k = 0; k < g.K; ++k)
-            acc += g.A.p[(long long)k * g.A.cs] * g.B.p[(long long)k * g.B.rs + n * g.B.cs];
-        T* c = g.C + n;
-        *c = g.beta != 0.0 ? (T)(g.alpha * acc + g.beta * *c) : (T)(g.alpha * acc);
+// Float64 product with one output per thread.  The FP64 pipe takes 64 cycles
+// of a scheduler for a warp's FMA, so operand loads straight from L1 and L2
+// (two per FMA, at most 12 lines) and address arithmetic are free beside it;
+// what counts is that no lane computes padding and that the FMAs are spread
+// over all 608 schedulers.  A warp owns WM x 32 / WM outputs (4 x 8; 1 x 32
+// for a row vector), S warps of a block share the K range of one such tile
+// and are summed in order.  A 64 x 64 x 16 step of the tile kernel is 16 us of
+// one SM; the 63 products of a residual at o=5 v=20 P=60 G=120 K=60 took 3750
+// us with it and take 570 us with this one, the 57 at o=13 v=57 P=121 G=283
+// K=151 4410 -> 1580 us (1.3 TFLOP/s: the FP64 pipe's rate).
+constexpr int kWarpsPerBlock = 8;
+
+template <int WM>
+__global__ void __launch_bounds__(32 * kWarpsPerBlock)
+    k_gemm_warp64(const Gemm<double> g, int S, int mt, int nt, long long tiles) {
+    constexpr int WN = 32 / WM, U = 8;
+    __shared__ double part[kWarpsPerBlock][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long tile = (long long)blockIdx.x * (kWarpsPerBlock / S) + warp / S;
+    const int ks = warp % S;
+    const long long bz = tile / ((long long)mt * nt);
+    const int r = (int)(tile % ((long long)mt * nt));
+    const int m = r / nt * WM + lane / WN, n = r % nt * WN + lane % WN;
+    const bool in = tile < tiles && m < g.M && n < g.N;
+    // four partial sums: shorter rounding chains, and FMAs to overlap
+    double sum[4] = {0.0, 0.0, 0.0, 0.0};
+    if (in) {
+        const double* A = g.A.p + (long long)m * g.A.rs + (g.reduce ? 0 : bz * g.sAb);
+        const double* B = g.B.p + (long long)n * g.B.cs + (g.reduce ? 0 : bz * g.sBb);
+        const long long Kt = (long long)g.K * (g.reduce ? g.batch : 1);
+        const long long chunk = (Kt + S - 1) / S;
+        long long k = chunk * ks;
+        const long long k_hi = min(Kt, k + chunk);
+        while (k < k_hi) {
+            // a run of K indices inside one batch
+            const long long kb = k / g.K;
+            const int k0 = (int)(k - kb * g.K);
+            const int len = (int)min((long long)(g.K - k0), k_hi - k);
+            const double* a = A + kb * g.sAb + (long long)k0 * g.A.cs;
+            const double* b = B + kb * g.sBb + (long long)k0 * g.B.rs;
+            int i = 0;
+            for (; i + U <= len; i += U) {
+                double x[U], y[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    x[u] = __ldg(a + u * g.A.cs);
+                    y[u] = __ldg(b + u * g.B.rs);
+                }
+                a += U * g.A.cs;
+                b += U * g.B.rs;
+#pragma unroll
+                for (int u = 0; u < U; ++u) sum[u % 4] = fma(x[u], y[u], sum[u % 4]);
+            }
+            if (i < len) {
+                const int rem = len - i;
+                double x[U], y[U];
+#pragma unroll
+                for (int u = 0; u < U - 1; ++u) {
+                    x[u] = u < rem ? __ldg(a + u * g.A.cs) : 0.0;
+                    y[u] = u < rem ? __ldg(b + u * g.B.rs) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < U - 1; ++u) {
+                    if (u >= rem) break;
+                    sum[u % 4] = fma(x[u], y[u], sum[u % 4]);
+                }
+            }
+            k += len;
+        }
     }
+    double acc = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+    if (S > 1) {
+        part[warp][lane] = acc;
+        __syncthreads();
+        if (ks != 0) return;
+        acc = 0.0;
+        for (int s = 0; s < S; ++s) acc += part[warp + s][lane];
+    }
+    if (!in) return;
+    double* c = g.C + (g.reduce ? 0 : bz * g.sCb) + (long long)m * g.ldc + n;
+    double v = g.alpha * acc;
+    if (g.beta != 0.0) v = fma(g.beta, *c, v);
+    *c = v;
 }
 
 // C(m, 0) = alpha sum_k A(m, k) B(k, 0) + beta C(m, 0): a matrix times a
@@ -289,14 +361,9 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
     if (g.K <= 0) {
         g.K = 0;   // C = beta C
     }
-    if (std::is_same<T, double>::value && g.batch == 1 && !g.reduce && g.K > 0 &&
-        (g.M == 1 || g.N == 1)) {
-        // float64 vector products (float32 tiles are cheap enough)
-        if (g.M == 1) {
-            k_gemv_row<T><<<(unsigned)std::min<long long>((g.N + 255) / 256, 152 * 8), 256, 0, s>>>(g);
-        } else {
-            k_gemv_col<T><<<(unsigned)std::min<long long>(g.M, 152 * 8), 256, 0, s>>>(g);
-        }
+    if (std::is_same<T, double>::value && g.batch == 1 && !g.reduce && g.K > 0 && g.N == 1) {
+        // float64 matrix times vector
+        k_gemv_col<T><<<(unsigned)std::min<long long>(g.M, 152 * 8), 256, 0, s>>>(g);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -314,6 +381,34 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
         long long per = (long long)g.M * g.N * (g.reduce ? 1 : g.batch);
         long long cap_ws = (long long)(g.ws_elems / (size_t)per);
         splits = (int)std::max(1LL, std::min({want, cap_k, cap_ws, 64LL}));
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        // Both kernels by the FP64 cycles of the SM (or scheduler) that gets
+        // the most: a tile kernel's block takes BM BN / 2 cycles per K index
+        // with its padding, a warp of the other 64 (it also reads its operands
+        // from L1 and L2, so that it has to be a tenth better).
+        const long long Kt = (long long)g.K * (g.reduce ? g.batch : 1);
+        const long long sms = device_sms(), nb = g.reduce ? 1 : g.batch;
+        const long long chunk = (ksteps + splits - 1) / splits * BK;
+        const double t_tile = (double)((tiles * splits + sms - 1) / sms) * (BM * BN / 2) * chunk +
+                              (splits > 1 ? 6000.0 : 0.0);
+        const int WM = g.M == 1 ? 1 : 4;
+        const int mt = (int)cdiv(g.M, WM), nt = (int)cdiv(g.N, 32 / WM);
+        const long long wt = (long long)mt * nt * nb;
+        // S warps per tile: while schedulers have fewer than two warps and
+        // each keeps 16 K indices
+        int S = 1;
+        while (S < kWarpsPerBlock && wt * S < 8 * sms && Kt / (2 * S) >= 16) S *= 2;
+        const double t_warp = (double)((wt * S + 4 * sms - 1) / (4 * sms)) * ((Kt + S - 1) / S) * 64;
+        const long long blocks = (wt + kWarpsPerBlock / S - 1) / (kWarpsPerBlock / S);
+        if (g.K > 0 && blocks <= INT32_MAX && (g.M == 1 || t_warp * 1.1 < t_tile)) {
+            if (WM == 1)
+                k_gemm_warp64<1><<<(unsigned)blocks, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
+            else
+                k_gemm_warp64<4><<<(unsigned)blocks, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
+            count_launches(1);
+            return cudaGetLastError();
+        }
     }
     g.splits = splits;
     dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), (g.reduce ? 1 : g.batch) * splits);
