@@ -188,19 +188,20 @@ Err Engine<T>::mm(int M, int N, int Kd, View<T> A, View<T> B, T* C, long long ld
         // the estimated time beats the CUDA cores (1 TFLOP/s): 28 slice-pair
         // products at the 1.2 PFLOP/s of bf16 products the fused kernel
         // reaches on large shapes, slicing (8 + 8 bytes read, 14 written per
-        // operand element), the float64 tile written once, 5 launches.
+        // operand element), the float64 tile written once, and 30 us of
+        // launches and of tiles' first loads and last drains.
         const double out = (double)M * N * (reduce ? 1 : batch);
         const double opnd = ((double)M + N) * Kd * batch;
         const double t_tc = 28.0 * fl / 1.2e15 + opnd * 30.0 / 5e12 + out * 8.0 / 5e12 +
-                            5.0 * 5e-6;
+                            30e-6;
         const bool use_tc = step_f64tc();
-        if (use_tc && fl >= 3.0e7 && Kd >= 16 && t_tc < fl / 1.0e12) {
+        if (use_tc && fl >= 3.0e7 && Kd >= 8 && t_tc < fl / 1.0e12) {
             cudaError_t e = gemm_f64_tc(g, f64ws, st);
             if (e == cudaSuccess) return Err{};
             if (e != cudaErrorMemoryAllocation) THC_CUDA(e);
             why = "workspace";
         } else if (use_tc && fl >= 3.0e7) {
-            why = Kd < 16 ? "K < 16" : "cost model";
+            why = Kd < 8 ? "K < 8" : "cost model";
         }
     }
     if (why && debug_products())

@@ -234,11 +234,13 @@ constexpr int kWarpsPerBlock = 8;
 template <int WM>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock)
     k_gemm_warp64(const Gemm<double> g, int S, int mt, int nt, long long tiles) {
+    // blockIdx.y of g.splits shares a K range over blocks; their sums go to
+    // g.ws for gemm_splitk_reduce
     constexpr int WN = 32 / WM, U = 8;
     __shared__ double part[kWarpsPerBlock][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long tile = (long long)blockIdx.x * (kWarpsPerBlock / S) + warp / S;
-    const int ks = warp % S;
+    const int ks = blockIdx.y * S + warp % S;
     const long long bz = tile / ((long long)mt * nt);
     const int r = (int)(tile % ((long long)mt * nt));
     const int m = r / nt * WM + lane / WN, n = r % nt * WN + lane % WN;
@@ -249,7 +251,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock)
         const double* A = g.A.p + (long long)m * g.A.rs + (g.reduce ? 0 : bz * g.sAb);
         const double* B = g.B.p + (long long)n * g.B.cs + (g.reduce ? 0 : bz * g.sBb);
         const long long Kt = (long long)g.K * (g.reduce ? g.batch : 1);
-        const long long chunk = (Kt + S - 1) / S;
+        const int parts = S * g.splits;
+        const long long chunk = (Kt + parts - 1) / parts;
         long long k = chunk * ks;
         const long long k_hi = min(Kt, k + chunk);
         while (k < k_hi) {
@@ -293,11 +296,16 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock)
     if (S > 1) {
         part[warp][lane] = acc;
         __syncthreads();
-        if (ks != 0) return;
+        if (warp % S != 0) return;
         acc = 0.0;
         for (int s = 0; s < S; ++s) acc += part[warp + s][lane];
     }
     if (!in) return;
+    if (g.splits > 1) {
+        const long long MN = (long long)g.M * g.N;
+        g.ws[(bz * g.splits + blockIdx.y) * MN + (long long)m * g.N + n] = acc;
+        return;
+    }
     double* c = g.C + (g.reduce ? 0 : bz * g.sCb) + (long long)m * g.ldc + n;
     double v = g.alpha * acc;
     if (g.beta != 0.0) v = fma(g.beta, *c, v);
@@ -395,18 +403,34 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
         const int WM = g.M == 1 ? 1 : 4;
         const int mt = (int)cdiv(g.M, WM), nt = (int)cdiv(g.N, 32 / WM);
         const long long wt = (long long)mt * nt * nb;
-        // S warps per tile: while schedulers have fewer than two warps and
-        // each keeps 16 K indices
-        int S = 1;
+        // S warps per tile, then gs blocks of them: while schedulers have
+        // fewer than two warps and each warp keeps 16 (32) K indices
+        int S = 1, gs = 1;
         while (S < kWarpsPerBlock && wt * S < 8 * sms && Kt / (2 * S) >= 16) S *= 2;
-        const double t_warp = (double)((wt * S + 4 * sms - 1) / (4 * sms)) * ((Kt + S - 1) / S) * 64;
+        if (S == kWarpsPerBlock && g.ws)
+            while (gs < 64 && wt * S * gs < 8 * sms && Kt / (2 * S * gs) >= 32 &&
+                   (size_t)(2 * gs) * g.M * g.N * nb <= g.ws_elems)
+                gs *= 2;
+        const long long parts = (long long)S * gs;
+        const double t_warp = (double)((wt * parts + 4 * sms - 1) / (4 * sms)) *
+                                  ((Kt + parts - 1) / parts) * 64 +
+                              (gs > 1 ? 6000.0 : 0.0);
         const long long blocks = (wt + kWarpsPerBlock / S - 1) / (kWarpsPerBlock / S);
         if (g.K > 0 && blocks <= INT32_MAX && (g.M == 1 || t_warp * 1.1 < t_tile)) {
+            g.splits = gs;
+            const dim3 wgrid((unsigned)blocks, (unsigned)gs);
             if (WM == 1)
-                k_gemm_warp64<1><<<(unsigned)blocks, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
+                k_gemm_warp64<1><<<wgrid, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
             else
-                k_gemm_warp64<4><<<(unsigned)blocks, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
-            count_launches(1);
+                k_gemm_warp64<4><<<wgrid, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            count_launches(gs > 1 ? 2 : 1);
+            if (gs > 1) {
+                const long long total = (long long)g.M * g.N * nb;
+                const unsigned nbk = (unsigned)std::min<long long>((total + 255) / 256, 152LL * 32);
+                gemm_splitk_reduce<double><<<nbk, 256, 0, s>>>(g);
+            }
             return cudaGetLastError();
         }
     }

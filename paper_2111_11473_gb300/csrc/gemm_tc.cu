@@ -825,31 +825,58 @@ __device__ __forceinline__ void f64_tile(double (*tile)[PK_K + 1], const double*
     }
 }
 
+// One operand of a product: rows r < R, K indices k < Kd of batches b < nb at
+// src[b bs + r rs + k ks]; its slices and row exponents.  A launch covers both
+// operands of a product: blocks 0 .. nblk(A) - 1 and the rest.
+struct SliceOp {
+    const double* src;
+    long long rs, ks, bs;
+    int R, nb;
+    __nv_bfloat16* out;
+    int* expo;
+};
+struct SlicePair {
+    SliceOp op[2];
+    long long blocks0;   // blocks of op[0]
+    int Kd, Kp, reduce;
+    long long Ktot;
+};
+
+// The tile of this block of 64 K indices x 32 rows: k tile fastest, then row
+// tile, then batch.
+struct SliceTile {
+    int k0, r0, b;
+};
+__device__ __forceinline__ SliceTile slice_tile(const SlicePair& p, const SliceOp& op, long long blk) {
+    const int kt = (p.Kp + PK_K - 1) / PK_K, rt = (op.R + PK_R - 1) / PK_R;
+    SliceTile t;
+    t.k0 = (int)(blk % kt) * PK_K;
+    blk /= kt;
+    t.r0 = (int)(blk % rt) * PK_R;
+    t.b = (int)(blk / rt);
+    return t;
+}
+
 // expo[bo * R + r] = max over the row of the biased exponent field (atomic
 // over the K tiles; the array starts at zero = all-zero row).
-__global__ void __launch_bounds__(256) k_row_exp(const double* src, long long rs, long long ks,
-                                                 long long bs, int R, int Kd, int reduce,
-                                                 int* expo) {
+__global__ void __launch_bounds__(256) k_row_exp(const __grid_constant__ SlicePair p) {
     __shared__ double tile[PK_R][PK_K + 1];
-    const int b = blockIdx.z;
-    const int k0 = blockIdx.x * PK_K;
-    const double* s = src + (long long)b * bs;
-    const int bo = reduce ? 0 : b;
+    const bool second = blockIdx.x >= p.blocks0;
+    const SliceOp& op = p.op[second];
+    const SliceTile c = slice_tile(p, op, blockIdx.x - (second ? p.blocks0 : 0));
     const int t = threadIdx.x;
-    for (int r0 = blockIdx.y * PK_R; r0 < R; r0 += gridDim.y * PK_R) {
-        f64_tile(tile, s, rs, ks, R, Kd, r0, k0);
-        __syncthreads();
-        const int rr = t >> 3, oct = t & 7;
-        int m = 0;
+    f64_tile(tile, op.src + c.b * op.bs, op.rs, op.ks, op.R, p.Kd, c.r0, c.k0);
+    __syncthreads();
+    const int rr = t >> 3, oct = t & 7;
+    int m = 0;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) m = max(m, f64_field(tile[rr][oct * 8 + e]));
-        // the 8 threads of a row are consecutive lanes of one warp
+    for (int e = 0; e < 8; ++e) m = max(m, f64_field(tile[rr][oct * 8 + e]));
+    // the 8 threads of a row are consecutive lanes of one warp
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o, 8));
-        const int r = r0 + rr;
-        if (oct == 0 && r < R && m > 0) atomicMax(&expo[(long long)bo * R + r], m);
-        __syncthreads();
-    }
+    for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o, 8));
+    const int r = c.r0 + rr;
+    if (oct == 0 && r < op.R && m > 0)
+        atomicMax(&op.expo[(p.reduce ? 0 : (long long)c.b * op.R) + r], m);
 }
 
 // Bits of the float32 whose upper half is the bf16 digit (byte n of w) - 128:
@@ -892,43 +919,106 @@ __device__ __forceinline__ void f64_digits(double x, int fe, unsigned (&d)[kSlic
 // K step instead of 6000).  A reduced product's batches follow one another
 // along k (Kp indices each, Kp a multiple of 8).  Written up to the next
 // multiple of 16, which is as far as the product reads.
-__global__ void __launch_bounds__(256, 5) k_slice64(const double* src, long long rs, long long ks,
-                                                    long long bs, int R, int Kd, int Kp,
-                                                    long long Ktot, int reduce, const int* expo,
-                                                    __nv_bfloat16* out) {
+__device__ __forceinline__ void slice_store(const SlicePair& p, const SliceOp& op, int b, int r, int k,
+                                            const double* x, int fe) {
+    unsigned v[kSlices][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        unsigned d0[kSlices], d1[kSlices];
+        f64_digits(x[2 * j], fe, d0);
+        f64_digits(x[2 * j + 1], fe, d1);
+#pragma unroll
+        for (int q = 0; q < kSlices; ++q) v[q][j] = __byte_perm(d0[q], d1[q], 0x7632);
+    }
+    const long long nkb = (p.Ktot + BK - 1) / BK;
+    const long long kg = (p.reduce ? (long long)b * p.Kp : 0) + k, bo = p.reduce ? 0 : b;
+    __nv_bfloat16* o = op.out + ((bo * nkb + kg / BK) * kSlices * op.R + r) * BK + kg % BK;
+    const long long plane = (long long)op.R * BK;
+#pragma unroll
+    for (int q = 0; q < kSlices; ++q)
+        *reinterpret_cast<uint4*>(o + q * plane) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
+}
+
+// True for the 8 K indices from k on that have to be written: the batch's own
+// and, after the last one, the zeros up to a multiple of 16.
+__device__ __forceinline__ bool slice_written(const SlicePair& p, int b, int nb, int k) {
+    if (k < p.Kp) return true;
+    return (!p.reduce || b == nb - 1) &&
+           (p.reduce ? (long long)b * p.Kp : 0) + k < (p.Ktot + 15) / 16 * 16;
+}
+
+__global__ void __launch_bounds__(256, 5) k_slice64(const __grid_constant__ SlicePair p) {
     __shared__ double tile[PK_R][PK_K + 1];
-    const int b = blockIdx.z;
-    const int k0 = blockIdx.x * PK_K;
-    const double* s = src + (long long)b * bs;
-    const int bo = reduce ? 0 : b;
-    const long long kofs = reduce ? (long long)b * Kp : 0;
-    const bool last = !reduce || b == (int)gridDim.z - 1;   // its zeros pad Ktot to 16
-    const long long nkb = (Ktot + BK - 1) / BK;
-    const int t = threadIdx.x;
-    for (int r0 = blockIdx.y * PK_R; r0 < R; r0 += gridDim.y * PK_R) {
-        f64_tile(tile, s, rs, ks, R, Kd, r0, k0);
-        __syncthreads();
-        const int rr = t >> 3, oct = t & 7;
-        const int r = r0 + rr, k = k0 + oct * 8;
-        const long long kg = kofs + k;
-        if (r < R && (k < Kp || (last && kg < (Ktot + 15) / 16 * 16))) {
-            const int fe = expo[(long long)bo * R + r];
-            unsigned v[kSlices][4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                unsigned d0[kSlices], d1[kSlices];
-                f64_digits(tile[rr][oct * 8 + 2 * j], fe, d0);
-                f64_digits(tile[rr][oct * 8 + 2 * j + 1], fe, d1);
-#pragma unroll
-                for (int q = 0; q < kSlices; ++q) v[q][j] = __byte_perm(d0[q], d1[q], 0x7632);
-            }
-            __nv_bfloat16* o = out + (((long long)bo * nkb + kg / BK) * kSlices * R + r) * BK + kg % BK;
-            const long long plane = (long long)R * BK;
-#pragma unroll
-            for (int q = 0; q < kSlices; ++q)
-                *reinterpret_cast<uint4*>(o + q * plane) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
+    const bool second = blockIdx.x >= p.blocks0;
+    const SliceOp& op = p.op[second];
+    const SliceTile c = slice_tile(p, op, blockIdx.x - (second ? p.blocks0 : 0));
+    f64_tile(tile, op.src + c.b * op.bs, op.rs, op.ks, op.R, p.Kd, c.r0, c.k0);
+    __syncthreads();
+    const int rr = threadIdx.x >> 3, oct = threadIdx.x & 7;
+    const int r = c.r0 + rr, k = c.k0 + oct * 8;
+    if (r < op.R && slice_written(p, c.b, op.nb, k))
+        slice_store(p, op, c.b, r, k, &tile[rr][oct * 8],
+                    op.expo[(p.reduce ? 0 : (long long)c.b * op.R) + r]);
+}
+
+// Exponents and slices in one pass for rows that fit shared memory (separate
+// batches, K <= kFusedK): a block holds SR rows with all their K indices, so
+// that the operand is read once and no exponent array has to be cleared.
+constexpr int SR = 16;            // rows per block
+constexpr int kFusedK = 512;      // at most 75 KB of shared memory: three blocks per SM
+
+// Place of K index k in a row (8 threads read 8 groups of 8 at once), and the
+// odd number of doubles of a row of Kw (a multiple of 16).
+__host__ __device__ __forceinline__ int row_at(int k) { return k + (k >> 3); }
+__host__ __device__ __forceinline__ int row_pitch(int Kw) { return Kw / 8 * 9 + 1; }
+
+__global__ void __launch_bounds__(256) k_slice_rows(const __grid_constant__ SlicePair p) {
+    extern __shared__ __align__(16) double rows[];   // [SR][pitch]
+    __shared__ int fe[SR];
+    const bool second = blockIdx.x >= p.blocks0;
+    const SliceOp& op = p.op[second];
+    const long long blk = blockIdx.x - (second ? p.blocks0 : 0);
+    const int rt = (op.R + SR - 1) / SR;
+    const int r0 = (int)(blk % rt) * SR, b = (int)(blk / rt);
+    const double* s = op.src + b * op.bs;
+    // K indices held: the written ones
+    const int Kw = (p.Kp + 15) / 16 * 16, pitch = row_pitch(Kw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (op.ks <= op.rs) {
+        for (int rr = warp; rr < SR; rr += 8) {
+            const int r = r0 + rr;
+#pragma unroll 4
+            for (int k = lane; k < Kw; k += 32)
+                rows[rr * pitch + row_at(k)] = (r < op.R && k < p.Kd) ? s[(long long)r * op.rs + (long long)k * op.ks] : 0.0;
         }
-        __syncthreads();
+    } else {
+        // half a warp along the rows
+        const int rr = threadIdx.x & (SR - 1), r = r0 + rr;
+#pragma unroll 4
+        for (int k = threadIdx.x / SR; k < Kw; k += 256 / SR)
+            rows[rr * pitch + row_at(k)] = (r < op.R && k < p.Kd) ? s[(long long)r * op.rs + (long long)k * op.ks] : 0.0;
+    }
+    __syncthreads();
+    for (int rr = warp; rr < SR; rr += 8) {
+        int m = 0;
+        for (int k = lane; k < Kw; k += 32) m = max(m, f64_field(rows[rr * pitch + row_at(k)]));
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) {
+            fe[rr] = m;
+            if (r0 + rr < op.R) op.expo[(long long)b * op.R + r0 + rr] = m;
+        }
+    }
+    __syncthreads();
+    // 8 K indices per thread: 8 threads write 128 contiguous bytes of a slice
+    const int octs = Kw / 8;
+    for (int e = threadIdx.x; e < SR * ((octs + 7) / 8) * 8; e += 256) {
+        const int oct = e / (8 * SR) * 8 + (e & 7), rr = (e >> 3) & (SR - 1);
+        if (oct < octs && r0 + rr < op.R) {
+            double x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = rows[rr * pitch + oct * 9 + j];
+            slice_store(p, op, b, r0 + rr, oct * 8, x, fe[rr]);
+        }
     }
 }
 
@@ -1683,20 +1773,38 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     int* eA = ws.expo;
     int* eB = ws.expo + (long long)Mr * nba;
     // Row exponents and slices of both operands.
-    const int red = g.reduce ? 1 : 0;
-    if ((e = cudaMemsetAsync(ws.expo, 0, sizeof(int) * ((long long)Mr * nba + (long long)Nr * nbb),
-                             s)) != cudaSuccess)
-        return e;
-    struct Side { View<double> v; long long sbat; int R; int nbg; __nv_bfloat16* sl; int* ex; };
-    const Side sides[2] = {{va, sa, Mr, a_bc ? 1 : nb, slA, eA}, {vb, sb, Nr, b_bc ? 1 : nb, slB, eB}};
-    for (const Side& sd : sides) {
-        const dim3 grid(cdiv(Kp, PK_K), std::min<unsigned>(cdiv(sd.R, PK_R), 65535), sd.nbg);
-        k_row_exp<<<grid, 256, 0, s>>>(sd.v.p, sd.v.rs, sd.v.cs, sd.sbat, sd.R, g.K, red, sd.ex);
-        k_slice64<<<grid, 256, 0, s>>>(sd.v.p, sd.v.rs, sd.v.cs, sd.sbat, sd.R, g.K, (int)Kp, Ktot,
-                                       red, sd.ex, sd.sl);
+    SlicePair p{};
+    p.op[0] = SliceOp{va.p, va.rs, va.cs, sa, Mr, a_bc ? 1 : nb, slA, eA};
+    p.op[1] = SliceOp{vb.p, vb.rs, vb.cs, sb, Nr, b_bc ? 1 : nb, slB, eB};
+    p.Kd = g.K;
+    p.Kp = (int)Kp;
+    p.Ktot = Ktot;
+    p.reduce = g.reduce ? 1 : 0;
+    const bool fused = !g.reduce && g.K <= kFusedK;
+    const long long kt = fused ? 1 : cdiv(Kp, PK_K);
+    long long blocks[2];
+    for (int i = 0; i < 2; ++i)
+        blocks[i] = kt * cdiv(p.op[i].R, fused ? SR : PK_R) * p.op[i].nb;
+    if (blocks[0] + blocks[1] > INT32_MAX) return cudaErrorInvalidValue;
+    p.blocks0 = blocks[0];
+    const unsigned sgrid = (unsigned)(blocks[0] + blocks[1]);
+    if (fused) {
+        const int sbytes = SR * row_pitch((int)rup(Kp, 16)) * (int)sizeof(double);
+        if ((e = smem_optin((const void*)k_slice_rows, SR * row_pitch(kFusedK) * (int)sizeof(double))) !=
+            cudaSuccess)
+            return e;
+        k_slice_rows<<<sgrid, 256, sbytes, s>>>(p);
+        count_launches(1);
+    } else {
+        if ((e = cudaMemsetAsync(ws.expo, 0,
+                                 sizeof(int) * ((long long)Mr * nba + (long long)Nr * nbb), s)) !=
+            cudaSuccess)
+            return e;
+        k_row_exp<<<sgrid, 256, 0, s>>>(p);
+        k_slice64<<<sgrid, 256, 0, s>>>(p);
         count_launches(2);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     CUtensorMap mA, mB;
     if ((e = make_map_slices(&mA, slA, ksteps, Mr, nba, BM, 1)) != cudaSuccess) return e;
     if ((e = make_map_slices(&mB, slB, ksteps, Nr, nbb, FN, kSlices)) != cudaSuccess) return e;
