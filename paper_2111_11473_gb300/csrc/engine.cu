@@ -685,6 +685,11 @@ Err Engine<T>::init_finish() {
         gall_resident = gall_fits;
         tri_df = std::is_same<T, double>::value && pol[THC_STEP_TRIANGLE] == THC_POL_FP64_TC;
         tri_pair = std::is_same<T, float>::value && triangle_pair_ok(P);
+        // The triangle's sums with bounds: grid chunks are whole bound chunks
+        // (i_chunk set by the caller may not be).
+        bool tri_bias = tri_df && G >= kBiasMinPoints;
+        if (tri_bias && cfg.i_chunk == 0 && ic < G) ic = std::max(kBiasChunk, ic / kBiasChunk * kBiasChunk);
+        tri_bias = tri_bias && (ic >= G || ic % kBiasChunk == 0);
         if (gall_resident) {
             THC_TRY(Gall.alloc((size_t)G * PP));
             THC_TRY(mm(P, P, o, tr(yo, P), View<T>{U6.p, (long long)G * P, 1}, Gall.p, P, 1, 0,
@@ -694,14 +699,24 @@ Err Engine<T>::init_finish() {
                 if (tri_df)
                     THC_CUDA(split_df(Gall.p, (long long)G * PP,
                                       reinterpret_cast<float2*>(Gall.p), st));
+                if (tri_bias) {
+                    THC_TRY(MG4.alloc((size_t)cdiv(G, kBiasChunk) * PP));
+                    THC_CUDA(pair_max(reinterpret_cast<const float2*>(Gall.p), G, P, MG4.p, st));
+                }
             }
         } else {
             THC_TRY(Gch.alloc((size_t)ic * PP));
+            if (tri_bias) THC_TRY(MG4.alloc((size_t)cdiv(ic, kBiasChunk) * PP));
         }
         if (tri_df) {
             const size_t pairs = (size_t)ic * ((x6 + 1) / 2) * P;
             THC_TRY(E4.alloc(pairs));
             THC_TRY(F4.alloc(pairs));
+            if (tri_bias) {
+                const size_t bounds = (size_t)cdiv(ic, kBiasChunk) * ((x6 + 1) / 2) * P;
+                THC_TRY(ME4.alloc(bounds));
+                THC_TRY(MF4.alloc(bounds));
+            }
         }
         const long long xP = (long long)x6 * P;
         // slabs of C_i, D_a, E and F: an even number of rows for the paired triangle
@@ -872,6 +887,9 @@ Err Engine<T>::init_finish() {
         THC_TRY(poison(f64part));
         THC_TRY(poison(E4));
         THC_TRY(poison(F4));
+        THC_TRY(poison(ME4));
+        THC_TRY(poison(MF4));
+        if (!gall_resident) THC_TRY(poison(MG4));
     }
     THC_CUDA(cudaStreamSynchronize(st));
     pending = false;
@@ -957,11 +975,14 @@ Err Engine<T>::alg6(T* sgm) {
             if constexpr (std::is_same<T, double>::value) {
                 if (tri_df) {
                     // float pairs of E, F (and of a rebuilt G chunk, in place)
-                    THC_CUDA(split_df_pairs(Ech.p, nI, nX, P, E4.p, st));
-                    THC_CUDA(split_df_pairs(Fch.p, nI, nX, P, F4.p, st));
-                    if (!gall_resident)
+                    THC_CUDA(split_df_pairs(Ech.p, nI, nX, P, E4.p, ME4.p, st));
+                    THC_CUDA(split_df_pairs(Fch.p, nI, nX, P, F4.p, MF4.p, st));
+                    if (!gall_resident) {
                         THC_CUDA(split_df(Gch.p, (long long)nI * PP,
                                           reinterpret_cast<float2*>(Gch.p), st));
+                        if (MG4.p)
+                            THC_CUDA(pair_max(reinterpret_cast<const float2*>(Gch.p), nI, P, MG4.p, st));
+                    }
                 }
             }
             // H^XYZ += (E^XY F^XZ + E^XZ F^XY) G^YZ   (line 11)
@@ -970,8 +991,10 @@ Err Engine<T>::alg6(T* sgm) {
             if (prof.on) prof.flops[THC_STEP_TRIANGLE] += 5.0 * nI * (double)nX * P * P;
             if constexpr (std::is_same<T, double>::value) {
                 if (tri_df)
-                    THC_CUDA(triangle_df(H.p, E4.p, F4.p, reinterpret_cast<const float2*>(Gp), P,
-                                         nX, nI, st));
+                    THC_CUDA(triangle_df(H.p, E4.p, F4.p, reinterpret_cast<const float2*>(Gp), ME4.p,
+                                         MF4.p,
+                                         gall_resident && MG4.p ? MG4.p + I0 / kBiasChunk * PP : MG4.p,
+                                         P, nX, nI, st));
                 else
                     THC_CUDA(triangle(H.p, Ech.p, Fch.p, Gp, P, nX, nI, st));
             } else if (tri_pair) {

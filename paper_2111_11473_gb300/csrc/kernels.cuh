@@ -90,12 +90,20 @@ cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, in
 // {h(x), h(x+1), l(x), l(x+1)} of E^{xY} for the row pairs x = 2q, 2q + 1
 // (split_df_pairs); G2: nI x P x P float2 {h, l} (split_df); H: nX x P x P
 // float64, accumulated into.
-cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out,
+// With bounds, also the largest |h| of every kBiasChunk grid points
+// (ceil(nI / kBiasChunk) x ceil(nX/2) x P).
+constexpr int kBiasChunk = 16;
+cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, float2* bounds,
                            cudaStream_t s);
-// out[i] = {fl32(in[i]), fl32(in[i] - fl32(in[i]))}; out may alias in.
+// The same of G: M[chunk][Y][Z] = max |G_h^YZ|, |G_h^ZY| (ceil(nI / kBiasChunk) x P x P).
+cudaError_t pair_max(const float2* G2, int nI, int P, float* M, cudaStream_t s);
+// Grid points from which the sums with bounds (ME, MF, MG not null) are the
+// more accurate ones.
+constexpr int kBiasMinPoints = 512;
 cudaError_t split_df(const double* in, long long n, float2* out, cudaStream_t s);
-cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2, int P,
-                        int nX, int nI, cudaStream_t s);
+cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
+                        const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
+                        cudaStream_t s);
 
 // Float32 triangle over X pairs in packed lanes (triangle_pair.cu), for P a
 // multiple of 4 and at most kPairMaxP.  E2, F2: nI x ceil(nX/2) x P float2

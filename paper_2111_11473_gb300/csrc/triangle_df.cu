@@ -321,6 +321,443 @@ __global__ void __launch_bounds__(DTH, 1)
             }
 }
 
+// ---------------------------------------------------------------------------
+// The same sums with fewer operations: TwoSum (six operations, because it does
+// not know which addend is larger) is replaced by additions to constants that
+// are known to be larger.  For a bound b >= |x| and a power of two 2^k >= 2 b,
+// c = 1.5 2^k:  s = fl(x + c) stays in [2^k, 2^(k+1)), so s - c is x rounded
+// to a multiple of u = 2^(k-23), exactly, and x - (s - c) has at most u / 2
+// (Rump, Ogita and Oishi's extraction).  With x = a b in an FMA:
+//   h = fma(a, b, c),  z = c - h,  r = fma(a, b, z):   a b = -z + r
+// up to the rounding of r (2^-25 of u / 2).  t = E^XY F^XZ + E^XZ F^XY is
+// formed this way from its two products (12 packed operations instead of 16),
+// and t G is added to the accumulator as an integer: the low bits of s are
+// (s - c) / u, so the sum over grid points of the bits of s, minus those of c,
+// is exact in 32 bits for up to 512 points and takes an integer addition per
+// lane; the remainder and the low-order products t_h g_l + t_l g_h go to a
+// float32 sum.  6 packed operations per accumulation instead of 12: 24 per
+// (X pair, Y, Z) pair of mirror outputs instead of 40.
+// The bounds come from the largest |E|, |F|, |G| of BC grid points at a time
+// (k_split_pairs and k_pair_max write them), for every (X, Y, Z) of its own;
+// after BC points the integer and float32 sums are added to a float pair in
+// shared memory.  Accuracy: an error u per term relative to the chunk's
+// bound instead of relative to the running sum, so it does not grow with the
+// number of grid points as the TwoSum form's does: on Gaussian operands, rms
+// over the sum of |terms|, 2^-46.1 / -46.6 / -47.1 for 300 / 600 / 1200 points
+// against 2^-46.7 / -46.2 / -45.7.  Hence the rule kBiasMinPoints: below it
+// the other kernel is the more accurate one (and the step is short).
+constexpr int BS = 2;                       // grid points per pipeline stage
+constexpr int BST = 3;                      // stages
+constexpr int BC = kBiasChunk;              // grid points per chunk of common bounds
+constexpr int BTH = 256;                    // threads: 16 x 16, each 2 x 2 (Y, Z) of two X pairs
+static_assert(BC % BS == 0 && BC <= 512, "chunks are whole stages; 512 x 2^22 fits 32 bits");
+
+struct BiasSmem {
+    struct {
+        float4 ey[BS][2][DT], ez[BS][2][DT], fy[BS][2][DT], fz[BS][2][DT];
+        // {h, l} of G^YZ, rows Y, and of G^ZY, rows Z: column c of row r at
+        // 2 ((c / 2) ^ (r & 15)) + c % 2, so that rows (16-byte copies, reads
+        // of G^YZ) and columns (reads of G^ZY) are free of bank conflicts
+        float2 g1[BS][DT][DT];
+        float2 g2[BS][DT][DT];
+    } st[BST];
+    // bounds of a chunk (two chunks in flight)
+    struct {
+        float2 ey[2][DT], ez[2][DT], fy[2][DT], fz[2][DT];   // [x pair][.]
+        float g[DT][DT];
+    } mx[2];
+    ulonglong2 sum[16][BTH];          // float pairs {high, low} of the thread's 16 accumulators
+};
+
+// 1.5 2^k with 2^(k-1) above b (a thousandth above the true bound).
+__device__ __forceinline__ f2 bias_of(f2 b) {
+    float x, y;
+    upk(b, x, y);
+    auto one = [](float v) {
+        const unsigned e = min(__float_as_uint(v * 1.001f) & 0x7F800000u, 0x7D800000u);
+        return __uint_as_float(e + 0x01400000u);
+    };
+    return pk(one(x), one(y));
+}
+__device__ __forceinline__ f2 max2(f2 a, f2 b) {
+    float a0, a1, b0, b1;
+    upk(a, a0, a1);
+    upk(b, b0, b1);
+    return pk(fmaxf(a0, b0), fmaxf(a1, b1));
+}
+
+// t = E^XY F^XZ + F^XY E^XZ for one Y and two Z (float pairs .x + .y), s the
+// biases of both products.  Both Z are taken operation by operation:
+// neighbours share an operand, which the register caches then keep (measured
+// 5.14 -> 4.93 ms at P = 200, 200 X, 600 grid points).
+__device__ __forceinline__ void bias_dot2(ulonglong2 ey, ulonglong2 fy, const ulonglong2 (&ez)[2],
+                                          const ulonglong2 (&fz)[2], const f2 (&s)[2], f2 (&th)[2],
+                                          f2 (&tl)[2]) {
+    f2 z1[2], z2[2], r1[2], r2[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) z1[j] = fma2(ey.x, fz[j].x, s[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) z2[j] = fma2(fy.x, ez[j].x, s[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        z1[j] = sub2(s[j], z1[j]);
+        z2[j] = sub2(s[j], z2[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) r1[j] = fma2(ey.x, fz[j].x, z1[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) r2[j] = fma2(fy.x, ez[j].x, z2[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) r1[j] = fma2(ey.x, fz[j].y, r1[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) r2[j] = fma2(fy.x, ez[j].y, r2[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) r1[j] = fma2(ey.y, fz[j].x, r1[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) r2[j] = fma2(fy.y, ez[j].x, r2[j]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        th[j] = neg2(add2(z1[j], z2[j]));
+        tl[j] = add2(r1[j], r2[j]);
+    }
+}
+
+struct BiasAcc {
+    unsigned i0, i1;   // sums of the bits of s, per lane
+    f2 lo;             // remainders and low-order products
+};
+
+// Both mirror outputs of a unit, operation by operation.
+__device__ __forceinline__ void bias_acc(BiasAcc& a, BiasAcc& b, f2 th, f2 tl, f2 gH, f2 gL, f2 kH,
+                                         f2 kL, f2 c) {
+    const f2 s = fma2(th, gH, c), t = fma2(th, kH, c);
+    const f2 y = sub2(c, s), z = sub2(c, t);
+    f2 p = fma2(th, gH, y), q = fma2(th, kH, z);
+    p = fma2(th, gL, p);
+    q = fma2(th, kL, q);
+    p = fma2(tl, gH, p);
+    q = fma2(tl, kH, q);
+    a.i0 += (unsigned)s;
+    a.i1 += (unsigned)(s >> 32);
+    b.i0 += (unsigned)t;
+    b.i1 += (unsigned)(t >> 32);
+    a.lo = add2(a.lo, p);
+    b.lo = add2(b.lo, q);
+}
+
+// sum += the accumulator's value after n points under bias c; clears it.
+__device__ __forceinline__ void bias_fold(BiasAcc& a, f2 c, unsigned n, ulonglong2& sum) {
+    const unsigned c0 = (unsigned)c, c1 = (unsigned)(c >> 32);
+    const int d0 = (int)(a.i0 - n * c0), d1 = (int)(a.i1 - n * c1);
+    // (s - c) / u summed: |d| < 2^31 as two exact floats, high 20 and low 12 bits
+    f2 dh = (f2)(0x4B400000u + (unsigned)(d0 >> 12)) | (f2)(0x4B400000u + (unsigned)(d1 >> 12)) << 32;
+    f2 dl = (f2)(0x4B000000u | (d0 & 4095)) | (f2)(0x4B000000u | (d1 & 4095)) << 32;
+    dh = sub2(dh, pk(12582912.f, 12582912.f));
+    dl = sub2(dl, pk(8388608.f, 8388608.f));
+    const f2 p = c & 0x7F8000007F800000ull;   // 2^k = 2^23 u
+    const f2 A = prod2(prod2(dh, pk(0x1p-11f, 0x1p-11f)), p);
+    const f2 B = prod2(prod2(dl, pk(0x1p-23f, 0x1p-23f)), p);
+    const f2 vh = add2(A, B);
+    const f2 vl = sub2(B, sub2(vh, A));       // |A| >= |B| or A = 0
+    const f2 S = sum.x;
+    const f2 t = add2(S, vh);                 // TwoSum(S, vh)
+    const f2 z = sub2(t, S);
+    const f2 e = add2(sub2(S, sub2(t, z)), sub2(vh, z));
+    const f2 l = add2(add2(sum.y, e), add2(vl, a.lo));
+    const f2 hi = add2(t, l);                 // renormalise
+    sum.x = hi;
+    sum.y = sub2(l, sub2(hi, t));
+    a.i0 = a.i1 = 0u;
+    a.lo = 0ull;
+}
+
+// Copy bytes (4, 8 or 16) global -> shared, the last `bytes - n` of them zeros.
+template <int BYTES>
+__device__ __forceinline__ void cp_n(void* dst, const void* src, int n) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n));
+    else if (BYTES == 8)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n));
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n));
+}
+
+// Grid as k_triangle_df.  ME, MF: bounds [chunk][x pair][P] (lanes x, x + 1);
+// MG: [chunk][P][P], symmetric.  EVEN: P is even, rows of G start on 16-byte
+// boundaries and are copied two columns at a time.
+// A packed FMA of three distinct register pairs measures 3.3 cycles of a
+// scheduler on GB300 and a packed addition 2.3 (peak: 2): the operations here
+// are bound by register reads, 138 per unit of two X and two mirror outputs
+// against 208 in the TwoSum form, so what comes besides them counts.  The copy
+// addresses advance by constants, which is why a thread copies a two-column
+// piece of two rows of every G tile and one element of E and of F.  P = 400,
+// 400 rows X, 1200 grid points: 58.8 ms (the TwoSum kernel 68.7); P = 200, 200
+// X, 600 points 4.93 ms (5.75).  512 threads of half the outputs: 5.30.
+template <bool EVEN>
+__global__ void __launch_bounds__(BTH, 1)
+    k_triangle_bias(double* H, const float4* E4, const float4* F4, const float2* G2,
+                    const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI) {
+    extern __shared__ __align__(16) unsigned char df_raw[];
+    BiasSmem& sm = *reinterpret_cast<BiasSmem*>(df_raw);
+    const int nb = (P + DT - 1) / DT;
+    int pidx = blockIdx.y, Yb = 0;
+    while (pidx >= nb - Yb) {
+        pidx -= nb - Yb;
+        ++Yb;
+    }
+    const int Zb = Yb + pidx;
+    const int Y0 = Yb * DT, Z0 = Zb * DT, X0 = blockIdx.x * DX;
+    const int nXp = (nX + 1) / 2, xp0 = X0 / 2;
+    const bool diag = Yb == Zb;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const long long PP = (long long)P * P, XP = (long long)nXp * P;
+
+    // Copies of this thread: columns 2 tx, 2 tx + 1 of rows ty and ty + 16 of
+    // both G tiles for every grid point, and one column of one row of E and of
+    // F per stage.
+    const char *g1p, *g2p, *ep, *fp;
+    int g1n[2], g2n[2], en;   // bytes inside the array
+    const long long row16 = 16LL * P * 8;
+    {
+        const int c1 = Z0 + 2 * tx, c2 = Y0 + 2 * tx;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            g1n[q] = Y0 + ty + 16 * q < P ? 8 * max(0, min(2, P - c1)) : 0;
+            g2n[q] = Z0 + ty + 16 * q < P ? 8 * max(0, min(2, P - c2)) : 0;
+        }
+        g1p = reinterpret_cast<const char*>(G2 + (g1n[0] ? (long long)(Y0 + ty) * P + c1 : 0));
+        g2p = reinterpret_cast<const char*>(G2 + (g2n[0] ? (long long)(Z0 + ty) * P + c2 : 0));
+    }
+    // warp w: Z side (or Y), grid point cs of the stage, X pair cx
+    const int w = tid >> 5, c = tid & 31;
+    const int cz = (w >> 2) & 1, cs = (w >> 1) & 1, cx = w & 1;
+    const char *mp, *np;      // the bounds of the same elements, per chunk
+    {
+        const int col = (cz ? Z0 : Y0) + c;
+        const bool ok = xp0 + cx < nXp && col < P;
+        const long long at = ok ? (long long)(xp0 + cx) * P + col : 0;
+        en = ok ? 16 : 0;
+        const long long first = cs < nI ? cs * XP * 16 : 0;
+        ep = reinterpret_cast<const char*>(E4 + at) + first;
+        fp = reinterpret_cast<const char*>(F4 + at) + first;
+        mp = reinterpret_cast<const char*>(ME + at);
+        np = reinterpret_cast<const char*>(MF + at);
+    }
+    const int gsw = 2 * (tx ^ ty);
+    auto load = [&](int k, int b) {
+        const int I0 = k * BS;
+        auto& st = sm.st[b];
+        const bool whole = I0 + BS <= nI;   // else the grid points beyond are zeros
+#pragma unroll
+        for (int s = 0; s < BS; ++s)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const bool in = whole || I0 + s < nI;
+                const int n1 = in ? g1n[q] : 0, n2 = in ? g2n[q] : 0;
+                const char* p1 = n1 ? g1p + s * PP * 8 + q * row16 : reinterpret_cast<const char*>(G2);
+                const char* p2 = n2 ? g2p + s * PP * 8 + q * row16 : reinterpret_cast<const char*>(G2);
+                if (EVEN) {
+                    cp_n<16>(&st.g1[s][ty + 16 * q][gsw], p1, n1);
+                    cp_n<16>(&st.g2[s][ty + 16 * q][gsw], p2, n2);
+                } else {
+                    cp_n<8>(&st.g1[s][ty + 16 * q][gsw], p1, min(n1, 8));
+                    cp_n<8>(&st.g1[s][ty + 16 * q][gsw + 1], n1 > 8 ? p1 + 8 : p1, max(n1 - 8, 0));
+                    cp_n<8>(&st.g2[s][ty + 16 * q][gsw], p2, min(n2, 8));
+                    cp_n<8>(&st.g2[s][ty + 16 * q][gsw + 1], n2 > 8 ? p2 + 8 : p2, max(n2 - 8, 0));
+                }
+            }
+        {
+            const bool in = whole || I0 + cs < nI;
+            cp_n<16>(cz ? &st.ez[cs][cx][c] : &st.ey[cs][cx][c],
+                     in ? ep : reinterpret_cast<const char*>(E4), in ? en : 0);
+            cp_n<16>(cz ? &st.fz[cs][cx][c] : &st.fy[cs][cx][c],
+                     in ? fp : reinterpret_cast<const char*>(F4), in ? en : 0);
+        }
+        // the chunk's bounds with its first stage
+        if (I0 % BC == 0) {
+            auto& mx = sm.mx[(I0 / BC) & 1];
+            if (cs == 0) {
+                cp_n<8>(cz ? &mx.ez[cx][c] : &mx.ey[cx][c], mp, en / 2);
+                cp_n<8>(cz ? &mx.fz[cx][c] : &mx.fy[cx][c], np, en / 2);
+            }
+            mp += XP * 8;
+            np += XP * 8;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float* m = MG + I0 / BC * PP +
+                                 (g1n[q] ? (long long)(Y0 + ty + 16 * q) * P + Z0 + 2 * tx : 0);
+                cp_n<4>(&mx.g[ty + 16 * q][2 * tx], m, min(g1n[q] / 2, 4));
+                cp_n<4>(&mx.g[ty + 16 * q][2 * tx + 1], g1n[q] > 8 ? m + 1 : m, max(g1n[q] / 2 - 4, 0));
+            }
+        }
+        g1p += BS * PP * 8;
+        g2p += BS * PP * 8;
+        ep += BS * XP * 16;
+        fp += BS * XP * 16;
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+
+    // [x pair][i][j]: H^XYZ and H^XZY, Y = ty + 16 i, Z = tx + 16 j
+    BiasAcc h1[2][2][2], h2[2][2][2];
+    f2 sg[2][2][2], cb[2][2][2];   // biases of t's products and of t G
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                h1[a][i][j] = BiasAcc{0u, 0u, 0ull};
+                h2[a][i][j] = BiasAcc{0u, 0u, 0ull};
+                sg[a][i][j] = cb[a][i][j] = 0ull;
+                sm.sum[(a * 4 + i * 2 + j) * 2][tid] = make_ulonglong2(0ull, 0ull);
+                sm.sum[(a * 4 + i * 2 + j) * 2 + 1][tid] = make_ulonglong2(0ull, 0ull);
+            }
+    auto fold = [&](unsigned n) {
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int u = (a * 4 + i * 2 + j) * 2;
+                    bias_fold(h1[a][i][j], cb[a][i][j], n, sm.sum[u][tid]);
+                    bias_fold(h2[a][i][j], cb[a][i][j], n, sm.sum[u + 1][tid]);
+                }
+    };
+    const int nsteps = (nI + BS - 1) / BS;
+#pragma unroll
+    for (int k = 0; k < BST - 1; ++k) {
+        if (k < nsteps) load(k, k);
+        else asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    int inchunk = 0;   // grid points summed under the present biases
+    int b = 0;         // stage of step k
+    for (int k = 0; k < nsteps; ++k) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(BST - 2) : "memory");
+        __syncthreads();   // stage k is there, stage k - 1 is free
+        if (k + BST - 1 < nsteps) load(k + BST - 1, b == 0 ? BST - 1 : b - 1);
+        else asm volatile("cp.async.commit_group;\n" ::: "memory");
+        if (k * BS % BC == 0) {
+            if (k > 0) fold((unsigned)inchunk);
+            inchunk = 0;
+            const auto& mx = sm.mx[(k * BS / BC) & 1];
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const f2 ey = reinterpret_cast<const f2&>(mx.ey[a][ty + 16 * i]);
+                        const f2 fy = reinterpret_cast<const f2&>(mx.fy[a][ty + 16 * i]);
+                        const f2 ez = reinterpret_cast<const f2&>(mx.ez[a][tx + 16 * j]);
+                        const f2 fz = reinterpret_cast<const f2&>(mx.fz[a][tx + 16 * j]);
+                        const float g = mx.g[ty + 16 * i][tx + 16 * j];
+                        const f2 p1 = prod2(ey, fz), p2 = prod2(ez, fy);
+                        sg[a][i][j] = bias_of(max2(p1, p2));
+                        cb[a][i][j] = bias_of(prod2(add2(p1, p2), pk(g, g)));
+                    }
+        }
+        const auto& cur = sm.st[b];
+#pragma unroll
+        for (int st = 0; st < BS; ++st) {
+            // G^(Y_i, Z_j) and G^(Z_j, Y_i), the same value in both lanes
+            f2 g1h[2][2], g1l[2][2], g2h[2][2], g2l[2][2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float2 u = cur.g1[st][ty + 16 * i][2 * ((tx / 2 + 8 * j) ^ ty) + (tx & 1)];
+                    const float2 v = cur.g2[st][tx + 16 * j][2 * ((ty / 2 + 8 * i) ^ tx) + (ty & 1)];
+                    g1h[i][j] = pk(u.x, u.x);
+                    g1l[i][j] = pk(u.y, u.y);
+                    g2h[i][j] = pk(v.x, v.x);
+                    g2l[i][j] = pk(v.y, v.y);
+                }
+#pragma unroll
+            for (int xp = 0; xp < 2; ++xp) {
+                ulonglong2 ey[2], fy[2], ez[2], fz[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    ey[i] = reinterpret_cast<const ulonglong2&>(cur.ey[st][xp][ty + 16 * i]);
+                    fy[i] = reinterpret_cast<const ulonglong2&>(cur.fy[st][xp][ty + 16 * i]);
+                    ez[i] = reinterpret_cast<const ulonglong2&>(cur.ez[st][xp][tx + 16 * i]);
+                    fz[i] = reinterpret_cast<const ulonglong2&>(cur.fz[st][xp][tx + 16 * i]);
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    f2 th[2], tl[2];
+                    bias_dot2(ey[i], fy[i], ez, fz, sg[xp][i], th, tl);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        bias_acc(h1[xp][i][j], h2[xp][i][j], th[j], tl[j], g1h[i][j], g1l[i][j],
+                                 g2h[i][j], g2l[i][j], cb[xp][i][j]);
+                }
+            }
+        }
+        inchunk += BS;
+        b = b + 1 == BST ? 0 : b + 1;
+    }
+    if (nsteps > 0) fold((unsigned)inchunk);
+    // On a diagonal pair both accumulators cover the same tile and count
+    // every (Y, Z) twice.
+    const double scale = diag ? 0.5 : 1.0;
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        if (m == 1 && diag) __syncthreads();   // mirror targets overlap other threads' first targets
+#pragma unroll
+        for (int xp = 0; xp < 2; ++xp)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int Y = Y0 + ty + 16 * i, Z = Z0 + tx + 16 * j;
+                    if (Y >= P || Z >= P) continue;
+                    const ulonglong2 v = sm.sum[(xp * 4 + i * 2 + j) * 2 + m][tid];
+                    float a0, a1, b0, b1;
+                    upk(v.x, a0, a1);
+                    upk(v.y, b0, b1);
+                    const int x = X0 + 2 * xp;
+                    const long long at = m == 0 ? (long long)Y * P + Z : (long long)Z * P + Y;
+                    if (x < nX) H[x * PP + at] += scale * ((double)a0 + (double)b0);
+                    if (x + 1 < nX) H[(x + 1) * PP + at] += scale * ((double)a1 + (double)b1);
+                }
+    }
+}
+
+// M[chunk][Y][Z] = max over the chunk's grid points of |G_h^YZ| and |G_h^ZY|.
+// Block: one 32 x 32 tile and its mirror (grid x: tile pairs, y: chunks).
+__global__ void __launch_bounds__(256) k_pair_max(const float2* G2, int nI, int P, float* M) {
+    __shared__ float t1[32][33], t2[32][33];
+    const int nb = (P + 31) / 32;
+    int pidx = blockIdx.x, Yb = 0;
+    while (pidx >= nb - Yb) {
+        pidx -= nb - Yb;
+        ++Yb;
+    }
+    const int Y0 = Yb * 32, Z0 = (Yb + pidx) * 32, ch = blockIdx.y;
+    const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+    const long long PP = (long long)P * P;
+    const int lo = ch * BC, hi = min(nI, lo + BC);
+    for (int r = r0; r < 32; r += 8) {
+        float a = 0.f, b = 0.f;
+        const bool ok1 = Y0 + r < P && Z0 + c < P, ok2 = Z0 + r < P && Y0 + c < P;
+        for (int I = lo; I < hi; ++I) {
+            if (ok1) a = fmaxf(a, fabsf(G2[I * PP + (long long)(Y0 + r) * P + Z0 + c].x));
+            if (ok2) b = fmaxf(b, fabsf(G2[I * PP + (long long)(Z0 + r) * P + Y0 + c].x));
+        }
+        t1[r][c] = a;
+        t2[r][c] = b;
+    }
+    __syncthreads();
+    for (int r = r0; r < 32; r += 8) {
+        if (Y0 + r < P && Z0 + c < P)
+            M[ch * PP + (long long)(Y0 + r) * P + Z0 + c] = fmaxf(t1[r][c], t2[c][r]);
+        if (Z0 + r < P && Y0 + c < P)
+            M[ch * PP + (long long)(Z0 + r) * P + Y0 + c] = fmaxf(t2[r][c], t1[c][r]);
+    }
+}
+
 // {h, l} = {fl32(d), fl32(d - fl32(d))}.  The float64 form takes four
 // float64-pipe operations (1/64 of the float32 rate on GB300: it kept the
 // split kernels' float64 pipe 88 % busy), so for 2^-60 <= |d| < 2^60 the
@@ -363,23 +800,31 @@ __device__ __forceinline__ void split1(double d, float& h, float& l) {
 }
 
 // One block per output row (I, q) at a time, threads along the P columns
-// (no 64-bit division per element).
-__global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* out) {
-    const int nXp = (nX + 1) / 2;
-    const long long rows = (long long)nI * nXp;
+// (no 64-bit division per element).  With M, a block takes the rows of one q
+// for the BC grid points of a chunk and also writes the largest |h| of every
+// column, M[chunk][q][P].
+__global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* out, float2* M) {
+    const int nXp = (nX + 1) / 2, per = M ? BC : 1;
+    const long long rows = (long long)((nI + per - 1) / per) * nXp;
     for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const long long I = row / nXp;
-        const int x = 2 * (int)(row - I * nXp);
-        const double* e0 = E + (I * nX + x) * P;
-        float4* o = out + row * P;
+        const long long ch = row / nXp;
+        const int q = (int)(row - ch * nXp), x = 2 * q;
+        const int lo = (int)ch * per, hi = min(nI, lo + per);
         const bool two = x + 1 < nX;
         for (int c = threadIdx.x; c < P; c += blockDim.x) {
-            const double d0 = e0[c];
-            const double d1 = two ? e0[P + c] : 0.0;
-            float h0, l0, h1, l1;
-            split1(d0, h0, l0);
-            split1(d1, h1, l1);
-            o[c] = make_float4(h0, h1, l0, l1);
+            float m0 = 0.f, m1 = 0.f;
+            for (int I = lo; I < hi; ++I) {
+                const double* e0 = E + ((long long)I * nX + x) * P;
+                const double d0 = e0[c];
+                const double d1 = two ? e0[P + c] : 0.0;
+                float h0, l0, h1, l1;
+                split1(d0, h0, l0);
+                split1(d1, h1, l1);
+                out[((long long)I * nXp + q) * P + c] = make_float4(h0, h1, l0, l1);
+                m0 = fmaxf(m0, fabsf(h0));
+                m1 = fmaxf(m1, fabsf(h1));
+            }
+            if (M) M[row * P + c] = make_float2(m0, m1);
         }
     }
 }
@@ -401,13 +846,20 @@ unsigned grid_for(long long n) {
 
 }  // namespace
 
-cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out,
+cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, float2* bounds,
                            cudaStream_t s) {
-    const long long n = (long long)nI * ((nX + 1) / 2) * P;
-    if (n <= 0) return cudaSuccess;
-    const long long rows = (long long)nI * ((nX + 1) / 2);
-    k_split_pairs<<<(unsigned)std::min<long long>(rows, 152LL * 16), 128, 0, s>>>(E, nI, nX, P,
-                                                                               out);
+    if (nI <= 0 || nX <= 0 || P <= 0) return cudaSuccess;
+    const long long rows = (long long)(bounds ? cdiv(nI, BC) : nI) * ((nX + 1) / 2);
+    k_split_pairs<<<(unsigned)std::min<long long>(rows, 152LL * 16), 128, 0, s>>>(E, nI, nX, P, out,
+                                                                                  bounds);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t pair_max(const float2* G2, int nI, int P, float* M, cudaStream_t s) {
+    if (nI <= 0 || P <= 0) return cudaSuccess;
+    const unsigned nb = cdiv(P, 32);
+    k_pair_max<<<dim3(nb * (nb + 1) / 2, cdiv(nI, BC)), 256, 0, s>>>(G2, nI, P, M);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -419,15 +871,25 @@ cudaError_t split_df(const double* in, long long n, float2* out, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2, int P,
-                        int nX, int nI, cudaStream_t s) {
+cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
+                        const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
+                        cudaStream_t s) {
     if (nX <= 0 || nI <= 0) return cudaSuccess;
     const unsigned nb = cdiv(P, DT);
-    const int smem = (int)(2 * sizeof(DfStage));
-    cudaError_t e = smem_optin((const void*)k_triangle_df, smem);
+    const bool bias = ME && MF && MG, even = P % 2 == 0;
+    const void* kern = !bias ? (const void*)k_triangle_df
+                             : (even ? (const void*)k_triangle_bias<true>
+                                     : (const void*)k_triangle_bias<false>);
+    const int smem = (int)(bias ? sizeof(BiasSmem) : 2 * sizeof(DfStage));
+    cudaError_t e = smem_optin(kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid(cdiv(nX, DX), nb * (nb + 1) / 2);
-    k_triangle_df<<<grid, DTH, smem, s>>>(H, E4, F4, G2, P, nX, nI);
+    if (bias && even)
+        k_triangle_bias<true><<<grid, BTH, smem, s>>>(H, E4, F4, G2, ME, MF, MG, P, nX, nI);
+    else if (bias)
+        k_triangle_bias<false><<<grid, BTH, smem, s>>>(H, E4, F4, G2, ME, MF, MG, P, nX, nI);
+    else
+        k_triangle_df<<<grid, DTH, smem, s>>>(H, E4, F4, G2, P, nX, nI);
     count_launches(1);
     return cudaGetLastError();
 }
