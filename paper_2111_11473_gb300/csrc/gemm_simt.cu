@@ -393,8 +393,10 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
     if constexpr (std::is_same<T, double>::value) {
         // Both kernels by the FP64 cycles of the SM (or scheduler) that gets
         // the most: a tile kernel's block takes BM BN / 2 cycles per K index
-        // with its padding, a warp of the other 64 (it also reads its operands
-        // from L1 and L2, so that it has to be a tenth better).
+        // with its padding, a warp of the other 64.  The latter also reads its
+        // operands from L1 and L2: it has to be a tenth better, and half where
+        // the operands are long (400 x 400 x 240000: 138 against 177 million
+        // cycles here, but 10 % slower).
         const long long Kt = (long long)g.K * (g.reduce ? g.batch : 1);
         const long long sms = device_sms(), nb = g.reduce ? 1 : g.batch;
         const long long chunk = (ksteps + splits - 1) / splits * BK;
@@ -416,7 +418,9 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
                                   ((Kt + parts - 1) / parts) * 64 +
                               (gs > 1 ? 6000.0 : 0.0);
         const long long blocks = (wt + kWarpsPerBlock / S - 1) / (kWarpsPerBlock / S);
-        if (g.K > 0 && blocks <= INT32_MAX && (g.M == 1 || t_warp * 1.1 < t_tile)) {
+        const double fmas = (double)g.M * g.N * nb * Kt;
+        if (g.K > 0 && blocks <= INT32_MAX &&
+            (g.M == 1 || t_warp * (fmas < 1e9 ? 1.1 : 1.5) < t_tile)) {
             g.splits = gs;
             const dim3 wgrid((unsigned)blocks, (unsigned)gs);
             if (WM == 1)

@@ -2,6 +2,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -17,6 +18,12 @@ inline unsigned nblocks(long long n) {
     if (b > 152LL * 64) b = 152LL * 64;   // grid-stride beyond 64 blocks per SM
     return (unsigned)(b < 1 ? 1 : b);
 }
+
+// Blocks and threads of kernels whose blocks take whole rows of P elements.
+inline unsigned row_blocks(long long rows) {
+    return (unsigned)std::max<long long>(1, std::min<long long>(rows, 152LL * 64));
+}
+inline unsigned row_threads(int P) { return (unsigned)std::min(NT, (P + 31) / 32 * 32); }
 
 template <typename T>
 __global__ void k_split(const T* full, int nb, int o, int v, Blocks<T> out) {
@@ -101,15 +108,33 @@ __global__ void k_to_double(const T* in, double* out, long long n) {
 template <typename T>
 __global__ void k_alg1(const T* Bbar, const T* Btil, const T* oo, const T* vv,
                        T* C1, T* Ccross, int P, int nb) {
+    // HBM bound: U vectors' loads in flight per thread (one at a time took 0.65
+    // ms for 600 vectors at P = 400 in float64, of which the bytes take 0.34)
+    constexpr int U = 8;
     const long long PP = (long long)P * P;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < PP;
          idx += (long long)gridDim.x * blockDim.x) {
         const int X = (int)(idx / P), Y = (int)(idx % P);
         const T wo = oo[idx], wv = vv[idx];
         T cross = Ccross[idx];
-        for (int a = 0; a < nb; ++a) {
+        T* out = C1 + (long long)X * nb * P + Y;
+        int a = 0;
+        for (; a + U <= nb; a += U) {
+            T bb[U], bt[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                bb[u] = __ldcs(Bbar + (a + u) * PP + idx);
+                bt[u] = __ldcs(Btil + (a + u) * PP + idx);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                out[(long long)(a + u) * P] = wv * bb[u] - wo * bt[u];
+                cross += bb[u] * bt[u];
+            }
+        }
+        for (; a < nb; ++a) {
             const T bb = Bbar[a * PP + idx], bt = Btil[a * PP + idx];
-            C1[((long long)X * nb + a) * P + Y] = wv * bb - wo * bt;
+            out[(long long)a * P] = wv * bb - wo * bt;
             cross += bb * bt;
         }
         Ccross[idx] = cross;
@@ -133,15 +158,18 @@ __global__ void k_diag_reduce(const T* y, const T* M, int R, int P, int nb, T* o
 template <typename T>
 __global__ void k_w_single(const T* TA, int ldta, const T* Tc, const T* E, T* W, int P,
                            int nb) {
-    const long long PP = (long long)P * P, total = PP * nb;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int a = (int)(idx / PP);
-        const long long e = idx % PP;
-        const int Y = (int)(e / P), Z = (int)(e % P);
-        T w = -Tc[e] * E[idx];
-        if (Y == Z) w += T(2) * TA[(long long)Y * ldta + a];
-        W[idx] = w;
+    // one row Y of one vector per block turn: no 64-bit division per element
+    const long long PP = (long long)P * P, rows = (long long)P * nb;
+    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
+        const int a = (int)(row / P), Y = (int)(row % P);
+        const T* t = Tc + (long long)Y * P;
+        const T* e = E + a * PP + (long long)Y * P;
+        T* w = W + a * PP + (long long)Y * P;
+        for (int Z = threadIdx.x; Z < P; Z += blockDim.x) {
+            T v = -t[Z] * e[Z];
+            if (Y == Z) v += T(2) * TA[(long long)Y * ldta + a];
+            w[Z] = v;
+        }
     }
 }
 
@@ -177,10 +205,13 @@ __global__ void k_hadamard2(T* out, long long n, const T* a, const T* b, const T
 
 template <typename T>
 __global__ void k_hadamard_batched(T* M, const T* z, long long per, int nb) {
-    const long long total = per * nb;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x)
-        M[i] *= z[i % per];
+    // grid y: batches; grid x: elements of one
+    for (int b = blockIdx.y; b < nb; b += gridDim.y) {
+        T* m = M + b * per;
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per;
+             i += (long long)gridDim.x * blockDim.x)
+            m[i] *= z[i];
+    }
 }
 
 template <typename T>
@@ -198,19 +229,20 @@ __global__ void k_kr(const T* A, const T* B, int na, int nbr, int P, T* out) {
 template <typename T>
 __global__ void k_scale_rows(const T* y, int R, int P, const T* w, int x0, int nx,
                              T* out) {
-    const long long per = (long long)R * P, total = per * nx;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(idx / per);
-        const long long e = idx % per;
-        const int Y = (int)(e % P);
-        out[idx] = y[e] * w[(long long)(x0 + x) * P + Y];
+    // one row of one x per block turn: no 64-bit division per element
+    const long long rows = (long long)R * nx;
+    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
+        const int x = (int)(row / R), r = (int)(row % R);
+        const T* a = y + (long long)r * P;
+        const T* b = w + (long long)(x0 + x) * P;
+        T* o = out + row * P;
+        for (int Y = threadIdx.x; Y < P; Y += blockDim.x) o[Y] = a[Y] * b[Y];
     }
 }
 
 // Tile of the float64 triangle kernel: TXB amplitude indices X and a pair of
 // TYZ x TYZ (Y, Z) tiles per block.
-constexpr int TXB = 4, TYZ = 32;
+constexpr int TXB = 4;
 
 // Float32 triangle kernel.  A block owns a 32 x 32 x 32 (X, Y, Z) tile of H;
 // lane = X, and the 16 warps form a 4 x 4 grid of 8 x 8 (Y, Z) register tiles.
@@ -227,6 +259,7 @@ constexpr int TXB = 4, TYZ = 32;
 // halved and added one after the other.
 constexpr int SIST = 2;
 
+template <int TYZ>
 struct TriSym64Stage {
     double g1[SIST][TYZ][TYZ + 1];   // G^YZ, rows Y
     double g2[SIST][TYZ][TYZ + 1];   // G^ZY, rows Z
@@ -241,7 +274,8 @@ __device__ __forceinline__ void cp_async8(double* dst, const double* src, bool o
 }
 
 // Stage grid points I0 .. I0 + SIST - 1 of the block's tiles (zeros outside).
-__device__ __forceinline__ void sym64_load(TriSym64Stage& st, const double* E, const double* F,
+template <int TYZ>
+__device__ __forceinline__ void sym64_load(TriSym64Stage<TYZ>& st, const double* E, const double* F,
                                            const double* G, int P, int nX, int nI, int I0,
                                            int X0, int Y0, int Z0) {
     const long long PP = (long long)P * P, XP = (long long)nX * P;
@@ -276,11 +310,16 @@ __device__ __forceinline__ void sym64_load(TriSym64Stage& st, const double* E, c
 // accumulators land on the same tile, count every element twice, and are
 // halved and added one after the other.  Operands of the next pair of grid
 // points are staged with cp.async while the current pair is computed.
+// Tiles of TYZ = 32 (2 x 2 (Y, Z) per thread) or 16 (one each) for sizes whose
+// 32-wide tiles leave SMs without a block: the FP64 pipe of an SM bounds a
+// block (P = 60, 120 grid points: 45 blocks 574 us, 150 blocks of 16 -> 149).
+template <int TYZ>
 __global__ void __launch_bounds__(256) k_triangle_sym64(double* H, const double* E,
-                                                        const double* F, const double* G,
-                                                        int P, int nX, int nI) {
+                                                            const double* F, const double* G,
+                                                            int P, int nX, int nI) {
+    constexpr int R = TYZ / 16;
     extern __shared__ __align__(16) unsigned char sym64_raw[];
-    TriSym64Stage* stg = reinterpret_cast<TriSym64Stage*>(sym64_raw);
+    auto* stg = reinterpret_cast<TriSym64Stage<TYZ>*>(sym64_raw);
     const int nb = (P + TYZ - 1) / TYZ;
     int pidx = blockIdx.x, Yb = 0;
     while (pidx >= nb - Yb) {
@@ -291,17 +330,17 @@ __global__ void __launch_bounds__(256) k_triangle_sym64(double* H, const double*
     const int Y0 = Yb * TYZ, Z0 = Zb * TYZ, X0 = blockIdx.y * TXB;
     const bool diag = Yb == Zb;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    double a1[TXB][2][2], a2[TXB][2][2];
+    double a1[TXB][R][R], a2[TXB][R][R];
 #pragma unroll
     for (int x = 0; x < TXB; ++x)
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < R; ++i)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) a1[x][i][j] = a2[x][i][j] = 0;
+            for (int j = 0; j < R; ++j) a1[x][i][j] = a2[x][i][j] = 0;
     const int nsteps = (nI + SIST - 1) / SIST;
     if (nsteps > 0) sym64_load(stg[0], E, F, G, P, nX, nI, 0, X0, Y0, Z0);
     for (int k = 0; k < nsteps; ++k) {
-        const TriSym64Stage& cur = stg[k & 1];
+        const auto& cur = stg[k & 1];
         if (k + 1 < nsteps) {
             sym64_load(stg[(k + 1) & 1], E, F, G, P, nX, nI, (k + 1) * SIST, X0, Y0, Z0);
             asm volatile("cp.async.wait_group 1;\n" ::: "memory");
@@ -311,28 +350,28 @@ __global__ void __launch_bounds__(256) k_triangle_sym64(double* H, const double*
         __syncthreads();
 #pragma unroll
         for (int st = 0; st < SIST; ++st) {
-            double g1[2][2], g2[2][2];
+            double g1[R][R], g2[R][R];
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                for (int j = 0; j < R; ++j) {
                     g1[i][j] = cur.g1[st][ty + 16 * i][tx + 16 * j];   // G^(Y_i, Z_j)
                     g2[i][j] = cur.g2[st][tx + 16 * j][ty + 16 * i];   // G^(Z_j, Y_i)
                 }
 #pragma unroll
             for (int x = 0; x < TXB; ++x) {
-                double ey[2], fy[2], ez[2], fz[2];
+                double ey[R], fy[R], ez[R], fz[R];
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
+                for (int i = 0; i < R; ++i) {
                     ey[i] = cur.ey[st][x][ty + 16 * i];
                     fy[i] = cur.fy[st][x][ty + 16 * i];
                     ez[i] = cur.ez[st][x][tx + 16 * i];
                     fz[i] = cur.fz[st][x][tx + 16 * i];
                 }
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                for (int i = 0; i < R; ++i)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
+                    for (int j = 0; j < R; ++j) {
                         double t = ey[i] * fz[j];
                         t = fma(ez[j], fy[i], t);
                         a1[x][i][j] = fma(t, g1[i][j], a1[x][i][j]);
@@ -348,11 +387,11 @@ __global__ void __launch_bounds__(256) k_triangle_sym64(double* H, const double*
         const int X = X0 + x;
         if (X >= nX) continue;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < R; ++i) {
             const int Y = Y0 + ty + 16 * i;
             if (Y >= P) continue;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < R; ++j) {
                 const int Z = Z0 + tx + 16 * j;
                 if (Z < P) H[((long long)X * P + Y) * P + Z] += scale * a1[x][i][j];
             }
@@ -364,11 +403,11 @@ __global__ void __launch_bounds__(256) k_triangle_sym64(double* H, const double*
         const int X = X0 + x;
         if (X >= nX) continue;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < R; ++i) {
             const int Y = Y0 + ty + 16 * i;
             if (Y >= P) continue;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < R; ++j) {
                 const int Z = Z0 + tx + 16 * j;
                 if (Z < P) H[((long long)X * P + Z) * P + Y] += scale * a2[x][i][j];
             }
@@ -610,7 +649,7 @@ cudaError_t diag_reduce(const T* y, const T* M, int R, int P, int nb, T* out, in
 template <typename T>
 cudaError_t w_single(const T* TA, int ldta, const T* Tc, const T* E, T* W, int P, int nb,
                      cudaStream_t s) {
-    k_w_single<T><<<nblocks((long long)nb * P * P), NT, 0, s>>>(TA, ldta, Tc, E, W, P, nb);
+    k_w_single<T><<<row_blocks((long long)nb * P), row_threads(P), 0, s>>>(TA, ldta, Tc, E, W, P, nb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -640,7 +679,8 @@ cudaError_t hadamard2(T* out, long long n, const T* a, const T* b, const T* c,
 
 template <typename T>
 cudaError_t hadamard_batched(T* M, const T* z, long long per, int nb, cudaStream_t s) {
-    k_hadamard_batched<T><<<nblocks(per * nb), NT, 0, s>>>(M, z, per, nb);
+    const dim3 grid(nblocks(per), (unsigned)std::max(1, std::min(nb, 65535)));
+    k_hadamard_batched<T><<<grid, NT, 0, s>>>(M, z, per, nb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -656,7 +696,7 @@ cudaError_t khatri_rao(const T* A, const T* B, int na, int nbr, int P, T* out,
 template <typename T>
 cudaError_t scale_rows(const T* y, int R, int P, const T* w, int x0, int nx, T* out,
                        cudaStream_t s) {
-    k_scale_rows<T><<<nblocks((long long)R * P * nx), NT, 0, s>>>(y, R, P, w, x0, nx, out);
+    k_scale_rows<T><<<row_blocks((long long)R * nx), row_threads(P), 0, s>>>(y, R, P, w, x0, nx, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -675,12 +715,17 @@ cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, in
         return cudaGetLastError();
     }
     if constexpr (std::is_same<T, double>::value) {
-        const unsigned nb = cdiv(P, TYZ);
-        dim3 grid(nb * (nb + 1) / 2, cdiv(nX, TXB));
-        const int smem = (int)(2 * sizeof(TriSym64Stage));
-        cudaError_t e = smem_optin((const void*)k_triangle_sym64, smem);
+        // Tile by the work of the SM that gets the most, in 16-wide tiles.
+        auto pairs = [&](int t) { const long long nb = cdiv(P, t); return nb * (nb + 1) / 2; };
+        const long long xb = cdiv(nX, TXB), sms = device_sms();
+        const bool small = 1.1 * ((pairs(16) * xb + sms - 1) / sms) < 4.0 * ((pairs(32) * xb + sms - 1) / sms);
+        const dim3 grid((unsigned)pairs(small ? 16 : 32), (unsigned)xb);
+        const int smem = (int)(2 * (small ? sizeof(TriSym64Stage<16>) : sizeof(TriSym64Stage<32>)));
+        cudaError_t e = smem_optin(small ? (const void*)k_triangle_sym64<16>
+                                         : (const void*)k_triangle_sym64<32>, smem);
         if (e != cudaSuccess) return e;
-        k_triangle_sym64<<<grid, 256, smem, s>>>(H, E, F, G, P, nX, nI);
+        if (small) k_triangle_sym64<16><<<grid, 256, smem, s>>>(H, E, F, G, P, nX, nI);
+        else k_triangle_sym64<32><<<grid, 256, smem, s>>>(H, E, F, G, P, nX, nI);
         count_launches(1);
         return cudaGetLastError();
     }
