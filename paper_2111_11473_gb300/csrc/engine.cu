@@ -659,7 +659,9 @@ Err Engine<T>::init_finish() {
     //      orbital) take at most a quarter of the free memory (48 GiB at
     //      most); all P rows in one block when they fit, else the fewest
     //      blocks that do, rounded up to the triangle kernel's 32-row tile.
-    const size_t gall_bytes = (size_t)G * PP * sizeof(T);
+    ldp = std::is_same<T, float>::value && triangle_pair_ok(P) ? (P + 3) / 4 * 4 : P;
+    const long long PL = (long long)P * ldp;   // elements of one G_I or one X of H
+    const size_t gall_bytes = (size_t)G * PL * sizeof(T);
     const bool gall_fits = cfg.workspace_bytes == 0 ? gall_bytes <= (size_t)48 << 30
                                                     : gall_bytes <= cfg.workspace_bytes / 4;
     {
@@ -668,7 +670,7 @@ Err Engine<T>::init_finish() {
                                                     : 48LL << 30;
         if (cfg.workspace_bytes == 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess)
             budget6 = std::min<long long>(budget6, (long long)(free_b / 4));
-        const long long perX = (2 * PP + (long long)(o + v) * P) * TB;
+        const long long perX = (2 * PL + (long long)(o + v) * ldp) * TB;
         if (cfg.x_block6 > 0) {
             x6 = std::min(cfg.x_block6, P);
         } else if (perX * P <= budget6) {
@@ -680,13 +682,13 @@ Err Engine<T>::init_finish() {
         // Grid points per chunk: the E and F chunks take at most 4 GB; a
         // rebuilt G chunk takes a twelfth of the free memory, 4-12 GiB (more
         // grid points per triangle launch: fewer read-modify-writes of H).
-        long long icl = (4LL << 30) / (2LL * x6 * P * TB);
+        long long icl = (4LL << 30) / (2LL * x6 * ldp * TB);
         if (!gall_fits) {
             long long gbudget = 4LL << 30;
             if (cfg.workspace_bytes == 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess)
                 gbudget = std::max<long long>(gbudget, std::min<long long>(
                                                            12LL << 30, (long long)(free_b / 12)));
-            icl = std::min<long long>(icl, gbudget / (PP * TB));
+            icl = std::min<long long>(icl, gbudget / (PL * TB));
         }
         ic = cfg.i_chunk > 0 ? std::min(cfg.i_chunk, G)
                              : (int)std::max<long long>(1, std::min<long long>(G, icl));
@@ -733,9 +735,9 @@ Err Engine<T>::init_finish() {
         if (tri_bias && cfg.i_chunk == 0 && ic < G) ic = std::max(kBiasChunk, ic / kBiasChunk * kBiasChunk);
         tri_bias = tri_bias && (ic >= G || ic % kBiasChunk == 0);
         if (gall_resident) {
-            THC_TRY(Gall.alloc((size_t)G * PP));
-            THC_TRY(mm(P, P, o, tr(yo, P), View<T>{U6.p, (long long)G * P, 1}, Gall.p, P, 1, 0,
-                       G, 0, P, PP));
+            THC_TRY(Gall.alloc((size_t)G * PL));
+            THC_TRY(mm(P, P, o, tr(yo, P), View<T>{U6.p, (long long)G * P, 1}, Gall.p, ldp, 1, 0,
+                       G, 0, P, PL));
             if constexpr (std::is_same<T, double>::value) {
                 // The float64-accurate triangle reads G_I^YZ as float pairs.
                 if (tri_df)
@@ -747,7 +749,7 @@ Err Engine<T>::init_finish() {
                 }
             }
         } else {
-            THC_TRY(Gch.alloc((size_t)ic * PP));
+            THC_TRY(Gch.alloc((size_t)ic * PL));
             if (tri_bias) THC_TRY(MG4.alloc((size_t)cdiv(ic, kBiasChunk) * PP));
         }
         if (tri_df) {
@@ -760,15 +762,14 @@ Err Engine<T>::init_finish() {
                 THC_TRY(MF4.alloc(bounds));
             }
         }
-        const long long xP = (long long)x6 * P;
         // slabs of C_i, D_a, E and F: an even number of rows for the paired triangle
-        const long long xPs = (long long)(tri_pair ? x6 + (x6 & 1) : x6) * P;
+        const long long xPs = (long long)(tri_pair ? x6 + (x6 & 1) : x6) * ldp;
         THC_TRY(A6.alloc(ov * P));
         THC_TRY(C6.alloc((size_t)o * xPs));
         THC_TRY(D6.alloc((size_t)v * xPs));
         THC_TRY(Ech.alloc((size_t)ic * xPs));
         THC_TRY(Fch.alloc((size_t)ic * xPs));
-        THC_TRY(H.alloc((size_t)x6 * PP));
+        THC_TRY(H.alloc((size_t)x6 * PL));
         THC_TRY(M6.alloc((size_t)x6 * o * P));
         THC_TRY(I6.alloc((size_t)x6 * ov));
     } else {
@@ -814,7 +815,7 @@ Err Engine<T>::init_finish() {
     // workspaces are sized from the largest).
     std::vector<Shape> shapes;
     {
-        const long long xP = (long long)(tri_pair ? x6 + (x6 & 1) : x6) * P;
+        const long long xP = (long long)(tri_pair ? x6 + (x6 & 1) : x6) * ldp;
         shapes = {
             {P, P, (long long)kb * P, 1}, {(long long)P * kb, P, P, 1}, {P, P, o, kb},
             {P, P, v, kb}, {v, P, v, kb}, {o, G, v, xb}, {G, G, o, xb}, {o, G, G, xb},
@@ -971,7 +972,7 @@ Err Engine<T>::set_state(const double* Zc, const double* t1in) {
 
 template <typename T>
 Err Engine<T>::alg6(T* sgm) {
-    const long long ov = (long long)o * v, PP = (long long)P * P;
+    const long long ov = (long long)o * v, PL = (long long)P * ldp;
     const T* yo = y.p;
     const T* yv = y.p + (long long)o * P;
     seg_begin(THC_STEP_ALG6_GEMM);
@@ -983,21 +984,21 @@ Err Engine<T>::alg6(T* sgm) {
         const int nX = std::min(x6, x_hi - X0);
         // row slabs of C_i, D_a, E, F: nX rows, or nX rounded up to even
         // with the rows of each pair interleaved for the paired triangle
-        const long long xP = (long long)(tri_pair ? nX + (nX & 1) : nX) * P;
+        const long long xP = (long long)(tri_pair ? nX + (nX & 1) : nX) * ldp;
         seg_begin(THC_STEP_ALG6_GEMM);
         // C_i^XY (line 4) and D_a^XY (line 5) for the block's X
-        THC_TRY(mm(nX, P, v, tr(yv + X0, P), rm(A6.p, P), C6.p, P, 1, 0, o, 0, (long long)v * P,
+        THC_TRY(mm(nX, P, v, tr(yv + X0, P), rm(A6.p, P), C6.p, ldp, 1, 0, o, 0, (long long)v * P,
                    xP));
-        THC_TRY(mm(nX, P, o, tr(yo + X0, P), View<T>{A6.p, (long long)v * P, 1}, D6.p, P, 1, 0,
+        THC_TRY(mm(nX, P, o, tr(yo + X0, P), View<T>{A6.p, (long long)v * P, 1}, D6.p, ldp, 1, 0,
                    v, 0, P, xP));
         if constexpr (std::is_same<T, float>::value) {
             if (tri_pair) {
                 // E and F inherit the column order of C_i and D_a (lines 8-9)
-                THC_CUDA(pair_rows(C6.p, o, xP, nX, P, st));
-                THC_CUDA(pair_rows(D6.p, v, xP, nX, P, st));
+                THC_CUDA(pair_rows(C6.p, o, xP, nX, ldp, st));
+                THC_CUDA(pair_rows(D6.p, v, xP, nX, ldp, st));
             }
         }
-        THC_CUDA(cudaMemsetAsync(H.p, 0, sizeof(T) * nX * PP, st));
+        THC_CUDA(cudaMemsetAsync(H.p, 0, sizeof(T) * nX * PL, st));
         for (int I0 = 0; I0 < G; I0 += ic) {
             const int nI = std::min(ic, G - I0);
             seg_begin(THC_STEP_ALG6_GEMM);
@@ -1007,11 +1008,11 @@ Err Engine<T>::alg6(T* sgm) {
                        Fch.p, xP, 1, 0));
             const T* Gp;
             if (gall_resident) {
-                Gp = Gall.p + (long long)I0 * PP;
+                Gp = Gall.p + (long long)I0 * PL;
             } else {
                 THC_TRY(mm(P, P, o, tr(yo, P),
-                           View<T>{U6.p + (long long)I0 * P, (long long)G * P, 1}, Gch.p, P, 1,
-                           0, nI, 0, P, PP));
+                           View<T>{U6.p + (long long)I0 * P, (long long)G * P, 1}, Gch.p, ldp, 1,
+                           0, nI, 0, P, PL));
                 Gp = Gch.p;
             }
             if constexpr (std::is_same<T, double>::value) {
@@ -1020,7 +1021,7 @@ Err Engine<T>::alg6(T* sgm) {
                     THC_CUDA(split_df_pairs(Ech.p, nI, nX, P, E4.p, ME4.p, st));
                     THC_CUDA(split_df_pairs(Fch.p, nI, nX, P, F4.p, MF4.p, st));
                     if (!gall_resident) {
-                        THC_CUDA(split_df(Gch.p, (long long)nI * PP,
+                        THC_CUDA(split_df(Gch.p, (long long)nI * PL,
                                           reinterpret_cast<float2*>(Gch.p), st));
                         if (MG4.p)
                             THC_CUDA(pair_max(reinterpret_cast<const float2*>(Gch.p), nI, P, MG4.p, st));
@@ -1035,14 +1036,14 @@ Err Engine<T>::alg6(T* sgm) {
                 if (tri_df)
                     THC_CUDA(triangle_df(H.p, E4.p, F4.p, reinterpret_cast<const float2*>(Gp), ME4.p,
                                          MF4.p,
-                                         gall_resident && MG4.p ? MG4.p + I0 / kBiasChunk * PP : MG4.p,
+                                         gall_resident && MG4.p ? MG4.p + I0 / kBiasChunk * PL : MG4.p,
                                          P, nX, nI, st));
                 else
                     THC_CUDA(triangle(H.p, Ech.p, Fch.p, Gp, P, nX, nI, st));
             } else if (tri_pair) {
                 THC_CUDA(triangle_pair(H.p, reinterpret_cast<const float2*>(Ech.p),
-                                       reinterpret_cast<const float2*>(Fch.p), Gp, P, nX, nI, st,
-                                       tcerr.p));
+                                       reinterpret_cast<const float2*>(Fch.p), Gp, P, ldp, nX, nI,
+                                       st, tcerr.p));
             } else {
                 THC_CUDA(triangle(H.p, Ech.p, Fch.p, Gp, P, nX, nI, st));
             }
@@ -1050,7 +1051,7 @@ Err Engine<T>::alg6(T* sgm) {
         }
         seg_begin(THC_STEP_ALG6_POST);
         // I_ia = sum_YZ y_i^Z y_a^Y H^XYZ (line 14); sigma^XX' += sum_ia y_i^X' y_a^X' I_ia
-        THC_TRY(mm(o, P, P, rm(yo, P), View<T>{H.p, 1, P}, M6.p, P, 1, 0, nX, 0, PP,
+        THC_TRY(mm(o, P, P, rm(yo, P), View<T>{H.p, 1, ldp}, M6.p, P, 1, 0, nX, 0, PL,
                    (long long)o * P));
         THC_TRY(mm(o, v, P, rm(M6.p, P), tr(yv, P), I6.p, v, 1, 0, nX, (long long)o * P, 0, ov));
         THC_TRY(mm(nX, P, (int)ov, rm(I6.p, ov), rm(KRy.p, P), sgm + (long long)X0 * P, P, 1, 1));

@@ -174,6 +174,8 @@ struct Engine {
     // Mixed triangle over X pairs in packed lanes (C_i, D_a, E, F with the rows
     // of a pair interleaved, slabs of an even number of rows).
     bool tri_pair = false;
+    int ldp = 0;                            // pitch of the rows of C_i, D_a, E, F, G_I and H:
+                                            // P, rounded up to 4 for the paired triangle
     DBuf<float4> E4, F4;
     // Its bounds per kBiasChunk grid points (E, F of a grid chunk; G of all grid
     // points when resident, else of the chunk); empty = the TwoSum kernel.

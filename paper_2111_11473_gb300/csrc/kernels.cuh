@@ -80,7 +80,7 @@ cudaError_t scale_rows(const T* y, int R, int P, const T* w, int x0, int nx,
 // for a block of nX rows X (X < nX <= P, Y, Z < P): H is nX x P x P, E and F
 // are nI x nX x P, G is nI x P x P.  Float64: mirror (Y, Z) tiles on the
 // FP64 pipe; float32: 32^3 tiles through cp.async (the mixed path takes
-// triangle_pair when P is a multiple of 4).
+// triangle_pair up to P = kPairMaxP).
 template <typename T>
 cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, int nI,
                      cudaStream_t s);
@@ -105,16 +105,17 @@ cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const flo
                         const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
                         cudaStream_t s);
 
-// Float32 triangle over X pairs in packed lanes (triangle_pair.cu), for P a
-// multiple of 4 and at most kPairMaxP.  E2, F2: nI x ceil(nX/2) x P float2
-// {E^{2q,Y}, E^{2q+1,Y}} (16-byte aligned); G: nI x P x P; H: nX x P x P,
-// accumulated into.  err (device int) receives 1 if a bounded wait expired.
+// Float32 triangle over X pairs in packed lanes (triangle_pair.cu), for P at
+// most kPairMaxP.  Rows have a pitch of ld >= P, a multiple of 4: E2, F2: nI x
+// ceil(nX/2) x ld float2 {E^{2q,Y}, E^{2q+1,Y}} (16-byte aligned); G: nI x P x
+// ld; H: nX x P x ld, accumulated into (zeros are added beyond P).  err (device
+// int) receives 1 if a bounded wait expired.
 constexpr int kPairMaxP = 28000;
 bool triangle_pair_ok(int P);
 cudaError_t triangle_pair(float* H, const float2* E2, const float2* F2, const float* G, int P,
-                          int nX, int nI, cudaStream_t s, int* err);
+                          int ld, int nX, int nI, cudaStream_t s, int* err);
 // In place: for each of nslab slabs at A + b stride (stride >= nX rounded up
-// to even, times P), rows 2q, 2q + 1 of P floats become the interleaved
+// to even, times P, P a multiple of 4), rows 2q, 2q + 1 of P floats become the interleaved
 // pairs of triangle_pair's layout (0 in the second lane of an odd last row).
 cudaError_t pair_rows(float* A, long long nslab, long long stride, int nX, int P,
                       cudaStream_t s);

@@ -127,12 +127,16 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
     return d;
 }
 
+// Rows of H, E2, F2 and G have a pitch of ld >= P, a multiple of 4 (16-byte
+// rows for the copies and for the stores of four outputs; what lies beyond P
+// is read as zero, and zeros are added there in H).
 // Grid: x = block of QP X pairs (fastest, so that the blocks running together
 // share the G tiles of one mirror pair in L2), y = pair of mirror tiles.
 __global__ void __launch_bounds__(256, 1)
     k_triangle_pair(float* H, const __grid_constant__ CUtensorMap tmE,
                     const __grid_constant__ CUtensorMap tmF,
-                    const __grid_constant__ CUtensorMap tmG, int P, int nX, int nI, int* err) {
+                    const __grid_constant__ CUtensorMap tmG, int P, int ld, int nX, int nI,
+                    int* err) {
     extern __shared__ __align__(1024) unsigned char q_raw[];
     QSmem& sm = *reinterpret_cast<QSmem*>((reinterpret_cast<uintptr_t>(q_raw) + 1023) &
                                           ~uintptr_t(1023));
@@ -234,15 +238,20 @@ __global__ void __launch_bounds__(256, 1)
                     fz[2 * hh + 1] = f3.y;
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < 4; ++i) {
+                    // t = E^XY F^XZ + E^XZ F^XY for X = 2q, 2q + 1; neighbours
+                    // share an operand (8.55 -> 8.45 ms at the sizes above)
+                    f2 t[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) t[j] = mul2(ey[i], fz[j]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) t[j] = fma2(fy[i], ez[j], t[j]);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        // t = E^XY F^XZ + E^XZ F^XY for X = 2q, 2q + 1
-                        f2 t = mul2(ey[i], fz[j]);
-                        t = fma2(ez[j], fy[i], t);
-                        a1[p][i][j] = fma2(t, gb1[i][j], a1[p][i][j]);
-                        a2[p][i][j] = fma2(t, gb2[i][j], a2[p][i][j]);
+                        a1[p][i][j] = fma2(t[j], gb1[i][j], a1[p][i][j]);
+                        a2[p][i][j] = fma2(t[j], gb2[i][j], a2[p][i][j]);
                     }
+                }
             }
         }
         // The last warp to finish with the stage refills it at once with
@@ -290,7 +299,7 @@ __global__ void __launch_bounds__(256, 1)
             for (int L = 0; L < 2; ++L) {
                 if (X + L >= nX) continue;
                 const float* v = L ? v1 : v0;
-                float4* h = reinterpret_cast<float4*>(H + ((long long)(X + L) * P + Y) * P + Zs);
+                float4* h = reinterpret_cast<float4*>(H + ((long long)(X + L) * P + Y) * ld + Zs);
                 float4 c = *h;
                 c.x += scale * v[0];
                 c.y += scale * v[1];
@@ -317,7 +326,7 @@ __global__ void __launch_bounds__(256, 1)
             for (int L = 0; L < 2; ++L) {
                 if (X + L >= nX) continue;
                 const float* v = L ? v1 : v0;
-                float4* h = reinterpret_cast<float4*>(H + ((long long)(X + L) * P + Z) * P + Ys);
+                float4* h = reinterpret_cast<float4*>(H + ((long long)(X + L) * P + Z) * ld + Ys);
                 float4 c = *h;
                 c.x += scale * v[0];
                 c.y += scale * v[1];
@@ -353,10 +362,10 @@ __global__ void __launch_bounds__(256) k_pair_rows(float* A, long long nslab, lo
 PFN_cuTensorMapEncodeTiled_v12000 g_q_encode = nullptr;
 std::once_flag g_q_once;
 
-// 3-D map (x, rows, nI) of elements of `esize` bytes (x contiguous, rows of
-// x elements), box (bx, by, QI), 128-byte swizzle, zero fill outside.
+// 3-D map (x, rows, nI) of elements of `esize` bytes (x contiguous, rows
+// `ld` elements apart), box (bx, by, QI), 128-byte swizzle, zero fill outside.
 cudaError_t q_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int esize, long long x,
-                  long long rows, int nI, int bx, int by) {
+                  long long ld, long long rows, int nI, int bx, int by) {
     std::call_once(g_q_once, [] {
         cudaDriverEntryPointQueryResult q;
         void* fn = nullptr;
@@ -367,7 +376,7 @@ cudaError_t q_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int 
     });
     if (!g_q_encode) return cudaErrorNotSupported;
     cuuint64_t dims[3] = {(cuuint64_t)x, (cuuint64_t)rows, (cuuint64_t)nI};
-    cuuint64_t strides[2] = {(cuuint64_t)(x * esize), (cuuint64_t)(x * rows * esize)};
+    cuuint64_t strides[2] = {(cuuint64_t)(ld * esize), (cuuint64_t)(ld * rows * esize)};
     cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)QI};
     cuuint32_t es[3] = {1, 1, 1};
     CUresult r = g_q_encode(m, dt, 3, const_cast<void*>(base), dims, strides, box, es,
@@ -378,12 +387,12 @@ cudaError_t q_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int 
 
 }  // namespace
 
-bool triangle_pair_ok(int P) { return P > 0 && P % 4 == 0 && P <= kPairMaxP; }
+bool triangle_pair_ok(int P) { return P > 0 && P <= kPairMaxP; }
 
 cudaError_t pair_rows(float* A, long long nslab, long long stride, int nX, int P,
                       cudaStream_t s) {
     if (nslab <= 0 || nX <= 0) return cudaSuccess;
-    if (!triangle_pair_ok(P) || stride < (long long)(nX + (nX & 1)) * P || stride % 2)
+    if (!triangle_pair_ok(P) || P % 4 || stride < (long long)(nX + (nX & 1)) * P || stride % 2)
         return cudaErrorInvalidValue;
     const long long work = nslab * ((nX + 1) / 2);
     const unsigned grid = (unsigned)std::min<long long>(work, 152LL * 8);
@@ -398,23 +407,23 @@ cudaError_t pair_rows(float* A, long long nslab, long long stride, int nX, int P
 }
 
 cudaError_t triangle_pair(float* H, const float2* E2, const float2* F2, const float* G, int P,
-                          int nX, int nI, cudaStream_t s, int* err) {
+                          int ld, int nX, int nI, cudaStream_t s, int* err) {
     if (nX <= 0 || nI <= 0) return cudaSuccess;
-    if (!triangle_pair_ok(P) || !err || (uintptr_t)E2 % 16 || (uintptr_t)F2 % 16 ||
+    if (!triangle_pair_ok(P) || ld < P || ld % 4 || !err || (uintptr_t)E2 % 16 || (uintptr_t)F2 % 16 ||
         (uintptr_t)G % 16)
         return cudaErrorInvalidValue;
     const int nXp = (nX + 1) / 2;
     CUtensorMap mE, mF, mG;
-    cudaError_t e = q_map(&mE, E2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, nXp, nI, 16, QP);
-    if (e == cudaSuccess) e = q_map(&mF, F2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, nXp, nI, 16, QP);
-    if (e == cudaSuccess) e = q_map(&mG, G, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, P, P, nI, QT, QT);
+    cudaError_t e = q_map(&mE, E2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, ld, nXp, nI, 16, QP);
+    if (e == cudaSuccess) e = q_map(&mF, F2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, ld, nXp, nI, 16, QP);
+    if (e == cudaSuccess) e = q_map(&mG, G, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, P, ld, P, nI, QT, QT);
     if (e != cudaSuccess) return e;
     const int smem = (int)sizeof(QSmem) + 1024;
     e = smem_optin((const void*)k_triangle_pair, smem);
     if (e != cudaSuccess) return e;
     const unsigned nb = cdiv(P, QT);
     dim3 grid(cdiv(nXp, QP), nb * (nb + 1) / 2);
-    k_triangle_pair<<<grid, 256, smem, s>>>(H, mE, mF, mG, P, nX, nI, err);
+    k_triangle_pair<<<grid, 256, smem, s>>>(H, mE, mF, mG, P, ld, nX, nI, err);
     count_launches(1);
     return cudaGetLastError();
 }
