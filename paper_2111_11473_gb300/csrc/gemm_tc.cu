@@ -2,14 +2,15 @@
 //
 // C = alpha * A B + beta * C with float32 operands and output.  Each operand
 // is split into bf16 hi/lo parts (x = hi + lo to 2^-17 relative) by a pack
-// pass that also makes it K-major and pads it to the tile grid.  The product
-// kernel runs hi*hi + hi*lo + lo*hi (or hi*hi only) as tcgen05.mma kind::f16
-// with a float32 accumulator in tensor memory:
+// pass that also makes it K-major.  The product kernel runs
+// hi*hi + hi*lo + lo*hi (or hi*hi only) as tcgen05.mma kind::f16 with a
+// float32 accumulator in tensor memory:
 //   - TMA (cp.async.bulk.tensor, 128-byte swizzle) stages 128 x 64 tiles of
-//     both operands through a 3-deep shared-memory ring on mbarriers;
-//   - one elected thread issues the MMAs and commits each stage back to the
-//     producer; a final commit releases the epilogue;
-//   - four warps read the 128 x BN accumulator with tcgen05.ld and write C.
+//     one operand and bn x 64 tiles of the other through a shared-memory ring
+//     on mbarriers and fills what lies outside the operands with zeros;
+//   - one elected lane of a converged warp issues the MMAs and commits each
+//     stage back to the producer; a final commit releases the epilogue;
+//   - eight warps read the 128 x bn accumulator with tcgen05.ld and write C.
 // Every mbarrier wait is bounded: on expiry the kernel raises an error flag
 // that the host turns into THC_ERR_TIMEOUT, and frees its tensor memory.
 #include <cuda.h>
@@ -102,44 +103,60 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
         : "memory");
 }
 
-// Shared-memory ring depth per tile width (a stage holds the 128 x 64 hi/lo
-// tiles of A and the BN x 64 hi/lo tiles of B).
-template <int BN>
-struct TcStages {
-    static constexpr int value = BN == 128 ? 3 : (BN == 64 ? 4 : 5);
-};
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.b32 %0, 1, 0, q;\n}\n"
+        : "=r"(p));
+    return p != 0;
+}
 
-template <int BN>
-struct TcSmem {
-    static constexpr int ST = TcStages<BN>::value;
-    __nv_bfloat16 a_hi[ST][BM * BK];
-    __nv_bfloat16 a_lo[ST][BM * BK];
-    __nv_bfloat16 b_hi[ST][BN * BK];
-    __nv_bfloat16 b_lo[ST][BN * BK];
-    uint64_t full[ST];
-    uint64_t empty[ST];
+// Tile: 128 rows x bn columns, bn a multiple of 16 up to 256 chosen per
+// product.  What bounds a product is either the write of C (short K) or the
+// operand tiles' way from L2 to shared memory (a 128 x 128 tile takes 64 KB
+// per 64-wide K step for 384 cycles of MMAs, a 128 x 256 tile 96 KB for 768),
+// hence the widest tile that the columns fill, two accumulators of up to 256
+// columns so that the epilogue of one tile overlaps the main loop of the next,
+// and eight epilogue warps (four took 5.5 us per 128 x 128 tile, which made
+// the products of K = 40 take 347 us where C is written in 57).
+constexpr int kMaxBN = 256;
+constexpr int kMaxStages = 8;
+constexpr int kEpiWarps = 8;
+constexpr int kTcThreads = 64 + 32 * kEpiWarps;   // producer, MMA issuer, epilogue
+constexpr int kEpiCols = 16;                      // columns staged at once
+constexpr int kRingBytes = 208 * 1024;            // ring space within the 227 KB of an SM
+
+// Control block, after the operand ring in shared memory.
+struct TcCtl {
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
     uint64_t acc_full[2];     // accumulator buffer b holds a finished tile
     uint64_t acc_empty[2];    // the epilogue has drained accumulator buffer b
-    float epi[4][32 * 33];    // per epilogue warp: a 32 x 32 tile, padded rows
     uint64_t drain;
     uint32_t tmem;
     int fail;
+    float epi[kEpiWarps][32 * (kEpiCols + 1)];   // per epilogue warp: 32 rows, padded
 };
 
-constexpr int kEpiWarps = 4;
-constexpr int kTcThreads = 64 + 32 * kEpiWarps;   // producer, MMA issuer, epilogue
-
 struct TcArgs {
-    int M, N;              // real accumulator rows (UMMA M side) and columns
+    int M, N;              // real accumulator rows (UMMA M side, all batches of a
+                           // collapsed product) and columns
+    int Mb;                // rows per batch: row i is row i % Mb of batch bo + i / Mb
+    int bn;                // tile columns
+    int stages;            // ring depth
     int nbo;               // output batches
+    int Ktot;              // packed K per output batch
     int ksteps;            // 64-wide K steps per output batch
     int splits;
     int mblocks, nblocks;
     long long ntiles;      // mblocks * nblocks * nbo * splits
     float* C;              // output (or partials when splits > 1)
     long long crs, ccs, cbs;   // C(i, j) of batch b at C[b*cbs + i*crs + j*ccs]
-    float alpha, beta;
+    long long split_stride;    // partials of one split
+    float alpha, beta;     // alpha 1 when splits > 1
     int nprod;
+    int vec;               // C rows take 32-byte stores
     int a_bcast, b_bcast;  // operand shared by every batch: packed once, batch coord 0
     int* err;
 };
@@ -148,7 +165,7 @@ struct TileCoord {
     int m0, n0, bo, split, k_lo, nk;
 };
 
-__device__ __forceinline__ TileCoord tile_coord(const TcArgs& a, long long t, int BN) {
+__device__ __forceinline__ TileCoord tile_coord(const TcArgs& a, long long t) {
     TileCoord c;
     const int splits = a.splits, ksteps = a.ksteps;
     const int nbk = (int)(t % a.nblocks);
@@ -158,7 +175,7 @@ __device__ __forceinline__ TileCoord tile_coord(const TcArgs& a, long long t, in
     c.bo = (int)(r / splits);
     c.split = (int)(r % splits);
     c.m0 = mbk * BM;
-    c.n0 = nbk * BN;
+    c.n0 = nbk * a.bn;
     const int chunk = (ksteps + splits - 1) / splits;
     c.k_lo = c.split * chunk;
     c.nk = max(0, min(ksteps, c.k_lo + chunk) - c.k_lo);
@@ -203,23 +220,41 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// Eight floats of a row: one 32-byte access (a full sector) per lane.
+__device__ __forceinline__ void st8(float* p, const float* v) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "f"(v[0]),
+                 "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void ld8(const float* p, float* v) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                   "=f"(v[6]), "=f"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+
 // Persistent warp-specialised product: warp 0 streams operand tiles with TMA,
 // warp 1 issues the MMAs into one of two tensor-memory accumulators, and
-// warps 2-5 drain the other accumulator to C, so that the epilogue of one
+// warps 2-9 drain the other accumulator to C, so that the epilogue of one
 // tile overlaps the main loop of the next.  Tiles are taken round-robin.
-template <int BN, bool RMW>
+template <bool RMW>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
               const __grid_constant__ CUtensorMap tb_hi, const __grid_constant__ CUtensorMap tb_lo,
               const TcArgs args) {
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     // 1024-byte alignment of the tile ring (required by the 128-byte swizzle)
-    using Sm = TcSmem<BN>;
-    constexpr int ST = Sm::ST;
-    Sm& sm = *reinterpret_cast<Sm*>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) &
-                                    ~uintptr_t(1023));
+    unsigned char* ring = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~uintptr_t(1023));
+    const bool three = args.nprod == 3;
+    const uint32_t a_bytes = BM * BK * 2, b_bytes = (uint32_t)args.bn * BK * 2;
+    const uint32_t stage_bytes = (three ? 2 : 1) * (a_bytes + b_bytes);
+    const int ST = args.stages;
+    // stage: [A hi | B hi | A lo | B lo]
+    TcCtl& sm = *reinterpret_cast<TcCtl*>(ring + (size_t)ST * stage_bytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr uint32_t kCols = 2 * BN < 32 ? 32 : 2 * BN;
+    constexpr uint32_t kCols = 2 * kMaxBN;
     volatile int* fail = &sm.fail;
 
     if (threadIdx.x == 0) {
@@ -245,99 +280,129 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = sm.tmem;
-    const uint32_t a_bytes = BM * BK * 2, b_bytes = BN * BK * 2;
-    const uint32_t stage_bytes = (args.nprod == 3 ? 2 : 1) * (a_bytes + b_bytes);
 
     if (warp == 0) {
         if (lane == 0) {
             // TMA producer
-            long long it = 0;
-            long long last[ST];
-            for (int s = 0; s < ST; ++s) last[s] = -1;
-            for (long long t = blockIdx.x; t < args.ntiles && !*fail; t += gridDim.x) {
-                const TileCoord c = tile_coord(args, t, BN);
+            int s = 0, issued = 0;
+            uint32_t par = 0;           // parity of the pass over the ring
+            bool wrapped = false, ok = true;
+            for (long long t = blockIdx.x; t < args.ntiles && ok && !*fail; t += gridDim.x) {
+                const TileCoord c = tile_coord(args, t);
                 const int ba = args.a_bcast ? 0 : c.bo, bb = args.b_bcast ? 0 : c.bo;
-                for (int i = 0; i < c.nk; ++i, ++it) {
-                    const int s = (int)(it % ST);
-                    if (it >= ST && !mbar_wait_or_fail(&sm.empty[s], (uint32_t)(((it / ST) - 1) & 1), fail))
-                        break;
-                    const int kc = (c.k_lo + i) * BK;
-                    mbar_expect_tx(&sm.full[s], stage_bytes);
-                    tma_load_3d(sm.a_hi[s], &ta_hi, &sm.full[s], kc, c.m0, ba);
-                    tma_load_3d(sm.b_hi[s], &tb_hi, &sm.full[s], kc, c.n0, bb);
-                    if (args.nprod == 3) {
-                        tma_load_3d(sm.a_lo[s], &ta_lo, &sm.full[s], kc, c.m0, ba);
-                        tma_load_3d(sm.b_lo[s], &tb_lo, &sm.full[s], kc, c.n0, bb);
-                    }
-                    last[s] = it;
-                }
-            }
-            // Every load this thread issued has landed before the CTA exits
-            // (immediate unless a wait above gave up).
-            for (int s = 0; s < ST; ++s)
-                if (last[s] >= 0) mbar_wait(&sm.full[s], (uint32_t)((last[s] / ST) & 1));
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer
-            const uint32_t idesc = instr_desc(BM, BN);
-            long long it = 0;
-            int tl = 0;
-            for (long long t = blockIdx.x; t < args.ntiles && !*fail; t += gridDim.x, ++tl) {
-                const TileCoord c = tile_coord(args, t, BN);
-                const int buf = tl & 1;
-                if (tl >= 2 && !mbar_wait_or_fail(&sm.acc_empty[buf], (uint32_t)(((tl >> 1) - 1) & 1), fail))
-                    break;
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t dst = tmem + (uint32_t)(buf * BN);
-                bool ok = true;
-                for (int i = 0; i < c.nk; ++i, ++it) {
-                    const int s = (int)(it % ST);
-                    if (!mbar_wait_or_fail(&sm.full[s], (uint32_t)((it / ST) & 1), fail)) {
+                for (int i = 0; i < c.nk; ++i) {
+                    if (wrapped && !mbar_wait_or_fail(&sm.empty[s], par ^ 1u, fail)) {
                         ok = false;
                         break;
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t ah = smem_u32(sm.a_hi[s]), bh = smem_u32(sm.b_hi[s]);
-                    const uint32_t al = smem_u32(sm.a_lo[s]), bl = smem_u32(sm.b_lo[s]);
+                    const int kc = (c.k_lo + i) * BK;
+                    unsigned char* st = ring + (size_t)s * stage_bytes;
+                    mbar_expect_tx(&sm.full[s], stage_bytes);
+                    tma_load_3d(st, &ta_hi, &sm.full[s], kc, c.m0, ba);
+                    tma_load_3d(st + a_bytes, &tb_hi, &sm.full[s], kc, c.n0, bb);
+                    if (three) {
+                        tma_load_3d(st + a_bytes + b_bytes, &ta_lo, &sm.full[s], kc, c.m0, ba);
+                        tma_load_3d(st + 2 * a_bytes + b_bytes, &tb_lo, &sm.full[s], kc, c.n0, bb);
+                    }
+                    issued = max(issued, s + 1);
+                    if (++s == ST) {
+                        s = 0;
+                        par ^= 1u;
+                        wrapped = true;
+                    }
+                }
+            }
+            // Every load this thread issued has landed before the CTA exits
+            // (immediate unless a wait above gave up): stages below s were
+            // last filled in this pass over the ring, the others in the one before.
+            for (int e = 0; e < issued; ++e) mbar_wait(&sm.full[e], e < s ? par : par ^ 1u);
+        }
+    } else if (warp == 1) {
+        // MMA issuer: the whole warp runs the loop and one elected lane
+        // issues, so that the descriptors stay in uniform registers.
+        const uint32_t idesc = instr_desc(BM, args.bn);
+        const uint64_t base = smem_desc(smem_u32(ring));
+        const uint64_t dstage = stage_bytes >> 4, dbh = a_bytes >> 4,
+                       dal = (a_bytes + b_bytes) >> 4, dbl = (2 * a_bytes + b_bytes) >> 4;
+        constexpr uint64_t dk = (uint64_t)(UK * 2) >> 4;   // along K inside the swizzle atom
+        auto wait_all = [&](uint64_t* bar, uint32_t parity) {
+            return __all_sync(0xffffffffu, mbar_wait_or_fail(bar, parity, fail)) != 0;
+        };
+        int s = 0, tl = 0;
+        uint32_t par = 0;
+        bool ok = true;
+        for (long long t = blockIdx.x; t < args.ntiles && ok; t += gridDim.x, ++tl) {
+            const TileCoord c = tile_coord(args, t);
+            const int buf = tl & 1;
+            if (tl >= 2 && !wait_all(&sm.acc_empty[buf], (uint32_t)(((tl >> 1) - 1) & 1))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t dst = tmem + (uint32_t)(buf * kMaxBN);
+            for (int i = 0; i < c.nk; ++i) {
+                if (!wait_all(&sm.full[s], par)) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint64_t d0 = base + (uint64_t)s * dstage;
+                // 16-wide steps that hold data (Ktot is a multiple of 16)
+                const int kks = min(BK / UK, (args.Ktot - (c.k_lo + i) * BK) / UK);
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < BK / UK; ++kk) {
-                        const uint32_t off = kk * UK * 2;   // bytes along K inside the swizzle atom
-                        const uint32_t acc0 = (i > 0 || kk > 0) ? 1u : 0u;
-                        mma_bf16(dst, smem_desc(ah + off), smem_desc(bh + off), idesc, acc0);
-                        if (args.nprod == 3) {
-                            mma_bf16(dst, smem_desc(ah + off), smem_desc(bl + off), idesc, 1u);
-                            mma_bf16(dst, smem_desc(al + off), smem_desc(bh + off), idesc, 1u);
+                        if (kk < kks) {
+                            const uint64_t a = d0 + kk * dk;
+                            mma_bf16(dst, a, a + dbh, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                            if (three) {
+                                mma_bf16(dst, a, a + dbl, idesc, 1u);
+                                mma_bf16(dst, a + dal, a + dbh, idesc, 1u);
+                            }
                         }
                     }
                     mma_commit(&sm.empty[s]);
                 }
-                if (!ok) break;
-                mma_commit(&sm.acc_full[buf]);
+                __syncwarp();
+                if (++s == ST) {
+                    s = 0;
+                    par ^= 1u;
+                }
             }
-            // All MMAs this thread issued have completed before TMEM is freed.
-            mma_commit(&sm.drain);
-            mbar_wait(&sm.drain, 0);
+            if (ok && elect_one()) mma_commit(&sm.acc_full[buf]);
+            __syncwarp();
         }
+        // All MMAs this warp issued have completed before TMEM is freed.
+        if (elect_one()) mma_commit(&sm.drain);
+        __syncwarp();
+        mbar_wait(&sm.drain, 0);
     } else {
-        // Epilogue: warp w reads accumulator lanes 32 (w % 4) .. 32 (w % 4) + 31
-        // in 32-column chunks; a row-major C is written through a shared-memory
-        // transpose so that every store instruction covers one 128-byte row.
+        // Epilogue: warp w reads accumulator lanes 32 (w % 4) .. + 31 (one row
+        // per lane) in 32-column chunks, every second chunk.  Rows of C that
+        // take it are written by 32-byte stores straight from the registers;
+        // other row-major outputs go through a shared-memory transpose, so that
+        // a store instruction covers two runs of 16 columns; outputs with
+        // contiguous rows need neither.
         const int q = warp & 3;
-        float* stg = sm.epi[q];
+        const int ew = warp - 2;
+        float* stg = sm.epi[ew];
         int tl = 0;
         for (long long t = blockIdx.x; t < args.ntiles; t += gridDim.x, ++tl) {
-            const TileCoord c = tile_coord(args, t, BN);
+            const TileCoord c = tile_coord(args, t);
             const int buf = tl & 1;
             if (!mbar_wait_or_fail(&sm.acc_full[buf], (uint32_t)((tl >> 1) & 1), fail)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            float* Cb = args.C + (long long)c.bo * args.cbs +
-                        (args.splits > 1 ? (long long)c.split * args.nbo * args.cbs : 0);
-            const int i_base = c.m0 + q * 32;
+            const int i = c.m0 + q * 32 + lane;
+            const bool iok = i < args.M;
+            long long roff = 0;
+            if (iok) {
+                const int b = i / args.Mb;
+                roff = (long long)(c.bo + b) * args.cbs + (long long)(i - b * args.Mb) * args.crs +
+                       (long long)c.split * args.split_stride;
+            }
+            const int jend = min(args.N, c.n0 + args.bn);
 #pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 32) {
+            for (int c0 = 32 * (ew >> 2); c.n0 + c0 < jend; c0 += 64) {
                 uint32_t r[32];
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c0);
+                const uint32_t taddr =
+                    tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * kMaxBN + c0);
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x32.b32"
                     " {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -350,66 +415,71 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                       "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                     : "r"(taddr));
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                float val[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    val[j] = c.nk > 0 ? args.alpha * __uint_as_float(r[j]) : 0.f;
                 const int j0 = c.n0 + c0;
-                // RMW (beta != 0, no split): the 32 old values of C are loaded
+                // RMW (beta != 0, no split): the old values of C are loaded
                 // before any is used, so that their latencies overlap.
-                constexpr bool rmw = RMW;
-                if (args.ccs == 1) {
+                if (args.vec) {
+                    if (iok) {
+                        float* p = args.C + roff + j0;
+                        if constexpr (RMW) {
+                            float old[32];
+#pragma unroll
+                            for (int g = 0; g < 4; ++g)
+                                if (j0 + 8 * g < jend) ld8(p + 8 * g, old + 8 * g);
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) val[j] = fmaf(args.beta, old[j], val[j]);
+                        }
+#pragma unroll
+                        for (int g = 0; g < 4; ++g)
+                            if (j0 + 8 * g < jend) st8(p + 8 * g, val + 8 * g);
+                    }
+                } else if (args.ccs == 1) {
+#pragma unroll
+                    for (int h = 0; h < 32 / kEpiCols; ++h) {
+#pragma unroll
+                        for (int j = 0; j < kEpiCols; ++j)
+                            stg[lane * (kEpiCols + 1) + j] = val[h * kEpiCols + j];
+                        __syncwarp();
+                        const int jc = lane & (kEpiCols - 1), j = j0 + h * kEpiCols + jc;
+                        const int rsub = lane / kEpiCols;
+                        float old[kEpiCols];
+#pragma unroll
+                        for (int rr = 0; rr < 16; ++rr) {
+                            const int row = 2 * rr + rsub;
+                            const long long off = __shfl_sync(0xffffffffu, roff, row) + j;
+                            const bool ok = c.m0 + q * 32 + row < args.M && j < jend;
+                            if constexpr (RMW) old[rr] = ok ? args.C[off] : 0.f;
+                            else if (ok) args.C[off] = stg[row * (kEpiCols + 1) + jc];
+                        }
+                        if constexpr (RMW) {
+#pragma unroll
+                            for (int rr = 0; rr < 16; ++rr) {
+                                const int row = 2 * rr + rsub;
+                                const long long off = __shfl_sync(0xffffffffu, roff, row) + j;
+                                if (c.m0 + q * 32 + row < args.M && j < jend)
+                                    args.C[off] = fmaf(args.beta, old[rr],
+                                                       stg[row * (kEpiCols + 1) + jc]);
+                            }
+                        }
+                        __syncwarp();
+                    }
+                } else if (iok) {
+                    float* p = args.C + roff + (long long)j0 * args.ccs;
+                    if constexpr (RMW) {
+                        float old[32];
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            old[j] = j0 + j < jend ? p[(long long)j * args.ccs] : 0.f;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) val[j] = fmaf(args.beta, old[j], val[j]);
+                    }
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        stg[lane * 33 + j] = c.nk > 0 ? __uint_as_float(r[j]) : 0.f;
-                    __syncwarp();
-                    const int j = j0 + lane;
-                    const bool jok = j < args.N;
-                    float old[32];
-                    if constexpr (rmw) {
-#pragma unroll
-                        for (int rr = 0; rr < 32; ++rr) {
-                            const int i = i_base + rr;
-                            old[rr] = (jok && i < args.M) ? Cb[(long long)i * args.crs + j] : 0.f;
-                        }
-                    }
-                    if constexpr (rmw) {
-#pragma unroll
-                        for (int rr = 0; rr < 32; ++rr) {
-                            const int i = i_base + rr;
-                            if (i < args.M && jok)
-                                Cb[(long long)i * args.crs + j] =
-                                    fmaf(args.beta, old[rr], args.alpha * stg[rr * 33 + lane]);
-                        }
-                    } else {
-#pragma unroll 4
-                        for (int rr = 0; rr < 32; ++rr) {
-                            const int i = i_base + rr;
-                            if (i < args.M && jok) {
-                                const float val = stg[rr * 33 + lane];
-                                Cb[(long long)i * args.crs + j] =
-                                    args.splits > 1 ? val : args.alpha * val;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                } else {
-                    const int i = i_base + lane;
-                    if (i < args.M) {
-                        float old[32];
-                        if constexpr (rmw) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                old[j] = (j0 + j < args.N)
-                                             ? Cb[(long long)i * args.crs + (long long)(j0 + j) * args.ccs]
-                                             : 0.f;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            if (j0 + j < args.N) {
-                                const float val = c.nk > 0 ? __uint_as_float(r[j]) : 0.f;
-                                float* p = Cb + (long long)i * args.crs + (long long)(j0 + j) * args.ccs;
-                                if constexpr (rmw) *p = fmaf(args.beta, old[j], args.alpha * val);
-                                else *p = args.splits > 1 ? val : args.alpha * val;
-                            }
-                        }
-                    }
+                        if (j0 + j < jend) p[(long long)j * args.ccs] = val[j];
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -425,63 +495,125 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                      "r"(kCols));
 }
 
-// Pack a strided float32 operand into bf16 hi/lo, K-major, padded:
-// out[bo][r][kb*Kp + k] = split(src(b, r, k)), r < Rp, k < Kp, with
-// (bo, kb) = (b, 0) for batched products and (0, b) for batch-reduced ones.
-// A 32 (r) x 64 (k) tile goes through shared memory so that the global reads
-// run along whichever index of the source is contiguous, and every thread
-// then writes 8 consecutive k of one row as one 16-byte store of hi and lo.
-constexpr int PK_R = 32, PK_K = 64;
+// A strided float32 operand to pack into bf16 hi/lo, K-major:
+// out[b][r][k] = split(src(b, r, k)), r < R, k < Kp (Kd rounded up to 16, so
+// that rows start on 32-byte sectors), or out[r][b*Kp + k] for batch-reduced
+// products.  Nothing is padded to tiles: the product's TMA loads read zeros
+// beyond the operand.
+struct PackOp {
+    const float* src;
+    long long rs, ks, bs;
+    int R, Kd, Kp, nb, reduce;
+    int vec;               // 16-byte loads along k
+    long long units;       // blocks' worth of work
+    __nv_bfloat16* hi;
+    __nv_bfloat16* lo;     // null: hi only
+};
+constexpr int PK_R = 32, PK_K = 64;    // strided sources: tile through shared memory
+constexpr int PK_U = 4;                // contiguous sources: octets of k per thread
 
-__global__ void __launch_bounds__(256) k_pack(const float* src, long long rs, long long ks,
-                                              long long bs, int R, int Kd, int nb, int Rp, int Kp,
-                                              int reduce, __nv_bfloat16* hi, __nv_bfloat16* lo) {
-    __shared__ float tile[PK_R][PK_K + 1];
-    const int b = blockIdx.z;
-    const int k0 = blockIdx.x * PK_K;
-    const float* s = src + (long long)b * bs;
-    const bool kfast = ks <= rs;
-    const long long Ktot = reduce ? (long long)nb * Kp : Kp;
-    const int bo = reduce ? 0 : b, kb = reduce ? b : 0;
+__device__ __forceinline__ void pack_octet(const PackOp& op, long long row, int b, int r, int k,
+                                           const float* v) {
+    union { __nv_bfloat16 b[8]; uint4 u; } vh, vl;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const __nv_bfloat16 hh = __float2bfloat16_rn(v[e]);
+        vh.b[e] = hh;
+        vl.b[e] = __float2bfloat16_rn(v[e] - __bfloat162float(hh));
+    }
+    const long long o = op.reduce ? (long long)r * op.nb * op.Kp + (long long)b * op.Kp + k
+                                  : row * op.Kp + k;
+    *reinterpret_cast<uint4*>(op.hi + o) = vh.u;
+    if (op.lo) *reinterpret_cast<uint4*>(op.lo + o) = vl.u;
+}
+
+// One block's unit of a source that is contiguous along k: 1024 octets of k,
+// four per thread, their loads issued together (HBM bound: 8 bytes per element).
+__device__ __forceinline__ void pack_contiguous(const PackOp& op, long long u) {
+    const unsigned oc = (unsigned)op.Kp >> 3;
+    const long long rows = (long long)op.nb * op.R, base = u * (256 * PK_U);
+    const long long row0 = base / oc;
+    const unsigned rem = (unsigned)(base - row0 * oc);
+    float4 x[PK_U][2];
+    long long row[PK_U];
+    int b[PK_U], r[PK_U], k[PK_U];
+#pragma unroll
+    for (int h = 0; h < PK_U; ++h) {
+        const unsigned l = rem + h * 256 + threadIdx.x;
+        row[h] = row0 + l / oc;
+        k[h] = (int)(l % oc) * 8;
+        b[h] = (int)((unsigned)row[h] / (unsigned)op.R);
+        r[h] = (int)row[h] - b[h] * op.R;
+        const float* s = op.src + b[h] * op.bs + r[h] * op.rs + k[h];
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        x[h][0] = row[h] < rows && k[h] < op.Kd ? *reinterpret_cast<const float4*>(s) : z;
+        x[h][1] = row[h] < rows && k[h] + 4 < op.Kd ? *reinterpret_cast<const float4*>(s + 4) : z;
+    }
+#pragma unroll
+    for (int h = 0; h < PK_U; ++h) {
+        if (row[h] < rows) {
+            const float v[8] = {x[h][0].x, x[h][0].y, x[h][0].z, x[h][0].w,
+                                x[h][1].x, x[h][1].y, x[h][1].z, x[h][1].w};
+            pack_octet(op, row[h], b[h], r[h], k[h], v);
+        }
+    }
+}
+
+// One block's unit of any other source: a 32 (r) x 64 (k) tile goes through
+// shared memory so that the global reads run along whichever index of the
+// source is contiguous, and every thread then writes 8 consecutive k of one
+// row as one 16-byte store of hi and lo.
+__device__ __forceinline__ void pack_tile(const PackOp& op, long long u,
+                                          float (*tile)[PK_K + 1]) {
+    const int tk = (op.Kp + PK_K - 1) / PK_K, tr = (op.R + PK_R - 1) / PK_R;
+    const int k0 = (int)(u % tk) * PK_K;
+    const long long v = u / tk;
+    const int r0 = (int)(v % tr) * PK_R, b = (int)(v / tr);
+    const float* s = op.src + (long long)b * op.bs;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    for (int r0 = blockIdx.y * PK_R; r0 < Rp; r0 += gridDim.y * PK_R) {
-        if (kfast) {
-            // warp w reads rows w, w + 8, ...; lanes run along k (two halves of 32)
-            for (int rr = warp; rr < PK_R; rr += 8) {
-                const int r = r0 + rr;
+    float x[8];
+    if (op.ks <= op.rs) {
+        // warp w reads rows w, w + 8, ...; lanes run along k (two halves of 32)
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = k0 + h * 32 + lane;
-                    tile[rr][h * 32 + lane] =
-                        (r < R && k < Kd) ? s[(long long)r * rs + (long long)k * ks] : 0.f;
-                }
-            }
+        for (int e = 0; e < 8; ++e) {
+            const int r = r0 + warp + 8 * (e >> 1), k = k0 + (e & 1) * 32 + lane;
+            x[e] = (r < op.R && k < op.Kd) ? s[(long long)r * op.rs + (long long)k * op.ks] : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) tile[warp + 8 * (e >> 1)][(e & 1) * 32 + lane] = x[e];
+    } else {
+        // warp w reads columns w, w + 8, ...; lanes run along r
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int r = r0 + lane, k = k0 + warp + 8 * e;
+            x[e] = (r < op.R && k < op.Kd) ? s[(long long)r * op.rs + (long long)k * op.ks] : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) tile[lane][warp + 8 * e] = x[e];
+    }
+    __syncthreads();
+    const int rr = t >> 3, r = r0 + rr, k = k0 + (t & 7) * 8;   // 32 rows x 8 octets of k
+    if (r < op.R && k < op.Kp) {
+        float w[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = tile[rr][(t & 7) * 8 + e];
+        pack_octet(op, (long long)b * op.R + r, b, r, k, w);
+    }
+    __syncthreads();
+}
+
+// Both operands of a product in one launch (one launch each cost 2 to 3 us
+// more per product, and most operands are packed in 4 to 10).
+__global__ void __launch_bounds__(256) k_pack(const PackOp a, const PackOp b) {
+    __shared__ float tile[PK_R][PK_K + 1];
+    for (long long u = blockIdx.x; u < a.units + b.units; u += gridDim.x) {
+        if (u < a.units) {
+            if (a.vec) pack_contiguous(a, u);
+            else pack_tile(a, u, tile);
         } else {
-            // warp w reads columns w, w + 8, ...; lanes run along r
-            for (int kk = warp; kk < PK_K; kk += 8) {
-                const int r = r0 + lane, k = k0 + kk;
-                tile[lane][kk] = (r < R && k < Kd) ? s[(long long)r * rs + (long long)k * ks] : 0.f;
-            }
+            if (b.vec) pack_contiguous(b, u - a.units);
+            else pack_tile(b, u - a.units, tile);
         }
-        __syncthreads();
-        {
-            const int rr = t >> 3, oct = t & 7;   // 32 rows x 8 octets of k
-            const int r = r0 + rr, k = k0 + oct * 8;
-            if (r < Rp && k < Kp) {
-                union { __nv_bfloat16 b[8]; uint4 u; } vh, vl;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float v = tile[rr][oct * 8 + e];
-                    const __nv_bfloat16 hh = __float2bfloat16_rn(v);
-                    vh.b[e] = hh;
-                    vl.b[e] = __float2bfloat16_rn(v - __bfloat162float(hh));
-                }
-                const long long o = ((long long)bo * Rp + r) * Ktot + (long long)kb * Kp + k;
-                *reinterpret_cast<uint4*>(hi + o) = vh.u;
-                if (lo) *reinterpret_cast<uint4*>(lo + o) = vl.u;
-            }
-        }
-        __syncthreads();
     }
 }
 
@@ -530,18 +662,20 @@ cudaError_t make_map(CUtensorMap* map, const __nv_bfloat16* base, long long Ktot
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int BN>
 cudaError_t launch_tc(const CUtensorMap* maps, const TcArgs& a, cudaStream_t s) {
-    const int smem = (int)sizeof(TcSmem<BN>) + 1024;
-    cudaError_t e = smem_optin((const void*)k_gemm_tc<BN, false>, smem);
-    if (e == cudaSuccess) e = smem_optin((const void*)k_gemm_tc<BN, true>, smem);
+    const int stage = (a.nprod == 3 ? 2 : 1) * (BM + a.bn) * BK * 2;
+    const int smem = a.stages * stage + (int)sizeof(TcCtl) + 1024;
+    constexpr int kMost = kRingBytes + (int)sizeof(TcCtl) + 1024;
+    static_assert(kMost <= 227 * 1024, "ring and control block exceed an SM's shared memory");
+    cudaError_t e = smem_optin((const void*)k_gemm_tc<false>, kMost);
+    if (e == cudaSuccess) e = smem_optin((const void*)k_gemm_tc<true>, kMost);
     if (e != cudaSuccess) return e;
     const long long sms = device_sms();
     const unsigned grid = (unsigned)std::min<long long>(a.ntiles, sms);
     if (a.splits == 1 && a.beta != 0.f)
-        k_gemm_tc<BN, true><<<grid, kTcThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
+        k_gemm_tc<true><<<grid, kTcThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
     else
-        k_gemm_tc<BN, false><<<grid, kTcThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
+        k_gemm_tc<false><<<grid, kTcThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -598,54 +732,55 @@ void PackCache::release() {
 
 namespace {
 
-// Pack one operand into the workspace, or (use_cache) take it from the cache
-// of constant packs, packing it there on first use.  A cached operand that
+// Packed K of one batch: rows of packed operands start on 32-byte sectors.
+long long pack_k(int K) { return rup(std::max(K, 1), UK); }
+
+// Units of work of packing one operand (nb batches of R rows).
+PackOp pack_op(const float* p, long long rs, long long ks, long long bs, int R, int Kd, int nb,
+               int Kp, int reduce, __nv_bfloat16* hi, __nv_bfloat16* lo) {
+    PackOp op{p, rs, ks, bs, R, Kd, Kp, nb, reduce, 0, 0, hi, lo};
+    const long long rows = (long long)nb * R;
+    op.vec = ks == 1 && Kd % 4 == 0 && rs % 4 == 0 && (nb == 1 || bs % 4 == 0) &&
+             reinterpret_cast<uintptr_t>(p) % 16 == 0 && rows < INT32_MAX;
+    op.units = op.vec ? (rows * (Kp / 8) + 256 * PK_U - 1) / (256 * PK_U)
+                      : (long long)cdiv(Kp, PK_K) * cdiv(R, PK_R) * nb;
+    return op;
+}
+
+// Where one operand's packed form goes: the workspace, or (use_cache) the
+// cache of constant packs, where a form made before is taken as it is (units
+// = 0) and a new one gets its own buffer (*made).  A cached operand that
 // cannot be stored (budget or allocation) is an error, never a workspace
 // write: the workspace was sized without it.
-cudaError_t pack_operand(const float* p, long long rs, long long cs, long long bs, int R, int Kd,
-                         int nb_eff, int nb_grid, int Rp, int Kp, int reduce, int nprod,
-                         __nv_bfloat16* ws_hi, __nv_bfloat16* ws_lo, bool use_cache,
-                         PackCache* cache, cudaStream_t s, __nv_bfloat16** out_hi,
-                         __nv_bfloat16** out_lo) {
-    const dim3 grid(cdiv(Kp, PK_K), std::min<unsigned>(cdiv(Rp, PK_R), 65535), nb_grid);
-    if (use_cache) {
-        for (const PackCache::Entry& e : cache->entries)
-            if (e.p == p && e.rs == rs && e.cs == cs && e.bs == bs && e.R == R && e.Kd == Kd &&
-                e.nb == nb_eff && e.Rp == Rp && e.Kp == Kp && e.reduce == reduce &&
-                e.nprod == nprod) {
-                *out_hi = e.hi;
-                *out_lo = e.lo;
-                return cudaSuccess;
-            }
-        const long long Ktot = reduce ? (long long)nb_eff * Kp : Kp;
-        const size_t elems = (size_t)Rp * Ktot * (reduce ? 1 : nb_grid);
-        const size_t bytes = elems * 2 * (nprod == 3 ? 2 : 1);
-        if (cache->bytes + bytes > cache->budget) return cudaErrorMemoryAllocation;
-        __nv_bfloat16* buf = nullptr;
-        if (cudaMalloc(&buf, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return cudaErrorMemoryAllocation;
-        }
-        PackCache::Entry e{p, rs, cs, bs, R, Kd, nb_eff, Rp, Kp, reduce, nprod, buf,
-                           nprod == 3 ? buf + elems : nullptr};
-        k_pack<<<grid, 256, 0, s>>>(p, rs, cs, bs, R, Kd, nb_eff, Rp, Kp, reduce, e.hi, e.lo);
-        count_launches(1);
-        cudaError_t err = cudaGetLastError();
-        if (err != cudaSuccess) {
-            cudaFree(buf);
-            return err;
-        }
-        cache->entries.push_back(e);
-        cache->bytes += bytes;
-        *out_hi = e.hi;
-        *out_lo = e.lo;
+cudaError_t pack_target(const float* p, long long rs, long long cs, long long bs, int R, int Kd,
+                        int nb, int nb_packed, int Kp, int reduce, int nprod,
+                        __nv_bfloat16* ws_hi, __nv_bfloat16* ws_lo, bool use_cache,
+                        PackCache* cache, PackOp* op, PackCache::Entry* made) {
+    made->hi = nullptr;
+    if (!use_cache) {
+        *op = pack_op(p, rs, cs, bs, R, Kd, nb_packed, Kp, reduce, ws_hi, ws_lo);
         return cudaSuccess;
     }
-    k_pack<<<grid, 256, 0, s>>>(p, rs, cs, bs, R, Kd, nb_eff, Rp, Kp, reduce, ws_hi, ws_lo);
-    count_launches(1);
-    *out_hi = ws_hi;
-    *out_lo = ws_lo;
-    return cudaGetLastError();
+    for (const PackCache::Entry& e : cache->entries)
+        if (e.p == p && e.rs == rs && e.cs == cs && e.bs == bs && e.R == R && e.Kd == Kd &&
+            e.nb == nb && e.Rp == R && e.Kp == Kp && e.reduce == reduce && e.nprod == nprod) {
+            *op = PackOp{};
+            op->hi = e.hi;
+            op->lo = e.lo;
+            return cudaSuccess;
+        }
+    const size_t elems = (size_t)R * Kp * nb_packed;
+    const size_t bytes = elems * 2 * (nprod == 3 ? 2 : 1);
+    if (cache->bytes + bytes > cache->budget) return cudaErrorMemoryAllocation;
+    __nv_bfloat16* buf = nullptr;
+    if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return cudaErrorMemoryAllocation;
+    }
+    *made = PackCache::Entry{p, rs, cs, bs, R, Kd, nb, R, Kp, reduce, nprod, buf,
+                             nprod == 3 ? buf + elems : nullptr};
+    *op = pack_op(p, rs, cs, bs, R, Kd, nb_packed, Kp, reduce, made->hi, made->lo);
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -655,17 +790,23 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
     cudaError_t e = get_encode();
     if (e != cudaSuccess) return e;
-    // Orientation: the UMMA M side (128-row tiles) takes the larger of M, N.
-    const bool swap = g.N > g.M;
-    const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
-    int BN = 128;
-    if (Nr <= 32) BN = 32;
-    else if (Nr <= 64) BN = 64;
-    const long long Kp = rup(std::max(g.K, 1), BK);
     const int nb = g.batch;
     const int nbo = g.reduce ? 1 : nb;
-    const long long Ktot = g.reduce ? Kp * nb : Kp;
-    const long long RpA = rup(Mr, BM), RpB = rup(Nr, BN);
+    const bool bc = !g.reduce && nb > 1;
+    const bool m_bc = bc && g.sAb == 0, n_bc = bc && g.sBb == 0;
+    // Orientation: the UMMA M side (128-row tiles) takes the larger of M, N;
+    // if one operand is shared by every batch, the rows of the other one's
+    // batches (packed one after the other), so that a batch leaves no ragged
+    // row tile of its own (400 rows fill 4 tiles of 128 to 78 %).
+    bool swap = g.N > g.M, collapse = false;
+    if (m_bc != n_bc && (long long)nb * (m_bc ? g.N : g.M) < INT32_MAX) {
+        swap = m_bc;
+        collapse = true;
+    }
+    const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
+    const int Kp = (int)pack_k(g.K);
+    const long long Ktot = g.reduce ? (long long)Kp * nb : Kp;
+    if (Ktot > INT32_MAX) return cudaErrorMemoryAllocation;
     // Operand views: UMMA-A rows r, K index k.
     // Unswapped: A side = A(m, k), B side = B(k, n) read as (n, k).
     View<float> va = g.A, vb{g.B.p, g.B.cs, g.B.rs};
@@ -674,23 +815,21 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
         std::swap(va, vb);
         std::swap(sa, sb);
     }
-    const bool a_bc = !g.reduce && nb > 1 && sa == 0;
-    const bool b_bc = !g.reduce && nb > 1 && sb == 0;
+    const bool a_bc = swap ? n_bc : m_bc, b_bc = swap ? m_bc : n_bc;
     const int nba = a_bc ? 1 : nbo, nbb = b_bc ? 1 : nbo;
-    const size_t needA = (size_t)(RpA * Ktot * nba), needB = (size_t)(RpB * Ktot * nbb);
+    const size_t needA = (size_t)(Mr * Ktot * nba), needB = (size_t)(Nr * Ktot * nbb);
     // Operands served from the cache of constant packs take no workspace.
     const int red = g.reduce ? 1 : 0;
     const size_t bytesA = needA * 2 * (nprod == 3 ? 2 : 1);
     const size_t bytesB = needB * 2 * (nprod == 3 ? 2 : 1);
-    const bool a_cached = cache && cache->serves(va.p, bytesA, va.rs, va.cs, sa, Mr, g.K, nb,
-                                                 (int)RpA, (int)Kp, red, nprod);
+    const bool a_cached =
+        cache && cache->serves(va.p, bytesA, va.rs, va.cs, sa, Mr, g.K, nb, Mr, Kp, red, nprod);
     // B is checked against the budget left after A's (possibly new) entry.
     bool b_cached = false;
     if (cache) {
         const size_t held = cache->bytes;
         if (a_cached) cache->bytes += bytesA;
-        b_cached = cache->serves(vb.p, bytesB, vb.rs, vb.cs, sb, Nr, g.K, nb, (int)RpB, (int)Kp,
-                                 red, nprod);
+        b_cached = cache->serves(vb.p, bytesB, vb.rs, vb.cs, sb, Nr, g.K, nb, Nr, Kp, red, nprod);
         cache->bytes = held;
     }
     const size_t need = (nprod == 3 ? 2 : 1) * ((a_cached ? 0 : needA) + (b_cached ? 0 : needB));
@@ -701,59 +840,108 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
     __nv_bfloat16* b_hi = a_hi + wsA;
     __nv_bfloat16* a_lo = nprod == 3 ? b_hi + wsB : nullptr;
     __nv_bfloat16* b_lo = nprod == 3 ? a_lo + wsA : nullptr;
-    if ((e = pack_operand(va.p, va.rs, va.cs, sa, Mr, g.K, nb, a_bc ? 1 : nb, (int)RpA, (int)Kp,
-                          red, nprod, a_hi, a_lo, a_cached, cache, s, &a_hi, &a_lo)) !=
-        cudaSuccess)
-        return e;
-    if ((e = pack_operand(vb.p, vb.rs, vb.cs, sb, Nr, g.K, nb, b_bc ? 1 : nb, (int)RpB, (int)Kp,
-                          red, nprod, b_hi, b_lo, b_cached, cache, s, &b_hi, &b_lo)) !=
-        cudaSuccess)
-        return e;
-    CUtensorMap maps[4];
-    if ((e = make_map(&maps[0], a_hi, Ktot, RpA, nba, BM)) != cudaSuccess) return e;
-    if ((e = make_map(&maps[1], nprod == 3 ? a_lo : a_hi, Ktot, RpA, nba, BM)) != cudaSuccess) return e;
-    if ((e = make_map(&maps[2], b_hi, Ktot, RpB, nbb, BN)) != cudaSuccess) return e;
-    if ((e = make_map(&maps[3], nprod == 3 ? b_lo : b_hi, Ktot, RpB, nbb, BN)) != cudaSuccess) return e;
+    PackOp pa{}, pb{};
+    PackCache::Entry made[2];
+    made[1].hi = nullptr;
+    e = pack_target(va.p, va.rs, va.cs, sa, Mr, g.K, nb, a_bc ? 1 : nb, Kp, red, nprod, a_hi, a_lo,
+                    a_cached, cache, &pa, &made[0]);
+    if (e == cudaSuccess) {
+        // the second operand sees the budget that the first one's new form leaves
+        const size_t held = cache ? cache->bytes : 0;
+        if (made[0].hi) cache->bytes += bytesA;
+        e = pack_target(vb.p, vb.rs, vb.cs, sb, Nr, g.K, nb, b_bc ? 1 : nb, Kp, red, nprod, b_hi,
+                        b_lo, b_cached, cache, &pb, &made[1]);
+        if (cache) cache->bytes = held;
+    }
+    if (e == cudaSuccess && pa.units + pb.units > 0) {
+        const unsigned grid = (unsigned)std::min<long long>(pa.units + pb.units, 1 << 30);
+        k_pack<<<grid, 256, 0, s>>>(pa, pb);
+        count_launches(1);
+        e = cudaGetLastError();
+    }
+    for (int i = 0; i < 2; ++i) {
+        if (!made[i].hi) continue;
+        if (e != cudaSuccess) {
+            cudaFree(made[i].hi);
+        } else {
+            cache->entries.push_back(made[i]);
+            cache->bytes += i ? bytesB : bytesA;
+        }
+    }
+    if (e != cudaSuccess) return e;
 
     TcArgs a{};
-    a.M = Mr;
+    a.M = collapse ? nb * Mr : Mr;
     a.N = Nr;
-    a.nbo = nbo;
-    a.ksteps = (int)(Ktot / BK);
+    a.Mb = Mr;
+    a.nbo = collapse ? 1 : nbo;
+    a.Ktot = (int)Ktot;
+    a.ksteps = (int)((Ktot + BK - 1) / BK);
     a.nprod = nprod;
     a.a_bcast = a_bc ? 1 : 0;
     a.b_bcast = b_bc ? 1 : 0;
     a.err = ws.err;
     a.alpha = (float)g.alpha;
     a.beta = (float)g.beta;
-    // C(m, n) = g.C[b*sCb + m*ldc + n]; accumulator (i, j) is (m, n) or (n, m).
-    const long long crs = swap ? 1 : g.ldc, ccs = swap ? g.ldc : 1;
-    const int mblocks = (int)(RpA / BM), nblocks = (int)(RpB / BN);
-    const long long tiles = (long long)mblocks * nblocks * nbo;
+    a.mblocks = (int)cdiv(a.M, BM);
+    // Columns: as few tiles as 256 columns allow, of equal width; narrower
+    // ones (down to 64) where the product would leave SMs idle and K is too
+    // short to be split instead.
+    const long long sms = device_sms(), rowtiles = (long long)a.mblocks * a.nbo;
+    int nblocks = (int)cdiv(Nr, kMaxBN);
+    if (a.ksteps < 16)
+        while (rowtiles * nblocks < sms && Nr > 64 * nblocks) ++nblocks;
+    a.bn = (int)rup(cdiv(Nr, nblocks), 16);
+    a.nblocks = (int)cdiv(Nr, a.bn);
+    const long long tiles = rowtiles * a.nblocks;
+    // K splits: the count with the fewest K steps on the busiest SM.
     int splits = 1;
-    if (tiles < 152 && a.ksteps >= 8 && ws.partial) {
-        splits = (int)std::min<long long>({(152 + tiles - 1) / tiles, a.ksteps / 4, 32});
-        const long long per = (long long)Mr * Nr;
-        while (splits > 1 && (size_t)(per * nbo * splits) > ws.partial_elems) --splits;
+    if (tiles < sms && a.ksteps >= 8 && ws.partial) {
+        const long long per = (long long)Mr * Nr * nbo;
+        const int most = (int)std::min<long long>(
+            {2 * sms / tiles, a.ksteps / 4, 32, per > 0 ? (long long)ws.partial_elems / per : 1});
+        long long best = a.ksteps;
+        for (int t = 2; t <= most; ++t) {
+            const long long steps =
+                (tiles * t + sms - 1) / sms * (((long long)a.ksteps + t - 1) / t);
+            if (steps < best) {
+                best = steps;
+                splits = t;
+            }
+        }
     }
     a.splits = splits;
-    a.mblocks = mblocks;
-    a.nblocks = nblocks;
     a.ntiles = tiles * splits;
+    const int stage = (nprod == 3 ? 2 : 1) * (BM + a.bn) * BK * 2;
+    a.stages = std::min(kMaxStages, kRingBytes / stage);
+    // C(m, n) = g.C[b*sCb + m*ldc + n]; accumulator (i, j) is (m, n) or (n, m).
+    const long long crs = swap ? 1 : g.ldc, ccs = swap ? g.ldc : 1;
     if (splits > 1) {
         a.C = ws.partial;
         a.crs = Nr;
         a.ccs = 1;
         a.cbs = (long long)Mr * Nr;
+        a.split_stride = a.cbs * nbo;
+        a.alpha = 1.f;
     } else {
         a.C = g.C;
         a.crs = crs;
         a.ccs = ccs;
         a.cbs = g.reduce ? 0 : g.sCb;
     }
-    if (BN == 32) e = launch_tc<32>(maps, a, s);
-    else if (BN == 64) e = launch_tc<64>(maps, a, s);
-    else e = launch_tc<128>(maps, a, s);
+    a.vec = a.ccs == 1 && a.crs % 8 == 0 && (nbo == 1 || a.cbs % 8 == 0) && Nr % 8 == 0 &&
+            reinterpret_cast<uintptr_t>(a.C) % 32 == 0;
+    CUtensorMap maps[4];
+    // a collapsed operand is one list of rows
+    const long long rowsA = a.M, rowsB = Nr;
+    const int mba = collapse ? 1 : nba, mbb = nbb;
+    if ((e = make_map(&maps[0], pa.hi, Ktot, rowsA, mba, BM)) != cudaSuccess) return e;
+    if ((e = make_map(&maps[1], nprod == 3 ? pa.lo : pa.hi, Ktot, rowsA, mba, BM)) != cudaSuccess)
+        return e;
+    if ((e = make_map(&maps[2], pb.hi, Ktot, rowsB, mbb, a.bn)) != cudaSuccess) return e;
+    if ((e = make_map(&maps[3], nprod == 3 ? pb.lo : pb.hi, Ktot, rowsB, mbb, a.bn)) != cudaSuccess)
+        return e;
+    e = launch_tc(maps, a, s);
     if (e != cudaSuccess) return e;
     if (splits > 1) {
         const long long total = (long long)Mr * Nr * nbo;
@@ -1188,15 +1376,6 @@ __device__ __forceinline__ unsigned f64_fresh(int i) {
 }
 __device__ __forceinline__ unsigned f64_drained(int i, int nk) {
     return i == nk - 1 ? 0x7fu : f64_fresh(i + 1);
-}
-
-// One lane of a converged warp.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile(
-        "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.b32 %0, 1, 0, q;\n}\n"
-        : "=r"(p));
-    return p != 0;
 }
 
 // Slices sl .. of rows row .. in K block kb of batch b.
@@ -1945,6 +2124,11 @@ cudaError_t gemm_tc_selftest(int cases, unsigned long long seed, double* max_rel
         g.K = 1 + (int)(st_next(s) % 900);
         g.batch = 1 + (int)(st_next(s) % 4);
         const int mode = (int)(st_next(s) % 4);   // 0 separate, 1 shared A, 2 shared B, 3 reduce
+        if (c % 3 == 2) {   // rows that take wide loads and stores
+            g.M = (g.M + 7) / 8 * 8;
+            g.N = (g.N + 7) / 8 * 8;
+            g.K = (g.K + 3) / 4 * 4;
+        }
         g.reduce = mode == 3 && g.batch > 1;
         const bool ta = st_next(s) & 1, tb = st_next(s) & 1;
         const int nprod = (st_next(s) % 3 == 0) ? 1 : 3;
