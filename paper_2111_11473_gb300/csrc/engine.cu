@@ -226,18 +226,9 @@ Err Engine<T>::mm(int M, int N, int Kd, View<T> A, View<T> B, T* C, long long ld
             why = "K < 16";
         }
     } else {
-        // float64 products by exact integer slices on the tensor cores, when
-        // the estimated time beats the CUDA cores (1 TFLOP/s): 28 slice-pair
-        // products at the 1.2 PFLOP/s of bf16 products the fused kernel
-        // reaches on large shapes, slicing (8 + 8 bytes read, 14 written per
-        // operand element), the float64 tile written once, and 30 us of
-        // launches and of tiles' first loads and last drains.
-        const double out = (double)M * N * (reduce ? 1 : batch);
-        const double opnd = ((double)M + N) * Kd * batch;
-        const double t_tc = 28.0 * fl / 1.2e15 + opnd * 30.0 / 5e12 + out * 8.0 / 5e12 +
-                            30e-6;
+        // float64 products by exact integer slices on the tensor cores
         const bool use_tc = step_f64tc();
-        if (use_tc && fl >= 3.0e7 && Kd >= 8 && t_tc < fl / 1.0e12) {
+        if (use_tc && f64_tc_pays(M, N, Kd, batch, reduce)) {
             cudaError_t e = gemm_f64_tc(g, f64ws, st);
             if (e == cudaSuccess) return Err{};
             if (e != cudaErrorMemoryAllocation) THC_CUDA(e);

@@ -98,6 +98,18 @@ struct F64TcWorkspace {
 void gemm_f64_tc_sizes(int M, int N, int K, int batch, bool reduce, size_t* slice_elems,
                        size_t* part_elems, size_t* expo_elems);
 cudaError_t gemm_f64_tc(const Gemm<double>& g, const F64TcWorkspace& ws, cudaStream_t s);
+// Whether a float64 product is estimated to take less time by slices than on
+// the CUDA cores (1 TFLOP/s): 28 slice-pair products at the 1.2 PFLOP/s of
+// bf16 products the fused kernel reaches on large shapes, slicing (8 + 8 bytes
+// read, 14 written per operand element), the float64 tile written once, and 30
+// us of launches and of tiles' first loads and last drains.
+inline bool f64_tc_pays(int M, int N, int K, int batch, bool reduce) {
+    const double fl = 2.0 * M * N * (double)K * batch;
+    const double out = (double)M * N * (reduce ? 1 : batch);
+    const double opnd = ((double)M + N) * K * batch;
+    const double t_tc = 28.0 * fl / 1.2e15 + opnd * 30.0 / 5e12 + out * 8.0 / 5e12 + 30e-6;
+    return fl >= 3.0e7 && K >= 8 && t_tc < fl / 1.0e12;
+}
 // Randomised check of gemm_f64_tc against the float64 CUDA-core product.
 cudaError_t gemm_f64_tc_selftest(int cases, unsigned long long seed, double* max_rel,
                                  int* failures, cudaStream_t st);
