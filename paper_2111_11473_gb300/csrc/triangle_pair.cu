@@ -130,8 +130,9 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 // Rows of H, E2, F2 and G have a pitch of ld >= P, a multiple of 4 (16-byte
 // rows for the copies and for the stores of four outputs; what lies beyond P
 // is read as zero, and zeros are added there in H).
-// Grid: x = block of QP X pairs (fastest, so that the blocks running together
-// share the G tiles of one mirror pair in L2), y = pair of mirror tiles.
+// Grid: block of QP X pairs (fastest, so that the blocks running together share
+// the G tiles of one mirror pair in L2), pair of mirror tiles (in one
+// dimension: the pairs of P > 11552 exceed the second one's 65535 blocks).
 __global__ void __launch_bounds__(256, 1)
     k_triangle_pair(float* H, const __grid_constant__ CUtensorMap tmE,
                     const __grid_constant__ CUtensorMap tmF,
@@ -141,13 +142,14 @@ __global__ void __launch_bounds__(256, 1)
     QSmem& sm = *reinterpret_cast<QSmem*>((reinterpret_cast<uintptr_t>(q_raw) + 1023) &
                                           ~uintptr_t(1023));
     const int nb = (P + QT - 1) / QT;
-    int pidx = blockIdx.y, Yb = 0;
+    const int nxb = ((nX + 1) / 2 + QP - 1) / QP, xb = (int)(blockIdx.x % (unsigned)nxb);
+    int pidx = (int)(blockIdx.x / (unsigned)nxb), Yb = 0;
     while (pidx >= nb - Yb) {
         pidx -= nb - Yb;
         ++Yb;
     }
     const int Zb = Yb + pidx;
-    const int Y0 = Yb * QT, Z0 = Zb * QT, q0 = blockIdx.x * QP;
+    const int Y0 = Yb * QT, Z0 = Zb * QT, q0 = xb * QP;
     const bool diag = Yb == Zb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int xs = warp >> 2, wy = (warp >> 1) & 1, wz = warp & 1;
@@ -421,9 +423,9 @@ cudaError_t triangle_pair(float* H, const float2* E2, const float2* F2, const fl
     const int smem = (int)sizeof(QSmem) + 1024;
     e = smem_optin((const void*)k_triangle_pair, smem);
     if (e != cudaSuccess) return e;
-    const unsigned nb = cdiv(P, QT);
-    dim3 grid(cdiv(nXp, QP), nb * (nb + 1) / 2);
-    k_triangle_pair<<<grid, 256, smem, s>>>(H, mE, mF, mG, P, ld, nX, nI, err);
+    const long long nb = cdiv(P, QT), grid = cdiv(nXp, QP) * (nb * (nb + 1) / 2);
+    if (grid > INT32_MAX) return cudaErrorInvalidValue;
+    k_triangle_pair<<<(unsigned)grid, 256, smem, s>>>(H, mE, mF, mG, P, ld, nX, nI, err);
     count_launches(1);
     return cudaGetLastError();
 }
