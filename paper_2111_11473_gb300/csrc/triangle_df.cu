@@ -109,218 +109,6 @@ __device__ __forceinline__ void df_acc(f2& Sh, f2& Sl, f2 th, f2 tl, f2 thn, f2 
     Sh = s;
 }
 
-constexpr int DX = 4;     // amplitude indices X per block (two lane pairs)
-constexpr int DT = 32;    // Y and Z tile
-constexpr int DS = 4;     // grid points per pipeline stage
-constexpr int DTH = 256;  // threads: 16 x 16, each a 2 x 2 (Y, Z) block
-
-static_assert(DS * 2 * DT == DTH, "one E/F element per thread and stage");
-static_assert(DT * DT == 4 * DTH / 8 * 8 && DTH / DT * 4 == DT, "four G rows per thread");
-
-struct DfStage {
-    float4 ey[DS][2][DT];         // E^{x,Y} of the Y tile, {h(x), h(x+1), l(x), l(x+1)}
-    float4 ez[DS][2][DT];         // E^{x,Z} of the Z tile
-    float4 fy[DS][2][DT];
-    float4 fz[DS][2][DT];
-    float2 g1[DS][DT][DT + 1];    // {h, l} of G^YZ, rows Y
-    float2 g2[DS][DT][DT + 1];    // {h, l} of G^ZY, rows Z
-};
-
-__device__ __forceinline__ void cpa16(void* dst, const void* src, bool ok) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src),
-                 "r"(ok ? 16 : 0));
-}
-__device__ __forceinline__ void cpa8(void* dst, const void* src, bool ok) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src),
-                 "r"(ok ? 8 : 0));
-}
-
-// Per-thread copy plan of the block's tiles, fixed for the whole launch.
-// G tiles: thread tid copies column c = tid % 32 of rows r0 + 8 q (q < 4) of
-// both tiles for each grid point of a stage; E, F: thread tid copies the
-// element (s, xp, c) = (tid / 64, tid / 32 % 2, tid % 32) of the four arrays.
-struct DfPlan {
-    int g1off[4], g2off[4];   // (Y0 + r) P + Z0 + c, (Z0 + r) P + Y0 + c
-    unsigned gok;             // bit q: g1 row in range, bit 4 + q: g2 row in range
-    long long qoff;           // (xp0 + xp) P
-    int cy, cz;               // Y0 + c, Z0 + c
-    bool qok, yok, zok;
-};
-
-__device__ __forceinline__ DfPlan df_plan(int P, int nXp, int xp0, int Y0, int Z0) {
-    DfPlan pl;
-    const int tid = threadIdx.x, c = tid & 31, r0 = tid >> 5;
-    pl.gok = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int r = r0 + 8 * q;
-        pl.g1off[q] = (Y0 + r) * P + Z0 + c;
-        pl.g2off[q] = (Z0 + r) * P + Y0 + c;
-        if (Y0 + r < P && Z0 + c < P) pl.gok |= 1u << q;
-        if (Z0 + r < P && Y0 + c < P) pl.gok |= 1u << (4 + q);
-    }
-    const int xp = (tid >> 5) & 1;
-    pl.qoff = (long long)(xp0 + xp) * P;
-    pl.qok = xp0 + xp < nXp;
-    pl.cy = Y0 + c;
-    pl.cz = Z0 + c;
-    pl.yok = Y0 + c < P;
-    pl.zok = Z0 + c < P;
-    return pl;
-}
-
-// Stage grid points I0 .. I0 + DS - 1 of the block's tiles (zeros outside).
-__device__ __forceinline__ void df_load(DfStage& st, const DfPlan& pl, const float4* E4,
-                                        const float4* F4, const float2* G2, int P, int nXp,
-                                        int nI, int I0) {
-    const long long PP = (long long)P * P, XP = (long long)nXp * P;
-    const int tid = threadIdx.x, c = tid & 31, r0 = tid >> 5;
-#pragma unroll
-    for (int s = 0; s < DS; ++s) {
-        const int I = I0 + s;
-        const bool iok = I < nI;
-        const float2* Gi = G2 + (iok ? I * PP : 0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const bool ok1 = iok && (pl.gok >> q & 1u);
-            const bool ok2 = iok && (pl.gok >> (4 + q) & 1u);
-            cpa8(&st.g1[s][r0 + 8 * q][c], ok1 ? Gi + pl.g1off[q] : G2, ok1);
-            cpa8(&st.g2[s][r0 + 8 * q][c], ok2 ? Gi + pl.g2off[q] : G2, ok2);
-        }
-    }
-    {
-        const int s = tid >> 6, xp = (tid >> 5) & 1;
-        const int I = I0 + s;
-        const bool okx = I < nI && pl.qok;
-        const long long base = (okx ? I * XP + pl.qoff : 0);
-        const bool oy = okx && pl.yok, oz = okx && pl.zok;
-        cpa16(&st.ey[s][xp][c], oy ? E4 + base + pl.cy : E4, oy);
-        cpa16(&st.ez[s][xp][c], oz ? E4 + base + pl.cz : E4, oz);
-        cpa16(&st.fy[s][xp][c], oy ? F4 + base + pl.cy : F4, oy);
-        cpa16(&st.fz[s][xp][c], oz ? F4 + base + pl.cz : F4, oz);
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-
-// Grid: x = block of DX rows X (fastest, so that the blocks running together
-// share the G tiles of one (Y, Z) pair in L2), y = pair of mirror tiles.
-__global__ void __launch_bounds__(DTH, 1)
-    k_triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2, int P,
-                  int nX, int nI) {
-    extern __shared__ __align__(16) unsigned char df_raw[];
-    DfStage* stg = reinterpret_cast<DfStage*>(df_raw);
-    const int nb = (P + DT - 1) / DT;
-    int pidx = blockIdx.y, Yb = 0;
-    while (pidx >= nb - Yb) {
-        pidx -= nb - Yb;
-        ++Yb;
-    }
-    const int Zb = Yb + pidx;
-    const int Y0 = Yb * DT, Z0 = Zb * DT, X0 = blockIdx.x * DX;
-    const int nXp = (nX + 1) / 2, xp0 = X0 / 2;
-    const bool diag = Yb == Zb;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    // Accumulators of -H for the mirror outputs: [x pair][i][j]
-    f2 h1[2][2][2], l1[2][2][2], h2[2][2][2], l2[2][2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) h1[a][i][j] = l1[a][i][j] = h2[a][i][j] = l2[a][i][j] = 0ull;
-    const int nsteps = (nI + DS - 1) / DS;
-    const DfPlan plan = df_plan(P, nXp, xp0, Y0, Z0);
-    if (nsteps > 0) df_load(stg[0], plan, E4, F4, G2, P, nXp, nI, 0);
-    for (int k = 0; k < nsteps; ++k) {
-        const DfStage& cur = stg[k & 1];
-        if (k + 1 < nsteps) {
-            df_load(stg[(k + 1) & 1], plan, E4, F4, G2, P, nXp, nI, (k + 1) * DS);
-            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        }
-        __syncthreads();
-#pragma unroll
-        for (int st = 0; st < DS; ++st) {
-            // G^(Y_i, Z_j) and G^(Z_j, Y_i), the same value in both lanes
-            f2 g1h[2][2], g1l[2][2], g2h[2][2], g2l[2][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const float2 a = cur.g1[st][ty + 16 * i][tx + 16 * j];
-                    const float2 b = cur.g2[st][tx + 16 * j][ty + 16 * i];
-                    g1h[i][j] = pk(a.x, a.x);
-                    g1l[i][j] = pk(a.y, a.y);
-                    g2h[i][j] = pk(b.x, b.x);
-                    g2l[i][j] = pk(b.y, b.y);
-                }
-#pragma unroll
-            for (int xp = 0; xp < 2; ++xp) {
-                // {h(x), h(x+1)} and {l(x), l(x+1)} as two 64-bit lanes
-                ulonglong2 ey[2], fy[2], ez[2], fz[2];
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    ey[i] = reinterpret_cast<const ulonglong2&>(cur.ey[st][xp][ty + 16 * i]);
-                    fy[i] = reinterpret_cast<const ulonglong2&>(cur.fy[st][xp][ty + 16 * i]);
-                    ez[i] = reinterpret_cast<const ulonglong2&>(cur.ez[st][xp][tx + 16 * i]);
-                    fz[i] = reinterpret_cast<const ulonglong2&>(cur.fz[st][xp][tx + 16 * i]);
-                }
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        f2 th, tl;
-                        df_dot2(ey[i].x, ey[i].y, fz[j].x, fz[j].y, ez[j].x, ez[j].y, fy[i].x,
-                                fy[i].y, th, tl);
-                        const f2 thn = neg2(th);
-                        df_acc(h1[xp][i][j], l1[xp][i][j], th, tl, thn, g1h[i][j], g1l[i][j]);
-                        df_acc(h2[xp][i][j], l2[xp][i][j], th, tl, thn, g2h[i][j], g2l[i][j]);
-                    }
-            }
-        }
-        __syncthreads();   // the buffer is refilled by the next step's load
-    }
-    // On a diagonal pair both accumulators cover the same tile and count
-    // every (Y, Z) twice.
-    const double scale = diag ? -0.5 : -1.0;
-#pragma unroll
-    for (int xp = 0; xp < 2; ++xp)
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int Y = Y0 + ty + 16 * i, Z = Z0 + tx + 16 * j;
-                if (Y >= P || Z >= P) continue;
-                float a0, a1, b0, b1;
-                upk(h1[xp][i][j], a0, a1);
-                upk(l1[xp][i][j], b0, b1);
-                const int x = X0 + 2 * xp;
-                if (x < nX) H[((long long)x * P + Y) * P + Z] += scale * ((double)a0 + (double)b0);
-                if (x + 1 < nX)
-                    H[((long long)(x + 1) * P + Y) * P + Z] += scale * ((double)a1 + (double)b1);
-            }
-    if (diag) __syncthreads();   // mirror targets overlap other threads' first targets
-#pragma unroll
-    for (int xp = 0; xp < 2; ++xp)
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int Y = Y0 + ty + 16 * i, Z = Z0 + tx + 16 * j;
-                if (Y >= P || Z >= P) continue;
-                float a0, a1, b0, b1;
-                upk(h2[xp][i][j], a0, a1);
-                upk(l2[xp][i][j], b0, b1);
-                const int x = X0 + 2 * xp;
-                if (x < nX) H[((long long)x * P + Z) * P + Y] += scale * ((double)a0 + (double)b0);
-                if (x + 1 < nX)
-                    H[((long long)(x + 1) * P + Z) * P + Y] += scale * ((double)a1 + (double)b1);
-            }
-}
-
 // ---------------------------------------------------------------------------
 // The same sums with fewer operations: TwoSum (six operations, because it does
 // not know which addend is larger) is replaced by additions to constants that
@@ -346,27 +134,49 @@ __global__ void __launch_bounds__(DTH, 1)
 // over the sum of |terms|, 2^-46.1 / -46.6 / -47.1 for 300 / 600 / 1200 points
 // against 2^-46.7 / -46.2 / -45.7.  Hence the rule kBiasMinPoints: below it
 // the other kernel is the more accurate one (and the step is short).
+constexpr int BC = kBiasChunk;              // grid points per chunk of common bounds
+
+// A block of 128 threads takes 8 rows X (4 lane pairs) and a pair of mirror 16
+// x 16 (Y, Z) tiles; its two halves of 8 x 8 threads take two X pairs each, and
+// a thread 2 x 2 (Y, Z) of both.  Two blocks share an SM, so that one computes
+// while the other waits for its copies.  The tile is small because mirror pairs
+// of tiles cover the diagonal and the ragged edge with work that counts for
+// nothing: 32-wide tiles do 1.16 times the needed work at P = 400, 1.43 at 200
+// and 2.0 at 100, 16-wide ones 1.04, 1.16 and 1.42.
+constexpr int DT = 16;                      // Y and Z tile
+constexpr int DP = 4;                       // X pairs per block
+constexpr int DX = 2 * DP;
+constexpr int DTH = 128;
 constexpr int BS = 2;                       // grid points per pipeline stage
 constexpr int BST = 3;                      // stages
-constexpr int BC = kBiasChunk;              // grid points per chunk of common bounds
-constexpr int BTH = 256;                    // threads: 16 x 16, each 2 x 2 (Y, Z) of two X pairs
+static_assert(DTH == 2 * DP * DT && DTH == DT * DT / 2, "one copy per thread, array and grid point");
 static_assert(BC % BS == 0 && BC <= 512, "chunks are whole stages; 512 x 2^22 fits 32 bits");
 
-struct BiasSmem {
-    struct {
-        float4 ey[BS][2][DT], ez[BS][2][DT], fy[BS][2][DT], fz[BS][2][DT];
-        // {h, l} of G^YZ, rows Y, and of G^ZY, rows Z: column c of row r at
-        // 2 ((c / 2) ^ (r & 15)) + c % 2, so that rows (16-byte copies, reads
-        // of G^YZ) and columns (reads of G^ZY) are free of bank conflicts
-        float2 g1[BS][DT][DT];
-        float2 g2[BS][DT][DT];
-    } st[BST];
+struct DfStage {
+    // {h(x), h(x+1), l(x), l(x+1)} of E^{x,Y} of the Y tile etc.: [x pair][.]
+    float4 ey[BS][DP][DT], ez[BS][DP][DT], fy[BS][DP][DT], fz[BS][DP][DT];
+    // {h, l} of G^YZ, rows Y, and of G^ZY, rows Z: column c of row r at
+    // 2 ((c / 2) ^ swz(r)) + c % 2, so that rows (16-byte copies), reads of
+    // four rows by eight columns (G^YZ) and of eight by four (G^ZY) take no
+    // more shared-memory cycles than their bytes
+    float2 g1[BS][DT][DT];
+    float2 g2[BS][DT][DT];
+};
+__device__ __forceinline__ int swz(int r) { return (r & 1) << 2 | (r >> 1 & 3); }
+
+template <bool BIAS>
+struct DfSmem {
+    DfStage st[BST];
+};
+template <>
+struct DfSmem<true> {
+    DfStage st[BST];
     // bounds of a chunk (two chunks in flight)
     struct {
-        float2 ey[2][DT], ez[2][DT], fy[2][DT], fz[2][DT];   // [x pair][.]
+        float2 ey[DP][DT], ez[DP][DT], fy[DP][DT], fz[DP][DT];   // [x pair][.]
         float g[DT][DT];
     } mx[2];
-    ulonglong2 sum[16][BTH];          // float pairs {high, low} of the thread's 16 accumulators
+    ulonglong2 sum[16][DTH];          // float pairs {high, low} of the thread's 16 accumulators
 };
 
 // 1.5 2^k with 2^(k-1) above b (a thousandth above the true bound).
@@ -483,112 +293,116 @@ __device__ __forceinline__ void cp_n(void* dst, const void* src, int n) {
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n));
 }
 
-// Grid as k_triangle_df.  ME, MF: bounds [chunk][x pair][P] (lanes x, x + 1);
-// MG: [chunk][P][P], symmetric.  EVEN: P is even, rows of G start on 16-byte
-// boundaries and are copied two columns at a time.
+// The two forms of the accumulators, for the kernel below: mirror outputs
+// [x pair][i][j] of H^XYZ and H^XZY, Y = ty + 8 i, Z = tx + 8 j.
+template <bool BIAS>
+struct DfAcc {
+    // float pairs of -H, updated by TwoSum
+    f2 h1[2][2][2], l1[2][2][2], h2[2][2][2], l2[2][2][2];
+};
+template <>
+struct DfAcc<true> {
+    BiasAcc h1[2][2][2], h2[2][2][2];
+    f2 sg[2][2][2], cb[2][2][2];   // biases of t's products and of t G
+};
+
+// Grid: block of DX rows X (fastest, so that the blocks running together share
+// the G tiles of one (Y, Z) pair in L2), pair of mirror tiles.
+// BIAS: bounds ME, MF: [chunk][x pair][P] (lanes x, x + 1); MG: [chunk][P][P],
+// symmetric.  EVEN: P is even, rows of G start on 16-byte boundaries and are
+// copied two columns at a time.
 // A packed FMA of three distinct register pairs measures 3.3 cycles of a
 // scheduler on GB300 and a packed addition 2.3 (peak: 2): the operations here
 // are bound by register reads, 138 per unit of two X and two mirror outputs
 // against 208 in the TwoSum form, so what comes besides them counts.  The copy
 // addresses advance by constants, which is why a thread copies a two-column
-// piece of two rows of every G tile and one element of E and of F.  P = 400,
-// 400 rows X, 1200 grid points: 58.8 ms (the TwoSum kernel 68.7); P = 200, 200
-// X, 600 points 4.93 ms (5.75).  512 threads of half the outputs: 5.30.
-template <bool EVEN>
-__global__ void __launch_bounds__(BTH, 1)
-    k_triangle_bias(double* H, const float4* E4, const float4* F4, const float2* G2,
-                    const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI) {
+// piece of one row of every G tile and one element of E and of F per grid
+// point.  P = 400, 400 rows X, 1200 grid points: 44.3 ms (32-wide tiles and one
+// block of 256 threads per SM: 58.5; their TwoSum form 68.7); P = 200, 200 X,
+// 600 points: 3.19 ms (4.93); TwoSum form, P = 100, 300 points: 0.41 (0.60).
+template <bool BIAS, bool EVEN>
+__global__ void __launch_bounds__(DTH, 2)
+    k_triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
+                  const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI) {
     extern __shared__ __align__(16) unsigned char df_raw[];
-    BiasSmem& sm = *reinterpret_cast<BiasSmem*>(df_raw);
+    DfSmem<BIAS>& sm = *reinterpret_cast<DfSmem<BIAS>*>(df_raw);
     const int nb = (P + DT - 1) / DT;
-    int pidx = blockIdx.y, Yb = 0;
+    const int nxb = (nX + DX - 1) / DX, xb = (int)(blockIdx.x % (unsigned)nxb);
+    int pidx = (int)(blockIdx.x / (unsigned)nxb), Yb = 0;
     while (pidx >= nb - Yb) {
         pidx -= nb - Yb;
         ++Yb;
     }
     const int Zb = Yb + pidx;
-    const int Y0 = Yb * DT, Z0 = Zb * DT, X0 = blockIdx.x * DX;
-    const int nXp = (nX + 1) / 2, xp0 = X0 / 2;
+    const int Y0 = Yb * DT, Z0 = Zb * DT, X0 = xb * DX;
+    const int nXp = (nX + 1) / 2, xp0 = xb * DP;
     const bool diag = Yb == Zb;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3 & 7, xg = tid >> 6 << 1;
     const long long PP = (long long)P * P, XP = (long long)nXp * P;
 
-    // Copies of this thread: columns 2 tx, 2 tx + 1 of rows ty and ty + 16 of
-    // both G tiles for every grid point, and one column of one row of E and of
-    // F per stage.
+    // Copies of this thread per grid point: columns 2 gc, 2 gc + 1 of row gr of
+    // both G tiles, and one column of one row of E and of F.
+    const int gr = tid >> 3, gc = tid & 7;
     const char *g1p, *g2p, *ep, *fp;
-    int g1n[2], g2n[2], en;   // bytes inside the array
-    const long long row16 = 16LL * P * 8;
+    int g1n, g2n, en;         // bytes inside the array
     {
-        const int c1 = Z0 + 2 * tx, c2 = Y0 + 2 * tx;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            g1n[q] = Y0 + ty + 16 * q < P ? 8 * max(0, min(2, P - c1)) : 0;
-            g2n[q] = Z0 + ty + 16 * q < P ? 8 * max(0, min(2, P - c2)) : 0;
-        }
-        g1p = reinterpret_cast<const char*>(G2 + (g1n[0] ? (long long)(Y0 + ty) * P + c1 : 0));
-        g2p = reinterpret_cast<const char*>(G2 + (g2n[0] ? (long long)(Z0 + ty) * P + c2 : 0));
+        const int c1 = Z0 + 2 * gc, c2 = Y0 + 2 * gc;
+        g1n = Y0 + gr < P ? 8 * max(0, min(2, P - c1)) : 0;
+        g2n = Z0 + gr < P ? 8 * max(0, min(2, P - c2)) : 0;
+        g1p = reinterpret_cast<const char*>(G2 + (g1n ? (long long)(Y0 + gr) * P + c1 : 0));
+        g2p = reinterpret_cast<const char*>(G2 + (g2n ? (long long)(Z0 + gr) * P + c2 : 0));
     }
-    // warp w: Z side (or Y), grid point cs of the stage, X pair cx
-    const int w = tid >> 5, c = tid & 31;
-    const int cz = (w >> 2) & 1, cs = (w >> 1) & 1, cx = w & 1;
-    const char *mp, *np;      // the bounds of the same elements, per chunk
+    // Z side (or Y), X pair cx, column c
+    const int cz = tid >> 6, cx = tid >> 4 & 3, c = tid & 15;
+    const char *mp = nullptr, *np = nullptr;      // the bounds of the same elements, per chunk
     {
         const int col = (cz ? Z0 : Y0) + c;
         const bool ok = xp0 + cx < nXp && col < P;
         const long long at = ok ? (long long)(xp0 + cx) * P + col : 0;
         en = ok ? 16 : 0;
-        const long long first = cs < nI ? cs * XP * 16 : 0;
-        ep = reinterpret_cast<const char*>(E4 + at) + first;
-        fp = reinterpret_cast<const char*>(F4 + at) + first;
-        mp = reinterpret_cast<const char*>(ME + at);
-        np = reinterpret_cast<const char*>(MF + at);
+        ep = reinterpret_cast<const char*>(E4 + at);
+        fp = reinterpret_cast<const char*>(F4 + at);
+        if (BIAS) {
+            mp = reinterpret_cast<const char*>(ME + at);
+            np = reinterpret_cast<const char*>(MF + at);
+        }
     }
-    const int gsw = 2 * (tx ^ ty);
+    const int gsw = 2 * (gc ^ swz(gr));
     auto load = [&](int k, int b) {
         const int I0 = k * BS;
         auto& st = sm.st[b];
-        const bool whole = I0 + BS <= nI;   // else the grid points beyond are zeros
 #pragma unroll
-        for (int s = 0; s < BS; ++s)
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const bool in = whole || I0 + s < nI;
-                const int n1 = in ? g1n[q] : 0, n2 = in ? g2n[q] : 0;
-                const char* p1 = n1 ? g1p + s * PP * 8 + q * row16 : reinterpret_cast<const char*>(G2);
-                const char* p2 = n2 ? g2p + s * PP * 8 + q * row16 : reinterpret_cast<const char*>(G2);
-                if (EVEN) {
-                    cp_n<16>(&st.g1[s][ty + 16 * q][gsw], p1, n1);
-                    cp_n<16>(&st.g2[s][ty + 16 * q][gsw], p2, n2);
-                } else {
-                    cp_n<8>(&st.g1[s][ty + 16 * q][gsw], p1, min(n1, 8));
-                    cp_n<8>(&st.g1[s][ty + 16 * q][gsw + 1], n1 > 8 ? p1 + 8 : p1, max(n1 - 8, 0));
-                    cp_n<8>(&st.g2[s][ty + 16 * q][gsw], p2, min(n2, 8));
-                    cp_n<8>(&st.g2[s][ty + 16 * q][gsw + 1], n2 > 8 ? p2 + 8 : p2, max(n2 - 8, 0));
-                }
+        for (int s = 0; s < BS; ++s) {
+            const bool in = I0 + s < nI;        // else the grid point's values are zeros
+            const int n1 = in ? g1n : 0, n2 = in ? g2n : 0, n = in ? en : 0;
+            const char* p1 = n1 ? g1p + s * PP * 8 : reinterpret_cast<const char*>(G2);
+            const char* p2 = n2 ? g2p + s * PP * 8 : reinterpret_cast<const char*>(G2);
+            if (EVEN) {
+                cp_n<16>(&st.g1[s][gr][gsw], p1, n1);
+                cp_n<16>(&st.g2[s][gr][gsw], p2, n2);
+            } else {
+                cp_n<8>(&st.g1[s][gr][gsw], p1, min(n1, 8));
+                cp_n<8>(&st.g1[s][gr][gsw + 1], n1 > 8 ? p1 + 8 : p1, max(n1 - 8, 0));
+                cp_n<8>(&st.g2[s][gr][gsw], p2, min(n2, 8));
+                cp_n<8>(&st.g2[s][gr][gsw + 1], n2 > 8 ? p2 + 8 : p2, max(n2 - 8, 0));
             }
-        {
-            const bool in = whole || I0 + cs < nI;
-            cp_n<16>(cz ? &st.ez[cs][cx][c] : &st.ey[cs][cx][c],
-                     in ? ep : reinterpret_cast<const char*>(E4), in ? en : 0);
-            cp_n<16>(cz ? &st.fz[cs][cx][c] : &st.fy[cs][cx][c],
-                     in ? fp : reinterpret_cast<const char*>(F4), in ? en : 0);
+            cp_n<16>(cz ? &st.ez[s][cx][c] : &st.ey[s][cx][c],
+                     n ? ep + s * XP * 16 : reinterpret_cast<const char*>(E4), n);
+            cp_n<16>(cz ? &st.fz[s][cx][c] : &st.fy[s][cx][c],
+                     n ? fp + s * XP * 16 : reinterpret_cast<const char*>(F4), n);
         }
-        // the chunk's bounds with its first stage
-        if (I0 % BC == 0) {
-            auto& mx = sm.mx[(I0 / BC) & 1];
-            if (cs == 0) {
+        if constexpr (BIAS) {
+            // the chunk's bounds with its first stage
+            if (I0 % BC == 0) {
+                auto& mx = sm.mx[(I0 / BC) & 1];
                 cp_n<8>(cz ? &mx.ez[cx][c] : &mx.ey[cx][c], mp, en / 2);
                 cp_n<8>(cz ? &mx.fz[cx][c] : &mx.fy[cx][c], np, en / 2);
-            }
-            mp += XP * 8;
-            np += XP * 8;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
+                mp += XP * 8;
+                np += XP * 8;
                 const float* m = MG + I0 / BC * PP +
-                                 (g1n[q] ? (long long)(Y0 + ty + 16 * q) * P + Z0 + 2 * tx : 0);
-                cp_n<4>(&mx.g[ty + 16 * q][2 * tx], m, min(g1n[q] / 2, 4));
-                cp_n<4>(&mx.g[ty + 16 * q][2 * tx + 1], g1n[q] > 8 ? m + 1 : m, max(g1n[q] / 2 - 4, 0));
+                                 (g1n ? (long long)(Y0 + gr) * P + Z0 + 2 * gc : 0);
+                cp_n<4>(&mx.g[gr][2 * gc], m, min(g1n / 2, 4));
+                cp_n<4>(&mx.g[gr][2 * gc + 1], g1n > 8 ? m + 1 : m, max(g1n / 2 - 4, 0));
             }
         }
         g1p += BS * PP * 8;
@@ -598,32 +412,36 @@ __global__ void __launch_bounds__(BTH, 1)
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
 
-    // [x pair][i][j]: H^XYZ and H^XZY, Y = ty + 16 i, Z = tx + 16 j
-    BiasAcc h1[2][2][2], h2[2][2][2];
-    f2 sg[2][2][2], cb[2][2][2];   // biases of t's products and of t G
+    DfAcc<BIAS> A;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                h1[a][i][j] = BiasAcc{0u, 0u, 0ull};
-                h2[a][i][j] = BiasAcc{0u, 0u, 0ull};
-                sg[a][i][j] = cb[a][i][j] = 0ull;
-                sm.sum[(a * 4 + i * 2 + j) * 2][tid] = make_ulonglong2(0ull, 0ull);
-                sm.sum[(a * 4 + i * 2 + j) * 2 + 1][tid] = make_ulonglong2(0ull, 0ull);
+                if constexpr (BIAS) {
+                    A.h1[a][i][j] = BiasAcc{0u, 0u, 0ull};
+                    A.h2[a][i][j] = BiasAcc{0u, 0u, 0ull};
+                    A.sg[a][i][j] = A.cb[a][i][j] = 0ull;
+                    sm.sum[(a * 4 + i * 2 + j) * 2][tid] = make_ulonglong2(0ull, 0ull);
+                    sm.sum[(a * 4 + i * 2 + j) * 2 + 1][tid] = make_ulonglong2(0ull, 0ull);
+                } else {
+                    A.h1[a][i][j] = A.l1[a][i][j] = A.h2[a][i][j] = A.l2[a][i][j] = 0ull;
+                }
             }
     auto fold = [&](unsigned n) {
+        if constexpr (BIAS) {
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+            for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+                for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int u = (a * 4 + i * 2 + j) * 2;
-                    bias_fold(h1[a][i][j], cb[a][i][j], n, sm.sum[u][tid]);
-                    bias_fold(h2[a][i][j], cb[a][i][j], n, sm.sum[u + 1][tid]);
-                }
+                    for (int j = 0; j < 2; ++j) {
+                        const int u = (a * 4 + i * 2 + j) * 2;
+                        bias_fold(A.h1[a][i][j], A.cb[a][i][j], n, sm.sum[u][tid]);
+                        bias_fold(A.h2[a][i][j], A.cb[a][i][j], n, sm.sum[u + 1][tid]);
+                    }
+        }
     };
     const int nsteps = (nI + BS - 1) / BS;
 #pragma unroll
@@ -638,25 +456,27 @@ __global__ void __launch_bounds__(BTH, 1)
         __syncthreads();   // stage k is there, stage k - 1 is free
         if (k + BST - 1 < nsteps) load(k + BST - 1, b == 0 ? BST - 1 : b - 1);
         else asm volatile("cp.async.commit_group;\n" ::: "memory");
-        if (k * BS % BC == 0) {
-            if (k > 0) fold((unsigned)inchunk);
-            inchunk = 0;
-            const auto& mx = sm.mx[(k * BS / BC) & 1];
+        if constexpr (BIAS) {
+            if (k * BS % BC == 0) {
+                if (k > 0) fold((unsigned)inchunk);
+                inchunk = 0;
+                const auto& mx = sm.mx[(k * BS / BC) & 1];
 #pragma unroll
-            for (int a = 0; a < 2; ++a)
+                for (int a = 0; a < 2; ++a)
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                    for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const f2 ey = reinterpret_cast<const f2&>(mx.ey[a][ty + 16 * i]);
-                        const f2 fy = reinterpret_cast<const f2&>(mx.fy[a][ty + 16 * i]);
-                        const f2 ez = reinterpret_cast<const f2&>(mx.ez[a][tx + 16 * j]);
-                        const f2 fz = reinterpret_cast<const f2&>(mx.fz[a][tx + 16 * j]);
-                        const float g = mx.g[ty + 16 * i][tx + 16 * j];
-                        const f2 p1 = prod2(ey, fz), p2 = prod2(ez, fy);
-                        sg[a][i][j] = bias_of(max2(p1, p2));
-                        cb[a][i][j] = bias_of(prod2(add2(p1, p2), pk(g, g)));
-                    }
+                        for (int j = 0; j < 2; ++j) {
+                            const f2 ey = reinterpret_cast<const f2&>(mx.ey[xg + a][ty + 8 * i]);
+                            const f2 fy = reinterpret_cast<const f2&>(mx.fy[xg + a][ty + 8 * i]);
+                            const f2 ez = reinterpret_cast<const f2&>(mx.ez[xg + a][tx + 8 * j]);
+                            const f2 fz = reinterpret_cast<const f2&>(mx.fz[xg + a][tx + 8 * j]);
+                            const float g = mx.g[ty + 8 * i][tx + 8 * j];
+                            const f2 p1 = prod2(ey, fz), p2 = prod2(ez, fy);
+                            A.sg[a][i][j] = bias_of(max2(p1, p2));
+                            A.cb[a][i][j] = bias_of(prod2(add2(p1, p2), pk(g, g)));
+                        }
+            }
         }
         const auto& cur = sm.st[b];
 #pragma unroll
@@ -667,8 +487,10 @@ __global__ void __launch_bounds__(BTH, 1)
             for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const float2 u = cur.g1[st][ty + 16 * i][2 * ((tx / 2 + 8 * j) ^ ty) + (tx & 1)];
-                    const float2 v = cur.g2[st][tx + 16 * j][2 * ((ty / 2 + 8 * i) ^ tx) + (ty & 1)];
+                    const float2 u =
+                        cur.g1[st][ty + 8 * i][2 * ((tx / 2 + 4 * j) ^ swz(ty)) + (tx & 1)];
+                    const float2 v =
+                        cur.g2[st][tx + 8 * j][2 * ((ty / 2 + 4 * i) ^ swz(tx)) + (ty & 1)];
                     g1h[i][j] = pk(u.x, u.x);
                     g1l[i][j] = pk(u.y, u.y);
                     g2h[i][j] = pk(v.x, v.x);
@@ -676,22 +498,37 @@ __global__ void __launch_bounds__(BTH, 1)
                 }
 #pragma unroll
             for (int xp = 0; xp < 2; ++xp) {
+                // {h(x), h(x+1)} and {l(x), l(x+1)} as two 64-bit lanes
                 ulonglong2 ey[2], fy[2], ez[2], fz[2];
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    ey[i] = reinterpret_cast<const ulonglong2&>(cur.ey[st][xp][ty + 16 * i]);
-                    fy[i] = reinterpret_cast<const ulonglong2&>(cur.fy[st][xp][ty + 16 * i]);
-                    ez[i] = reinterpret_cast<const ulonglong2&>(cur.ez[st][xp][tx + 16 * i]);
-                    fz[i] = reinterpret_cast<const ulonglong2&>(cur.fz[st][xp][tx + 16 * i]);
+                    ey[i] = reinterpret_cast<const ulonglong2&>(cur.ey[st][xg + xp][ty + 8 * i]);
+                    fy[i] = reinterpret_cast<const ulonglong2&>(cur.fy[st][xg + xp][ty + 8 * i]);
+                    ez[i] = reinterpret_cast<const ulonglong2&>(cur.ez[st][xg + xp][tx + 8 * i]);
+                    fz[i] = reinterpret_cast<const ulonglong2&>(cur.fz[st][xg + xp][tx + 8 * i]);
                 }
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    f2 th[2], tl[2];
-                    bias_dot2(ey[i], fy[i], ez, fz, sg[xp][i], th, tl);
+                    if constexpr (BIAS) {
+                        f2 th[2], tl[2];
+                        bias_dot2(ey[i], fy[i], ez, fz, A.sg[xp][i], th, tl);
 #pragma unroll
-                    for (int j = 0; j < 2; ++j)
-                        bias_acc(h1[xp][i][j], h2[xp][i][j], th[j], tl[j], g1h[i][j], g1l[i][j],
-                                 g2h[i][j], g2l[i][j], cb[xp][i][j]);
+                        for (int j = 0; j < 2; ++j)
+                            bias_acc(A.h1[xp][i][j], A.h2[xp][i][j], th[j], tl[j], g1h[i][j],
+                                     g1l[i][j], g2h[i][j], g2l[i][j], A.cb[xp][i][j]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            f2 th, tl;
+                            df_dot2(ey[i].x, ey[i].y, fz[j].x, fz[j].y, ez[j].x, ez[j].y, fy[i].x,
+                                    fy[i].y, th, tl);
+                            const f2 thn = neg2(th);
+                            df_acc(A.h1[xp][i][j], A.l1[xp][i][j], th, tl, thn, g1h[i][j],
+                                   g1l[i][j]);
+                            df_acc(A.h2[xp][i][j], A.l2[xp][i][j], th, tl, thn, g2h[i][j],
+                                   g2l[i][j]);
+                        }
+                    }
                 }
             }
         }
@@ -701,7 +538,7 @@ __global__ void __launch_bounds__(BTH, 1)
     if (nsteps > 0) fold((unsigned)inchunk);
     // On a diagonal pair both accumulators cover the same tile and count
     // every (Y, Z) twice.
-    const double scale = diag ? 0.5 : 1.0;
+    const double scale = (diag ? 0.5 : 1.0) * (BIAS ? 1.0 : -1.0);
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
         if (m == 1 && diag) __syncthreads();   // mirror targets overlap other threads' first targets
@@ -711,18 +548,37 @@ __global__ void __launch_bounds__(BTH, 1)
             for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const int Y = Y0 + ty + 16 * i, Z = Z0 + tx + 16 * j;
+                    const int Y = Y0 + ty + 8 * i, Z = Z0 + tx + 8 * j;
                     if (Y >= P || Z >= P) continue;
-                    const ulonglong2 v = sm.sum[(xp * 4 + i * 2 + j) * 2 + m][tid];
                     float a0, a1, b0, b1;
-                    upk(v.x, a0, a1);
-                    upk(v.y, b0, b1);
-                    const int x = X0 + 2 * xp;
+                    if constexpr (BIAS) {
+                        const ulonglong2 v = sm.sum[(xp * 4 + i * 2 + j) * 2 + m][tid];
+                        upk(v.x, a0, a1);
+                        upk(v.y, b0, b1);
+                    } else {
+                        upk(m == 0 ? A.h1[xp][i][j] : A.h2[xp][i][j], a0, a1);
+                        upk(m == 0 ? A.l1[xp][i][j] : A.l2[xp][i][j], b0, b1);
+                    }
+                    const int x = X0 + 2 * (xg + xp);
                     const long long at = m == 0 ? (long long)Y * P + Z : (long long)Z * P + Y;
                     if (x < nX) H[x * PP + at] += scale * ((double)a0 + (double)b0);
                     if (x + 1 < nX) H[(x + 1) * PP + at] += scale * ((double)a1 + (double)b1);
                 }
     }
+}
+
+template <bool BIAS, bool EVEN>
+cudaError_t launch_df(double* H, const float4* E4, const float4* F4, const float2* G2,
+                      const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
+                      cudaStream_t s) {
+    const int smem = (int)sizeof(DfSmem<BIAS>);
+    const cudaError_t e = smem_optin((const void*)k_triangle_df<BIAS, EVEN>, smem);
+    if (e != cudaSuccess) return e;
+    const long long nb = cdiv(P, DT), grid = cdiv(nX, DX) * (nb * (nb + 1) / 2);
+    if (grid > INT32_MAX) return cudaErrorInvalidValue;
+    k_triangle_df<BIAS, EVEN><<<(unsigned)grid, DTH, smem, s>>>(H, E4, F4, G2, ME, MF, MG, P, nX, nI);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 // M[chunk][Y][Z] = max over the chunk's grid points of |G_h^YZ| and |G_h^ZY|.
@@ -875,23 +731,11 @@ cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const flo
                         const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
                         cudaStream_t s) {
     if (nX <= 0 || nI <= 0) return cudaSuccess;
-    const unsigned nb = cdiv(P, DT);
-    const bool bias = ME && MF && MG, even = P % 2 == 0;
-    const void* kern = !bias ? (const void*)k_triangle_df
-                             : (even ? (const void*)k_triangle_bias<true>
-                                     : (const void*)k_triangle_bias<false>);
-    const int smem = (int)(bias ? sizeof(BiasSmem) : 2 * sizeof(DfStage));
-    cudaError_t e = smem_optin(kern, smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(cdiv(nX, DX), nb * (nb + 1) / 2);
-    if (bias && even)
-        k_triangle_bias<true><<<grid, BTH, smem, s>>>(H, E4, F4, G2, ME, MF, MG, P, nX, nI);
-    else if (bias)
-        k_triangle_bias<false><<<grid, BTH, smem, s>>>(H, E4, F4, G2, ME, MF, MG, P, nX, nI);
-    else
-        k_triangle_df<<<grid, DTH, smem, s>>>(H, E4, F4, G2, P, nX, nI);
-    count_launches(1);
-    return cudaGetLastError();
+    if (ME && MF && MG)
+        return P % 2 ? launch_df<true, false>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s)
+                     : launch_df<true, true>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s);
+    return P % 2 ? launch_df<false, false>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s)
+                 : launch_df<false, true>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s);
 }
 
 }  // namespace thc
