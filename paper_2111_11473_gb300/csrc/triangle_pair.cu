@@ -10,18 +10,20 @@
 // the kernel issues one packed multiply and three packed FMAs: 2 FMA-pipe
 // lanes per (I, X, Y, Z) term, where the unpaired form takes 3.
 //
-// Block: 16 X (8 pairs) x a mirror pair of 32 x 32 (Y, Z) tiles, 256
-// threads.  Warp w takes pairs 4 (w / 4) .. + 3, Y half (w / 2) % 2 and Z
-// half w % 2; lane (lx, ly, lz) = (lane / 16, lane / 4 % 4, lane % 4) owns
-// the pairs 4 (w / 4) + lx + 2p (p < 2), Y = 16 ((w / 2) % 2) + 4 ly + (0..3)
-// and Z = 16 (w % 2) + 4 lz + (0..3): 64 packed accumulators per thread.
-// One thread streams the operands with 3-D TMA boxes (128-byte swizzle)
-// through a ring of QS stages of QI grid points; every wait is bounded.
-// The last warp to finish with a stage issues its refill.  Measured at
-// P = 400, 400 rows X, 1200 grid points: two stages of six grid points
-// 8.54 ms (0.56 of the FP32 peak in algorithmic flops), three of four 9.33,
-// four of three 9.89, five of two 10.57; with the refills issued by one
-// thread of warp 0 instead, 9.16, 9.85, 10.6 and 12.2 ms.
+// Block: 32 X (16 pairs) x a mirror pair of 16 x 16 (Y, Z) tiles, 128 threads,
+// two blocks per SM.  The tile is small because mirror pairs of tiles compute
+// the diagonal twice and the ragged edge for nothing (32-wide tiles 1.16 times
+// the needed work at P = 400, 16-wide ones 1.04).  Warp w takes pairs 4 w ..
+// + 3; lane (ly, lx, lz) = (lane / 8, lane / 4 % 2, lane % 4) owns the pairs
+// 4 w + lx + 2p (p < 2), Y = 4 ly + (0..3) and Z = 4 lz + (0..3): 64 packed
+// accumulators per thread.  One thread streams the operands with 3-D TMA
+// boxes (swizzled) through a ring of QS stages of QI grid points; every wait
+// is bounded.  The last warp to finish with a stage issues its refill.
+// Bound: register reads of the packed FMAs (three distinct register pairs take
+// 3.3 cycles of a scheduler, 2 at best).  Measured at P = 400, 400 rows X, 1200
+// grid points: two stages of five grid points 7.99 ms (0.60 of the FP32 peak
+// in algorithmic flops), two of four 8.25, three of three 8.98, five of two
+// 9.04; blocks of 256 threads, 16 X and 32-wide tiles took 8.49.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -36,25 +38,25 @@ namespace {
 typedef unsigned long long f2;   // two float32 lanes: low word = lane 0 (X = 2q)
 
 #ifndef THC_PAIR_QI
-#define THC_PAIR_QI 6
+#define THC_PAIR_QI 5
 #endif
 #ifndef THC_PAIR_QS
 #define THC_PAIR_QS 2
 #endif
-constexpr int QT = 32;            // Y and Z tile
-constexpr int QP = 8;             // X pairs per block
+constexpr int QT = 16;            // Y and Z tile
+constexpr int QP = 16;            // X pairs per block
+constexpr int QTH = 128;          // threads: a warp per four X pairs
 constexpr int QI = THC_PAIR_QI;   // grid points per stage
 constexpr int QS = THC_PAIR_QS;   // ring stages
 constexpr long long kQWait = 4000000000LL;
 
 struct QSmem {
-    // E2, F2 half tiles: [stage][half][grid point][pair][16 pairs of floats]
-    // (128-byte rows, 1 KB per (half, grid point)).
-    f2 ey[QS][2][QI][QP][16];
-    f2 ez[QS][2][QI][QP][16];
-    f2 fy[QS][2][QI][QP][16];
-    f2 fz[QS][2][QI][QP][16];
-    float g1[QS][QI][QT][QT];   // G^YZ, rows Y
+    // E2, F2 tiles: [stage][grid point][pair][16 pairs of floats], 128-byte rows
+    f2 ey[QS][QI][QP][QT];
+    f2 ez[QS][QI][QP][QT];
+    f2 fy[QS][QI][QP][QT];
+    f2 fz[QS][QI][QP][QT];
+    float g1[QS][QI][QT][QT];   // G^YZ, rows Y (64 bytes)
     float g2[QS][QI][QT][QT];   // G^ZY, rows Z
     unsigned long long full[QS];
     unsigned cnt[QS];     // warps done with the stage, over all its uses
@@ -99,9 +101,10 @@ __device__ __forceinline__ ulonglong2 lds_pairs(unsigned tile, int row, int chun
     asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];\n" : "=l"(v.x), "=l"(v.y) : "r"(a));
     return v;
 }
+// The same of a 64-byte row (chunk c of row r at c ^ (r / 2 & 3)).
 __device__ __forceinline__ float4 lds_f4(unsigned tile, int row, int chunk) {
     float4 v;
-    const unsigned a = tile + (unsigned)(row * 128) + ((unsigned)(chunk ^ (row & 7)) << 4);
+    const unsigned a = tile + (unsigned)(row * 64) + ((unsigned)(chunk ^ (row >> 1 & 3)) << 4);
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                  : "r"(a));
@@ -133,7 +136,7 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 // Grid: block of QP X pairs (fastest, so that the blocks running together share
 // the G tiles of one mirror pair in L2), pair of mirror tiles (in one
 // dimension: the pairs of P > 11552 exceed the second one's 65535 blocks).
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(QTH, 2)
     k_triangle_pair(float* H, const __grid_constant__ CUtensorMap tmE,
                     const __grid_constant__ CUtensorMap tmF,
                     const __grid_constant__ CUtensorMap tmG, int P, int ld, int nX, int nI,
@@ -152,10 +155,9 @@ __global__ void __launch_bounds__(256, 1)
     const int Y0 = Yb * QT, Z0 = Zb * QT, q0 = xb * QP;
     const bool diag = Yb == Zb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int xs = warp >> 2, wy = (warp >> 1) & 1, wz = warp & 1;
-    const int lx = lane >> 4, ly = (lane >> 2) & 3, lz = lane & 3;
+    const int lz = lane & 3, lx = (lane >> 2) & 1, ly = lane >> 3;
     const int nst = (nI + QI - 1) / QI;
-    const unsigned stage_bytes = 8u * QI * QP * 128u + 2u * QI * QT * QT * 4u;
+    const unsigned stage_bytes = 4u * QI * QP * QT * 8u + 2u * QI * QT * QT * 4u;
     if (threadIdx.x == 0) {
         for (int s = 0; s < QS; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&sm.full[s])));
@@ -173,13 +175,10 @@ __global__ void __launch_bounds__(256, 1)
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(
                          su32(&sm.full[s])),
                      "r"(stage_bytes));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            q_tma(&sm.ey[s][h][0][0][0], &tmE, &sm.full[s], Y0 + 16 * h, q0, I0);
-            q_tma(&sm.ez[s][h][0][0][0], &tmE, &sm.full[s], Z0 + 16 * h, q0, I0);
-            q_tma(&sm.fy[s][h][0][0][0], &tmF, &sm.full[s], Y0 + 16 * h, q0, I0);
-            q_tma(&sm.fz[s][h][0][0][0], &tmF, &sm.full[s], Z0 + 16 * h, q0, I0);
-        }
+        q_tma(&sm.ey[s][0][0][0], &tmE, &sm.full[s], Y0, q0, I0);
+        q_tma(&sm.ez[s][0][0][0], &tmE, &sm.full[s], Z0, q0, I0);
+        q_tma(&sm.fy[s][0][0][0], &tmF, &sm.full[s], Y0, q0, I0);
+        q_tma(&sm.fz[s][0][0][0], &tmF, &sm.full[s], Z0, q0, I0);
         q_tma(&sm.g1[s][0][0][0], &tmG, &sm.full[s], Z0, Y0, I0);
         q_tma(&sm.g2[s][0][0][0], &tmG, &sm.full[s], Y0, Z0, I0);
     };
@@ -207,22 +206,22 @@ __global__ void __launch_bounds__(256, 1)
             f2 gb1[4][4], gb2[4][4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4 u = lds_f4(g1t, 16 * wy + 4 * ly + i, 4 * wz + lz);
+                const float4 u = lds_f4(g1t, 4 * ly + i, lz);
                 gb1[i][0] = bcast(u.x);
                 gb1[i][1] = bcast(u.y);
                 gb1[i][2] = bcast(u.z);
                 gb1[i][3] = bcast(u.w);
-                const float4 w = lds_f4(g2t, 16 * wz + 4 * lz + i, 4 * wy + ly);
+                const float4 w = lds_f4(g2t, 4 * lz + i, ly);
                 gb2[0][i] = bcast(w.x);
                 gb2[1][i] = bcast(w.y);
                 gb2[2][i] = bcast(w.z);
                 gb2[3][i] = bcast(w.w);
             }
-            const unsigned eyt = su32(&sm.ey[s][wy][ti][0][0]), ezt = su32(&sm.ez[s][wz][ti][0][0]);
-            const unsigned fyt = su32(&sm.fy[s][wy][ti][0][0]), fzt = su32(&sm.fz[s][wz][ti][0][0]);
+            const unsigned eyt = su32(&sm.ey[s][ti][0][0]), ezt = su32(&sm.ez[s][ti][0][0]);
+            const unsigned fyt = su32(&sm.fy[s][ti][0][0]), fzt = su32(&sm.fz[s][ti][0][0]);
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                const int q = 4 * xs + 2 * p + lx;
+                const int q = 4 * warp + 2 * p + lx;
                 f2 ey[4], fy[4], ez[4], fz[4];
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
@@ -263,7 +262,7 @@ __global__ void __launch_bounds__(256, 1)
         if (lane == 0) {
             __threadfence_block();
             const unsigned done = atomicAdd(&sm.cnt[s], 1u);
-            if (done % 8u == 7u && k + QS < nst) {
+            if (done % (QTH / 32u) == QTH / 32u - 1u && k + QS < nst) {
                 __threadfence_block();
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 issue(k + QS);
@@ -287,12 +286,12 @@ __global__ void __launch_bounds__(256, 1)
     const float scale = diag ? 0.5f : 1.f;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-        const int X = 2 * (q0 + 4 * xs + 2 * p + lx);
-        const int Zs = Z0 + 16 * wz + 4 * lz;
+        const int X = 2 * (q0 + 4 * warp + 2 * p + lx);
+        const int Zs = Z0 + 4 * lz;
         if (Zs >= P) continue;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int Y = Y0 + 16 * wy + 4 * ly + i;
+            const int Y = Y0 + 4 * ly + i;
             if (Y >= P) continue;
             float v0[4], v1[4];
 #pragma unroll
@@ -314,12 +313,12 @@ __global__ void __launch_bounds__(256, 1)
     if (diag) __syncthreads();   // mirror targets overlap other threads' first targets
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-        const int X = 2 * (q0 + 4 * xs + 2 * p + lx);
-        const int Ys = Y0 + 16 * wy + 4 * ly;
+        const int X = 2 * (q0 + 4 * warp + 2 * p + lx);
+        const int Ys = Y0 + 4 * ly;
         if (Ys >= P) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int Z = Z0 + 16 * wz + 4 * lz + j;
+            const int Z = Z0 + 4 * lz + j;
             if (Z >= P) continue;
             float v0[4], v1[4];
 #pragma unroll
@@ -365,9 +364,9 @@ PFN_cuTensorMapEncodeTiled_v12000 g_q_encode = nullptr;
 std::once_flag g_q_once;
 
 // 3-D map (x, rows, nI) of elements of `esize` bytes (x contiguous, rows
-// `ld` elements apart), box (bx, by, QI), 128-byte swizzle, zero fill outside.
+// `ld` elements apart), box (bx, by, QI), zero fill outside.
 cudaError_t q_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int esize, long long x,
-                  long long ld, long long rows, int nI, int bx, int by) {
+                  long long ld, long long rows, int nI, int bx, int by, CUtensorMapSwizzle sw) {
     std::call_once(g_q_once, [] {
         cudaDriverEntryPointQueryResult q;
         void* fn = nullptr;
@@ -382,7 +381,7 @@ cudaError_t q_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int 
     cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)QI};
     cuuint32_t es[3] = {1, 1, 1};
     CUresult r = g_q_encode(m, dt, 3, const_cast<void*>(base), dims, strides, box, es,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -416,16 +415,21 @@ cudaError_t triangle_pair(float* H, const float2* E2, const float2* F2, const fl
         return cudaErrorInvalidValue;
     const int nXp = (nX + 1) / 2;
     CUtensorMap mE, mF, mG;
-    cudaError_t e = q_map(&mE, E2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, ld, nXp, nI, 16, QP);
-    if (e == cudaSuccess) e = q_map(&mF, F2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, ld, nXp, nI, 16, QP);
-    if (e == cudaSuccess) e = q_map(&mG, G, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, P, ld, P, nI, QT, QT);
+    cudaError_t e = q_map(&mE, E2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, ld, nXp, nI, QT, QP,
+                          CU_TENSOR_MAP_SWIZZLE_128B);
+    if (e == cudaSuccess)
+        e = q_map(&mF, F2, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, P, ld, nXp, nI, QT, QP,
+                  CU_TENSOR_MAP_SWIZZLE_128B);
+    if (e == cudaSuccess)
+        e = q_map(&mG, G, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, P, ld, P, nI, QT, QT,
+                  CU_TENSOR_MAP_SWIZZLE_64B);
     if (e != cudaSuccess) return e;
     const int smem = (int)sizeof(QSmem) + 1024;
     e = smem_optin((const void*)k_triangle_pair, smem);
     if (e != cudaSuccess) return e;
     const long long nb = cdiv(P, QT), grid = cdiv(nXp, QP) * (nb * (nb + 1) / 2);
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
-    k_triangle_pair<<<(unsigned)grid, 256, smem, s>>>(H, mE, mF, mG, P, ld, nX, nI, err);
+    k_triangle_pair<<<(unsigned)grid, QTH, smem, s>>>(H, mE, mF, mG, P, ld, nX, nI, err);
     count_launches(1);
     return cudaGetLastError();
 }
