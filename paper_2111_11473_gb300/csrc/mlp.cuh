@@ -26,7 +26,7 @@ struct Mlp {
     // scratch for batches of up to cap samples
     long long cap = 0;
     float *a1 = nullptr, *a2 = nullptr, *d1 = nullptr, *d2 = nullptr;
-    float *y = nullptr, *dy = nullptr, *ones = nullptr, *red = nullptr;
+    float *y = nullptr, *dy = nullptr, *red = nullptr;
     float *xb = nullptr, *jb = nullptr, *tb = nullptr;
     float* splitk = nullptr;
     size_t splitk_elems = 0;
