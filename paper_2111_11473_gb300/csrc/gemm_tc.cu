@@ -1020,6 +1020,7 @@ struct SliceOp {
     const double* src;
     long long rs, ks, bs;
     int R, nb;
+    int flat;            // the batches' rows form one list (b R + r) of the slices
     __nv_bfloat16* out;
     int* expo;
 };
@@ -1119,9 +1120,12 @@ __device__ __forceinline__ void slice_store(const SlicePair& p, const SliceOp& o
         for (int q = 0; q < kSlices; ++q) v[q][j] = __byte_perm(d0[q], d1[q], 0x7632);
     }
     const long long nkb = (p.Ktot + BK - 1) / BK;
-    const long long kg = (p.reduce ? (long long)b * p.Kp : 0) + k, bo = p.reduce ? 0 : b;
-    __nv_bfloat16* o = op.out + ((bo * nkb + kg / BK) * kSlices * op.R + r) * BK + kg % BK;
-    const long long plane = (long long)op.R * BK;
+    const long long kg = (p.reduce ? (long long)b * p.Kp : 0) + k;
+    const long long bo = p.reduce || op.flat ? 0 : b;
+    const long long rows = op.flat ? (long long)op.nb * op.R : op.R;
+    const long long row = op.flat ? (long long)b * op.R + r : r;
+    __nv_bfloat16* o = op.out + ((bo * nkb + kg / BK) * kSlices * rows + row) * BK + kg % BK;
+    const long long plane = rows * BK;
 #pragma unroll
     for (int q = 0; q < kSlices; ++q)
         *reinterpret_cast<uint4*>(o + q * plane) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
@@ -1332,7 +1336,9 @@ struct F64Smem {
 };
 
 struct F64Args {
-    int M, N;                // real accumulator rows (A side) and columns (B side)
+    int M, N;                // real accumulator rows (A side, all batches of a
+                             // collapsed product) and columns (B side)
+    int Mb;                  // rows per batch: row i is row i % Mb of batch bo + i / Mb
     int nbo, mblocks, nblocks, ksteps, splits;
     int last_kk;             // 16-deep sub-steps of the last K step
     long long ntiles;        // mblocks * nblocks * nbo * splits
@@ -1341,6 +1347,7 @@ struct F64Args {
     const int* eB;
     double* C;               // output, or float64 partials when splits > 1
     long long crs, ccs, cbs;
+    long long split_stride;  // partials of one split
     double alpha, beta;
     int alpha_exp;           // alpha = +-2^alpha_exp, or kNoPow2
     int hshift;              // fractional bits below the int64 sums' unit
@@ -1787,9 +1794,10 @@ __global__ void __launch_bounds__(kF64Threads, 1)
             __syncwarp();
             if (i >= args.M || ncols <= 0) continue;
             f64_finish(H, T, eb, args.hshift, fa, ebase, aneg, range_ok, ncols);
-            double* Cr = args.C + (long long)c.bo * args.cbs +
-                         (partial ? (long long)c.split * args.nbo * args.cbs : 0) +
-                         (long long)i * args.crs + (long long)col0 * args.ccs;
+            const int ib = i / args.Mb;
+            double* Cr = args.C + (long long)(c.bo + ib) * args.cbs +
+                         (partial ? (long long)c.split * args.split_stride : 0) +
+                         (long long)(i - ib * args.Mb) * args.crs + (long long)col0 * args.ccs;
             if (general) {
 #pragma unroll
                 for (int j = 0; j < FC; ++j) {
@@ -1925,11 +1933,17 @@ namespace {
 cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cudaStream_t s) {
     cudaError_t e = get_encode();
     if (e != cudaSuccess) return e;
-    const bool swap = g.N > g.M;
-    const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
-    const long long Kp = rup(std::max(g.K, 1), 8);
     const int nb = g.batch;
     const int nbo = g.reduce ? 1 : nb;
+    // The larger side takes the 128-row tiles; if one operand is shared by
+    // every batch, the rows of all batches of the other one, as one list:
+    // otherwise every batch has a ragged tile (131 rows fill two tiles of 128
+    // to a half, 200 and 400 rows 0.78 of theirs).
+    const bool m_bc = !g.reduce && nb > 1 && g.sAb == 0, n_bc = !g.reduce && nb > 1 && g.sBb == 0;
+    const bool flat = m_bc != n_bc && (long long)nb * (m_bc ? g.N : g.M) < INT32_MAX;
+    const bool swap = flat ? m_bc : g.N > g.M;
+    const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
+    const long long Kp = rup(std::max(g.K, 1), 8);
     const long long Ktot = f64_ktot(g.K, nb, g.reduce);
     View<double> va = g.A, vb{g.B.p, g.B.cs, g.B.rs};
     long long sa = g.sAb, sb = g.sBb;
@@ -1941,8 +1955,9 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     const bool b_bc = !g.reduce && nb > 1 && sb == 0;
     const int nba = a_bc ? 1 : nbo, nbb = b_bc ? 1 : nbo;
     const long long sliceA = (long long)Mr * kSlices * rup(Ktot, BK) * nba;
-    const int mblocks = (int)cdiv(Mr, BM), nblocks = (int)cdiv(Nr, FN);
-    const long long tiles = (long long)mblocks * nblocks * nbo;
+    const int rowsA = flat ? nb * Mr : Mr, tilesets = flat ? 1 : nbo;
+    const int mblocks = (int)cdiv(rowsA, BM), nblocks = (int)cdiv(Nr, FN);
+    const long long tiles = (long long)mblocks * nblocks * tilesets;
     const int ksteps = (int)((Ktot + BK - 1) / BK);
     const long long sms = device_sms();
     const int splits = f64_splits(tiles, ksteps, (long long)Mr * Nr * nbo, ws.part_elems, sms);
@@ -1953,8 +1968,8 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     int* eB = ws.expo + (long long)Mr * nba;
     // Row exponents and slices of both operands.
     SlicePair p{};
-    p.op[0] = SliceOp{va.p, va.rs, va.cs, sa, Mr, a_bc ? 1 : nb, slA, eA};
-    p.op[1] = SliceOp{vb.p, vb.rs, vb.cs, sb, Nr, b_bc ? 1 : nb, slB, eB};
+    p.op[0] = SliceOp{va.p, va.rs, va.cs, sa, Mr, a_bc ? 1 : nb, flat ? 1 : 0, slA, eA};
+    p.op[1] = SliceOp{vb.p, vb.rs, vb.cs, sb, Nr, b_bc ? 1 : nb, 0, slB, eB};
     p.Kd = g.K;
     p.Kp = (int)Kp;
     p.Ktot = Ktot;
@@ -1985,12 +2000,13 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     CUtensorMap mA, mB;
-    if ((e = make_map_slices(&mA, slA, ksteps, Mr, nba, BM, 1)) != cudaSuccess) return e;
+    if ((e = make_map_slices(&mA, slA, ksteps, rowsA, flat ? 1 : nba, BM, 1)) != cudaSuccess) return e;
     if ((e = make_map_slices(&mB, slB, ksteps, Nr, nbb, FN, kSlices)) != cudaSuccess) return e;
     F64Args a{};
-    a.M = Mr;
+    a.M = rowsA;
     a.N = Nr;
-    a.nbo = nbo;
+    a.Mb = Mr;
+    a.nbo = tilesets;
     a.mblocks = mblocks;
     a.nblocks = nblocks;
     a.ksteps = ksteps;
@@ -2025,6 +2041,7 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
         a.crs = swap ? 1 : Nr;
         a.ccs = swap ? Mr : 1;
         a.cbs = (long long)Mr * Nr;
+        a.split_stride = a.cbs * nbo;
     } else {
         a.C = g.C;
         a.crs = crs;
