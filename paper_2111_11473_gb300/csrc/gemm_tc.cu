@@ -509,7 +509,8 @@ struct PackOp {
     __nv_bfloat16* hi;
     __nv_bfloat16* lo;     // null: hi only
 };
-constexpr int PK_R = 32, PK_K = 64;    // strided sources: tile through shared memory
+constexpr int PK_R = 32, PK_K = 64;    // tiles of strided float64 sources
+constexpr int PT_R = 64;               // rows of a tile of strided float32 sources
 constexpr int PK_U = 4;                // contiguous sources: octets of k per thread
 
 __device__ __forceinline__ void pack_octet(const PackOp& op, long long row, int b, int r, int k,
@@ -559,45 +560,50 @@ __device__ __forceinline__ void pack_contiguous(const PackOp& op, long long u) {
     }
 }
 
-// One block's unit of any other source: a 32 (r) x 64 (k) tile goes through
+// One block's unit of any other source: a 64 (r) x 64 (k) tile goes through
 // shared memory so that the global reads run along whichever index of the
-// source is contiguous, and every thread then writes 8 consecutive k of one
-// row as one 16-byte store of hi and lo.
+// source is contiguous, and every thread then writes 8 consecutive k of a row
+// as one 16-byte store of hi and lo.  16 loads per thread are in flight (with
+// 32 rows and 8 loads, 600 x 400 x 400 took 228 us, of which its bytes take 114).
 __device__ __forceinline__ void pack_tile(const PackOp& op, long long u,
                                           float (*tile)[PK_K + 1]) {
-    const int tk = (op.Kp + PK_K - 1) / PK_K, tr = (op.R + PK_R - 1) / PK_R;
+    const int tk = (op.Kp + PK_K - 1) / PK_K, tr = (op.R + PT_R - 1) / PT_R;
     const int k0 = (int)(u % tk) * PK_K;
     const long long v = u / tk;
-    const int r0 = (int)(v % tr) * PK_R, b = (int)(v / tr);
+    const int r0 = (int)(v % tr) * PT_R, b = (int)(v / tr);
     const float* s = op.src + (long long)b * op.bs;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    float x[8];
+    float x[16];
     if (op.ks <= op.rs) {
         // warp w reads rows w, w + 8, ...; lanes run along k (two halves of 32)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
+        for (int e = 0; e < 16; ++e) {
             const int r = r0 + warp + 8 * (e >> 1), k = k0 + (e & 1) * 32 + lane;
             x[e] = (r < op.R && k < op.Kd) ? s[(long long)r * op.rs + (long long)k * op.ks] : 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) tile[warp + 8 * (e >> 1)][(e & 1) * 32 + lane] = x[e];
+        for (int e = 0; e < 16; ++e) tile[warp + 8 * (e >> 1)][(e & 1) * 32 + lane] = x[e];
     } else {
-        // warp w reads columns w, w + 8, ...; lanes run along r
+        // warp w reads columns w, w + 8, ...; lanes run along r (two halves of 32)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int r = r0 + lane, k = k0 + warp + 8 * e;
+        for (int e = 0; e < 16; ++e) {
+            const int r = r0 + (e & 1) * 32 + lane, k = k0 + warp + 8 * (e >> 1);
             x[e] = (r < op.R && k < op.Kd) ? s[(long long)r * op.rs + (long long)k * op.ks] : 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) tile[lane][warp + 8 * e] = x[e];
+        for (int e = 0; e < 16; ++e) tile[(e & 1) * 32 + lane][warp + 8 * (e >> 1)] = x[e];
     }
     __syncthreads();
-    const int rr = t >> 3, r = r0 + rr, k = k0 + (t & 7) * 8;   // 32 rows x 8 octets of k
-    if (r < op.R && k < op.Kp) {
-        float w[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) w[e] = tile[rr][(t & 7) * 8 + e];
-        pack_octet(op, (long long)b * op.R + r, b, r, k, w);
+    for (int h = 0; h < 2; ++h) {
+        // 32 rows x 8 octets of k
+        const int rr = (t >> 3) + 32 * h, r = r0 + rr, k = k0 + (t & 7) * 8;
+        if (r < op.R && k < op.Kp) {
+            float w[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) w[e] = tile[rr][(t & 7) * 8 + e];
+            pack_octet(op, (long long)b * op.R + r, b, r, k, w);
+        }
     }
     __syncthreads();
 }
@@ -605,7 +611,7 @@ __device__ __forceinline__ void pack_tile(const PackOp& op, long long u,
 // Both operands of a product in one launch (one launch each cost 2 to 3 us
 // more per product, and most operands are packed in 4 to 10).
 __global__ void __launch_bounds__(256) k_pack(const PackOp a, const PackOp b) {
-    __shared__ float tile[PK_R][PK_K + 1];
+    __shared__ float tile[PT_R][PK_K + 1];
     for (long long u = blockIdx.x; u < a.units + b.units; u += gridDim.x) {
         if (u < a.units) {
             if (a.vec) pack_contiguous(a, u);
@@ -743,7 +749,7 @@ PackOp pack_op(const float* p, long long rs, long long ks, long long bs, int R, 
     op.vec = ks == 1 && Kd % 4 == 0 && rs % 4 == 0 && (nb == 1 || bs % 4 == 0) &&
              reinterpret_cast<uintptr_t>(p) % 16 == 0 && rows < INT32_MAX;
     op.units = op.vec ? (rows * (Kp / 8) + 256 * PK_U - 1) / (256 * PK_U)
-                      : (long long)cdiv(Kp, PK_K) * cdiv(R, PK_R) * nb;
+                      : (long long)cdiv(Kp, PK_K) * cdiv(R, PT_R) * nb;
     return op;
 }
 
