@@ -27,6 +27,7 @@ unsigned nblk(long long n) { return (unsigned)std::min<long long>((n + 255) / 25
 
 // te[P][X] = eps_P^2 tau[P][X]
 __global__ void k_weight_rows(const double* tau, const double* eps, int N, int W, double* te) {
+    grid_wait();
     const long long tot = (long long)N * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
          e += (long long)gridDim.x * blockDim.x) {
@@ -38,6 +39,7 @@ __global__ void k_weight_rows(const double* tau, const double* eps, int N, int W
 // occ = 1: R[i][X] = sum_a M[(i,a)][X] yv[a][X];  occ = 0: R[a][X] = sum_i M[(i,a)][X] yo[i][X]
 __global__ void k_reduce_other(const double* M, const double* f, int o, int v, int W, int occ,
                                double* R) {
+    grid_wait();
     const int rows = occ ? o : v, other = occ ? v : o;
     const long long tot = (long long)rows * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
@@ -54,6 +56,7 @@ __global__ void k_reduce_other(const double* M, const double* f, int o, int v, i
 
 // KR[(i,a)][X] = yo[i][X] yv[a][X]
 __global__ void k_khatri_rao(const double* yo, const double* yv, int o, int v, int W, double* KR) {
+    grid_wait();
     const long long tot = (long long)o * v * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
          e += (long long)gridDim.x * blockDim.x) {
@@ -64,6 +67,7 @@ __global__ void k_khatri_rao(const double* yo, const double* yv, int o, int v, i
 }
 
 __global__ void k_mul(double* a, const double* b, long long n) {
+    grid_wait();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x)
         a[e] *= b[e];
@@ -72,6 +76,7 @@ __global__ void k_mul(double* a, const double* b, long long n) {
 // part[block] = sum over its elements of (eps_P (U - rec))^2, U, rec: (ov) x N
 __global__ void k_wsq(const double* U, const double* rec, const double* eps, long long rows,
                       int N, double* part) {
+    grid_wait();
     __shared__ double red[32];
     double s = 0;
     const long long tot = rows * N;
@@ -111,6 +116,7 @@ constexpr int kSolveSmem = 200 * 1024;   // rows of one block of the substitutio
 
 __global__ void __launch_bounds__(128) k_chol_panel(double* S, int W, int k0, double* D,
                                                     int* info) {
+    grid_wait();
     __shared__ double L[CB][CB + 1];
     __shared__ double col[2][CB];
     __shared__ double rinv[CB];
@@ -179,6 +185,7 @@ __global__ void __launch_bounds__(128) k_chol_panel(double* S, int W, int k0, do
 // Lower triangle beyond the panel at k0, a 16 x 16 tile per block:
 // S[i][j] -= sum_l X[i][l] X[j][l].
 __global__ void __launch_bounds__(256) k_chol_update(double* S, int W, int k0) {
+    grid_wait();
     __shared__ double xi[16][CB + 1], xj[16][CB + 1];
     int ti = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
     while ((long long)ti * (ti + 1) / 2 > blockIdx.x) --ti;
@@ -210,6 +217,7 @@ template <int RR>
 __global__ void __launch_bounds__(256) k_chol_solve(const double* S, int W, const double* D,
                                                     const double* B, int rows, double* out,
                                                     int in_smem) {
+    grid_wait();
     extern __shared__ double ybuf[];
     __shared__ double red[8][RR][CB];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -343,7 +351,7 @@ struct Als {
         cudaError_t e;
         if ((e = gemm(W, W, na, trv(A, W), rmv(A, W), S.p))) return e;
         if ((e = gemm(W, W, nb, trv(B, W), rmv(B, W), S2.p))) return e;
-        k_mul<<<nblk((long long)W * W), 256, 0, st>>>(S.p, S2.p, (long long)W * W);
+        launch_chained(k_mul, nblk((long long)W * W), 256, 0, st, S.p, S2.p, (long long)W * W);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -386,12 +394,12 @@ struct Als {
         cudaError_t e = cudaMemsetAsync(info.p, 0, sizeof(int), st);
         for (int k0 = 0; k0 < W && !e; k0 += CB) {
             const int rest = std::max(0, W - k0 - CB);
-            k_chol_panel<<<std::max(1u, cdiv(rest, 8)), 128, 0, st>>>(S.p, W, k0, diag.p,
-                                                                     (int*)info.p);
+            launch_chained(k_chol_panel, std::max(1u, cdiv(rest, 8)), 128, 0, st, S.p, W, k0,
+                           diag.p, (int*)info.p);
             count_launches(1);
             if (rest > 0) {
                 const long long T = cdiv(rest, 16);
-                k_chol_update<<<(unsigned)(T * (T + 1) / 2), 256, 0, st>>>(S.p, W, k0);
+                launch_chained(k_chol_update, (unsigned)(T * (T + 1) / 2), 256, 0, st, S.p, W, k0);
                 count_launches(1);
             }
             e = cudaGetLastError();
@@ -406,7 +414,8 @@ struct Als {
         if (!fits) smem = 0;
         cudaError_t e = smem_optin((const void*)k_chol_solve<RR>, kSolveSmem);
         if (e) return e;
-        k_chol_solve<RR><<<cdiv(rows, RR), 256, smem, st>>>(S.p, W, diag.p, R.p, rows, out, fits);
+        launch_chained(k_chol_solve<RR>, cdiv(rows, RR), 256, smem, st, S.p, W, diag.p, R.p, rows,
+                       out, fits);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -414,13 +423,13 @@ struct Als {
     cudaError_t objective(const double* U, const double* eps, const double* yo, const double* yv,
                           const double* tau, double* f) {
         cudaError_t e;
-        k_khatri_rao<<<nblk(ov * W), 256, 0, st>>>(yo, yv, o, v, W, KR.p);
+        launch_chained(k_khatri_rao, nblk(ov * W), 256, 0, st, yo, yv, o, v, W, KR.p);
         count_launches(1);
         if ((e = cudaGetLastError())) return e;
         if ((e = gemm((int)ov, N, W, rmv(KR.p, W), trv(tau, W), rec.p)))
             return e;
         const unsigned nb = nblk(ov * N);
-        k_wsq<<<nb, 256, 0, st>>>(U, rec.p, eps, ov, N, part.p);
+        launch_chained(k_wsq, nb, 256, 0, st, U, rec.p, eps, ov, N, part.p);
         count_launches(1);
         if ((e = cudaGetLastError())) return e;
         std::vector<double> hp(nb);
@@ -436,7 +445,7 @@ struct Als {
     cudaError_t sweep(const double* U, const double* eps, double* yo, double* yv, double* tau) {
         cudaError_t e;
         // y_o and y_v share M = U diag(eps^2) tau (tau is fixed in both updates)
-        k_weight_rows<<<nblk((long long)N * W), 256, 0, st>>>(tau, eps, N, W, te.p);
+        launch_chained(k_weight_rows, nblk((long long)N * W), 256, 0, st, tau, eps, N, W, te.p);
         count_launches(1);
         if ((e = cudaGetLastError())) return e;
         if ((e = gemm((int)ov, W, N, rmv(U, N), rmv(te.p, W), M.p)))
@@ -444,21 +453,21 @@ struct Als {
         // y_o: S = (y_v^T y_v) o (tau^T E tau)
         if ((e = gemm(W, W, N, trv(tau, W), rmv(te.p, W), SE.p))) return e;
         if ((e = gemm(W, W, v, trv(yv, W), rmv(yv, W), S.p))) return e;
-        k_mul<<<nblk((long long)W * W), 256, 0, st>>>(S.p, SE.p, (long long)W * W);
-        k_reduce_other<<<nblk((long long)o * W), 256, 0, st>>>(M.p, yv, o, v, W, 1, R.p);
+        launch_chained(k_mul, nblk((long long)W * W), 256, 0, st, S.p, SE.p, (long long)W * W);
+        launch_chained(k_reduce_other, nblk((long long)o * W), 256, 0, st, M.p, yv, o, v, W, 1, R.p);
         count_launches(2);
         if ((e = cudaGetLastError())) return e;
         if ((e = solve(o, yo))) return e;
         // y_v: S = (y_o^T y_o) o (tau^T E tau)
         if ((e = gemm(W, W, o, trv(yo, W), rmv(yo, W), S.p))) return e;
-        k_mul<<<nblk((long long)W * W), 256, 0, st>>>(S.p, SE.p, (long long)W * W);
-        k_reduce_other<<<nblk((long long)v * W), 256, 0, st>>>(M.p, yo, o, v, W, 0, R.p);
+        launch_chained(k_mul, nblk((long long)W * W), 256, 0, st, S.p, SE.p, (long long)W * W);
+        launch_chained(k_reduce_other, nblk((long long)v * W), 256, 0, st, M.p, yo, o, v, W, 0, R.p);
         count_launches(2);
         if ((e = cudaGetLastError())) return e;
         if ((e = solve(v, yv))) return e;
         // tau: S = (y_o^T y_o) o (y_v^T y_v), R = U^T KR(y_o, y_v)
         if ((e = gram2(yo, o, yv, v))) return e;
-        k_khatri_rao<<<nblk(ov * W), 256, 0, st>>>(yo, yv, o, v, W, KR.p);
+        launch_chained(k_khatri_rao, nblk(ov * W), 256, 0, st, yo, yv, o, v, W, KR.p);
         count_launches(1);
         if ((e = cudaGetLastError())) return e;
         if ((e = gemm(N, W, (int)ov, trv(U, N), rmv(KR.p, W), R.p)))

@@ -47,6 +47,7 @@ __global__ void k_outer_acc(const T* Acols, int P, int K, double* acc, double sc
 // memory and adds to out once (per-element atomics on three words took 214 us
 // at n = 400, 9 us now).
 __global__ void __launch_bounds__(256) k_asym(const double* a, int n, unsigned long long* out) {
+    grid_wait();
     __shared__ double t1[32][33], t2[32][33];
     __shared__ double red[2][8];
     __shared__ unsigned bad[8];
@@ -118,7 +119,7 @@ Err Engine<T>::check_sym(const double* a, int nn_, double rel, const char* what)
     unsigned long long h[3];
     THC_CUDA(cudaMemsetAsync(chk.p, 0, 3 * sizeof(unsigned long long), st));
     const unsigned nb_ = cdiv(nn_, 32);
-    k_asym<<<nb_ * (nb_ + 1) / 2, 256, 0, st>>>(a, nn_, chk.p);
+    launch_chained(k_asym, nb_ * (nb_ + 1) / 2, 256, 0, st, a, nn_, chk.p);
     count_launches(1);
     THC_CUDA(cudaGetLastError());
     THC_CUDA(cudaMemcpyAsync(h, chk.p, sizeof(h), cudaMemcpyDeviceToHost, st));

@@ -140,6 +140,7 @@ __device__ __forceinline__ void store_tiles(Smem<T, BM, BN>& sm, int buf, const 
 // register tile per thread, double-buffered shared memory.
 template <typename T, int BM, int BN>
 __global__ void __launch_bounds__(NT) gemm_kernel(const Gemm<T> g) {
+    grid_wait();
     __shared__ Smem<T, BM, BN> sm;
     constexpr int RI = BM / 16, RJ = BN / 16;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const Gemm<T> g) {
 
 template <typename T>
 __global__ void gemm_splitk_reduce(const Gemm<T> g) {
+    grid_wait();
     const long long MN = (long long)g.M * g.N;
     const int nb = g.reduce ? 1 : g.batch;
     const long long total = MN * nb;
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock)
     // blockIdx.y of g.splits shares a K range over blocks; their sums go to
     // g.ws for gemm_splitk_reduce
     constexpr int WN = 32 / WM, U = 8;
+    grid_wait();
     __shared__ double part[kWarpsPerBlock][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long tile = (long long)blockIdx.x * (kWarpsPerBlock / S) + warp / S;
@@ -341,6 +344,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock)
 // here), fixed-order reduction.
 template <typename T>
 __global__ void k_gemv_col(Gemm<T> g) {
+    grid_wait();
     __shared__ T part[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (long long m = blockIdx.x; m < g.M; m += gridDim.x) {
@@ -383,7 +387,7 @@ void tile_edges(long long M, long long N, long long nb, long long ksteps, int* B
 
 template <typename T, int BM, int BN>
 cudaError_t run(const Gemm<T>& g, dim3 grid, cudaStream_t s) {
-    gemm_kernel<T, BM, BN><<<grid, NT, 0, s>>>(g);
+    launch_chained(gemm_kernel<T, BM, BN>, grid, NT, 0, s, g);
     return cudaGetLastError();
 }
 
@@ -395,7 +399,7 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
     }
     if (std::is_same<T, double>::value && g.batch == 1 && !g.reduce && g.K > 0 && g.N == 1) {
         // float64 matrix times vector
-        k_gemv_col<T><<<(unsigned)std::min<long long>(g.M, 152 * 8), 256, 0, s>>>(g);
+        launch_chained(k_gemv_col<T>, (unsigned)std::min<long long>(g.M, 152 * 8), 256, 0, s, g);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -450,17 +454,15 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
             (g.M == 1 || t_warp * (fmas < 1e9 ? 1.1 : 1.5) < t_tile)) {
             g.splits = gs;
             const dim3 wgrid((unsigned)blocks, (unsigned)gs);
-            if (WM == 1)
-                k_gemm_warp64<1><<<wgrid, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
-            else
-                k_gemm_warp64<4><<<wgrid, 32 * kWarpsPerBlock, 0, s>>>(g, S, mt, nt, wt);
-            cudaError_t e = cudaGetLastError();
+            const cudaError_t e =
+                launch_chained(WM == 1 ? k_gemm_warp64<1> : k_gemm_warp64<4>, wgrid,
+                               32 * kWarpsPerBlock, 0, s, g, S, mt, nt, wt);
             if (e != cudaSuccess) return e;
             count_launches(gs > 1 ? 2 : 1);
             if (gs > 1) {
                 const long long total = (long long)g.M * g.N * nb;
                 const unsigned nbk = (unsigned)std::min<long long>((total + 255) / 256, 152LL * 32);
-                gemm_splitk_reduce<double><<<nbk, 256, 0, s>>>(g);
+                launch_chained(gemm_splitk_reduce<double>, nbk, 256, 0, s, g);
             }
             return cudaGetLastError();
         }
@@ -478,7 +480,7 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
     if (splits > 1) {
         long long total = (long long)g.M * g.N * (g.reduce ? 1 : g.batch);
         unsigned nbk = (unsigned)std::min<long long>((total + 255) / 256, 152LL * 32);
-        gemm_splitk_reduce<T><<<nbk, 256, 0, s>>>(g);
+        launch_chained(gemm_splitk_reduce<T>, nbk, 256, 0, s, g);
     }
     return cudaGetLastError();
 }

@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
               const __grid_constant__ CUtensorMap tb_hi, const __grid_constant__ CUtensorMap tb_lo,
               const TcArgs args) {
+    grid_wait();
     extern __shared__ __align__(1024) unsigned char tc_raw[];
     // 1024-byte alignment of the tile ring (required by the 128-byte swizzle)
     unsigned char* ring = reinterpret_cast<unsigned char*>(
@@ -611,6 +612,7 @@ __device__ __forceinline__ void pack_tile(const PackOp& op, long long u,
 // Both operands of a product in one launch (one launch each cost 2 to 3 us
 // more per product, and most operands are packed in 4 to 10).
 __global__ void __launch_bounds__(256) k_pack(const PackOp a, const PackOp b) {
+    grid_wait();
     __shared__ float tile[PT_R][PK_K + 1];
     for (long long u = blockIdx.x; u < a.units + b.units; u += gridDim.x) {
         if (u < a.units) {
@@ -626,6 +628,7 @@ __global__ void __launch_bounds__(256) k_pack(const PackOp a, const PackOp b) {
 __global__ void k_splitk_sum(const float* part, int splits, int nbo, int M, int N,
                              long long pcbs, float* C, long long crs, long long ccs,
                              long long cbs, float alpha, float beta) {
+    grid_wait();
     const long long MN = (long long)M * N, total = MN * nbo;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -679,9 +682,11 @@ cudaError_t launch_tc(const CUtensorMap* maps, const TcArgs& a, cudaStream_t s) 
     const long long sms = device_sms();
     const unsigned grid = (unsigned)std::min<long long>(a.ntiles, sms);
     if (a.splits == 1 && a.beta != 0.f)
-        k_gemm_tc<true><<<grid, kTcThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
+        launch_chained(k_gemm_tc<true>, grid, kTcThreads, smem, s, maps[0], maps[1], maps[2],
+                       maps[3], a);
     else
-        k_gemm_tc<false><<<grid, kTcThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
+        launch_chained(k_gemm_tc<false>, grid, kTcThreads, smem, s, maps[0], maps[1], maps[2],
+                       maps[3], a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -861,7 +866,7 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
     }
     if (e == cudaSuccess && pa.units + pb.units > 0) {
         const unsigned grid = (unsigned)std::min<long long>(pa.units + pb.units, 1 << 30);
-        k_pack<<<grid, 256, 0, s>>>(pa, pb);
+        launch_chained(k_pack, grid, 256, 0, s, pa, pb);
         count_launches(1);
         e = cudaGetLastError();
     }
@@ -952,9 +957,9 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
     if (splits > 1) {
         const long long total = (long long)Mr * Nr * nbo;
         const unsigned blocks = (unsigned)std::min<long long>((total + 255) / 256, 152 * 16);
-        k_splitk_sum<<<blocks, 256, 0, s>>>(ws.partial, splits, nbo, Mr, Nr, (long long)Mr * Nr,
-                                            g.C, crs, ccs, g.reduce ? 0 : g.sCb, (float)g.alpha,
-                                            (float)g.beta);
+        launch_chained(k_splitk_sum, blocks, 256, 0, s, ws.partial, splits, nbo, Mr, Nr,
+                       (long long)Mr * Nr, g.C, crs, ccs, g.reduce ? 0 : g.sCb, (float)g.alpha,
+                       (float)g.beta);
         count_launches(1);
         e = cudaGetLastError();
     }
@@ -1055,6 +1060,7 @@ __device__ __forceinline__ SliceTile slice_tile(const SlicePair& p, const SliceO
 // expo[bo * R + r] = max over the row of the biased exponent field (atomic
 // over the K tiles; the array starts at zero = all-zero row).
 __global__ void __launch_bounds__(256) k_row_exp(const __grid_constant__ SlicePair p) {
+    grid_wait();
     __shared__ double tile[PK_R][PK_K + 1];
     const bool second = blockIdx.x >= p.blocks0;
     const SliceOp& op = p.op[second];
@@ -1146,6 +1152,7 @@ __device__ __forceinline__ bool slice_written(const SlicePair& p, int b, int nb,
 }
 
 __global__ void __launch_bounds__(256, 5) k_slice64(const __grid_constant__ SlicePair p) {
+    grid_wait();
     __shared__ double tile[PK_R][PK_K + 1];
     const bool second = blockIdx.x >= p.blocks0;
     const SliceOp& op = p.op[second];
@@ -1171,6 +1178,7 @@ __host__ __device__ __forceinline__ int row_at(int k) { return k + (k >> 3); }
 __host__ __device__ __forceinline__ int row_pitch(int Kw) { return Kw / 8 * 9 + 1; }
 
 __global__ void __launch_bounds__(256) k_slice_rows(const __grid_constant__ SlicePair p) {
+    grid_wait();
     extern __shared__ __align__(16) double rows[];   // [SR][pitch]
     __shared__ int fe[SR];
     const bool second = blockIdx.x >= p.blocks0;
@@ -1464,6 +1472,7 @@ __device__ __forceinline__ void f64_finish(long long (&H)[FC], const float (&T)[
 __global__ void __launch_bounds__(kF64Threads, 1)
     k_gemm_f64s(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const F64Args args) {
+    grid_wait();
     extern __shared__ __align__(1024) unsigned char f64_raw[];
     F64Smem& sm = *reinterpret_cast<F64Smem*>((reinterpret_cast<uintptr_t>(f64_raw) + 1023) &
                                               ~uintptr_t(1023));
@@ -1841,6 +1850,7 @@ __global__ void __launch_bounds__(kF64Threads, 1)
 __global__ void k_f64_splitsum(const double* part, int splits, int nbo, int M, int N, int i_fast,
                                double* C, long long crs, long long ccs, long long cbs,
                                double alpha, double beta) {
+    grid_wait();
     const long long MN = (long long)M * N, tot = MN * nbo;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
          e += (long long)gridDim.x * blockDim.x) {
@@ -1993,15 +2003,15 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
         if ((e = smem_optin((const void*)k_slice_rows, SR * row_pitch(kFusedK) * (int)sizeof(double))) !=
             cudaSuccess)
             return e;
-        k_slice_rows<<<sgrid, 256, sbytes, s>>>(p);
+        launch_chained(k_slice_rows, sgrid, 256, sbytes, s, p);
         count_launches(1);
     } else {
         if ((e = cudaMemsetAsync(ws.expo, 0,
                                  sizeof(int) * ((long long)Mr * nba + (long long)Nr * nbb), s)) !=
             cudaSuccess)
             return e;
-        k_row_exp<<<sgrid, 256, 0, s>>>(p);
-        k_slice64<<<sgrid, 256, 0, s>>>(p);
+        launch_chained(k_row_exp, sgrid, 256, 0, s, p);
+        launch_chained(k_slice64, sgrid, 256, 0, s, p);
         count_launches(2);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -2057,14 +2067,14 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     const int smem = (int)sizeof(F64Smem) + 1024;
     if ((e = smem_optin((const void*)k_gemm_f64s, smem)) != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<long long>(a.ntiles, sms);
-    k_gemm_f64s<<<grid, kF64Threads, smem, s>>>(mA, mB, a);
+    launch_chained(k_gemm_f64s, grid, kF64Threads, smem, s, mA, mB, a);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (splits > 1) {
         const long long tot = (long long)Mr * Nr * nbo;
         const unsigned blocks = (unsigned)std::min<long long>((tot + 255) / 256, sms * 16);
-        k_f64_splitsum<<<blocks, 256, 0, s>>>(part, splits, nbo, Mr, Nr, swap ? 1 : 0, g.C, crs,
-                                              ccs, cbs, g.alpha, g.beta);
+        launch_chained(k_f64_splitsum, blocks, 256, 0, s, part, splits, nbo, Mr, Nr, swap ? 1 : 0,
+                       g.C, crs, ccs, cbs, g.alpha, g.beta);
         count_launches(1);
         e = cudaGetLastError();
     }

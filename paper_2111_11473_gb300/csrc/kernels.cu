@@ -27,6 +27,7 @@ inline unsigned row_threads(int P) { return (unsigned)std::min(NT, (P + 31) / 32
 
 template <typename T>
 __global__ void k_split(const T* full, int nb, int o, int v, Blocks<T> out) {
+    grid_wait();
     const int n = o + v;
     const long long total = (long long)nb * n * n;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
@@ -50,6 +51,7 @@ __global__ void k_split(const T* full, int nb, int o, int v, Blocks<T> out) {
 // write it transposed, so every global access runs along a row.
 template <typename T>
 __global__ void k_unpack_vv(const T* packed, int nb, int v, T* out) {
+    grid_wait();
     __shared__ T tile[32][33];
     const long long vt = (long long)v * (v + 1) / 2;
     const T* src = packed + (long long)blockIdx.z * vt;
@@ -75,6 +77,7 @@ __global__ void k_unpack_vv(const T* packed, int nb, int v, T* out) {
 
 template <typename T>
 __global__ void k_transpose(const T* in, T* out, int nb, int rows, int cols) {
+    grid_wait();
     __shared__ T tile[32][33];
     const int a = blockIdx.z;
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
@@ -93,6 +96,7 @@ __global__ void k_transpose(const T* in, T* out, int nb, int rows, int cols) {
 
 template <typename T>
 __global__ void k_convert(const double* in, T* out, long long n) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = (T)in[i];
@@ -100,6 +104,7 @@ __global__ void k_convert(const double* in, T* out, long long n) {
 
 template <typename T>
 __global__ void k_to_double(const T* in, double* out, long long n) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = (double)in[i];
@@ -108,6 +113,7 @@ __global__ void k_to_double(const T* in, double* out, long long n) {
 template <typename T>
 __global__ void k_alg1(const T* Bbar, const T* Btil, const T* oo, const T* vv,
                        T* C1, T* Ccross, int P, int nb) {
+    grid_wait();
     // HBM bound: U vectors' loads in flight per thread (one at a time took 0.65
     // ms for 600 vectors at P = 400 in float64, of which the bytes take 0.34)
     constexpr int U = 8;
@@ -144,6 +150,7 @@ __global__ void k_alg1(const T* Bbar, const T* Btil, const T* oo, const T* vv,
 template <typename T>
 __global__ void k_diag_reduce(const T* y, const T* M, int R, int P, int nb, T* out,
                               int ldo, int col0) {
+    grid_wait();
     const long long total = (long long)nb * P;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -158,6 +165,7 @@ __global__ void k_diag_reduce(const T* y, const T* M, int R, int P, int nb, T* o
 template <typename T>
 __global__ void k_w_single(const T* TA, int ldta, const T* Tc, const T* E, T* W, int P,
                            int nb) {
+    grid_wait();
     // one row Y of one vector per block turn: no 64-bit division per element
     const long long PP = (long long)P * P, rows = (long long)P * nb;
     for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
@@ -175,6 +183,7 @@ __global__ void k_w_single(const T* TA, int ldta, const T* Tc, const T* E, T* W,
 
 template <typename T>
 __global__ void k_eps_t1(const T* eps, const T* t1, int o, int v, T* out) {
+    grid_wait();
     const long long tot = (long long)o * v;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
          e += (long long)gridDim.x * blockDim.x) {
@@ -186,6 +195,7 @@ __global__ void k_eps_t1(const T* eps, const T* t1, int o, int v, T* out) {
 template <typename T>
 __global__ void k_lincomb(T* out, long long n, double a, const T* x, double b,
                           const T* y, double c, const T* z) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         T r = T(a) * x[i];
@@ -198,6 +208,7 @@ __global__ void k_lincomb(T* out, long long n, double a, const T* x, double b,
 template <typename T>
 __global__ void k_hadamard2(T* out, long long n, const T* a, const T* b, const T* c,
                             const T* d) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = c ? a[i] * b[i] - c[i] * d[i] : a[i] * b[i];
@@ -205,6 +216,7 @@ __global__ void k_hadamard2(T* out, long long n, const T* a, const T* b, const T
 
 template <typename T>
 __global__ void k_hadamard_batched(T* M, const T* z, long long per, int nb) {
+    grid_wait();
     // grid y: batches; grid x: elements of one
     for (int b = blockIdx.y; b < nb; b += gridDim.y) {
         T* m = M + b * per;
@@ -216,6 +228,7 @@ __global__ void k_hadamard_batched(T* M, const T* z, long long per, int nb) {
 
 template <typename T>
 __global__ void k_kr(const T* A, const T* B, int na, int nbr, int P, T* out) {
+    grid_wait();
     const long long total = (long long)na * nbr * P;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -229,6 +242,7 @@ __global__ void k_kr(const T* A, const T* B, int na, int nbr, int P, T* out) {
 template <typename T>
 __global__ void k_scale_rows(const T* y, int R, int P, const T* w, int x0, int nx,
                              T* out) {
+    grid_wait();
     // one row of one x per block turn: no 64-bit division per element
     const long long rows = (long long)R * nx;
     for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
@@ -317,6 +331,7 @@ template <int TYZ>
 __global__ void __launch_bounds__(256) k_triangle_sym64(double* H, const double* E,
                                                             const double* F, const double* G,
                                                             int P, int nX, int nI) {
+    grid_wait();
     constexpr int R = TYZ / 16;
     extern __shared__ __align__(16) unsigned char sym64_raw[];
     auto* stg = reinterpret_cast<TriSym64Stage<TYZ>*>(sym64_raw);
@@ -461,6 +476,7 @@ __device__ __forceinline__ void tri_load(TriStage& st, const float* E, const flo
 __global__ void __launch_bounds__(512, 1) k_triangle_f32(float* H, const float* E,
                                                          const float* F, const float* G,
                                                          int P, int nX, int nI) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char tri_smem[];
     TriStage* st = reinterpret_cast<TriStage*>(tri_smem);
     const int Z0 = blockIdx.x * TT, Y0 = blockIdx.y * TT, X0 = blockIdx.z * TT;
@@ -542,6 +558,7 @@ constexpr int NPART = 512;
 
 template <typename T>
 __global__ void k_dot_part(const T* a, const T* b, long long n, double* part) {
+    grid_wait();
     double acc = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
@@ -551,6 +568,7 @@ __global__ void k_dot_part(const T* a, const T* b, long long n, double* part) {
 }
 
 __global__ void k_sum_parts(const double* part, int n, double* out) {
+    grid_wait();
     double acc = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) acc += part[i];
     acc = block_sum(acc);
@@ -560,6 +578,7 @@ __global__ void k_sum_parts(const double* part, int n, double* out) {
 template <typename T>
 __global__ void k_singles_energy(const T* Lov, const T* Mo, const T* t1, int o, int v,
                                  double* part) {
+    grid_wait();
     const int k = blockIdx.x;
     const T* L = Lov + (long long)k * o * v;
     const T* M = Mo + (long long)k * o * o;
@@ -576,6 +595,7 @@ __global__ void k_singles_energy(const T* Lov, const T* Mo, const T* t1, int o, 
 }
 
 __global__ void k_nonfinite(const double* a, long long n, int* flag) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         if (!isfinite(a[i])) atomicOr(flag, 1);
@@ -583,6 +603,7 @@ __global__ void k_nonfinite(const double* a, long long n, int* flag) {
 
 template <typename T>
 __global__ void k_accumulate(double* acc, const T* part, long long n, double scale) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         acc[i] += scale * (double)part[i];
@@ -594,7 +615,7 @@ template <typename T>
 cudaError_t split_blocks(const T* full, int nb, int o, int v, Blocks<T> out,
                          cudaStream_t s) {
     long long n = (long long)nb * (o + v) * (o + v);
-    k_split<T><<<nblocks(n), NT, 0, s>>>(full, nb, o, v, out);
+    launch_chained(k_split<T>, nblocks(n), NT, 0, s, full, nb, o, v, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -602,7 +623,7 @@ cudaError_t split_blocks(const T* full, int nb, int o, int v, Blocks<T> out,
 template <typename T>
 cudaError_t unpack_vv(const T* packed, int nb, int v, T* out, cudaStream_t s) {
     dim3 grid(cdiv(v, 32), cdiv(v, 32), nb);
-    k_unpack_vv<T><<<grid, dim3(32, 8), 0, s>>>(packed, nb, v, out);
+    launch_chained(k_unpack_vv<T>, grid, dim3(32, 8), 0, s, packed, nb, v, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -611,21 +632,21 @@ template <typename T>
 cudaError_t transpose_batched(const T* in, T* out, int nb, int rows, int cols,
                               cudaStream_t s) {
     dim3 grid(cdiv(cols, 32), cdiv(rows, 32), nb);
-    k_transpose<T><<<grid, dim3(32, 8), 0, s>>>(in, out, nb, rows, cols);
+    launch_chained(k_transpose<T>, grid, dim3(32, 8), 0, s, in, out, nb, rows, cols);
     count_launches(1);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t convert(const double* in, T* out, long long n, cudaStream_t s) {
-    k_convert<T><<<nblocks(n), NT, 0, s>>>(in, out, n);
+    launch_chained(k_convert<T>, nblocks(n), NT, 0, s, in, out, n);
     count_launches(1);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t to_double(const T* in, double* out, long long n, cudaStream_t s) {
-    k_to_double<T><<<nblocks(n), NT, 0, s>>>(in, out, n);
+    launch_chained(k_to_double<T>, nblocks(n), NT, 0, s, in, out, n);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -633,7 +654,8 @@ cudaError_t to_double(const T* in, double* out, long long n, cudaStream_t s) {
 template <typename T>
 cudaError_t alg1_combine(const T* Bbar, const T* Btil, const T* oo, const T* vv,
                          T* C1, T* Ccross, int P, int nb, cudaStream_t s) {
-    k_alg1<T><<<nblocks((long long)P * P), NT, 0, s>>>(Bbar, Btil, oo, vv, C1, Ccross, P, nb);
+    launch_chained(k_alg1<T>, nblocks((long long)P * P), NT, 0, s, Bbar, Btil, oo, vv, C1, Ccross,
+                   P, nb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -641,7 +663,8 @@ cudaError_t alg1_combine(const T* Bbar, const T* Btil, const T* oo, const T* vv,
 template <typename T>
 cudaError_t diag_reduce(const T* y, const T* M, int R, int P, int nb, T* out, int ldo,
                         int col0, cudaStream_t s) {
-    k_diag_reduce<T><<<nblocks((long long)nb * P), NT, 0, s>>>(y, M, R, P, nb, out, ldo, col0);
+    launch_chained(k_diag_reduce<T>, nblocks((long long)nb * P), NT, 0, s, y, M, R, P, nb, out, ldo,
+                   col0);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -649,14 +672,15 @@ cudaError_t diag_reduce(const T* y, const T* M, int R, int P, int nb, T* out, in
 template <typename T>
 cudaError_t w_single(const T* TA, int ldta, const T* Tc, const T* E, T* W, int P, int nb,
                      cudaStream_t s) {
-    k_w_single<T><<<row_blocks((long long)nb * P), row_threads(P), 0, s>>>(TA, ldta, Tc, E, W, P, nb);
+    launch_chained(k_w_single<T>, row_blocks((long long)nb * P), row_threads(P), 0, s, TA, ldta, Tc,
+                   E, W, P, nb);
     count_launches(1);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t eps_t1(const T* eps, const T* t1, int o, int v, T* out, cudaStream_t s) {
-    k_eps_t1<T><<<nblocks((long long)o * v), NT, 0, s>>>(eps, t1, o, v, out);
+    launch_chained(k_eps_t1<T>, nblocks((long long)o * v), NT, 0, s, eps, t1, o, v, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -664,7 +688,7 @@ cudaError_t eps_t1(const T* eps, const T* t1, int o, int v, T* out, cudaStream_t
 template <typename T>
 cudaError_t lincomb(T* out, long long n, double a, const T* x, double b, const T* y,
                     double c, const T* z, cudaStream_t s) {
-    k_lincomb<T><<<nblocks(n), NT, 0, s>>>(out, n, a, x, b, y, c, z);
+    launch_chained(k_lincomb<T>, nblocks(n), NT, 0, s, out, n, a, x, b, y, c, z);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -672,7 +696,7 @@ cudaError_t lincomb(T* out, long long n, double a, const T* x, double b, const T
 template <typename T>
 cudaError_t hadamard2(T* out, long long n, const T* a, const T* b, const T* c,
                       const T* d, cudaStream_t s) {
-    k_hadamard2<T><<<nblocks(n), NT, 0, s>>>(out, n, a, b, c, d);
+    launch_chained(k_hadamard2<T>, nblocks(n), NT, 0, s, out, n, a, b, c, d);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -680,7 +704,7 @@ cudaError_t hadamard2(T* out, long long n, const T* a, const T* b, const T* c,
 template <typename T>
 cudaError_t hadamard_batched(T* M, const T* z, long long per, int nb, cudaStream_t s) {
     const dim3 grid(nblocks(per), (unsigned)std::max(1, std::min(nb, 65535)));
-    k_hadamard_batched<T><<<grid, NT, 0, s>>>(M, z, per, nb);
+    launch_chained(k_hadamard_batched<T>, grid, NT, 0, s, M, z, per, nb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -688,7 +712,7 @@ cudaError_t hadamard_batched(T* M, const T* z, long long per, int nb, cudaStream
 template <typename T>
 cudaError_t khatri_rao(const T* A, const T* B, int na, int nbr, int P, T* out,
                        cudaStream_t s) {
-    k_kr<T><<<nblocks((long long)na * nbr * P), NT, 0, s>>>(A, B, na, nbr, P, out);
+    launch_chained(k_kr<T>, nblocks((long long)na * nbr * P), NT, 0, s, A, B, na, nbr, P, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -696,7 +720,8 @@ cudaError_t khatri_rao(const T* A, const T* B, int na, int nbr, int P, T* out,
 template <typename T>
 cudaError_t scale_rows(const T* y, int R, int P, const T* w, int x0, int nx, T* out,
                        cudaStream_t s) {
-    k_scale_rows<T><<<row_blocks((long long)R * nx), row_threads(P), 0, s>>>(y, R, P, w, x0, nx, out);
+    launch_chained(k_scale_rows<T>, row_blocks((long long)R * nx), row_threads(P), 0, s, y, R, P, w,
+                   x0, nx, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -710,7 +735,7 @@ cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, in
         cudaError_t e = smem_optin((const void*)k_triangle_f32, smem);
         if (e != cudaSuccess) return e;
         dim3 grid(cdiv(P, TT), cdiv(P, TT), cdiv(nX, TT));
-        k_triangle_f32<<<grid, 512, smem, s>>>(H, E, F, G, P, nX, nI);
+        launch_chained(k_triangle_f32, grid, 512, smem, s, H, E, F, G, P, nX, nI);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -724,8 +749,8 @@ cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, in
         cudaError_t e = smem_optin(small ? (const void*)k_triangle_sym64<16>
                                          : (const void*)k_triangle_sym64<32>, smem);
         if (e != cudaSuccess) return e;
-        if (small) k_triangle_sym64<16><<<grid, 256, smem, s>>>(H, E, F, G, P, nX, nI);
-        else k_triangle_sym64<32><<<grid, 256, smem, s>>>(H, E, F, G, P, nX, nI);
+        if (small) launch_chained(k_triangle_sym64<16>, grid, 256, smem, s, H, E, F, G, P, nX, nI);
+        else launch_chained(k_triangle_sym64<32>, grid, 256, smem, s, H, E, F, G, P, nX, nI);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -735,23 +760,23 @@ cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, in
 template <typename T>
 cudaError_t dot(const T* a, const T* b, long long n, double* scratch, double* out,
                 cudaStream_t s) {
-    k_dot_part<T><<<NPART, NT, 0, s>>>(a, b, n, scratch);
+    launch_chained(k_dot_part<T>, NPART, NT, 0, s, a, b, n, scratch);
     count_launches(1);
-    k_sum_parts<<<1, NT, 0, s>>>(scratch, NPART, out);
+    launch_chained(k_sum_parts, 1, NT, 0, s, scratch, NPART, out);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t singles_energy(const T* Lov, const T* Mo, const T* t1, int K, int o, int v,
                            double* scratch, double* out, cudaStream_t s) {
-    k_singles_energy<T><<<K, NT, 0, s>>>(Lov, Mo, t1, o, v, scratch);
+    launch_chained(k_singles_energy<T>, K, NT, 0, s, Lov, Mo, t1, o, v, scratch);
     count_launches(1);
-    k_sum_parts<<<1, NT, 0, s>>>(scratch, K, out);
+    launch_chained(k_sum_parts, 1, NT, 0, s, scratch, K, out);
     return cudaGetLastError();
 }
 
 cudaError_t any_nonfinite(const double* a, long long n, int* flag, cudaStream_t s) {
-    k_nonfinite<<<nblocks(n), NT, 0, s>>>(a, n, flag);
+    launch_chained(k_nonfinite, nblocks(n), NT, 0, s, a, n, flag);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -759,7 +784,7 @@ cudaError_t any_nonfinite(const double* a, long long n, int* flag, cudaStream_t 
 template <typename T>
 cudaError_t accumulate(double* acc, const T* part, long long n, double scale,
                        cudaStream_t s) {
-    k_accumulate<T><<<nblocks(n), NT, 0, s>>>(acc, part, n, scale);
+    launch_chained(k_accumulate<T>, nblocks(n), NT, 0, s, acc, part, n, scale);
     count_launches(1);
     return cudaGetLastError();
 }

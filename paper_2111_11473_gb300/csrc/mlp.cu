@@ -32,6 +32,7 @@ unsigned col_threads(int H) { return (unsigned)std::min(NT, (H + 31) / 32 * 32);
 // a1 = tanh(X W1^T + b1)
 __global__ void k_layer1(const float* X, const float* W1, const float* b1, long long n, int H,
                          int run, float* a1) {
+    grid_wait();
     constexpr int F = kMlpFeatures;
     const long long r0 = (long long)blockIdx.x * run, r1 = min(n, r0 + run);
     for (int c = threadIdx.x; c < H; c += blockDim.x) {
@@ -52,6 +53,7 @@ __global__ void k_layer1(const float* X, const float* W1, const float* b1, long 
 // Z = tanh(Z + b2) in place, y = Z w3 + b3: a warp per row
 __global__ void k_head(float* Z, const float* b2, const float* w3, const float* b3, long long n,
                        int H, float* y) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const long long step = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n;
@@ -71,6 +73,7 @@ __global__ void k_head(float* Z, const float* b2, const float* w3, const float* 
 // dy = (2/n) (j (1 + y) - t) j ; part[block] = sum of r^2 (float64)
 __global__ void k_loss(const float* y, const float* j, const float* t, long long n, float* dy,
                        double* part) {
+    grid_wait();
     __shared__ double red[NT];
     double acc = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -89,6 +92,7 @@ __global__ void k_loss(const float* y, const float* j, const float* t, long long
 }
 
 __global__ void k_sum_d(const double* part, int n, double* out) {
+    grid_wait();
     __shared__ double red[NT];
     double acc = 0;
     for (int i = threadIdx.x; i < n; i += NT) acc += part[i];
@@ -105,6 +109,7 @@ __global__ void k_sum_d(const double* part, int n, double* out) {
 // of d2), w3 (of a2 dy) and b3 (of dy): part[block] = [b2 | w3 | b3]
 __global__ void k_head_grad(const float* dy, const float* w3, const float* a2, long long n, int H,
                             int run, float* d2, float* part) {
+    grid_wait();
     const long long r0 = (long long)blockIdx.x * run, r1 = min(n, r0 + run);
     float* out = part + (long long)blockIdx.x * (2 * H + 1);
     for (int c = threadIdx.x; c < H; c += blockDim.x) {
@@ -129,6 +134,7 @@ __global__ void k_head_grad(const float* dy, const float* w3, const float* a2, l
 // b1 (sums of d): part[block] = [W1 | b1]
 __global__ void k_layer1_grad(const float* d1, const float* a1, const float* X, long long n, int H,
                               int run, float* part) {
+    grid_wait();
     constexpr int F = kMlpFeatures;
     const long long r0 = (long long)blockIdx.x * run, r1 = min(n, r0 + run);
     float* out = part + (long long)blockIdx.x * (F + 1) * H;
@@ -149,6 +155,7 @@ __global__ void k_layer1_grad(const float* d1, const float* a1, const float* X, 
 
 // out[c] = sum over blocks of part[block][c], in a fixed order
 __global__ void k_sum_parts_f(const float* part, int nblk, int ncols, float* out) {
+    grid_wait();
     __shared__ float red[8][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
@@ -167,6 +174,7 @@ __global__ void k_sum_parts_f(const float* part, int nblk, int ncols, float* out
 
 __global__ void k_adam(float* th, const float* g, float* m, float* v, long long n, float lr,
                        float c1, float c2) {
+    grid_wait();
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
@@ -183,6 +191,7 @@ __global__ void k_adam(float* th, const float* g, float* m, float* v, long long 
 __global__ void k_gather(const float* X, const float* j, const float* t, long long n, int F,
                          long long off, long long stride, long long b0, long long nb, float* xb,
                          float* jb, float* tb) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nb;
          i += (long long)gridDim.x * blockDim.x) {
         const long long src = (off + (b0 + i) % n * stride) % n;
@@ -226,6 +235,7 @@ __global__ void k_features(const double* sig1, const double* eps, const double* 
                            const double* e, const double* x, const double* dprev,
                            const long long* idx, long long n, int o, int v, int r, double s1,
                            double s2, double logr, float* X, float* jj) {
+    grid_wait();
     const long long ov = (long long)o * v;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
@@ -250,6 +260,7 @@ __global__ void k_features(const double* sig1, const double* eps, const double* 
 
 __global__ void k_apply(const double* sig1, const double* eps, const double* sq, const double* e,
                         const float* y, int o, int v, int r, int blocks, double* step) {
+    grid_wait();
     const long long ov = (long long)o * v, tot = ov + (long long)r * r;
     for (long long el = blockIdx.x * (long long)blockDim.x + threadIdx.x; el < tot;
          el += (long long)gridDim.x * blockDim.x) {
@@ -273,8 +284,8 @@ cudaError_t mlp_features(const double* sig1, const double* eps, const double* sq
                          const double* e, const double* x, const double* dprev,
                          const long long* idx, long long n, int o, int v, int r, double s1,
                          double s2, double log_rnorm, float* X, float* jj, cudaStream_t st) {
-    k_features<<<nbl(n), NT, 0, st>>>(sig1, eps, sq, e, x, dprev, idx, n, o, v, r, s1, s2,
-                                      log_rnorm, X, jj);
+    launch_chained(k_features, nbl(n), NT, 0, st, sig1, eps, sq, e, x, dprev, idx, n, o, v, r, s1,
+                   s2, log_rnorm, X, jj);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -282,8 +293,8 @@ cudaError_t mlp_features(const double* sig1, const double* eps, const double* sq
 cudaError_t mlp_apply(const double* sig1, const double* eps, const double* sq, const double* e,
                       const float* y, int o, int v, int r, int blocks, double* step,
                       cudaStream_t st) {
-    k_apply<<<nbl((long long)o * v + (long long)r * r), NT, 0, st>>>(sig1, eps, sq, e, y, o, v, r,
-                                                                     blocks, step);
+    launch_chained(k_apply, nbl((long long)o * v + (long long)r * r), NT, 0, st, sig1, eps, sq, e,
+                   y, o, v, r, blocks, step);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -369,7 +380,8 @@ Err Mlp::forward(const float* X, long long n, float* yout) {
     THC_TRY(ensure(n));
     const int ni = (int)n;
     // a1 = tanh(X W1^T + b1)
-    k_layer1<<<run_blocks(n), col_threads(H), 0, st>>>(X, W1(), b1(), n, H, (int)row_run(n), a1);
+    launch_chained(k_layer1, run_blocks(n), col_threads(H), 0, st, X, W1(), b1(), n, H,
+                   (int)row_run(n), a1);
     count_launches(1);
     THC_CUDA(cudaGetLastError());
     // a2 = tanh(a1 W2^T + b2)   (tensor cores, bf16 weights, in bf16 mode)
@@ -386,8 +398,7 @@ Err Mlp::forward(const float* X, long long n, float* yout) {
     }
     if (!done) THC_TRY(mm32(*this, ni, H, H, View<float>{a1, H, 1}, View<float>{W2(), 1, H}, a2, H, 1, 0));
     // y = a2 w3 + b3
-    k_head<<<run_blocks(n), NT, 0, st>>>(a2, b2(), w3(), b3(),
-                                                                               n, H, yout);
+    launch_chained(k_head, run_blocks(n), NT, 0, st, a2, b2(), w3(), b3(), n, H, yout);
     count_launches(1);
     THC_CUDA(cudaGetLastError());
     return Err{};
@@ -400,8 +411,8 @@ Err Mlp::loss_grad(const float* X, const float* j, const float* t, long long n, 
     const int ni = (int)n;
     const unsigned nb = std::min<unsigned>(nbl(n), 1024);
     double* part = reinterpret_cast<double*>(red);
-    k_loss<<<nb, NT, 0, st>>>(y, j, t, n, dy, part);
-    k_sum_d<<<1, NT, 0, st>>>(part, (int)nb, part + 2048);
+    launch_chained(k_loss, nb, NT, 0, st, y, j, t, n, dy, part);
+    launch_chained(k_sum_d, 1, NT, 0, st, part, (int)nb, part + 2048);
     count_launches(2);
     THC_CUDA(cudaGetLastError());
     // layout of the gradient: [W1 | b1 | W2 | b2 | w3 | b3]
@@ -410,16 +421,17 @@ Err Mlp::loss_grad(const float* X, const float* j, const float* t, long long n, 
     float* gb2 = gW2 + (long long)H * H;
     const int run = (int)row_run(n), blocks = (int)run_blocks(n);
     // output layer and biases of the second
-    k_head_grad<<<blocks, col_threads(H), 0, st>>>(dy, w3(), a2, n, H, run, d2, splitk);
-    k_sum_parts_f<<<cdiv(2 * H + 1, 32), NT, 0, st>>>(splitk, blocks, 2 * H + 1, gb2);
+    launch_chained(k_head_grad, blocks, col_threads(H), 0, st, dy, w3(), a2, n, H, run, d2, splitk);
+    launch_chained(k_sum_parts_f, cdiv(2 * H + 1, 32), NT, 0, st, splitk, blocks, 2 * H + 1, gb2);
     count_launches(2);
     THC_CUDA(cudaGetLastError());
     // second layer
     THC_TRY(mm32(*this, H, H, ni, View<float>{d2, 1, H}, View<float>{a1, H, 1}, gW2, H, 1, 0));
     // first layer
     THC_TRY(mm32(*this, ni, H, H, View<float>{d2, H, 1}, View<float>{W2(), H, 1}, d1, H, 1, 0));
-    k_layer1_grad<<<blocks, col_threads(H), 0, st>>>(d1, a1, X, n, H, run, splitk);
-    k_sum_parts_f<<<cdiv((F + 1) * H, 32), NT, 0, st>>>(splitk, blocks, (F + 1) * H, gW1);
+    launch_chained(k_layer1_grad, blocks, col_threads(H), 0, st, d1, a1, X, n, H, run, splitk);
+    launch_chained(k_sum_parts_f, cdiv((F + 1) * H, 32), NT, 0, st, splitk, blocks, (F + 1) * H,
+                   gW1);
     count_launches(2);
     THC_CUDA(cudaGetLastError());
     if (loss) {
@@ -434,7 +446,7 @@ Err Mlp::loss_grad(const float* X, const float* j, const float* t, long long n, 
 Err Mlp::adam(float lr) {
     ++step;
     const float c1 = 1.f - std::pow(0.9f, (float)step), c2 = 1.f - std::pow(0.999f, (float)step);
-    k_adam<<<nbl(np), NT, 0, st>>>(theta, grad, m, v, np, lr, c1, c2);
+    launch_chained(k_adam, nbl(np), NT, 0, st, theta, grad, m, v, np, lr, c1, c2);
     count_launches(1);
     THC_CUDA(cudaGetLastError());
     return Err{};
@@ -457,7 +469,8 @@ Err Mlp::train(const float* X, const float* j, const float* t, long long n, int 
         long long cnt = 0;
         for (long long b0 = 0; b0 < n; b0 += B) {
             const long long nb = std::min(B, n - b0);
-            k_gather<<<nbl(nb), NT, 0, st>>>(X, j, t, n, F, off, stride, b0, nb, xb, jb, tb);
+            launch_chained(k_gather, nbl(nb), NT, 0, st, X, j, t, n, F, off, stride, b0, nb, xb, jb,
+                           tb);
             count_launches(1);
             THC_CUDA(cudaGetLastError());
             double l = 0;

@@ -24,6 +24,7 @@ View64 rm64(const double* p, long long ld) { return View64{p, ld, 1}; }
 View64 tr64(const double* p, long long ld) { return View64{p, 1, ld}; }
 
 __global__ void k_scale_diag(const double* y, const double* eps, int R, int P, double* out) {
+    grid_wait();
     const long long total = (long long)R * P;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x)
@@ -32,6 +33,7 @@ __global__ void k_scale_diag(const double* y, const double* eps, int R, int P, d
 
 __global__ void k_metric(const double* oo, const double* vv, const double* oe,
                          const double* ve, double* S, double* F, long long nn) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nn;
          i += (long long)gridDim.x * blockDim.x) {
         S[i] = oo[i] * vv[i];
@@ -42,6 +44,7 @@ __global__ void k_metric(const double* oo, const double* vv, const double* oe,
 // X[i][k] = V[(k0 + k) * P + i] / sqrt(s[k0 + k])   (cuSOLVER returns V column-major)
 __global__ void k_half_inverse(const double* V, const double* s, int P, int k0, int r,
                                double* X) {
+    grid_wait();
     const long long total = (long long)P * r;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -52,6 +55,7 @@ __global__ void k_half_inverse(const double* V, const double* s, int P, int k0, 
 
 // row-major W[i][k] from column-major eigenvectors
 __global__ void k_colmajor_to_rowmajor(const double* V, int r, double* W) {
+    grid_wait();
     const long long total = (long long)r * r;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -61,6 +65,7 @@ __global__ void k_colmajor_to_rowmajor(const double* V, int r, double* W) {
 }
 
 __global__ void k_symmetrize(double* A, int n) {
+    grid_wait();
     const long long total = (long long)n * n;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -77,6 +82,7 @@ __global__ void k_symmetrize(double* A, int n) {
 __global__ void k_jacobi(const double* sig1, const double* sq, const double* eps,
                          const double* e, int o, int v, int r, const double* x, double* step,
                          double* xnew) {
+    grid_wait();
     const long long ov = (long long)o * v, total = ov + (long long)r * r;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -96,6 +102,7 @@ __global__ void k_jacobi(const double* sig1, const double* sq, const double* eps
 
 __global__ void k_combine(const double* hx, const double* c, int m, long long len,
                           double* out) {
+    grid_wait();
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < len;
          idx += (long long)gridDim.x * blockDim.x) {
         double s = 0;
@@ -119,6 +126,7 @@ __device__ double block_sum64(double v) {
 
 // out[k] = <a_k, b> for m vectors a_k (stride len), one block per k.
 __global__ void k_multidot(const double* A, const double* b, long long len, double* out) {
+    grid_wait();
     const double* a = A + (long long)blockIdx.x * len;
     double s = 0;
     for (long long i = threadIdx.x; i < len; i += blockDim.x) s += a[i] * b[i];
@@ -130,6 +138,7 @@ unsigned nb(long long n) { return (unsigned)std::min<long long>((n + 255) / 256,
 
 // out = a + b (n elements)
 __global__ void k_add(const double* a, const double* b, long long n, double* out) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = a[i] + b[i];
@@ -137,6 +146,7 @@ __global__ void k_add(const double* a, const double* b, long long n, double* out
 
 // out = a - b
 __global__ void k_sub(const double* a, const double* b, long long n, double* out) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = a[i] - b[i];
@@ -144,6 +154,7 @@ __global__ void k_sub(const double* a, const double* b, long long n, double* out
 
 // out[k] = src[idx[k]]
 __global__ void k_gather64(const double* src, const long long* idx, long long n, double* out) {
+    grid_wait();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x)
         out[k] = src[idx[k]];
@@ -152,12 +163,14 @@ __global__ void k_gather64(const double* src, const long long* idx, long long n,
 // t[k] = (Tstar[idx[k]] - Tk[k]) / s[k]
 __global__ void k_targets(const double* Tstar, const long long* idx, const double* Tk,
                           const double* sk, long long n, float* t) {
+    grid_wait();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x)
         t[k] = (float)((Tstar[idx[k]] - Tk[k]) / sk[k]);
 }
 
 __global__ void k_fill64(double* p, long long n, double v) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         p[i] = v;
@@ -263,9 +276,9 @@ Err Solver::setup(Engine<T>& eng, double cutoff) {
     const double* yv = yd.p + (long long)o * P;
     THC_TRY(yo_e.alloc((size_t)o * P));
     THC_TRY(yv_e.alloc((size_t)v * P));
-    k_scale_diag<<<nb((long long)o * P), 256, 0, st>>>(yo, epsd.p, o, P, yo_e.p);
+    launch_chained(k_scale_diag, nb((long long)o * P), 256, 0, st, yo, epsd.p, o, P, yo_e.p);
     count_launches(1);
-    k_scale_diag<<<nb((long long)v * P), 256, 0, st>>>(yv, epsd.p + o, v, P, yv_e.p);
+    launch_chained(k_scale_diag, nb((long long)v * P), 256, 0, st, yv, epsd.p + o, v, P, yv_e.p);
     THC_CUDA(cudaGetLastError());
     for (DBuf<double>* b : {&oo, &vv, &oe, &ve, &F}) THC_TRY(b->alloc(PP));
     THC_TRY(Sd.alloc(PP));
@@ -273,10 +286,10 @@ Err Solver::setup(Engine<T>& eng, double cutoff) {
     THC_TRY(mm(st, P, P, v, tr64(yv, P), rm64(yv, P), vv.p, P, 1, 0));
     THC_TRY(mm(st, P, P, o, tr64(yo, P), rm64(yo_e.p, P), oe.p, P, 1, 0));
     THC_TRY(mm(st, P, P, v, tr64(yv, P), rm64(yv_e.p, P), ve.p, P, 1, 0));
-    k_metric<<<nb(PP), 256, 0, st>>>(oo.p, vv.p, oe.p, ve.p, Sd.p, F.p, PP);
+    launch_chained(k_metric, nb(PP), 256, 0, st, oo.p, vv.p, oe.p, ve.p, Sd.p, F.p, PP);
     count_launches(1);
     THC_CUDA(cudaGetLastError());
-    k_symmetrize<<<nb(PP), 256, 0, st>>>(F.p, P);
+    launch_chained(k_symmetrize, nb(PP), 256, 0, st, F.p, P);
     count_launches(1);
     // S = V diag(s) V^T
     THC_TRY(Wm.alloc(PP));
@@ -292,7 +305,7 @@ Err Solver::setup(Engine<T>& eng, double cutoff) {
     r = P - k0;
     DBuf<double> X, M, tmpPr;
     THC_TRY(X.alloc((size_t)P * r));
-    k_half_inverse<<<nb((long long)P * r), 256, 0, st>>>(Wm.p, sv.p, P, k0, r, X.p);
+    launch_chained(k_half_inverse, nb((long long)P * r), 256, 0, st, Wm.p, sv.p, P, k0, r, X.p);
     count_launches(1);
     THC_CUDA(cudaGetLastError());
     // M = X^T F X, eigenvectors W:  C = X W
@@ -300,13 +313,13 @@ Err Solver::setup(Engine<T>& eng, double cutoff) {
     THC_TRY(M.alloc((size_t)r * r));
     THC_TRY(mm(st, P, r, P, rm64(F.p, P), rm64(X.p, r), tmpPr.p, r, 1, 0));
     THC_TRY(mm(st, r, r, P, tr64(X.p, r), rm64(tmpPr.p, r), M.p, r, 1, 0));
-    k_symmetrize<<<nb((long long)r * r), 256, 0, st>>>(M.p, r);
+    launch_chained(k_symmetrize, nb((long long)r * r), 256, 0, st, M.p, r);
     count_launches(1);
     THC_TRY(e.alloc(r));
     THC_TRY(syevd(st, M.p, r, e.p));
     DBuf<double> W;
     THC_TRY(W.alloc((size_t)r * r));
-    k_colmajor_to_rowmajor<<<nb((long long)r * r), 256, 0, st>>>(M.p, r, W.p);
+    launch_chained(k_colmajor_to_rowmajor, nb((long long)r * r), 256, 0, st, M.p, r, W.p);
     count_launches(1);
     THC_TRY(C.alloc((size_t)P * r));
     THC_TRY(mm(st, P, r, r, rm64(X.p, r), rm64(W.p, r), C.p, r, 1, 0));
@@ -365,7 +378,7 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
         THC_TRY(eng.check_sym(Zc.p, P, 1e-12, "Zc"));
         THC_TRY(mm(st, P, r, P, rm64(Zc.p, P), rm64(SC.p, r), tmp.p, r, 1, 0));
         THC_TRY(mm(st, r, r, P, tr64(SC.p, r), rm64(tmp.p, r), x.p + ov, r, 1, 0));
-        k_symmetrize<<<nb(rr), 256, 0, st>>>(x.p + ov, r);
+        launch_chained(k_symmetrize, nb(rr), 256, 0, st, x.p + ov, r);
         count_launches(1);
     }
     resumable = false;
@@ -408,7 +421,7 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
                                  cudaMemcpyDeviceToDevice, st));
         THC_CUDA(cudaMemcpyAsync(he.p + (long long)slot * len, ev, sizeof(double) * len,
                                  cudaMemcpyDeviceToDevice, st));
-        k_multidot<<<m, 256, 0, st>>>(he.p, he.p + (long long)slot * len, len, dots.p);
+        launch_chained(k_multidot, m, 256, 0, st, he.p, he.p + (long long)slot * len, len, dots.p);
         count_launches(1);
         THC_CUDA(cudaGetLastError());
         std::vector<double> row(m);
@@ -430,7 +443,7 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
         if (nhist >= 2 && diis_coefficients(Bsub, nhist, c)) {
             THC_CUDA(cudaMemcpyAsync(dots.p, c.data(), sizeof(double) * nhist,
                                      cudaMemcpyHostToDevice, st));
-            k_combine<<<nb(len), 256, 0, st>>>(hx.p, dots.p, nhist, len, x.p);
+            launch_chained(k_combine, nb(len), 256, 0, st, hx.p, dots.p, nhist, len, x.p);
             count_launches(1);
             THC_CUDA(cudaGetLastError());
         } else {
@@ -442,7 +455,7 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
         // Zc = C T C^T
         THC_TRY(mm(st, P, r, r, rm64(C.p, r), rm64(x.p + ov, r), tmp.p, r, 1, 0));
         THC_TRY(mm(st, P, P, r, rm64(tmp.p, r), tr64(C.p, r), Zc.p, P, 1, 0));
-        k_symmetrize<<<nb(PP), 256, 0, st>>>(Zc.p, P);
+        launch_chained(k_symmetrize, nb(PP), 256, 0, st, Zc.p, P);
         count_launches(1);
         THC_CUDA(cudaGetLastError());
         THC_TRY(eng.set_state(Zc.p, x.p));
@@ -452,9 +465,9 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
         // sigma_q = C^T sigma C
         THC_TRY(mm(st, P, r, P, rm64(eng.sig.p, P), rm64(C.p, r), tmp.p, r, 1, 0));
         THC_TRY(mm(st, r, r, P, tr64(C.p, r), rm64(tmp.p, r), sq.p, r, 1, 0));
-        k_multidot<<<1, 256, 0, st>>>(eng.sig1.p, eng.sig1.p, ov, dots.p);
+        launch_chained(k_multidot, 1, 256, 0, st, eng.sig1.p, eng.sig1.p, ov, dots.p);
         count_launches(1);
-        k_multidot<<<1, 256, 0, st>>>(sq.p, sq.p, rr, dots.p + 1);
+        launch_chained(k_multidot, 1, 256, 0, st, sq.p, sq.p, rr, dots.p + 1);
         THC_CUDA(cudaGetLastError());
         double h[4];
         THC_CUDA(cudaMemcpyAsync(h, dots.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -487,7 +500,7 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
                 // plain iterate.  Two rejections switch proposals off.
                 ++n_rej;
                 if (n_rej >= 2) mlp_off = true;
-                k_add<<<nb(len), 256, 0, st>>>(saved_x.p, saved_j.p, len, xnew.p);
+                launch_chained(k_add, nb(len), 256, 0, st, saved_x.p, saved_j.p, len, xnew.p);
                 count_launches(1);
                 THC_CUDA(cudaGetLastError());
                 if (m > 0 && saved_slot >= 0) {
@@ -510,17 +523,17 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
             converged = true;
             break;
         }
-        k_jacobi<<<nb(len), 256, 0, st>>>(eng.sig1.p, sq.p, epsd.p, e.p, o, v, r, x.p,
-                                           step.p, xnew.p);
+        launch_chained(k_jacobi, nb(len), 256, 0, st, eng.sig1.p, sq.p, epsd.p, e.p, o, v, r, x.p,
+                       step.p, xnew.p);
         count_launches(1);
         THC_CUDA(cudaGetLastError());
         bool mlp_used = false;
         if ((nrec > 0 || use_mlp) && it >= 2) {
             // scales of this iteration's singles and doubles Jacobi steps,
             // previous step
-            k_multidot<<<1, 256, 0, st>>>(step.p, step.p, ov, dots.p + 7);
-            k_multidot<<<1, 256, 0, st>>>(step.p + ov, step.p + ov, rr, dots.p + 8);
-            k_sub<<<nb(len), 256, 0, st>>>(x.p, xprev.p, len, dprev.p);
+            launch_chained(k_multidot, 1, 256, 0, st, step.p, step.p, ov, dots.p + 7);
+            launch_chained(k_multidot, 1, 256, 0, st, step.p + ov, step.p + ov, rr, dots.p + 8);
+            launch_chained(k_sub, nb(len), 256, 0, st, x.p, xprev.p, len, dprev.p);
             count_launches(3);
             THC_CUDA(cudaGetLastError());
             double ss[2] = {0, 0};
@@ -542,9 +555,10 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
                 THC_CUDA(mlp_features(eng.sig1.p, epsd.p, sq.p, e.p, x.p, dp, di, nrec_it, o, v, r,
                                       sc1, sc, lr, recX.p + n_rec * kMlpFeatures, recJ.p + n_rec,
                                       st));
-                k_gather64<<<nb(nrec_it), 256, 0, st>>>(x.p, di, nrec_it, recTk.p + n_rec);
-                k_fill64<<<nb(nrec), 256, 0, st>>>(recS.p + n_rec, nrec, sc);
-                k_fill64<<<nb(nrec1), 256, 0, st>>>(recS.p + n_rec + nrec, nrec1, sc1);
+                launch_chained(k_gather64, nb(nrec_it), 256, 0, st, x.p, di, nrec_it,
+                               recTk.p + n_rec);
+                launch_chained(k_fill64, nb(nrec), 256, 0, st, recS.p + n_rec, nrec, sc);
+                launch_chained(k_fill64, nb(nrec1), 256, 0, st, recS.p + n_rec + nrec, nrec1, sc1);
                 count_launches(3);
                 THC_CUDA(cudaGetLastError());
                 // hidx is reused next iteration: the copy must finish first
@@ -562,7 +576,7 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
                                          yb.p + r0));
                 THC_CUDA(mlp_apply(eng.sig1.p, epsd.p, sq.p, e.p, yb.p, o, v, r,
                                    opts.mlp_blocks > 0 ? opts.mlp_blocks : 3, smlp.p, st));
-                k_add<<<nb(len), 256, 0, st>>>(x.p, smlp.p, len, xnew.p);
+                launch_chained(k_add, nb(len), 256, 0, st, x.p, smlp.p, len, xnew.p);
                 count_launches(1);
                 THC_CUDA(cudaGetLastError());
                 mlp_used = true;
@@ -598,7 +612,8 @@ Err Solver::run(Engine<T>& eng, const thc_solve_opts& opts, double* Zc_io, doubl
     THC_CUDA(cudaMemcpyAsync(t1_io, eng.t1d.p, sizeof(double) * ov, cudaMemcpyDefault, st));
     THC_CUDA(cudaStreamSynchronize(st));
     if (converged && n_rec > 0) {
-        k_targets<<<nb(n_rec), 256, 0, st>>>(x.p, recIdx.p, recTk.p, recS.p, n_rec, recT.p);
+        launch_chained(k_targets, nb(n_rec), 256, 0, st, x.p, recIdx.p, recTk.p, recS.p, n_rec,
+                       recT.p);
         count_launches(1);
         THC_CUDA(cudaGetLastError());
         THC_CUDA(cudaStreamSynchronize(st));

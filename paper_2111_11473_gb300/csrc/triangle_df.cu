@@ -324,6 +324,7 @@ template <bool BIAS, bool EVEN>
 __global__ void __launch_bounds__(DTH, 2)
     k_triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
                   const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char df_raw[];
     DfSmem<BIAS>& sm = *reinterpret_cast<DfSmem<BIAS>*>(df_raw);
     const int nb = (P + DT - 1) / DT;
@@ -576,7 +577,8 @@ cudaError_t launch_df(double* H, const float4* E4, const float4* F4, const float
     if (e != cudaSuccess) return e;
     const long long nb = cdiv(P, DT), grid = cdiv(nX, DX) * (nb * (nb + 1) / 2);
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
-    k_triangle_df<BIAS, EVEN><<<(unsigned)grid, DTH, smem, s>>>(H, E4, F4, G2, ME, MF, MG, P, nX, nI);
+    launch_chained(k_triangle_df<BIAS, EVEN>, (unsigned)grid, DTH, smem, s, H, E4, F4, G2, ME, MF,
+                   MG, P, nX, nI);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -584,6 +586,7 @@ cudaError_t launch_df(double* H, const float4* E4, const float4* F4, const float
 // M[chunk][Y][Z] = max over the chunk's grid points of |G_h^YZ| and |G_h^ZY|.
 // Block: one 32 x 32 tile and its mirror (grid x: tile pairs, y: chunks).
 __global__ void __launch_bounds__(256) k_pair_max(const float2* G2, int nI, int P, float* M) {
+    grid_wait();
     __shared__ float t1[32][33], t2[32][33];
     const int nb = (P + 31) / 32;
     int pidx = blockIdx.x, Yb = 0;
@@ -660,6 +663,7 @@ __device__ __forceinline__ void split1(double d, float& h, float& l) {
 // for the BC grid points of a chunk and also writes the largest |h| of every
 // column, M[chunk][q][P].
 __global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* out, float2* M) {
+    grid_wait();
     const int nXp = (nX + 1) / 2, per = M ? BC : 1;
     const long long rows = (long long)((nI + per - 1) / per) * nXp;
     for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
@@ -688,6 +692,7 @@ __global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* ou
 // in and out may be the same buffer: element i's float64 value is replaced
 // by its float pair in the same eight bytes.
 __global__ void k_split_df(const double* in, long long n, float2* out) {
+    grid_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         float h, l;
@@ -706,8 +711,8 @@ cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, 
                            cudaStream_t s) {
     if (nI <= 0 || nX <= 0 || P <= 0) return cudaSuccess;
     const long long rows = (long long)(bounds ? cdiv(nI, BC) : nI) * ((nX + 1) / 2);
-    k_split_pairs<<<(unsigned)std::min<long long>(rows, 152LL * 16), 128, 0, s>>>(E, nI, nX, P, out,
-                                                                                  bounds);
+    launch_chained(k_split_pairs, (unsigned)std::min<long long>(rows, 152LL * 16), 128, 0, s, E, nI,
+                   nX, P, out, bounds);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -715,14 +720,14 @@ cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, 
 cudaError_t pair_max(const float2* G2, int nI, int P, float* M, cudaStream_t s) {
     if (nI <= 0 || P <= 0) return cudaSuccess;
     const unsigned nb = cdiv(P, 32);
-    k_pair_max<<<dim3(nb * (nb + 1) / 2, cdiv(nI, BC)), 256, 0, s>>>(G2, nI, P, M);
+    launch_chained(k_pair_max, dim3(nb * (nb + 1) / 2, cdiv(nI, BC)), 256, 0, s, G2, nI, P, M);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t split_df(const double* in, long long n, float2* out, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    k_split_df<<<grid_for(n), 256, 0, s>>>(in, n, out);
+    launch_chained(k_split_df, grid_for(n), 256, 0, s, in, n, out);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(QTH, 2)
                     const __grid_constant__ CUtensorMap tmF,
                     const __grid_constant__ CUtensorMap tmG, int P, int ld, int nX, int nI,
                     int* err) {
+    grid_wait();
     extern __shared__ __align__(1024) unsigned char q_raw[];
     QSmem& sm = *reinterpret_cast<QSmem*>((reinterpret_cast<uintptr_t>(q_raw) + 1023) &
                                           ~uintptr_t(1023));
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__(QTH, 2)
 // lane (its second row is the slab's padding, never read).
 __global__ void __launch_bounds__(256) k_pair_rows(float* A, long long nslab, long long stride,
                                                    int nX, int P) {
+    grid_wait();
     extern __shared__ float seg[];   // 2P floats
     const int nq = (nX + 1) / 2;
     for (long long w = blockIdx.x; w < nslab * nq; w += gridDim.x) {
@@ -402,7 +404,7 @@ cudaError_t pair_rows(float* A, long long nslab, long long stride, int nX, int P
         const cudaError_t e = smem_optin((const void*)k_pair_rows, smem);
         if (e != cudaSuccess) return e;
     }
-    k_pair_rows<<<grid, 256, smem, s>>>(A, nslab, stride, nX, P);
+    launch_chained(k_pair_rows, grid, 256, smem, s, A, nslab, stride, nX, P);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -429,7 +431,7 @@ cudaError_t triangle_pair(float* H, const float2* E2, const float2* F2, const fl
     if (e != cudaSuccess) return e;
     const long long nb = cdiv(P, QT), grid = cdiv(nXp, QP) * (nb * (nb + 1) / 2);
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
-    k_triangle_pair<<<(unsigned)grid, QTH, smem, s>>>(H, mE, mF, mG, P, ld, nX, nI, err);
+    launch_chained(k_triangle_pair, (unsigned)grid, QTH, smem, s, H, mE, mF, mG, P, ld, nX, nI, err);
     count_launches(1);
     return cudaGetLastError();
 }
