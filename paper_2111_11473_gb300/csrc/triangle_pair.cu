@@ -14,16 +14,17 @@
 // two blocks per SM.  The tile is small because mirror pairs of tiles compute
 // the diagonal twice and the ragged edge for nothing (32-wide tiles 1.16 times
 // the needed work at P = 400, 16-wide ones 1.04).  Warp w takes pairs 4 w ..
-// + 3; lane (ly, lx, lz) = (lane / 8, lane / 4 % 2, lane % 4) owns the pairs
+// + 3; lane (lx, ly, lz) owns the pairs
 // 4 w + lx + 2p (p < 2), Y = 4 ly + (0..3) and Z = 4 lz + (0..3): 64 packed
 // accumulators per thread.  One thread streams the operands with 3-D TMA
 // boxes (swizzled) through a ring of QS stages of QI grid points; every wait
 // is bounded.  The last warp to finish with a stage issues its refill.
 // Bound: register reads of the packed FMAs (three distinct register pairs take
 // 3.3 cycles of a scheduler, 2 at best).  Measured at P = 400, 400 rows X, 1200
-// grid points: two stages of five grid points 7.99 ms (0.60 of the FP32 peak
-// in algorithmic flops), two of four 8.25, three of three 8.98, five of two
-// 9.04; blocks of 256 threads, 16 X and 32-wide tiles took 8.49.
+// grid points: 7.31 ms (0.65 of the FP32 peak in algorithmic flops); with bank
+// conflicts of the G^ZY reads 7.99, and then two stages of four grid points
+// 8.25, three of three 8.98, five of two 9.04; blocks of 256 threads, 16 X and
+// 32-wide tiles 8.49.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -156,7 +157,11 @@ __global__ void __launch_bounds__(QTH, 2)
     const int Y0 = Yb * QT, Z0 = Zb * QT, q0 = xb * QP;
     const bool diag = Yb == Zb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int lz = lane & 3, lx = (lane >> 2) & 1, ly = lane >> 3;
+    // Each run of eight lanes takes two ly, two lz and both lx, so that no 16-byte
+    // load of it meets a bank conflict (with all four lz in a run, the rows of
+    // G^ZY did: 16 of 112 shared-memory cycles per grid point and warp).
+    const int lz = (lane & 1) | (lane >> 2 & 2), ly = (lane >> 1 & 1) | (lane >> 3 & 2);
+    const int lx = lane >> 2 & 1;
     const int nst = (nI + QI - 1) / QI;
     const unsigned stage_bytes = 4u * QI * QP * QT * 8u + 2u * QI * QT * QT * 4u;
     if (threadIdx.x == 0) {
