@@ -73,22 +73,26 @@ FP64_ALU_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 # float32 operations issued per (I, X, Y, Z) term by each triangle kernel:
 # float64 kernel 3.5 float64 flops (t shared by the mirror outputs); float32
-# kernel over X pairs (P a multiple of 4) 2 FMA-pipe lane operations (one
-# packed multiply and three packed FMAs per pair of X and pair of mirror
-# outputs), 3 for the unpaired float32 kernel; float-pair kernel 43 float32
-# operations per pair of mirror outputs (19 for t, 12 per accumulation).
+# kernel over X pairs 2 FMA-pipe lane operations (one packed multiply and three
+# packed FMAs per pair of X and pair of mirror outputs), 3 for the unpaired
+# float32 kernel; float-pair kernel 43 float32 operations per pair of mirror
+# outputs (19 for t, 12 per accumulation).  The float-pair fraction is stated
+# against this count of the TwoSum form at every size; from 512 grid points on
+# the kernel issues 24 packed operations in the place of 40, so that it can
+# come above that form's bound.
 TRI_ISSUED = {"fp64": 3.5, "mixed": 2.0, "fp64tc": 21.5}
 TRI_KERNEL = {"fp64": "k_triangle_sym64", "mixed": "k_triangle_pair", "fp64tc": "k_triangle_df"}
 
 
 def _mixed_triangle_unpaired():
-    """The paired float32 triangle needs P % 4 == 0 and P <= 28000."""
+    """Workloads stated against the unpaired kernel's 3 operations per term (it
+    runs for P > 28000 only; the paired kernel takes every other P)."""
     return WORKLOAD is not None and not (WORKLOAD["P"] % 4 == 0 and WORKLOAD["P"] <= 28000)
 
 # DRAM bytes (read + write) of one triangle launch at o=40, v=200, P=400,
-# G=1200, from one ncu capture of the kernel that runs at that precision
-# (None: not captured since the kernel last changed).
-TRIANGLE_TRAFFIC_BYTES = {"fp64": 97.58e9 + 0.52e9, "fp64tc": 36.653e9 + 0.517e9,
+# G=1200, from one ncu capture (fp64 and mixed: of the 32-wide tiles used
+# before; the 16-wide tiles of the mixed kernel read and write 22.5e9).
+TRIANGLE_TRAFFIC_BYTES = {"fp64": 97.58e9 + 0.52e9, "fp64tc": 65.397e9 + 0.514e9,
                           "mixed": 12.702e9 + 0.249e9}
 
 
@@ -431,7 +435,7 @@ def run_peaks():
     bf16 = _peaks().get("bf16_tflops")
     gemm = {}
     for mode, name, nprod in ((0, "bf16x3", 3), (1, "bf16x3_with_pack", 3), (2, "bf16x1", 1),
-                              (3, "float64_slices", 36)):
+                              (3, "float64_slices", 28)):
         ms = b.probe_gemm(mode, n, n, n, 10 if mode < 3 else 3, stream)
         alg = 2.0 * n ** 3 / (ms * 1e-3) / 1e12
         gemm[name] = {"ms": ms, "algorithmic_tflops": alg, "bf16_product_tflops": alg * nprod,
@@ -762,9 +766,9 @@ def main():
         ms_d, fl_d, n_d = prof[dom]
         achieved = fl_d / (ms_d * 1e-3) / 1e12
         if args.precision == "fp64tc":
-            # 36 bf16 products per float64 multiply-add (8 slices a side)
-            peak = _peaks().get("bf16_tflops", 1931.0) / 36.0
-            bound, src = "tensor", "measured bf16 burst peak / 36 (slice products)"
+            # 28 bf16 products per float64 multiply-add (7 slices a side)
+            peak = _peaks().get("bf16_tflops", 1931.0) / 28.0
+            bound, src = "tensor", "measured bf16 burst peak / 28 (slice products)"
         elif fp64:
             peak, bound, src = FP64_ALU_TFLOPS, "alu", "derived: 152 SMs x 2 fp64 FMA lanes x 2 x 2.07 GHz"
         else:
@@ -782,7 +786,7 @@ def main():
         "scaling": "weak", "vs_baseline": None, "dtype": "f64" if fp64 else "f32+bf16x3",
         "data": "synthetic",
         "config": {"workload": WORKLOAD_NAME, "precision": args.precision,
-                   "products": {"fp64tc": "float64 by 8 exact 7-bit integer slices per operand "
+                   "products": {"fp64tc": "float64 by 7 exact 8-bit integer slices per operand "
                                           "row on the tensor cores, combined in float64",
                                 "fp64": "float64 on the CUDA cores",
                                 "mixed": "float32 operands, bf16 hi/lo on the tensor cores"}[
