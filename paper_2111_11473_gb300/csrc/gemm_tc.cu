@@ -810,7 +810,7 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
     // batches (packed one after the other), so that a batch leaves no ragged
     // row tile of its own (400 rows fill 4 tiles of 128 to 78 %).
     bool swap = g.N > g.M, collapse = false;
-    if (m_bc != n_bc && (long long)nb * (m_bc ? g.N : g.M) < INT32_MAX) {
+    if (m_bc != n_bc && (long long)nb * (m_bc ? g.N : g.M) < INT32_MAX - BM) {
         swap = m_bc;
         collapse = true;
     }
@@ -1956,7 +1956,7 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
     // otherwise every batch has a ragged tile (131 rows fill two tiles of 128
     // to a half, 200 and 400 rows 0.78 of theirs).
     const bool m_bc = !g.reduce && nb > 1 && g.sAb == 0, n_bc = !g.reduce && nb > 1 && g.sBb == 0;
-    const bool flat = m_bc != n_bc && (long long)nb * (m_bc ? g.N : g.M) < INT32_MAX;
+    const bool flat = m_bc != n_bc && (long long)nb * (m_bc ? g.N : g.M) < INT32_MAX - BM;
     const bool swap = flat ? m_bc : g.N > g.M;
     const int Mr = swap ? g.N : g.M, Nr = swap ? g.M : g.N;
     const long long Kp = rup(std::max(g.K, 1), 8);
