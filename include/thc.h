@@ -72,7 +72,10 @@ typedef enum {
  * of two per row), combined in fixed point: each product term is within about
  * 1.2e-16 of its row and column scale, float64 rounding level; the triangle
  * (Alg. 6 line 11) runs in float pairs on the FP32 pipe, each term within
- * about 2^-45 of |E F G|.  Per-step choices: thc_config.policy. */
+ * about 2^-45 of |E F G| and an element of H within about 2^-43 of
+ * sum_I |E F G| (rms; from 512 grid points of a chunk on, operands that are
+ * even enough over the grid take sums with common bounds, decided tile by tile
+ * from the operands).  Per-step choices: thc_config.policy. */
 typedef enum { THC_PREC_FP64 = 0, THC_PREC_MIXED = 1, THC_PREC_FP64_TC = 2 } thc_precision;
 
 /* Steps of one residual evaluation (per-step policy, timing and flop counts). */
@@ -124,7 +127,10 @@ typedef struct {
     int n_k;                 /* K: number of Cholesky vectors */
     int precision;           /* thc_precision */
     int k_slab;              /* Cholesky vectors per fused slab, 0 = auto */
-    int i_chunk;             /* grid points per Alg. 6 chunk, 0 = auto */
+    int i_chunk;             /* grid points per Alg. 6 chunk, 0 = auto (in float
+                                pairs, chunks of 512 or more that are multiples
+                                of 16, or the whole grid, take the faster sums
+                                with common bounds) */
     int x_block;             /* amplitude-THC columns per Alg. 7 block, 0 = auto */
     size_t workspace_bytes;  /* device workspace limit, 0 = auto */
     double lsq_rel_cutoff;   /* drop metric eigenvalues below cutoff*max (1e-10) */

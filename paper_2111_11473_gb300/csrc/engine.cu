@@ -721,11 +721,12 @@ Err Engine<T>::init_finish() {
         gall_resident = gall_fits;
         tri_df = std::is_same<T, double>::value && pol[THC_STEP_TRIANGLE] == THC_POL_FP64_TC;
         tri_pair = std::is_same<T, float>::value && triangle_pair_ok(P);
-        // The triangle's sums with bounds: grid chunks are whole bound chunks
-        // (i_chunk set by the caller may not be).
+        // The triangle's sums with bounds take launches of kBiasMinPoints grid
+        // points or more that are whole bound chunks (i_chunk set by the caller
+        // may not be).
         bool tri_bias = tri_df && G >= kBiasMinPoints;
         if (tri_bias && cfg.i_chunk == 0 && ic < G) ic = std::max(kBiasChunk, ic / kBiasChunk * kBiasChunk);
-        tri_bias = tri_bias && (ic >= G || ic % kBiasChunk == 0);
+        tri_bias = tri_bias && ic >= kBiasMinPoints && (ic >= G || ic % kBiasChunk == 0);
         if (gall_resident) {
             THC_TRY(Gall.alloc((size_t)G * PL));
             THC_TRY(mm(P, P, o, tr(yo, P), View<T>{U6.p, (long long)G * P, 1}, Gall.p, ldp, 1, 0,
@@ -737,7 +738,7 @@ Err Engine<T>::init_finish() {
                                       reinterpret_cast<float2*>(Gall.p), st));
                 if (tri_bias) {
                     THC_TRY(MG4.alloc((size_t)cdiv(G, kBiasChunk) * PP));
-                    THC_CUDA(pair_max(reinterpret_cast<const float2*>(Gall.p), G, P, MG4.p, st));
+                    THC_CUDA(chunk_max(reinterpret_cast<const float2*>(Gall.p), G, P, MG4.p, st));
                 }
             }
         } else {
@@ -752,6 +753,7 @@ Err Engine<T>::init_finish() {
                 const size_t bounds = (size_t)cdiv(ic, kBiasChunk) * ((x6 + 1) / 2) * P;
                 THC_TRY(ME4.alloc(bounds));
                 THC_TRY(MF4.alloc(bounds));
+                THC_TRY(uneven4.alloc((size_t)triangle_df_tiles(P, x6)));
             }
         }
         // slabs of C_i, D_a, E and F: an even number of rows for the paired triangle
@@ -924,6 +926,7 @@ Err Engine<T>::init_finish() {
         THC_TRY(poison(F4));
         THC_TRY(poison(ME4));
         THC_TRY(poison(MF4));
+        THC_TRY(poison(uneven4));
         if (!gall_resident) THC_TRY(poison(MG4));
     }
     THC_CUDA(cudaStreamSynchronize(st));
@@ -1016,7 +1019,7 @@ Err Engine<T>::alg6(T* sgm) {
                         THC_CUDA(split_df(Gch.p, (long long)nI * PL,
                                           reinterpret_cast<float2*>(Gch.p), st));
                         if (MG4.p)
-                            THC_CUDA(pair_max(reinterpret_cast<const float2*>(Gch.p), nI, P, MG4.p, st));
+                            THC_CUDA(chunk_max(reinterpret_cast<const float2*>(Gch.p), nI, P, MG4.p, st));
                     }
                 }
             }
@@ -1029,7 +1032,7 @@ Err Engine<T>::alg6(T* sgm) {
                     THC_CUDA(triangle_df(H.p, E4.p, F4.p, reinterpret_cast<const float2*>(Gp), ME4.p,
                                          MF4.p,
                                          gall_resident && MG4.p ? MG4.p + I0 / kBiasChunk * PL : MG4.p,
-                                         P, nX, nI, st));
+                                         uneven4.p, P, nX, nI, st));
                 else
                     THC_CUDA(triangle(H.p, Ech.p, Fch.p, Gp, P, nX, nI, st));
             } else if (tri_pair) {

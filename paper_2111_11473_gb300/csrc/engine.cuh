@@ -179,8 +179,9 @@ struct Engine {
     DBuf<float4> E4, F4;
     // Its bounds per kBiasChunk grid points (E, F of a grid chunk; G of all grid
     // points when resident, else of the chunk); empty = the TwoSum kernel.
-    DBuf<float2> ME4, MF4;
-    DBuf<float> MG4;
+    DBuf<uint2> ME4, MF4;
+    DBuf<unsigned> MG4;
+    DBuf<int> uneven4;   // per tile of a launch: 1 = not even enough for the bounds
     // Alg. 7 scratch (C7, D7: P x G on the dense route, G x P transposed on
     // the blocked route).
     DBuf<T> R7, S7, C7, D7, Yv, M7, Yo, N7, E7, P7, G7;

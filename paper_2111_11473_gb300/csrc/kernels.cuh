@@ -90,20 +90,24 @@ cudaError_t triangle(T* H, const T* E, const T* F, const T* G, int P, int nX, in
 // {h(x), h(x+1), l(x), l(x+1)} of E^{xY} for the row pairs x = 2q, 2q + 1
 // (split_df_pairs); G2: nI x P x P float2 {h, l} (split_df); H: nX x P x P
 // float64, accumulated into.
-// With bounds, also the largest |h| of every kBiasChunk grid points
-// (ceil(nI / kBiasChunk) x ceil(nX/2) x P).
+// With bounds, also the largest |h| and the geometric mean of every kBiasChunk
+// grid points (ceil(nI / kBiasChunk) x ceil(nX/2) x P; bf16 halves).
 constexpr int kBiasChunk = 16;
-cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, float2* bounds,
+cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, uint2* bounds,
                            cudaStream_t s);
-// The same of G: M[chunk][Y][Z] = max |G_h^YZ|, |G_h^ZY| (ceil(nI / kBiasChunk) x P x P).
-cudaError_t pair_max(const float2* G2, int nI, int P, float* M, cudaStream_t s);
-// Grid points from which the sums with bounds (ME, MF, MG not null) are the
-// more accurate ones.
+// The same of G: M[chunk][Y][Z] of |G_h^YZ| (ceil(nI / kBiasChunk) x P x P).
+cudaError_t chunk_max(const float2* G2, int nI, int P, unsigned* M, cudaStream_t s);
+// Grid points of a launch from which the sums with bounds are the more accurate
+// ones on operands of one scale.
 constexpr int kBiasMinPoints = 512;
 cudaError_t split_df(const double* in, long long n, float2* out, cudaStream_t s);
+// uneven: triangle_df_tiles(P, nX) words for the choice between the two forms,
+// tile by tile; without them or the bounds (ME, MF, MG) every tile takes the
+// TwoSum form.
+long long triangle_df_tiles(int P, int nX);
 cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
-                        const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
-                        cudaStream_t s);
+                        const uint2* ME, const uint2* MF, const unsigned* MG, int* uneven, int P,
+                        int nX, int nI, cudaStream_t s);
 
 // Float32 triangle over X pairs in packed lanes (triangle_pair.cu), for P at
 // most kPairMaxP.  Rows have a pitch of ld >= P, a multiple of 4: E2, F2: nI x

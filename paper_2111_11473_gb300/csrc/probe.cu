@@ -1,10 +1,14 @@
 // Throughput probes behind the C ABI (diagnostics; no counterpart in the
 // paper): the CUDA-core FMA rates that serve as roofline denominators of the
-// triangle kernels, and timed tensor-core products at a given shape.
+// triangle kernels, and timed tensor-core products at a given shape.  Also the
+// triangle kernels alone on given operands, for tests (not in thc.h).
+#include <algorithm>
 #include <string>
+#include <vector>
 
 #include "common.cuh"
 #include "gemm_tc.cuh"
+#include "kernels.cuh"
 
 namespace thc {
 
@@ -225,4 +229,110 @@ extern "C" thc_status thc_probe_gemm(int mode, int M, int N, int K, int iters, d
     }
     *ms_out = ms / iters;
     return THC_OK;
+}
+
+// H^XYZ = sum_I (E^XY F^XZ + E^XZ F^XY) G^YZ by one triangle kernel.  Host arrays:
+// E, F: nI x nX x P, G: nI x P x P, H: nX x P x P.  kind 0 float64, 1 float pairs
+// (as a float64 tensor-core context launches them; *tiles and *uneven, nullable,
+// receive the number of its tiles and of those that took the TwoSum form although
+// nI allows the other), 2 paired float32, 3 unpaired float32.
+extern "C" thc_status thc_diag_triangle(int kind, int P, int nX, int nI, const double* E,
+                                        const double* F, const double* G, double* H, int* tiles,
+                                        int* uneven, void* stream) {
+    using namespace thc;
+    if (kind < 0 || kind > 3 || P <= 0 || nX <= 0 || nX > P || nI <= 0 || !E || !F || !G || !H) {
+        set_thread_error("thc_diag_triangle: bad size or NULL pointer");
+        return THC_ERR_ARG;
+    }
+    cudaStream_t st = (cudaStream_t)stream;
+    const long long nE = (long long)nI * nX * P, nG = (long long)nI * P * P;
+    const long long nH = (long long)nX * P * P, nXp = (nX + 1) / 2;
+    std::vector<void*> held;
+    cudaError_t e = cudaSuccess;
+    auto make = [&](size_t bytes) -> void* {
+        void* p = nullptr;
+        if (e == cudaSuccess) e = cudaMalloc(&p, std::max<size_t>(bytes, 16));
+        if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, std::max<size_t>(bytes, 16), st);
+        if (p) held.push_back(p);
+        return p;
+    };
+    auto put = [&](const void* host, size_t bytes) -> void* {
+        void* p = make(bytes);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        return p;
+    };
+    int* err = (int*)make(sizeof(int));
+    std::vector<int> words;
+    if (kind <= 1) {
+        double* dE = (double*)put(E, nE * 8);
+        double* dF = (double*)put(F, nE * 8);
+        double* dG = (double*)put(G, nG * 8);
+        double* dH = (double*)make(nH * 8);
+        if (kind == 0) {
+            if (e == cudaSuccess) e = triangle(dH, dE, dF, dG, P, nX, nI, st);
+        } else {
+            const size_t nch = cdiv(nI, kBiasChunk);
+            float4* E4 = (float4*)make((size_t)nI * nXp * P * sizeof(float4));
+            float4* F4 = (float4*)make((size_t)nI * nXp * P * sizeof(float4));
+            uint2* ME = (uint2*)make(nch * nXp * P * sizeof(uint2));
+            uint2* MF = (uint2*)make(nch * nXp * P * sizeof(uint2));
+            unsigned* MG = (unsigned*)make(nch * P * P * sizeof(unsigned));
+            words.assign((size_t)triangle_df_tiles(P, nX), 0);
+            int* un = (int*)make(words.size() * sizeof(int));
+            float2* G2 = reinterpret_cast<float2*>(dG);
+            if (e == cudaSuccess) e = split_df_pairs(dE, nI, nX, P, E4, ME, st);
+            if (e == cudaSuccess) e = split_df_pairs(dF, nI, nX, P, F4, MF, st);
+            if (e == cudaSuccess) e = split_df(dG, nG, G2, st);
+            if (e == cudaSuccess) e = chunk_max(G2, nI, P, MG, st);
+            if (e == cudaSuccess) e = triangle_df(dH, E4, F4, G2, ME, MF, MG, un, P, nX, nI, st);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(words.data(), un, words.size() * sizeof(int),
+                                    cudaMemcpyDeviceToHost, st);
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(H, dH, nH * 8, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    } else {
+        const long long ld = kind == 2 ? (P + 3) / 4 * 4 : P;
+        const long long rows = kind == 2 ? 2 * nXp : nX;
+        std::vector<float> hE((size_t)nI * rows * ld), hF(hE.size()), hG((size_t)nI * P * ld);
+        for (long long I = 0; I < nI; ++I)
+            for (long long x = 0; x < nX; ++x)
+                for (long long y = 0; y < P; ++y) {
+                    const size_t from = (size_t)((I * nX + x) * P + y);
+                    const size_t to = (size_t)(kind == 2 ? ((I * nXp + x / 2) * ld + y) * 2 + x % 2
+                                                         : (I * nX + x) * P + y);
+                    hE[to] = (float)E[from];
+                    hF[to] = (float)F[from];
+                }
+        for (long long r = 0; r < (long long)nI * P; ++r)
+            for (long long z = 0; z < P; ++z) hG[(size_t)(r * ld + z)] = (float)G[r * P + z];
+        float* dE = (float*)put(hE.data(), hE.size() * 4);
+        float* dF = (float*)put(hF.data(), hF.size() * 4);
+        float* dG = (float*)put(hG.data(), hG.size() * 4);
+        std::vector<float> hH((size_t)nX * P * ld);
+        float* dH = (float*)make(hH.size() * 4);
+        if (e == cudaSuccess) {
+            if (kind == 2)
+                e = triangle_pair(dH, (const float2*)dE, (const float2*)dF, dG, P, (int)ld, nX, nI, st,
+                                  err);
+            else
+                e = triangle(dH, dE, dF, dG, P, nX, nI, st);
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(hH.data(), dH, hH.size() * 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        for (long long r = 0; r < (long long)nX * P; ++r)
+            for (long long z = 0; z < P; ++z) H[r * P + z] = hH[(size_t)(r * ld + z)];
+    }
+    int expired = 0;
+    if (e == cudaSuccess) e = cudaMemcpy(&expired, err, sizeof(int), cudaMemcpyDeviceToHost);
+    for (void* p : held) cudaFree(p);
+    if (tiles) *tiles = (int)words.size();
+    if (uneven) *uneven = (int)std::count(words.begin(), words.end(), 1);
+    if (e != cudaSuccess) {
+        set_thread_error(std::string("thc_diag_triangle: ") + cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? THC_ERR_OOM : THC_ERR_CUDA;
+    }
+    return expired ? THC_ERR_TIMEOUT : THC_OK;
 }

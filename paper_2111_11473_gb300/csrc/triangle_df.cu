@@ -60,13 +60,7 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 // -a in both lanes: a sign-bit flip on the integer pipe (the FMA pipe is the
 // busy one here; -0 for a zero lane, which no later sum can tell from +0).
 __device__ __forceinline__ f2 neg2(f2 a) {
-#ifdef THC_DF_SUBNEG
-    f2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(0ull), "l"(a));
-    return d;
-#else
     return a ^ 0x8000000080000000ull;
-#endif
 }
 // The rounded product fl(a b), written as fma(a, b, +0).  ptxas contracts a
 // packed mul.rn.f32x2 whose result feeds an add.rn.f32x2 into one fused
@@ -126,14 +120,19 @@ __device__ __forceinline__ void df_acc(f2& Sh, f2& Sl, f2 th, f2 tl, f2 thn, f2 
 // float32 sum.  6 packed operations per accumulation instead of 12: 24 per
 // (X pair, Y, Z) pair of mirror outputs instead of 40.
 // The bounds come from the largest |E|, |F|, |G| of BC grid points at a time
-// (k_split_pairs and k_pair_max write them), for every (X, Y, Z) of its own;
+// (k_split_pairs and k_chunk_max write them), for every (X, Y, Z) of its own;
 // after BC points the integer and float32 sums are added to a float pair in
-// shared memory.  Accuracy: an error u per term relative to the chunk's
-// bound instead of relative to the running sum, so it does not grow with the
-// number of grid points as the TwoSum form's does: on Gaussian operands, rms
-// over the sum of |terms|, 2^-46.1 / -46.6 / -47.1 for 300 / 600 / 1200 points
-// against 2^-46.7 / -46.2 / -45.7.  Hence the rule kBiasMinPoints: below it
-// the other kernel is the more accurate one (and the step is short).
+// shared memory.
+// Accuracy: the error of a term is relative to the chunk's bound, not to the
+// term or the running sum.  It does not grow with the number of grid points as
+// the TwoSum form's does: on Gaussian operands, rms over W = sum_I |E F G|,
+// 2^-46.2 / -46.8 / -47.2 for 256 / 512 / 1200 points against 2^-47.3 / -46.6 /
+// -46.3.  But a bound is the product of three largest values, and where E, F
+// or G vary over the 16 points, or are large at different ones, it lies far
+// above the terms: 2^-36 with entries spread over 2^-40 .. 1, 2^-42.5 with
+// operands that decay over the grid as exp(-I / 2) (TwoSum: 2^-44.7, 2^-46.8).
+// So it is used where the data carry it: in launches of kBiasMinPoints grid
+// points or more, and there for the tiles that k_bias_check finds even enough.
 constexpr int BC = kBiasChunk;              // grid points per chunk of common bounds
 
 // A block of 128 threads takes 8 rows X (4 lane pairs) and a pair of mirror 16
@@ -173,8 +172,8 @@ struct DfSmem<true> {
     DfStage st[BST];
     // bounds of a chunk (two chunks in flight)
     struct {
-        float2 ey[DP][DT], ez[DP][DT], fy[DP][DT], fz[DP][DT];   // [x pair][.]
-        float g[DT][DT];
+        uint2 ey[DP][DT], ez[DP][DT], fy[DP][DT], fz[DP][DT];    // [x pair][.]
+        unsigned g1[DT][DT], g2[DT][DT];                         // G^YZ rows Y, G^ZY rows Z
     } mx[2];
     ulonglong2 sum[16][DTH];          // float pairs {high, low} of the thread's 16 accumulators
 };
@@ -189,6 +188,11 @@ __device__ __forceinline__ f2 bias_of(f2 b) {
     };
     return pk(one(x), one(y));
 }
+// The bounds of a chunk are bf16 halves: {largest of x, of x + 1}, {means} of E and
+// F, {largest, mean} of G.
+__device__ __forceinline__ float bf_lo(unsigned v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(unsigned v) { return __uint_as_float(v & 0xFFFF0000u); }
+__device__ __forceinline__ f2 bound2(uint2 v) { return pk(bf_lo(v.x), bf_hi(v.x)); }
 __device__ __forceinline__ f2 max2(f2 a, f2 b) {
     float a0, a1, b0, b1;
     upk(a, a0, a1);
@@ -239,9 +243,9 @@ struct BiasAcc {
 
 // Both mirror outputs of a unit, operation by operation.
 __device__ __forceinline__ void bias_acc(BiasAcc& a, BiasAcc& b, f2 th, f2 tl, f2 gH, f2 gL, f2 kH,
-                                         f2 kL, f2 c) {
-    const f2 s = fma2(th, gH, c), t = fma2(th, kH, c);
-    const f2 y = sub2(c, s), z = sub2(c, t);
+                                         f2 kL, f2 c, f2 d) {
+    const f2 s = fma2(th, gH, c), t = fma2(th, kH, d);
+    const f2 y = sub2(c, s), z = sub2(d, t);
     f2 p = fma2(th, gH, y), q = fma2(th, kH, z);
     p = fma2(th, gL, p);
     q = fma2(th, kL, q);
@@ -303,13 +307,12 @@ struct DfAcc {
 template <>
 struct DfAcc<true> {
     BiasAcc h1[2][2][2], h2[2][2][2];
-    f2 sg[2][2][2], cb[2][2][2];   // biases of t's products and of t G
+    f2 sg[2][2][2], cb[2][2][2], db[2][2][2];   // biases of t's products, of t G^YZ and of t G^ZY
 };
 
 // Grid: block of DX rows X (fastest, so that the blocks running together share
 // the G tiles of one (Y, Z) pair in L2), pair of mirror tiles.
-// BIAS: bounds ME, MF: [chunk][x pair][P] (lanes x, x + 1); MG: [chunk][P][P],
-// symmetric.  EVEN: P is even, rows of G start on 16-byte boundaries and are
+// BIAS: bounds ME, MF: [chunk][x pair][P]; MG: [chunk][P][P].  EVEN: P is even, rows of G start on 16-byte boundaries and are
 // copied two columns at a time.
 // A packed FMA of three distinct register pairs measures 3.3 cycles of a
 // scheduler on GB300 and a packed addition 2.3 (peak: 2): the operations here
@@ -317,14 +320,20 @@ struct DfAcc<true> {
 // against 208 in the TwoSum form, so what comes besides them counts.  The copy
 // addresses advance by constants, which is why a thread copies a two-column
 // piece of one row of every G tile and one element of E and of F per grid
-// point.  P = 400, 400 rows X, 1200 grid points: 44.3 ms (32-wide tiles and one
-// block of 256 threads per SM: 58.5; their TwoSum form 68.7); P = 200, 200 X,
-// 600 points: 3.19 ms (4.93); TwoSum form, P = 100, 300 points: 0.41 (0.60).
+// point.  P = 400, 400 rows X, 1200 grid points: 46.3 ms (with one bias for both
+// mirror outputs, which measures the smaller of H^XYZ and H^XZY by the larger's
+// bound, 44.3; 32-wide tiles and one block of 256 threads per SM: 58.5; their
+// TwoSum form 68.7), and 0.37 for k_bias_check; TwoSum form, P = 100, 300 points:
+// 0.41 (0.60).
+// uneven (may be null for the TwoSum form): a block runs where its tile's word
+// asks for its form.
 template <bool BIAS, bool EVEN>
 __global__ void __launch_bounds__(DTH, 2)
     k_triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
-                  const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI) {
+                  const uint2* ME, const uint2* MF, const unsigned* MG, const int* uneven, int P,
+                  int nX, int nI) {
     grid_wait();
+    if (BIAS ? uneven[blockIdx.x] != 0 : uneven && uneven[blockIdx.x] == 0) return;
     extern __shared__ __align__(16) unsigned char df_raw[];
     DfSmem<BIAS>& sm = *reinterpret_cast<DfSmem<BIAS>*>(df_raw);
     const int nb = (P + DT - 1) / DT;
@@ -400,10 +409,13 @@ __global__ void __launch_bounds__(DTH, 2)
                 cp_n<8>(cz ? &mx.fz[cx][c] : &mx.fy[cx][c], np, en / 2);
                 mp += XP * 8;
                 np += XP * 8;
-                const float* m = MG + I0 / BC * PP +
+                const unsigned* m = MG + I0 / BC * PP +
                                  (g1n ? (long long)(Y0 + gr) * P + Z0 + 2 * gc : 0);
-                cp_n<4>(&mx.g[gr][2 * gc], m, min(g1n / 2, 4));
-                cp_n<4>(&mx.g[gr][2 * gc + 1], g1n > 8 ? m + 1 : m, max(g1n / 2 - 4, 0));
+                cp_n<4>(&mx.g1[gr][2 * gc], m, min(g1n / 2, 4));
+                cp_n<4>(&mx.g1[gr][2 * gc + 1], g1n > 8 ? m + 1 : m, max(g1n / 2 - 4, 0));
+                m = MG + I0 / BC * PP + (g2n ? (long long)(Z0 + gr) * P + Y0 + 2 * gc : 0);
+                cp_n<4>(&mx.g2[gr][2 * gc], m, min(g2n / 2, 4));
+                cp_n<4>(&mx.g2[gr][2 * gc + 1], g2n > 8 ? m + 1 : m, max(g2n / 2 - 4, 0));
             }
         }
         g1p += BS * PP * 8;
@@ -423,7 +435,7 @@ __global__ void __launch_bounds__(DTH, 2)
                 if constexpr (BIAS) {
                     A.h1[a][i][j] = BiasAcc{0u, 0u, 0ull};
                     A.h2[a][i][j] = BiasAcc{0u, 0u, 0ull};
-                    A.sg[a][i][j] = A.cb[a][i][j] = 0ull;
+                    A.sg[a][i][j] = A.cb[a][i][j] = A.db[a][i][j] = 0ull;
                     sm.sum[(a * 4 + i * 2 + j) * 2][tid] = make_ulonglong2(0ull, 0ull);
                     sm.sum[(a * 4 + i * 2 + j) * 2 + 1][tid] = make_ulonglong2(0ull, 0ull);
                 } else {
@@ -440,7 +452,7 @@ __global__ void __launch_bounds__(DTH, 2)
                     for (int j = 0; j < 2; ++j) {
                         const int u = (a * 4 + i * 2 + j) * 2;
                         bias_fold(A.h1[a][i][j], A.cb[a][i][j], n, sm.sum[u][tid]);
-                        bias_fold(A.h2[a][i][j], A.cb[a][i][j], n, sm.sum[u + 1][tid]);
+                        bias_fold(A.h2[a][i][j], A.db[a][i][j], n, sm.sum[u + 1][tid]);
                     }
         }
     };
@@ -468,14 +480,16 @@ __global__ void __launch_bounds__(DTH, 2)
                     for (int i = 0; i < 2; ++i)
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
-                            const f2 ey = reinterpret_cast<const f2&>(mx.ey[xg + a][ty + 8 * i]);
-                            const f2 fy = reinterpret_cast<const f2&>(mx.fy[xg + a][ty + 8 * i]);
-                            const f2 ez = reinterpret_cast<const f2&>(mx.ez[xg + a][tx + 8 * j]);
-                            const f2 fz = reinterpret_cast<const f2&>(mx.fz[xg + a][tx + 8 * j]);
-                            const float g = mx.g[ty + 8 * i][tx + 8 * j];
-                            const f2 p1 = prod2(ey, fz), p2 = prod2(ez, fy);
+                            const f2 ey = bound2(mx.ey[xg + a][ty + 8 * i]);
+                            const f2 fy = bound2(mx.fy[xg + a][ty + 8 * i]);
+                            const f2 ez = bound2(mx.ez[xg + a][tx + 8 * j]);
+                            const f2 fz = bound2(mx.fz[xg + a][tx + 8 * j]);
+                            const float g1 = bf_lo(mx.g1[ty + 8 * i][tx + 8 * j]);
+                            const float g2 = bf_lo(mx.g2[tx + 8 * j][ty + 8 * i]);
+                            const f2 p1 = prod2(ey, fz), p2 = prod2(ez, fy), p = add2(p1, p2);
                             A.sg[a][i][j] = bias_of(max2(p1, p2));
-                            A.cb[a][i][j] = bias_of(prod2(add2(p1, p2), pk(g, g)));
+                            A.cb[a][i][j] = bias_of(prod2(p, pk(g1, g1)));
+                            A.db[a][i][j] = bias_of(prod2(p, pk(g2, g2)));
                         }
             }
         }
@@ -516,7 +530,7 @@ __global__ void __launch_bounds__(DTH, 2)
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
                             bias_acc(A.h1[xp][i][j], A.h2[xp][i][j], th[j], tl[j], g1h[i][j],
-                                     g1l[i][j], g2h[i][j], g2l[i][j], A.cb[xp][i][j]);
+                                     g1l[i][j], g2h[i][j], g2l[i][j], A.cb[xp][i][j], A.db[xp][i][j]);
                     } else {
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
@@ -568,52 +582,125 @@ __global__ void __launch_bounds__(DTH, 2)
     }
 }
 
-template <bool BIAS, bool EVEN>
-cudaError_t launch_df(double* H, const float4* E4, const float4* F4, const float2* G2,
-                      const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
-                      cudaStream_t s) {
-    const int smem = (int)sizeof(DfSmem<BIAS>);
-    const cudaError_t e = smem_optin((const void*)k_triangle_df<BIAS, EVEN>, smem);
-    if (e != cudaSuccess) return e;
-    const long long nb = cdiv(P, DT), grid = cdiv(nX, DX) * (nb * (nb + 1) / 2);
-    if (grid > INT32_MAX) return cudaErrorInvalidValue;
-    launch_chained(k_triangle_df<BIAS, EVEN>, (unsigned)grid, DTH, smem, s, H, E4, F4, G2, ME, MF,
-                   MG, P, nX, nI);
-    count_launches(1);
-    return cudaGetLastError();
-}
+// ---------------------------------------------------------------------------
+// Which tiles the sums with bounds are accurate enough for.  With b_c the bounds
+// of an output's chunks, the rms error of the bounded sum is close to 2^-46.5
+// sqrt(16 sum_c b_c^2), the TwoSum form's between 2^-47 and 2^-43.5 of W = sum_I
+// (|E^XY F^XZ| + |E^XZ F^XY|) |G^YZ|.  A lower bound of W follows from each factor by
+// itself: the sum of n terms is at least n times their geometric mean, which is
+// the product of the factors' geometric means.  With those of a chunk, a tile is
+// even if
+//   sqrt(16 max_c b_c sum_c b_c) <= kEven sum_c n_c (<E^XY><F^XZ> + <E^XZ><F^XY>) <G^YZ>
+// (max b sum b >= sum b^2 keeps squares out of float32's range), that is, if the
+// rms error is at most 2^-43.2 W.  The left side over the right one's sum is 4.1
+// to 6.5 on Gaussian operands at 512 grid points, 2.9 to 3.5 at 1200; 10 is where the
+// bounded form begins to be less accurate than TwoSum (by 0.4 bits, for entries
+// spread over a factor of 2, 512 points); a spread over 2^-4 .. 1 gives 70 and
+// more, a decay of exp(-I / 8) 260.  Sums outside 2^-100 .. 2^120 are refused as well
+// (the biases end at 1.5 2^126); all-zero outputs are not.
+// A block looks at 256 outputs of 32 X and one (Y, Z) tile and both mirrors, with
+// X pair q = Y + Z mod 16, so that every element of E, F and G of the tile enters
+// one of them: the ratio of bound to mean is the product of the factors', each at
+// least 1, and an uneven element shows in any output.  (All 4096 outputs took
+// 5.9 ms at the size above.)
+constexpr float kEven = 10.f;
+constexpr int CX = 32;                      // X per block
 
-// M[chunk][Y][Z] = max over the chunk's grid points of |G_h^YZ| and |G_h^ZY|.
-// Block: one 32 x 32 tile and its mirror (grid x: tile pairs, y: chunks).
-__global__ void __launch_bounds__(256) k_pair_max(const float2* G2, int nI, int P, float* M) {
+__global__ void __launch_bounds__(256)
+    k_bias_check(const uint2* ME, const uint2* MF, const unsigned* MG, int P, int nX, int nI,
+                 int* uneven) {
     grid_wait();
-    __shared__ float t1[32][33], t2[32][33];
-    const int nb = (P + 31) / 32;
-    int pidx = blockIdx.x, Yb = 0;
+    const int nb = (P + DT - 1) / DT, nxb = (nX + DX - 1) / DX, nsx = (nX + CX - 1) / CX;
+    const int sx = (int)(blockIdx.x % (unsigned)nsx);
+    const int pair = (int)(blockIdx.x / (unsigned)nsx);
+    int pidx = pair, Yb = 0;
     while (pidx >= nb - Yb) {
         pidx -= nb - Yb;
         ++Yb;
     }
-    const int Y0 = Yb * 32, Z0 = (Yb + pidx) * 32, ch = blockIdx.y;
-    const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
-    const long long PP = (long long)P * P;
-    const int lo = ch * BC, hi = min(nI, lo + BC);
-    for (int r = r0; r < 32; r += 8) {
-        float a = 0.f, b = 0.f;
-        const bool ok1 = Y0 + r < P && Z0 + c < P, ok2 = Z0 + r < P && Y0 + c < P;
-        for (int I = lo; I < hi; ++I) {
-            if (ok1) a = fmaxf(a, fabsf(G2[I * PP + (long long)(Y0 + r) * P + Z0 + c].x));
-            if (ok2) b = fmaxf(b, fabsf(G2[I * PP + (long long)(Z0 + r) * P + Y0 + c].x));
+    const int y = threadIdx.x & 15, q = threadIdx.x >> 4;
+    const int Y = Yb * DT + y, Z = (Yb + pidx) * DT + ((q - y) & 15);
+    const int nXp = (nX + 1) / 2, xp = sx * (CX / 2) + q;
+    const long long PP = (long long)P * P, XP = (long long)nXp * P;
+    bool good = true;
+    if (Y < P && Z < P && xp < nXp) {
+        const uint2 *ey = ME + (long long)xp * P + Y, *ez = ME + (long long)xp * P + Z;
+        const uint2 *fy = MF + (long long)xp * P + Y, *fz = MF + (long long)xp * P + Z;
+        const unsigned *g1 = MG + (long long)Y * P + Z, *g2 = MG + (long long)Z * P + Y;
+        float sb[2][2] = {}, mb[2][2] = {}, w[2][2] = {};   // [mirror][lane]
+        const int nch = (nI + BC - 1) / BC;
+#pragma unroll 4
+        for (int c = 0; c < nch; ++c) {
+            const uint2 a = ey[c * XP], b = ez[c * XP], d = fy[c * XP], e = fz[c * XP];
+            const unsigned g[2] = {g1[c * PP], g2[c * PP]};
+            const float n = (float)min(BC, nI - c * BC);
+            const float tb[2] = {fmaf(bf_lo(d.x), bf_lo(b.x), bf_lo(a.x) * bf_lo(e.x)),
+                                 fmaf(bf_hi(d.x), bf_hi(b.x), bf_hi(a.x) * bf_hi(e.x))};
+            const float tw[2] = {fmaf(bf_lo(d.y), bf_lo(b.y), bf_lo(a.y) * bf_lo(e.y)),
+                                 fmaf(bf_hi(d.y), bf_hi(b.y), bf_hi(a.y) * bf_hi(e.y))};
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int l = 0; l < 2; ++l) {
+                    const float v = tb[l] * bf_lo(g[m]);
+                    sb[m][l] += v;
+                    mb[m][l] = fmaxf(mb[m][l], v);
+                    w[m][l] = fmaf(tw[l], n * bf_hi(g[m]), w[m][l]);
+                }
         }
-        t1[r][c] = a;
-        t2[r][c] = b;
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int l = 0; l < 2; ++l) {
+                const float v = w[m][l] * (kEven / 4.f);
+                const bool in = mb[m][l] > 0x1p-100f && mb[m][l] < 0x1p120f;
+                good = good && (mb[m][l] == 0.f || (in && mb[m][l] / v * (sb[m][l] / v) <= 1.f));
+            }
     }
-    __syncthreads();
-    for (int r = r0; r < 32; r += 8) {
-        if (Y0 + r < P && Z0 + c < P)
-            M[ch * PP + (long long)(Y0 + r) * P + Z0 + c] = fmaxf(t1[r][c], t2[c][r]);
-        if (Z0 + r < P && Y0 + c < P)
-            M[ch * PP + (long long)(Z0 + r) * P + Y0 + c] = fmaxf(t2[r][c], t1[c][r]);
+    const int all = __syncthreads_and(good);
+    if (threadIdx.x < CX / DX && sx * (CX / DX) + (int)threadIdx.x < nxb)
+        uneven[(long long)pair * nxb + sx * (CX / DX) + threadIdx.x] = all ? 0 : 1;
+}
+
+template <bool BIAS, bool EVEN>
+cudaError_t launch_df(double* H, const float4* E4, const float4* F4, const float2* G2,
+                      const uint2* ME, const uint2* MF, const unsigned* MG, const int* uneven, int P,
+                      int nX, int nI, cudaStream_t s) {
+    const int smem = (int)sizeof(DfSmem<BIAS>);
+    const cudaError_t e = smem_optin((const void*)k_triangle_df<BIAS, EVEN>, smem);
+    if (e != cudaSuccess) return e;
+    const long long grid = triangle_df_tiles(P, nX);
+    if (grid > INT32_MAX) return cudaErrorInvalidValue;
+    launch_chained(k_triangle_df<BIAS, EVEN>, (unsigned)grid, DTH, smem, s, H, E4, F4, G2, ME, MF,
+                   MG, uneven, P, nX, nI);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+// Largest value (rounded up) and geometric mean (rounded down, from the sum of n
+// binary logarithms) in bf16; a zero makes the mean zero.
+__device__ __forceinline__ unsigned bf_up(float v) {
+    return (__float_as_uint(v) + 0xFFFFu) >> 16;
+}
+__device__ __forceinline__ unsigned bf_mean(float logs, int n) {
+    return __float_as_uint(exp2f(logs / (float)n)) >> 16;
+}
+
+// M[chunk][Y][Z] = {largest, mean} |G_h^YZ| of the chunk's grid points (grid y: chunks).
+__global__ void __launch_bounds__(256) k_chunk_max(const float2* G2, int nI, int P, unsigned* M) {
+    grid_wait();
+    const int ch = blockIdx.y, lo = ch * BC, n = min(nI - lo, BC);
+    const long long PP = (long long)P * P;
+    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < PP; e += gridDim.x * 256LL) {
+        const float2* g = G2 + lo * PP + e;
+        float m = 0.f, s = 0.f;
+#pragma unroll 4
+        for (int I = 0; I < n; ++I) {
+            const float v = fabsf(g[I * PP].x);
+            m = fmaxf(m, v);
+            s += __log2f(v);
+        }
+        M[ch * PP + e] = bf_up(m) | bf_mean(s, n) << 16;
     }
 }
 
@@ -660,9 +747,9 @@ __device__ __forceinline__ void split1(double d, float& h, float& l) {
 
 // One block per output row (I, q) at a time, threads along the P columns
 // (no 64-bit division per element).  With M, a block takes the rows of one q
-// for the BC grid points of a chunk and also writes the largest |h| of every
-// column, M[chunk][q][P].
-__global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* out, float2* M) {
+// for the BC grid points of a chunk and also writes the largest |h| and the
+// geometric mean of every column, M[chunk][q][P].
+__global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* out, uint2* M) {
     grid_wait();
     const int nXp = (nX + 1) / 2, per = M ? BC : 1;
     const long long rows = (long long)((nI + per - 1) / per) * nXp;
@@ -672,7 +759,7 @@ __global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* ou
         const int lo = (int)ch * per, hi = min(nI, lo + per);
         const bool two = x + 1 < nX;
         for (int c = threadIdx.x; c < P; c += blockDim.x) {
-            float m0 = 0.f, m1 = 0.f;
+            float m0 = 0.f, m1 = 0.f, s0 = 0.f, s1 = 0.f;
             for (int I = lo; I < hi; ++I) {
                 const double* e0 = E + ((long long)I * nX + x) * P;
                 const double d0 = e0[c];
@@ -683,8 +770,12 @@ __global__ void k_split_pairs(const double* E, int nI, int nX, int P, float4* ou
                 out[((long long)I * nXp + q) * P + c] = make_float4(h0, h1, l0, l1);
                 m0 = fmaxf(m0, fabsf(h0));
                 m1 = fmaxf(m1, fabsf(h1));
+                s0 += __log2f(fabsf(h0));
+                s1 += __log2f(fabsf(h1));
             }
-            if (M) M[row * P + c] = make_float2(m0, m1);
+            if (M)
+                M[row * P + c] = make_uint2(bf_up(m0) | bf_up(m1) << 16,
+                                            bf_mean(s0, hi - lo) | bf_mean(s1, hi - lo) << 16);
         }
     }
 }
@@ -707,7 +798,7 @@ unsigned grid_for(long long n) {
 
 }  // namespace
 
-cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, float2* bounds,
+cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, uint2* bounds,
                            cudaStream_t s) {
     if (nI <= 0 || nX <= 0 || P <= 0) return cudaSuccess;
     const long long rows = (long long)(bounds ? cdiv(nI, BC) : nI) * ((nX + 1) / 2);
@@ -717,10 +808,10 @@ cudaError_t split_df_pairs(const double* E, int nI, int nX, int P, float4* out, 
     return cudaGetLastError();
 }
 
-cudaError_t pair_max(const float2* G2, int nI, int P, float* M, cudaStream_t s) {
+cudaError_t chunk_max(const float2* G2, int nI, int P, unsigned* M, cudaStream_t s) {
     if (nI <= 0 || P <= 0) return cudaSuccess;
-    const unsigned nb = cdiv(P, 32);
-    launch_chained(k_pair_max, dim3(nb * (nb + 1) / 2, cdiv(nI, BC)), 256, 0, s, G2, nI, P, M);
+    const unsigned nb = (unsigned)std::min<long long>(((long long)P * P + 255) / 256, 152LL * 8);
+    launch_chained(k_chunk_max, dim3(nb, cdiv(nI, BC)), 256, 0, s, G2, nI, P, M);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -732,15 +823,30 @@ cudaError_t split_df(const double* in, long long n, float2* out, cudaStream_t s)
     return cudaGetLastError();
 }
 
+long long triangle_df_tiles(int P, int nX) {
+    const long long nb = cdiv(P, DT);
+    return cdiv(nX, DX) * (nb * (nb + 1) / 2);
+}
+
 cudaError_t triangle_df(double* H, const float4* E4, const float4* F4, const float2* G2,
-                        const float2* ME, const float2* MF, const float* MG, int P, int nX, int nI,
-                        cudaStream_t s) {
+                        const uint2* ME, const uint2* MF, const unsigned* MG, int* uneven, int P,
+                        int nX, int nI, cudaStream_t s) {
     if (nX <= 0 || nI <= 0) return cudaSuccess;
-    if (ME && MF && MG)
-        return P % 2 ? launch_df<true, false>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s)
-                     : launch_df<true, true>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s);
-    return P % 2 ? launch_df<false, false>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s)
-                 : launch_df<false, true>(H, E4, F4, G2, ME, MF, MG, P, nX, nI, s);
+    const bool bounds = ME && MF && MG && uneven && nI >= kBiasMinPoints;
+    if (bounds) {
+        const long long nb = cdiv(P, DT), grid = cdiv(nX, CX) * (nb * (nb + 1) / 2);
+        if (grid > INT32_MAX) return cudaErrorInvalidValue;
+        launch_chained(k_bias_check, (unsigned)grid, 256, 0, s, ME, MF, MG, P, nX, nI, uneven);
+        count_launches(1);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = P % 2 ? launch_df<true, false>(H, E4, F4, G2, ME, MF, MG, uneven, P, nX, nI, s)
+                      : launch_df<true, true>(H, E4, F4, G2, ME, MF, MG, uneven, P, nX, nI, s);
+        if (e != cudaSuccess) return e;
+    }
+    const int* rest = bounds ? uneven : nullptr;
+    return P % 2 ? launch_df<false, false>(H, E4, F4, G2, ME, MF, MG, rest, P, nX, nI, s)
+                 : launch_df<false, true>(H, E4, F4, G2, ME, MF, MG, rest, P, nX, nI, s);
 }
 
 }  // namespace thc
