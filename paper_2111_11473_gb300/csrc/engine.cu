@@ -650,7 +650,7 @@ Err Engine<T>::init_finish() {
     //      its packed copy for the post-products, D_a and C_i (x6 P each per
     //      orbital) take at most a quarter of the free memory (48 GiB at
     //      most); all P rows in one block when they fit, else the fewest
-    //      blocks that do, rounded up to the triangle kernel's 32-row tile.
+    //      blocks that do, rounded up to 32 rows.
     ldp = std::is_same<T, float>::value && triangle_pair_ok(P) ? (P + 3) / 4 * 4 : P;
     const long long PL = (long long)P * ldp;   // elements of one G_I or one X of H
     const size_t gall_bytes = (size_t)G * PL * sizeof(T);
@@ -722,11 +722,17 @@ Err Engine<T>::init_finish() {
         tri_df = std::is_same<T, double>::value && pol[THC_STEP_TRIANGLE] == THC_POL_FP64_TC;
         tri_pair = std::is_same<T, float>::value && triangle_pair_ok(P);
         // The triangle's sums with bounds take launches of kBiasMinPoints grid
-        // points or more that are whole bound chunks (i_chunk set by the caller
-        // may not be).
-        bool tri_bias = tri_df && G >= kBiasMinPoints;
-        if (tri_bias && cfg.i_chunk == 0 && ic < G) ic = std::max(kBiasChunk, ic / kBiasChunk * kBiasChunk);
-        tri_bias = tri_bias && ic >= kBiasMinPoints && (ic >= G || ic % kBiasChunk == 0);
+        // points or more that are whole bound chunks: an automatic chunk is
+        // rounded down to that, and the chunks are made of one length where the
+        // last one is then long enough too (G = 1800 at P = 600: 608, 608, 584
+        // points instead of 736, 736, 328).
+        if (tri_df && cfg.i_chunk == 0 && ic < G && ic >= kBiasMinPoints) {
+            ic = ic / kBiasChunk * kBiasChunk;
+            const int n = (G + ic - 1) / ic;
+            const int even = ((G + n - 1) / n + kBiasChunk - 1) / kBiasChunk * kBiasChunk;
+            if (G - (n - 1) * even >= kBiasMinPoints) ic = even;
+        }
+        const bool tri_bias = tri_df && ic >= kBiasMinPoints && (ic >= G || ic % kBiasChunk == 0);
         if (gall_resident) {
             THC_TRY(Gall.alloc((size_t)G * PL));
             THC_TRY(mm(P, P, o, tr(yo, P), View<T>{U6.p, (long long)G * P, 1}, Gall.p, ldp, 1, 0,
