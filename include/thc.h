@@ -468,7 +468,10 @@ thc_status thc_energy_noalloc(int n_occ, int n_vir, int n_p, int n_k,
  * projectors (Eqs. 15-16, App. I): U_ia^P ~ sum_W y_i^W y_a^W tau^PW,
  * minimising f = sum_P eps_P^2 sum_ia (U_ia^P - sum_W y_i^W y_a^W tau^PW)^2
  * by `iters` sweeps of alternating least squares (y_o, then y_v, then tau;
- * the y_o update is Eq. 16), float64 on the device.  The W x W normal
+ * the y_o update is Eq. 16), float64 on the device: the large products run as
+ * integer slices on the tensor cores (as THC_PREC_FP64_TC), except for elements
+ * whose sum |a b| is below the scale of their row and column, where float64 sums
+ * have the smaller error bound and are formed instead.  The W x W normal
  * equations are solved by Cholesky factorisation (App. I uses CG).
  *   U: (n_occ n_vir) x n_rr row-major, row (i, a) = i n_vir + a
  *   eps: n_rr projector eigenvalues (any sign)
@@ -477,7 +480,9 @@ thc_status thc_energy_noalloc(int n_occ, int n_vir, int n_p, int n_k,
  *   objective: nullable host array of `iters` doubles, f after every sweep
  * All arrays host or device; stream: cudaStream_t or NULL.  Returns
  * THC_ERR_NUMERIC if a normal-equation matrix stays singular after a ridge
- * of 1e-12 of its largest diagonal.  No context is needed.
+ * of 1e-12 of its largest diagonal, THC_ERR_TIMEOUT if a bounded wait of a
+ * tensor-core product expired (y_o, y_v and tau are left as they were), both
+ * before anything is written to them.  No context is needed.
  */
 thc_status thc_cp_als(int n_occ, int n_vir, int n_rr, int rank, const double* U,
                       const double* eps, double* y_o, double* y_v, double* tau, int iters,

@@ -6,9 +6,18 @@
 // (the MTTKRP of App. I's Eq. 46 as one GEMM plus a reduction over the
 // other orbital index); the W x W normal equations (Eqs. 44-45) are solved
 // by Cholesky factorisation instead of App. I's preconditioned CG.
-// The large products run as exact integer slices on the tensor cores where
-// that is estimated to be faster (gemm_tc.cu; the sums are closer to the
-// exact ones than those of the float64 CUDA cores).
+// The large products run as exact integer slices on the tensor cores
+// (gemm_tc.cu) where that is estimated to be faster and the operands allow it:
+// slices are cut below one power of two per row, so that an output in which the
+// large entries of a row of one operand meet small ones of the other's (U over
+// eigenvalues of several decades) would lose what float64 sums keep.  Every
+// product by slices is checked for that (k_slices_even); outputs that fail are done
+// again as float64 sums, the whole product on the CUDA cores if they are more than
+// a sixteenth.  With sums of |a b| at or above that scale the slices
+// are the more accurate ones: rms error over the sum of |a b|, U of rank 200
+// plus noise, 300 projectors, eigenvalues 1 .. 0.3: U te 2^-54.5 (float64 sums
+// 2^-53.1), U^T KR 2^-55.9 (2^-51.4), KR tau^T 2^-54.4 (2^-53.8); without the
+// check, eigenvalues over 6 decades and U large where they are small: 2^-33.8.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -284,8 +293,10 @@ struct Als {
     long long ov;
     cudaStream_t st;
     Dev S, S2, SE, M, KR, R, te, rec, part, ws, diag, info;
-    Dev slices, fpart, expo;
+    Dev slices, fpart, expo, list;
+    static constexpr int kRedo = 1 << 16;   // outputs of a product done again
     F64TcWorkspace tc;
+    bool expired = false;   // a bounded wait of a product
     std::string err;
 
     cudaError_t init() {
@@ -297,12 +308,15 @@ struct Als {
             (e = R.alloc((size_t)mx * W)) || (e = te.alloc((size_t)N * W)) ||
             (e = rec.alloc((size_t)ov * N)) || (e = part.alloc(152 * 16)) ||
             (e = ws.alloc(1 << 22)) || (e = diag.alloc((size_t)cdiv(W, CB) * kDiagDoubles)) ||
-            (e = info.alloc(1)))
+            (e = info.alloc(2)))
             return e;
-        if ((e = cudaMemsetAsync(info.p, 0, sizeof(double), st))) return e;
-        // Tensor-core products: room for the largest in one piece, at most 2
-        // GiB of slices (larger ones are cut); without the memory they stay on
-        // the CUDA cores.
+        return cudaMemsetAsync(info.p, 0, 2 * sizeof(double), st);
+    }
+
+    // Tensor-core products: room for the largest in one piece, at most 2 GiB of
+    // slices (larger ones are cut); without the memory the products stay on the
+    // CUDA cores.
+    void init_slices() {
         size_t sl = 0, pt = 0, ex = 0;
         const long long shapes[][3] = {{ov, W, N}, {W, W, N}, {W, W, v}, {W, W, o},
                                        {N, W, ov}, {ov, N, W}};
@@ -318,7 +332,8 @@ struct Als {
         }
         if (sl > 0) {
             sl = std::min<size_t>(sl, 1ULL << 30);
-            if (slices.alloc(sl / 4 + 1) || fpart.alloc(pt / 2 + 1) || expo.alloc(ex / 2 + 1)) {
+            if (slices.alloc(sl / 4 + 1) || fpart.alloc(pt / 2 + 1) || expo.alloc(ex / 2 + 1) ||
+                list.alloc(kRedo)) {
                 cudaGetLastError();   // not enough memory
             } else {
                 tc.slices = reinterpret_cast<__nv_bfloat16*>(slices.p);
@@ -328,9 +343,11 @@ struct Als {
                 tc.expo = reinterpret_cast<int*>(expo.p);
                 tc.expo_elems = ex;
                 tc.err = reinterpret_cast<int*>(info.p) + 1;
+                tc.redo = tc.err + 1;
+                tc.redo_list = reinterpret_cast<int2*>(list.p);
+                tc.redo_cap = kRedo;
             }
         }
-        return cudaSuccess;
     }
 
     // C (M x N) = A B, row-major views.
@@ -340,8 +357,17 @@ struct Als {
         g.A = A; g.B = B; g.C = C; g.ldc = n;
         g.ws = ws.p; g.ws_elems = 1 << 22;
         if (tc.slices && f64_tc_pays(m, n, k, 1, false)) {
-            const cudaError_t e = gemm_f64_tc(g, tc, st);
-            if (e != cudaErrorMemoryAllocation) return e;
+            int flags[3] = {0, 0, 0};   // a wait expired; -; too many outputs to do again
+            cudaError_t e = cudaMemsetAsync(tc.redo + 1, 0, sizeof(int), st);
+            if (!e) e = gemm_f64_tc(g, tc, st);
+            if (!e) e = cudaMemcpyAsync(flags, tc.err, sizeof(flags), cudaMemcpyDeviceToHost, st);
+            if (!e) e = cudaStreamSynchronize(st);
+            if (!e && flags[0]) {
+                expired = true;
+                return cudaErrorUnknown;
+            }
+            if (!e && !flags[2]) return cudaSuccess;
+            if (e && e != cudaErrorMemoryAllocation) return e;
         }
         return gemm_simt(g, st);
     }
@@ -493,6 +519,7 @@ extern "C" thc_status thc_cp_als(int n_occ, int n_vir, int n_rr, int rank, const
     a.ov = (long long)n_occ * n_vir;
     a.st = (cudaStream_t)stream;
     cudaError_t e = a.init();
+    if (!e) a.init_slices();
     // Device copies of the inputs and of the factors (updated in place).
     Dev dU, de, dyo, dyv, dt;
     const size_t nU = (size_t)a.ov * n_rr;
@@ -518,11 +545,8 @@ extern "C" thc_status thc_cp_als(int n_occ, int n_vir, int n_rr, int rank, const
     if (!e) e = cudaMemcpyAsync(y_o, dyo.p, sizeof(double) * no, cudaMemcpyDefault, a.st);
     if (!e) e = cudaMemcpyAsync(y_v, dyv.p, sizeof(double) * nv, cudaMemcpyDefault, a.st);
     if (!e) e = cudaMemcpyAsync(tau, dt.p, sizeof(double) * nt, cudaMemcpyDefault, a.st);
-    int expired = 0;
-    if (!e && a.tc.slices)
-        e = cudaMemcpyAsync(&expired, a.tc.err, sizeof(int), cudaMemcpyDeviceToHost, a.st);
     if (!e) e = cudaStreamSynchronize(a.st);
-    if (!e && expired) {
+    if (a.expired) {
         set_thread_error("thc_cp_als: a tensor-core kernel's bounded wait expired");
         return THC_ERR_TIMEOUT;
     }

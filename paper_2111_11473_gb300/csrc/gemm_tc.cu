@@ -1228,6 +1228,127 @@ __global__ void __launch_bounds__(256) k_slice_rows(const __grid_constant__ Slic
     }
 }
 
+// Lists the outputs (i, j) of a single product with
+//   sum_k |a_ik b_jk| < 2^(e_i + e_j)          (e: the exponents of the slices);
+// redo[0] counts them (the list ends at `cap`).
+// A product by slices is off by at most K 2^-53 2^(e_i + e_j) (rounding of the
+// operands and digit pairs left out, 8 units of 2^-56 per term), float64 sums
+// by K 2^-53 sum_k |a_ik b_jk| and more: where the sum reaches the scale, the
+// slices' bound is no larger.  It does not where the large entries of a row meet
+// the small ones of a column, and at a few outputs of heavy-tailed rows.  The sum
+// is bounded from below by the first digits, |a| >= (|a_1| - 0.502) 2^(e - 7): as 8-bit
+// integers 2 |a_1| - 1 (0.4 % above that at most, which kEnough allows for), four
+// products per instruction, and only until every output of the tile has enough: 60
+// of 300 K indices for Gaussian entries.  Zero rows are exact; those with a
+// non-finite entry and results outside 2^-700 .. 2^800 are left to float64 sums.
+// Tile of 32 x 32 outputs, 2 x 2 per thread: 12 us for 8000 x 200 x 300, 29 for
+// 300 x 200 x 8000 (few tiles, 10 K blocks each), 25 for 8000 x 300 x 200; with
+// float32 products 26, 46 and 59.
+constexpr unsigned kEnough = 66200u;     // (2 2^7)^2 and a hundredth
+__global__ void __launch_bounds__(256)
+    k_slices_even(const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int K,
+                  const int* eA, const int* eB, int* redo, int2* list, int cap) {
+    grid_wait();
+    __shared__ unsigned a[BK / 4][33], b[BK / 4][33];      // four K indices per word
+    const int nt = (N + 31) / 32;
+    const int m0 = (int)(blockIdx.x / (unsigned)nt) * 32, n0 = (int)(blockIdx.x % (unsigned)nt) * 32;
+    const int lr = threadIdx.x >> 3, lk = (threadIdx.x & 7) * 8;     // row and K octet loaded
+    const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+    unsigned sum[2][2] = {};
+    bool need[2][2], bad[2][2];   // a sum to look at; an output that is not for slices
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int m = m0 + tr + 16 * i, n = n0 + tc + 16 * j;
+            const bool in = m < M && n < N;
+            const int ea = in ? eA[m] : 0, eb = in ? eB[n] : 0, e = ea + eb;
+            const bool zero = ea == 0 || eb == 0;
+            bad[i][j] = max(ea, eb) == 2047 || (!zero && (e <= 2044 - 700 || e >= 2044 + 800));
+            need[i][j] = !zero && !bad[i][j];
+        }
+    // 2 |d| - 1 or 0 in the low byte of the float's bits
+    auto lower = [](unsigned half) {
+        return __float_as_uint(fmaxf(fmaf(2.f, fabsf(__uint_as_float(half << 16)), 8388607.f), 8388608.f)) &
+               0xFFu;
+    };
+    for (int k0 = 0;; k0 += BK) {
+        bool enough = true;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) enough = enough && (!need[i][j] || sum[i][j] >= kEnough);
+        // (also the barrier between the reads of a K block and its successor's writes)
+        if (__syncthreads_and(enough) || k0 >= K) break;
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        const long long at = (long long)(k0 / BK) * kSlices;
+        const uint4 va = m0 + lr < M
+            ? *reinterpret_cast<const uint4*>(A + (at * M + m0 + lr) * BK + lk) : z;
+        const uint4 vb = n0 + lr < N
+            ? *reinterpret_cast<const uint4*>(B + (at * N + n0 + lr) * BK + lk) : z;
+        const unsigned ua[4] = {va.x, va.y, va.z, va.w}, ub[4] = {vb.x, vb.y, vb.z, vb.w};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            unsigned wa = 0u, wb = 0u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int e = 4 * h + j;
+                if (k0 + lk + e < K) {            // (what follows is not written)
+                    wa |= lower(ua[e / 2] >> (16 * (e & 1)) & 0xFFFFu) << (8 * j);
+                    wb |= lower(ub[e / 2] >> (16 * (e & 1)) & 0xFFFFu) << (8 * j);
+                }
+            }
+            a[lk / 4 + h][lr] = wa;
+            b[lk / 4 + h][lr] = wb;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < BK / 4; ++k) {
+            const unsigned a0 = a[k][tr], a1 = a[k][tr + 16], b0 = b[k][tc], b1 = b[k][tc + 16];
+            sum[0][0] = __dp4a(a0, b0, sum[0][0]);
+            sum[0][1] = __dp4a(a0, b1, sum[0][1]);
+            sum[1][0] = __dp4a(a1, b0, sum[1][0]);
+            sum[1][1] = __dp4a(a1, b1, sum[1][1]);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) sum[i][j] = min(sum[i][j], 1u << 24);   // (no wrap)
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if ((bad[i][j] || (need[i][j] && sum[i][j] < kEnough)) &&
+                *(volatile int*)redo <= cap) {       // (more need not be counted)
+                const int at = atomicAdd(redo, 1);
+                if (at < cap) list[at] = make_int2(m0 + tr + 16 * i, n0 + tc + 16 * j);
+            }
+}
+
+// The listed outputs as float64 sums, a warp each; if there are more than `cap` of
+// them, or C's old values were needed, only says so in redo[1].
+__global__ void __launch_bounds__(256)
+    k_redo64(const double* A, long long ars, long long aks, const double* B, long long brs,
+             long long bks, int K, double alpha, double* C, long long crs, long long ccs, int* redo,
+             const int2* list, int cap) {
+    grid_wait();
+    const int n = redo[0], lane = threadIdx.x & 31;
+    if (n > cap) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) redo[1] = 1;
+        return;
+    }
+    for (int e = blockIdx.x * 8 + (threadIdx.x >> 5); e < n; e += gridDim.x * 8) {
+        const int2 ij = list[e];
+        const double *a = A + ij.x * ars, *b = B + ij.y * brs;
+        double s = 0.0;
+#pragma unroll 4
+        for (int k = lane; k < K; k += 32) s = fma(a[k * aks], b[k * bks], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) C[ij.x * crs + ij.y * ccs] = alpha * s;
+    }
+}
+
 __device__ __forceinline__ double pow2(int k) {
     return (k >= -1022 && k <= 1023) ? __longlong_as_double((long long)(k + 1023) << 52)
                                      : scalbn(1.0, k);
@@ -2015,6 +2136,19 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
         count_launches(2);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const bool redo = ws.redo && nb == 1;
+    // (a sixteenth of the outputs at most: the rest of the product is then worth it)
+    const int redo_cap = g.beta != 0.0 ? 0
+                       : (int)std::min<long long>(ws.redo_cap, (long long)Mr * Nr / 16);
+    if (redo) {
+        const long long grid = (long long)cdiv(Mr, 32) * cdiv(Nr, 32);
+        if (grid > INT32_MAX) return cudaErrorInvalidValue;
+        if ((e = cudaMemsetAsync(ws.redo, 0, sizeof(int), s)) != cudaSuccess) return e;
+        launch_chained(k_slices_even, (unsigned)grid, 256, 0, s, slA, slB, Mr, Nr, g.K, eA, eB,
+                       ws.redo, ws.redo_list, redo_cap);
+        count_launches(1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     CUtensorMap mA, mB;
     if ((e = make_map_slices(&mA, slA, ksteps, rowsA, flat ? 1 : nba, BM, 1)) != cudaSuccess) return e;
     if ((e = make_map_slices(&mB, slB, ksteps, Nr, nbb, FN, kSlices)) != cudaSuccess) return e;
@@ -2075,6 +2209,12 @@ cudaError_t gemm_f64_tc_one(const Gemm<double>& g, const F64TcWorkspace& ws, cud
         const unsigned blocks = (unsigned)std::min<long long>((tot + 255) / 256, sms * 16);
         launch_chained(k_f64_splitsum, blocks, 256, 0, s, part, splits, nbo, Mr, Nr, swap ? 1 : 0,
                        g.C, crs, ccs, cbs, g.alpha, g.beta);
+        count_launches(1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (redo) {
+        launch_chained(k_redo64, (unsigned)sms, 256, 0, s, va.p, va.rs, va.cs, vb.p, vb.rs, vb.cs,
+                       g.K, g.alpha, g.C, crs, ccs, ws.redo, ws.redo_list, redo_cap);
         count_launches(1);
         e = cudaGetLastError();
     }

@@ -92,6 +92,14 @@ struct F64TcWorkspace {
     int* expo = nullptr;               // per-row binary exponents
     size_t expo_elems = 0;
     int* err = nullptr;                // bounded-wait expiry flag
+    // Not null (single products only): outputs whose sum_k |a_k b_k| is below the
+    // scale that their slices are cut at, where float64 sums have the smaller
+    // error bound, are done again as such sums.  redo[0] counts those of a piece,
+    // and redo[1] is set to 1 (and never back) if they are too many for that: the
+    // product is then to be done on the CUDA cores.  redo_list holds redo_cap.
+    int* redo = nullptr;
+    int2* redo_list = nullptr;
+    int redo_cap = 0;
 };
 // Workspace one product takes in one piece (part: room for its largest
 // split-K count).
