@@ -281,7 +281,11 @@ __global__ void __launch_bounds__(256) k_chol_solve(const double* S, int W, cons
 
 struct Dev {
     double* p = nullptr;
-    ~Dev() { if (p) cudaFree(p); }
+    ~Dev() { release(); }
+    void release() {
+        if (p) cudaFree(p);
+        p = nullptr;
+    }
     cudaError_t alloc(size_t n) { return cudaMalloc(&p, n * sizeof(double)); }
 };
 
@@ -314,8 +318,8 @@ struct Als {
     }
 
     // Tensor-core products: room for the largest in one piece, at most 2 GiB of
-    // slices (larger ones are cut); without the memory the products stay on the
-    // CUDA cores.
+    // slices and 512 MiB of partial sums (larger ones are cut).  Optional, hence
+    // after everything else: without the memory the products stay on the CUDA cores.
     void init_slices() {
         size_t sl = 0, pt = 0, ex = 0;
         const long long shapes[][3] = {{ov, W, N}, {W, W, N}, {W, W, v}, {W, W, o},
@@ -332,9 +336,11 @@ struct Als {
         }
         if (sl > 0) {
             sl = std::min<size_t>(sl, 1ULL << 30);
+            pt = std::min<size_t>(pt, 1ULL << 27);
             if (slices.alloc(sl / 4 + 1) || fpart.alloc(pt / 2 + 1) || expo.alloc(ex / 2 + 1) ||
                 list.alloc(kRedo)) {
                 cudaGetLastError();   // not enough memory
+                for (Dev* d : {&slices, &fpart, &expo, &list}) d->release();
             } else {
                 tc.slices = reinterpret_cast<__nv_bfloat16*>(slices.p);
                 tc.slice_elems = sl;
@@ -519,7 +525,6 @@ extern "C" thc_status thc_cp_als(int n_occ, int n_vir, int n_rr, int rank, const
     a.ov = (long long)n_occ * n_vir;
     a.st = (cudaStream_t)stream;
     cudaError_t e = a.init();
-    if (!e) a.init_slices();
     // Device copies of the inputs and of the factors (updated in place).
     Dev dU, de, dyo, dyv, dt;
     const size_t nU = (size_t)a.ov * n_rr;
@@ -529,6 +534,7 @@ extern "C" thc_status thc_cp_als(int n_occ, int n_vir, int n_rr, int rank, const
     if (!e) e = dyo.alloc(no);
     if (!e) e = dyv.alloc(nv);
     if (!e) e = dt.alloc(nt);
+    if (!e) a.init_slices();
     if (!e) e = cudaMemcpyAsync(dU.p, U, sizeof(double) * nU, cudaMemcpyDefault, a.st);
     if (!e) e = cudaMemcpyAsync(de.p, eps, sizeof(double) * n_rr, cudaMemcpyDefault, a.st);
     if (!e) e = cudaMemcpyAsync(dyo.p, y_o, sizeof(double) * no, cudaMemcpyDefault, a.st);
