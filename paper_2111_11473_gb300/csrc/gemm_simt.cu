@@ -425,9 +425,10 @@ cudaError_t launch(Gemm<T> g, cudaStream_t s) {
         // Both kernels by the FP64 cycles of the SM (or scheduler) that gets
         // the most: a tile kernel's block takes BM BN / 2 cycles per K index
         // with its padding, a warp of the other 64.  The latter also reads its
-        // operands from L1 and L2: it has to be a tenth better, and half where
-        // the operands are long (400 x 400 x 240000: 138 against 177 million
-        // cycles here, but 10 % slower).
+        // operands from L1 and L2: it has to be a tenth better, and half for
+        // products of 1e9 multiply-adds or more, whose operands are re-read from
+        // L2 (400 x 400 x 240000: 138 against 177 million cycles here, but 10 %
+        // slower; such products fill the SMs with tiles anyway).
         const long long Kt = (long long)g.K * (g.reduce ? g.batch : 1);
         const long long sms = device_sms(), nb = g.reduce ? 1 : g.batch;
         const long long chunk = (ksteps + splits - 1) / splits * BK;

@@ -774,7 +774,7 @@ cudaError_t pack_target(const float* p, long long rs, long long cs, long long bs
     }
     for (const PackCache::Entry& e : cache->entries)
         if (e.p == p && e.rs == rs && e.cs == cs && e.bs == bs && e.R == R && e.Kd == Kd &&
-            e.nb == nb && e.Rp == R && e.Kp == Kp && e.reduce == reduce && e.nprod == nprod) {
+            e.nb == nb && e.Kp == Kp && e.reduce == reduce && e.nprod == nprod) {
             *op = PackOp{};
             op->hi = e.hi;
             op->lo = e.lo;
@@ -788,7 +788,7 @@ cudaError_t pack_target(const float* p, long long rs, long long cs, long long bs
         cudaGetLastError();
         return cudaErrorMemoryAllocation;
     }
-    *made = PackCache::Entry{p, rs, cs, bs, R, Kd, nb, R, Kp, reduce, nprod, buf,
+    *made = PackCache::Entry{p, rs, cs, bs, R, Kd, nb, Kp, reduce, nprod, buf,
                              nprod == 3 ? buf + elems : nullptr};
     *op = pack_op(p, rs, cs, bs, R, Kd, nb_packed, Kp, reduce, made->hi, made->lo);
     return cudaSuccess;
@@ -834,13 +834,13 @@ cudaError_t gemm_tc(const Gemm<float>& g, const TcWorkspace& ws, int nprod, cuda
     const size_t bytesA = needA * 2 * (nprod == 3 ? 2 : 1);
     const size_t bytesB = needB * 2 * (nprod == 3 ? 2 : 1);
     const bool a_cached =
-        cache && cache->serves(va.p, bytesA, va.rs, va.cs, sa, Mr, g.K, nb, Mr, Kp, red, nprod);
+        cache && cache->serves(va.p, bytesA, va.rs, va.cs, sa, Mr, g.K, nb, Kp, red, nprod);
     // B is checked against the budget left after A's (possibly new) entry.
     bool b_cached = false;
     if (cache) {
         const size_t held = cache->bytes;
         if (a_cached) cache->bytes += bytesA;
-        b_cached = cache->serves(vb.p, bytesB, vb.rs, vb.cs, sb, Nr, g.K, nb, Nr, Kp, red, nprod);
+        b_cached = cache->serves(vb.p, bytesB, vb.rs, vb.cs, sb, Nr, g.K, nb, Kp, red, nprod);
         cache->bytes = held;
     }
     const size_t need = (nprod == 3 ? 2 : 1) * ((a_cached ? 0 : needA) + (b_cached ? 0 : needB));
@@ -1430,8 +1430,9 @@ void gemm_f64_tc_sizes(int M, int N, int K, int batch, bool reduce, size_t* slic
 // merged ones average 110), and 40 MMAs are issued per K step.
 // A level is drained before its sum can pass 2^24: (q + 1) pairs x 64 x 2^14
 // per step, every 16, 8, 4, 4 and 2 steps for q = 0 .. 4 (exact); q = 5 and 6
-// weigh 2^-54 and less and are drained every 4 and 8 steps (a sum above 2^24
-// there is rounded by two of its units at most).
+// weigh 2^-54 and 2^-62 and are drained every 4 and 8 steps: digits of one sign
+// near the largest ones take their sums to 1.5 and 3.5 times 2^24, and each MMA
+// beyond 2^24 rounds the sum by one or two units, 2^-57 per term in all.
 // Measured with slicing and exponents (8 unsigned slices, one MMA per pair ->
 // this kernel): 4096^3 5.78 -> 2.65 ms (52 TFLOP/s of float64, 0.77 of the
 // measured bf16 peak on its 28 products), 400 x 400 x 240000 6.54 -> 3.27 ms,
@@ -2410,7 +2411,7 @@ cudaError_t gemm_f64_tc_selftest(int cases, unsigned long long seed, double* max
     al((void**)&simt, cap * 8);
     ws.slice_elems = (size_t)1 << 26;
     al((void**)&ws.slices, ws.slice_elems * 2);
-    ws.part_elems = (size_t)1 << 28;   // the 8 levels of the largest case (about 1.4e8)
+    ws.part_elems = (size_t)64 * cap;   // 32 float64 split-K sums of the largest output
     al((void**)&ws.part, ws.part_elems * 4);
     ws.expo_elems = (size_t)1 << 16;
     al((void**)&ws.expo, ws.expo_elems * 4);

@@ -28,7 +28,7 @@ struct PackCache {
     struct Entry {
         const float* p;
         long long rs, cs, bs;
-        int R, Kd, nb, Rp, Kp, reduce, nprod;
+        int R, Kd, nb, Kp, reduce, nprod;
         __nv_bfloat16* hi;
         __nv_bfloat16* lo;
     };
@@ -44,11 +44,11 @@ struct PackCache {
     }
     // True if this operand is (or, within the budget, will be) cached.
     bool serves(const float* p, size_t packed_bytes, long long rs, long long cs, long long bs,
-                int R, int Kd, int nb, int Rp, int Kp, int reduce, int nprod) const {
+                int R, int Kd, int nb, int Kp, int reduce, int nprod) const {
         if (!is_constant(p)) return false;
         for (const Entry& e : entries)
             if (e.p == p && e.rs == rs && e.cs == cs && e.bs == bs && e.R == R && e.Kd == Kd &&
-                e.nb == nb && e.Rp == Rp && e.Kp == Kp && e.reduce == reduce && e.nprod == nprod)
+                e.nb == nb && e.Kp == Kp && e.reduce == reduce && e.nprod == nprod)
                 return true;
         return bytes + packed_bytes <= budget;
     }

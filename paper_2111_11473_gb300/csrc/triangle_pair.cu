@@ -136,7 +136,7 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 // is read as zero, and zeros are added there in H).
 // Grid: block of QP X pairs (fastest, so that the blocks running together share
 // the G tiles of one mirror pair in L2), pair of mirror tiles (in one
-// dimension: the pairs of P > 11552 exceed the second one's 65535 blocks).
+// dimension: the pairs of P > 5776 exceed the second one's 65535 blocks).
 __global__ void __launch_bounds__(QTH, 2)
     k_triangle_pair(float* H, const __grid_constant__ CUtensorMap tmE,
                     const __grid_constant__ CUtensorMap tmF,
