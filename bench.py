@@ -76,10 +76,10 @@ FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 # kernel over X pairs 2 FMA-pipe lane operations (one packed multiply and three
 # packed FMAs per pair of X and pair of mirror outputs), 3 for the unpaired
 # float32 kernel; float-pair kernel 43 float32 operations per pair of mirror
-# outputs (19 for t, 12 per accumulation).  The float-pair fraction is stated
-# against this count of the TwoSum form at every size; from 512 grid points on
-# the kernel issues 24 packed operations in the place of 40, so that it can
-# come above that form's bound.
+# outputs (19 for t, 12 per accumulation).  The float-pair fractions `frac` and
+# `frac_issued` are stated against this count of the TwoSum form at every size;
+# in launches of 512 grid points or more even tiles issue 24 packed operations
+# per pair of X and of mirror outputs, 12 per term (`frac_issued_bounds`).
 TRI_ISSUED = {"fp64": 3.5, "mixed": 2.0, "fp64tc": 21.5}
 TRI_KERNEL = {"fp64": "k_triangle_sym64", "mixed": "k_triangle_pair", "fp64tc": "k_triangle_df"}
 
@@ -90,10 +90,12 @@ def _mixed_triangle_unpaired():
     return WORKLOAD is not None and not (WORKLOAD["P"] % 4 == 0 and WORKLOAD["P"] <= 28000)
 
 # DRAM bytes (read + write) of one triangle launch at o=40, v=200, P=400,
-# G=1200, from one ncu capture (fp64 and mixed: of the 32-wide tiles used
-# before; the 16-wide tiles of the mixed kernel read and write 22.5e9).
-TRIANGLE_TRAFFIC_BYTES = {"fp64": 97.58e9 + 0.52e9, "fp64tc": 65.397e9 + 0.514e9,
+# G=1200, from one ncu capture (fp64 and mixed: of kernels with 32-wide tiles;
+# TRIANGLE_TRAFFIC_NOW has the mixed kernel's 16-wide ones).
+TRIANGLE_TRAFFIC_BYTES = {"fp64": 97.58e9 + 0.52e9, "fp64tc": 57.670e9 + 0.514e9,
                           "mixed": 12.702e9 + 0.249e9}
+TRIANGLE_TRAFFIC_NOW = {"mixed": 22.41e9 + 0.253e9}
+BOUNDS_POINTS, BOUNDS_ISSUED = 512, 12.0
 
 
 def triangle_roofline(precision, flops, ms, launches, share):
@@ -118,20 +120,27 @@ def triangle_roofline(precision, flops, ms, launches, share):
            "bound": "alu", "achieved": achieved, "unit": "TFLOP/s",
            "achieved_counts": "algorithmic flops, 5 per (I, X, Y, Z) term",
            "frac_issued": issued / pipe,
-           "frac_issued_counts": "operations the kernel issues per term (%g) / pipe rate"
-                                 % n_issued,
+           "frac_issued_counts": "operations the kernel issues per term (%g%s) / pipe rate"
+                                 % (n_issued, ", its TwoSum form" if precision == "fp64tc" else ""),
            "frac_algorithmic": achieved / unit_peak,
            "frac_algorithmic_peak": unit_peak,
            "traffic": TRIANGLE_TRAFFIC_BYTES[precision] if WORKLOAD_NAME.startswith(
                "THC-RR-CCSD o=40 v=200 P=400 G=1200") else None,
-           "traffic_unit": "bytes per launch (ncu dram__bytes_read + write)",
+           "traffic_unit": "bytes per launch (ncu dram__bytes_read + write%s)"
+                           % ("" if precision == "fp64tc" else "; of 32-wide tiles"),
            "share_of_step": share}
+    if out["traffic"] is not None and precision in TRIANGLE_TRAFFIC_NOW:
+        out["traffic_now"] = TRIANGLE_TRAFFIC_NOW[precision]
     if precision == "fp64tc":
         # float64 result from float32 pairs: the bound is the FP32 pipe at
         # 21.5 operations per term
         out.update({"peak": peak, "frac": achieved / peak,
                     "peak_source": src + "; / 21.5 float32 operations per term x 5 flops",
                     "frac_of_fp64_alu_peak": achieved / FP64_ALU_TFLOPS})
+        if flops / launches >= 5.0 * BOUNDS_POINTS * WORKLOAD["P"] ** 3:
+            out["frac_issued_bounds"] = terms_per_s * BOUNDS_ISSUED / pipe
+            out["frac_issued_bounds_counts"] = ("operations of the sums with bounds per term (%g), "
+                                                "which even tiles take" % BOUNDS_ISSUED)
     else:
         out.update({"peak": unit_peak, "frac": achieved / unit_peak, "peak_source": src})
     return out
